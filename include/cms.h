@@ -149,16 +149,18 @@ CMS_API cms_status cms_hashes_buckets(const cms_hashes* h, int32_t t, int32_t si
 
 /*
  * cms_workspace_size - bytes of device workspace cms_sketch_product needs
- * for these shapes (A n1 x n2, B n2 x n3, storage dtype dt).  Host output.
+ * for these shapes (A n1 x n2, B n2 x n3, storage dtype dt), the larger of
+ * its two routes'.  Host output.
  * Errors: CMS_ERR_INVALID_ARG, CMS_ERR_UNSUPPORTED.
  */
 CMS_API cms_status cms_workspace_size(const cms_hashes* h, int64_t n1, int64_t n2,
                               int64_t n3, int32_t dt, size_t* bytes);
 
 /*
- * cms_plan_kernel - which fused kernel cms_sketch_product would run for
- * these arguments (the choice depends on b, n, the storage type, the
- * alignment of A and B and whether they alias), without running it:
+ * cms_plan_kernel - which fused kernel the transform route of
+ * cms_sketch_product would run for these arguments (the choice depends on b,
+ * n, the storage type, the alignment of A and B and whether they alias),
+ * without running it:
  *   CMS_KERNEL_SHARED_MEMORY      shared-memory Stockham FFTs (any 5-smooth b)
  *   CMS_KERNEL_LOCKSTEP           register FFTs, C = P Q, records in shared memory
  *   CMS_KERNEL_LOCKSTEP_TMEM      the same with the records in tensor memory
@@ -182,9 +184,16 @@ CMS_API cms_status cms_plan_kernel(const void* A, int64_t lda, const void* B, in
  * cms_sketch_product - COMPRESSEDPRODUCT(A, B, b, d) of Fig. 1 (Lemma 1):
  *   c[t][z] = sum over (i,j) with (h1_t(i)+h2_t(j)) mod b = z of
  *             s1_t(i) s2_t(j) (AB)_ij,
- * computed as in Sec. 2.2: per inner index k, count-sketch column k of A and
- * row k of B, FFT both, multiply pointwise and accumulate over k
- * (compensated FP32), then one inverse FFT per repetition.
+ * by the cheaper of two routes (an estimate from the sizes):
+ *   transform  as in Sec. 2.2: per inner index k, count-sketch column k of A
+ *              and row k of B, FFT both, multiply pointwise and accumulate
+ *              over k (compensated FP32), then one inverse FFT per repetition;
+ *   direct     where b is not much smaller than n1 n3: the entries of AB
+ *              from tensor-core tiles, each added to its bucket of every
+ *              repetition as the tile leaves the accumulators (integer sums,
+ *              so their order does not matter); AB is not stored.
+ * Either gives the same bits in every run.  An infinity or a NaN in A or B
+ * makes c NaN.
  *   A   : n1 x n2, column-major, column k at A + k*lda (lda >= n1), so a
  *         single pass reads each a_k contiguously (Sec. 2.2, "single pass").
  *   B   : n2 x n3, row-major, row k at B + k*ldb (ldb >= n3).
@@ -192,7 +201,8 @@ CMS_API cms_status cms_plan_kernel(const void* A, int64_t lda, const void* B, in
  *   h   : hashes with n >= max(n1, n3).
  *   c   : device float [d][b], written (not accumulated).
  *   ws  : device workspace of at least cms_workspace_size() bytes,
- *         256-byte aligned.
+ *         256-byte aligned (one that holds only the transform route's share
+ *         is accepted and selects that route).
  * Errors: CMS_ERR_INVALID_ARG, CMS_ERR_UNSUPPORTED (b not 5-smooth or shape
  * beyond the kernels' limits), CMS_ERR_WORKSPACE, CMS_ERR_CUDA.
  */
@@ -211,9 +221,9 @@ CMS_API cms_status cms_sketch_product(const void* A, int64_t lda, const void* B,
  *   Arguments are those of cms_sketch_product without ws / ws_bytes; the
  *   caller still passes A, B, the hashes and the output c.
  *   Scratch: a fixed 32 MiB device array owned by the library (held on every
- *   GPU that loads it until the process exits).  Shapes whose
- *   cms_workspace_size() exceeds 32 MiB are rejected with CMS_ERR_WORKSPACE
- *   (the covariance shape n = 2048, b = 65536, d = 5 needs about 18 MiB).
+ *   GPU that loads it until the process exits).  The direct route runs where
+ *   its layout fits in it; shapes whose transform route needs more than
+ *   32 MiB as well are rejected with CMS_ERR_WORKSPACE (the covariance shape n = 2048, b = 65536, d = 5 needs about 18 MiB).
  *   The call allocates nothing.  Its first call on a device looks up the
  *   array's device address (cudaGetSymbolAddress) with that device current;
  *   make that first call before any stream capture.  The address is cached
@@ -317,8 +327,9 @@ typedef struct cms_batch cms_batch;
  * on `stream`).  With flags & CMS_BATCH_AUTOTUNE, shapes not found in the
  * cache file `tune_cache` (may be NULL) are tuned by timing candidate
  * inner-index chunkings (and group sizes of the generic kernel) on the
- * instance's own data; results are written back to the file, one line per
- * key "b,n1,n2,n3,dt,d,SM count,kernel".
+ * instance's own data (for an instance on the direct route, that route
+ * against the transform route); results are written back to the file, one
+ * line per key "b,n1,n2,n3,dt,d,SM count,kernel".
  * The instances' pointers are captured: the same buffers are used by every
  * run.  Errors: CMS_ERR_INVALID_ARG, CMS_ERR_UNSUPPORTED, CMS_ERR_CUDA.
  */
@@ -326,8 +337,9 @@ CMS_API cms_status cms_batch_create(const cms_instance* items, int32_t count, in
                                     const char* tune_cache, void* stream, cms_batch** out);
 
 /*
- * cms_batch_run - compute every instance's sketch c: one persistent kernel
- * over all instances' tasks (longest first, taken from an atomic work
+ * cms_batch_run - compute every instance's sketch c: the instances that the
+ * direct route serves in two launches (packing, tiles), the others in one
+ * persistent kernel over all their tasks (longest first, taken from an atomic work
  * counter; each task writes only its own partial row, so results do not
  * depend on scheduling), then the fixed-order reduction and inverse FFT of
  * every instance in two launches (rows, then columns).  Asynchronous,

@@ -370,8 +370,12 @@ cms_status cms_workspace_size(const cms_hashes* h, int64_t n1, int64_t n2, int64
       r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &alias, &why, same, ld, same, ld);
       if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
       *bytes = std::max(*bytes, alias.ws_bytes);
+      DirectPlan direct;
+      if (choose_direct(h, alias, n1, n2, n3, dt, true, dp.sms, &direct)) *bytes = std::max(*bytes, direct.ws_bytes);
     }
   }
+  DirectPlan direct;
+  if (choose_direct(h, plan, n1, n2, n3, dt, false, dp.sms, &direct)) *bytes = std::max(*bytes, direct.ws_bytes);
   return CMS_OK;
 }
 
@@ -404,10 +408,19 @@ cms_status cms_sketch_product(const void* A, int64_t lda, const void* B, int64_t
   std::string why;
   int r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &plan, &why, A, lda, B, ldb);
   if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
-  if (!ws || ws_bytes < plan.ws_bytes)
+  DirectPlan direct;
+  const bool use = choose_direct(h, plan, n1, n2, n3, dt, A == B && lda == ldb && n1 == n3, dp.sms, &direct) &&
+                   ws_bytes >= direct.ws_bytes;
+  if (!ws || ws_bytes < (use ? direct.ws_bytes : plan.ws_bytes))
     return fail(CMS_ERR_WORKSPACE, "workspace missing or smaller than cms_workspace_size()");
   if (reinterpret_cast<uintptr_t>(ws) % 256 != 0)
     return fail(CMS_ERR_WORKSPACE, "workspace must be 256-byte aligned");
+  if (use) {
+    cudaError_t e = launch_direct(direct, h, A, lda, B, ldb, n1, n2, n3, dt, c, static_cast<char*>(ws),
+                                  static_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "cms_sketch_product");
+    return CMS_OK;
+  }
   cudaError_t e = launch_sketch(plan, h, A, lda, B, ldb, n1, n2, n3, dt, c, static_cast<char*>(ws),
                                 static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "cms_sketch_product");
@@ -812,8 +825,11 @@ cms_status cms_find_significant(const void* A, int64_t lda, const void* B, int64
     std::string why;
     int rc = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &plan, &why, Ao, la, Bo, lb);
     if (rc != CMS_OK) return fail(static_cast<cms_status>(rc), why);
-    if (plan.ws_bytes > L.mask - L.sk) return fail(CMS_ERR_WORKSPACE, "internal: sketch scratch too small");
-    e = launch_sketch(plan, h, Ao, la, Bo, lb, n1, n2, n3, dt, P + r * per, w + L.sk, s);
+    DirectPlan direct;
+    const bool use = choose_direct(h, plan, n1, n2, n3, dt, false, dp.sms, &direct) && direct.ws_bytes <= L.mask - L.sk;
+    if (!use && plan.ws_bytes > L.mask - L.sk) return fail(CMS_ERR_WORKSPACE, "internal: sketch scratch too small");
+    e = use ? launch_direct(direct, h, Ao, la, Bo, lb, n1, n2, n3, dt, P + r * per, w + L.sk, s)
+            : launch_sketch(plan, h, Ao, la, Bo, lb, n1, n2, n3, dt, P + r * per, w + L.sk, s);
     if (e != cudaSuccess) return cuda_fail(e, "cms_find_significant (sketch)");
   }
   cudaError_t e = launch_decode_significant(P, h, n1, n3, delta, rho, ij_out, capacity, count_out, w + L.dec, s);
@@ -849,8 +865,9 @@ cms_status cms_check_async(void* stream) {
   const uint32_t ws1 = read_clear_error_sketch();
   const uint32_t ws2 = read_clear_error_sketch_ws();
   const uint32_t ws3 = read_clear_error_sketch_wide();
-  const uint32_t ws = ws1 | ws2 | ws3;
-  if (w == 0xFFFFFFFFu || ws1 == 0xFFFFFFFFu || ws2 == 0xFFFFFFFFu || ws3 == 0xFFFFFFFFu)
+  const uint32_t ws4 = read_clear_error_direct();
+  const uint32_t ws = ws1 | ws2 | ws3 | ws4;
+  if (w == 0xFFFFFFFFu || ws1 == 0xFFFFFFFFu || ws2 == 0xFFFFFFFFu || ws3 == 0xFFFFFFFFu || ws4 == 0xFFFFFFFFu)
     return fail(CMS_ERR_CUDA, "could not read the device error words");
   if (ws) return fail(CMS_ERR_TIMEOUT, "a fused-kernel wait for its TMA copies gave up");
   if (w) return fail(CMS_ERR_DEVICE, "decode saw an index pair outside the hash domain");

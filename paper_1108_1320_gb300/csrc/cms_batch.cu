@@ -10,6 +10,8 @@
 //   * ONE persistent kernel over the tasks of every instance (longest
 //     first), and
 //   * per instance, the fixed-order reduction and inverse FFT.
+// Instances that the direct route serves (k_direct.cu) have no tasks there:
+// their packing and their tiles are one launch each for all of them.
 // cms_batch_run_graph captures that sequence once in a CUDA graph and
 // replays it.
 #include <atomic>
@@ -31,6 +33,10 @@ struct cms_batch {
   int device = 0;
   std::vector<cms_instance> items;
   std::vector<cms::SketchPlan> plans;
+  std::vector<cms::DirectPlan> direct;   // used where is_direct
+  std::vector<char> is_direct;
+  void* d_direct = nullptr;         // arguments of the direct launches
+  cms::DirectBatch direct_batch;
   std::vector<size_t> ws_off;       // workspace offset of each instance
   std::vector<int> order;           // instance order in the persistent launch
   char* ws = nullptr;
@@ -39,6 +45,7 @@ struct cms_batch {
   int* d_start = nullptr;
   int* d_next = nullptr;
   int total_tasks = 0;
+  int transform_tasks = 0;          // of the persistent kernel
   size_t smem = 0;
   int grid = 0;
   int launches = 0;
@@ -55,10 +62,10 @@ namespace {
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
-std::string tune_key(const cms_instance& it, const SketchPlan& p, int sms) {
+std::string tune_key(const cms_instance& it, const SketchPlan& p, int sms, bool direct = false) {
   std::ostringstream k;
   k << "b=" << p.b << ",n1=" << it.n1 << ",n2=" << it.n2 << ",n3=" << it.n3 << ",dt=" << it.dt
-    << ",d=" << p.d << ",sms=" << sms << ",kernel=" << (p.fast ? "fast" : "generic")
+    << ",d=" << p.d << ",sms=" << sms << ",kernel=" << (direct ? "direct" : p.fast ? "fast" : "generic")
     << (p.alias ? "-alias" : "");
   return k.str();
 }
@@ -129,16 +136,20 @@ cms_status cuda_fail(cudaError_t e, const char* where) {
   return CMS_ERR_CUDA;
 }
 
-// Time one configuration of one instance with the single-instance launch.
-cudaError_t time_plan(const SketchPlan& p, const cms_instance& it, char* ws, cudaStream_t s, double* ms) {
+// Time one configuration of one instance with the single-instance launch
+// (on the direct route when `direct` is given).
+cudaError_t time_plan(const SketchPlan& p, const cms_instance& it, char* ws, cudaStream_t s, double* ms,
+                      const DirectPlan* direct = nullptr) {
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
-  if (e == cudaSuccess)
-    e = launch_sketch(p, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, it.c, ws, s);  // warm-up
+  auto once = [&]() {
+    return direct ? launch_direct(*direct, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, it.c, ws, s)
+                  : launch_sketch(p, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, it.c, ws, s);
+  };
+  if (e == cudaSuccess) e = once();  // warm-up
   if (e == cudaSuccess) e = cudaEventRecord(a, s);
-  for (int r = 0; r < 2 && e == cudaSuccess; ++r)
-    e = launch_sketch(p, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, it.c, ws, s);
+  for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = once();
   if (e == cudaSuccess) e = cudaEventRecord(b, s);
   if (e == cudaSuccess) e = cudaEventSynchronize(b);
   float t = 0.f;
@@ -157,6 +168,8 @@ void release(cms_batch* b) {
   if (b->d_start) cudaFree(b->d_start);
   if (b->d_next) cudaFree(b->d_next);
   if (b->d_inv) cudaFree(b->d_inv);
+  if (b->d_direct) cudaFree(b->d_direct);
+  b->d_direct = nullptr;
   b->d_inv = nullptr;
   b->exec = nullptr;
   b->graph = nullptr;
@@ -183,10 +196,13 @@ double instance_work(const cms_instance& it) {
 }
 
 // Chunks of instance `it` (planned as p) under the batch budget: tasks in
-// proportion to its share of the batch's work, at least one per unit.
-int batch_chunks(const cms_instance& it, const SketchPlan& p, const cms_instance* items, int count, int sms) {
+// proportion to its share of the transform route's work, at least one per
+// unit.
+int batch_chunks(const cms_instance& it, const SketchPlan& p, const cms_instance* items,
+                 const std::vector<char>& skip, int count, int sms) {
   double total = 0.0;
-  for (int i = 0; i < count; ++i) total += instance_work(items[i]);
+  for (int i = 0; i < count; ++i)
+    if (!skip[i]) total += instance_work(items[i]);
   if (!(total > 0.0)) return 0;
   const double units = static_cast<double>(p.d) * (p.fast ? (p.nrows + 1) / 2 : p.nrows);
   const double tasks = static_cast<double>(kBatchWaves) * sms * instance_work(it) / total;
@@ -207,6 +223,8 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
   b->items.assign(items, items + count);
   b->plans.resize(count);
   b->ws_off.resize(count);
+  b->direct.resize(count);
+  b->is_direct.assign(count, 0);
   std::string why;
   // ---- plan every instance (tuned shapes come from the cache) ------------
   std::map<std::string, Tuned> cache = load_cache(tune_cache);
@@ -226,13 +244,39 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
     int r = make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &p, &why, it.A, it.lda, it.B, it.ldb,
                              true, 0, 0, false, false);
     if (r != CMS_OK) { delete b; return fail(static_cast<cms_status>(r), "instance " + std::to_string(i) + ": " + why); }
+    b->is_direct[i] = choose_direct(it.h, p, it.n1, it.n2, it.n3, it.dt,
+                                    it.A == it.B && it.lda == it.ldb && it.n1 == it.n3, sms, &b->direct[i]) ? 1 : 0;
+    b->plans[i] = p;
+    if (!b->is_direct[i]) continue;
+    // the direct route has no tiles to tune: the cache holds whether it was
+    // the faster route (nkc = 0), else the transform route's chunks
+    auto hit = cache.find(tune_key(it, p, sms, true));
+    if (hit != cache.end()) {
+      b->is_direct[i] = hit->second.nkc == 0;
+    } else if (flags & CMS_BATCH_AUTOTUNE) {
+      char* tws = nullptr;
+      cudaError_t e = cudaMalloc(&tws, std::max<size_t>(std::max(p.ws_bytes, b->direct[i].ws_bytes), 256));
+      double td = 0.0, tt = 0.0;
+      if (e == cudaSuccess) e = time_plan(p, it, tws, s, &td, &b->direct[i]);
+      if (e == cudaSuccess) e = time_plan(p, it, tws, s, &tt);
+      if (tws) cudaFree(tws);
+      if (e != cudaSuccess) { delete b; return cuda_fail(e, "cms_batch_create (autotune)"); }
+      b->is_direct[i] = td <= tt;
+      cache[tune_key(it, p, sms, true)] = Tuned{td <= tt ? 0 : p.nkc, 0, std::min(td, tt)};
+      cache_dirty = true;
+    }
+  }
+  for (int i = 0; i < count; ++i) {
+    if (b->is_direct[i]) continue;
+    const cms_instance& it = items[i];
+    SketchPlan p = b->plans[i];
     // k-chunking for the batch as a whole: each instance gets tasks in
     // proportion to its work out of a budget of kBatchWaves waves over the
     // SMs (the planner alone would split every instance to fill the GPU by
     // itself: many short tasks, each repeating its prologue and writing a
     // partial row)
     {
-      const int nkc = batch_chunks(it, p, items, count, sms);
+      const int nkc = batch_chunks(it, p, items, b->is_direct, count, sms);
       SketchPlan q;
       if (nkc > 0 && make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &q, &why, it.A, it.lda, it.B,
                                       it.ldb, true, nkc, 0, false, false) == CMS_OK)
@@ -284,7 +328,7 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
   size_t off = 0;
   for (int i = 0; i < count; ++i) {
     b->ws_off[i] = off;
-    off = align256(off + b->plans[i].ws_bytes);
+    off = align256(off + (b->is_direct[i] ? b->direct[i].ws_bytes : b->plans[i].ws_bytes));
   }
   b->ws_bytes = off;
   cudaError_t e = cudaMalloc(&b->ws, std::max<size_t>(off, 256));
@@ -297,13 +341,16 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
     const double per_k = static_cast<double>(p.C) * (p.fast ? 2.0 : 1.0);
     return per_k * static_cast<double>(p.kchunk) * (p.fast ? 0.2 : 1.0);
   };
+  b->order.erase(std::remove_if(b->order.begin(), b->order.end(), [&](int i) { return b->is_direct[i] != 0; }),
+                 b->order.end());
+  const int ntr = static_cast<int>(b->order.size());   // instances of the persistent kernel
   std::stable_sort(b->order.begin(), b->order.end(), [&](int x, int y) { return cost(x) > cost(y); });
   const size_t dsz = batch_desc_bytes();
-  std::vector<unsigned char> desc(dsz * count);
-  std::vector<int> start(count);
+  std::vector<unsigned char> desc(dsz * std::max(ntr, 1));
+  std::vector<int> start(std::max(ntr, 1));
   int total = 0;
   size_t smem = 0;
-  for (int q = 0; q < count; ++q) {
+  for (int q = 0; q < ntr; ++q) {
     const int i = b->order[q];
     const cms_instance& it = items[i];
     const SketchPlan& p = b->plans[i];
@@ -314,22 +361,24 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
     smem = std::max(smem, p.smem);
   }
   b->total_tasks = total;
+  b->transform_tasks = total;
   b->use_tmem = 0;
-  for (const auto& p : b->plans) b->use_tmem |= (p.fast && p.tmem_rec) ? 1 : 0;
+  for (int i : b->order) b->use_tmem |= (b->plans[i].fast && b->plans[i].tmem_rec) ? 1 : 0;
   if (b->use_tmem) smem = std::max(smem, kSmemOneBlockPerSm);
   b->smem = smem;
   b->grid = std::max(1, std::min(total, sms));
   if ((e = cudaMalloc(&b->d_desc, desc.size())) != cudaSuccess ||
-      (e = cudaMalloc(reinterpret_cast<void**>(&b->d_start), sizeof(int) * count)) != cudaSuccess ||
+      (e = cudaMalloc(reinterpret_cast<void**>(&b->d_start), sizeof(int) * start.size())) != cudaSuccess ||
       (e = cudaMalloc(reinterpret_cast<void**>(&b->d_next), sizeof(int))) != cudaSuccess ||
       (e = cudaMemcpy(b->d_desc, desc.data(), desc.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(b->d_start, start.data(), sizeof(int) * count, cudaMemcpyHostToDevice)) != cudaSuccess) {
+      (e = cudaMemcpy(b->d_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
     release(b);
     delete b;
     return cuda_fail(e, "cms_batch_create (descriptors)");
   }
   // constant twiddle tables of every instance
   for (int i = 0; i < count && e == cudaSuccess; ++i) {
+    if (b->is_direct[i]) continue;
     const SketchPlan& p = b->plans[i];
     char* w = b->ws + b->ws_off[i];
     e = launch_twiddle_tables(reinterpret_cast<float2*>(w + p.off_twC), static_cast<int>(p.C),
@@ -343,7 +392,14 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
     for (int i = 0; i < count; ++i) {
       const SketchPlan& p = b->plans[i];
       char* w = b->ws + b->ws_off[i];
-      specs[i] = InverseSpec{&p, reinterpret_cast<const float2*>(w + p.off_partial),
+      if (b->is_direct[i]) {
+        const DirectPlan& dp = b->direct[i];
+        specs[i] = InverseSpec{reinterpret_cast<unsigned long long*>(w + dp.off_acc),
+                               reinterpret_cast<const DirectScale*>(w + dp.off_scale), direct_scale_log2(dp.split),
+                               &p, nullptr, nullptr, nullptr, nullptr, items[i].c};
+        continue;
+      }
+      specs[i] = InverseSpec{nullptr, nullptr, 0, &p, reinterpret_cast<const float2*>(w + p.off_partial),
                              reinterpret_cast<float2*>(w + p.off_V), reinterpret_cast<const float2*>(w + p.off_twC),
                              reinterpret_cast<const float2*>(w + p.off_twR), items[i].c};
     }
@@ -351,8 +407,29 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
     if (e == cudaSuccess) e = build_inverse_batch(specs, b->d_inv, &b->inv, s);
     if (e != cudaSuccess) { release(b); delete b; return cuda_fail(e, "cms_batch_create (inverse arguments)"); }
   }
-  int launches = 2 + 2;   // counter reset + persistent kernel + batched inverse (rows, columns)
-  for (int i = 0; i < count; ++i) launches += b->plans[i].fast ? 0 : 1;
+  // the direct instances' packing and tiles, the longest tiles first
+  {
+    std::vector<int> ord;
+    for (int i = 0; i < count; ++i)
+      if (b->is_direct[i]) ord.push_back(i);
+    auto tile_cost = [&](int i) { return b->direct[i].sb_per_split * (b->direct[i].split ? 3 : 1); };
+    std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return tile_cost(x) > tile_cost(y); });
+    std::vector<DirectSpec> specs;
+    for (int i : ord) {
+      const cms_instance& it = items[i];
+      specs.push_back(DirectSpec{b->direct[i], it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt,
+                                 b->ws + b->ws_off[i]});
+    }
+    if (!specs.empty()) {
+      e = cudaMalloc(&b->d_direct, direct_batch_bytes(static_cast<int>(specs.size())));
+      if (e == cudaSuccess) e = build_direct_batch(specs, b->d_direct, &b->direct_batch, s);
+      if (e != cudaSuccess) { release(b); delete b; return cuda_fail(e, "cms_batch_create (direct arguments)"); }
+    }
+    b->total_tasks += b->direct_batch.tile_blocks;
+  }
+  // counter reset + persistent kernel, packing + tiles, batched inverse (rows, columns)
+  int launches = (ntr > 0 ? 2 : 0) + (ntr < count ? 2 : 0) + 2;
+  for (int i : b->order) launches += b->plans[i].fast ? 0 : 1;
   b->launches = launches;
   *out = b;
   return CMS_OK;
@@ -364,9 +441,10 @@ cms_status cms_batch_run(cms_batch* b, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
   for (size_t i = 0; i < b->items.size() && e == cudaSuccess; ++i)
-    if (!b->plans[i].fast) e = launch_frontend_twiddles(b->plans[i], b->items[i].h, b->ws + b->ws_off[i], s);
-  if (e == cudaSuccess)
-    e = launch_sketch_batched(b->d_desc, b->d_start, static_cast<int>(b->items.size()), b->total_tasks,
+    if (!b->is_direct[i] && !b->plans[i].fast) e = launch_frontend_twiddles(b->plans[i], b->items[i].h, b->ws + b->ws_off[i], s);
+  if (e == cudaSuccess) e = launch_direct_batched(b->direct_batch, s);
+  if (e == cudaSuccess && b->transform_tasks > 0)
+    e = launch_sketch_batched(b->d_desc, b->d_start, static_cast<int>(b->order.size()), b->transform_tasks,
                               b->d_next, b->smem, b->grid, b->use_tmem, s);
   if (e == cudaSuccess) e = launch_inverse_batched(b->inv, s);
   if (e != cudaSuccess) return cuda_fail(e, "cms_batch_run");

@@ -210,8 +210,14 @@ cudaError_t launch_inverse(const SketchPlan& plan, const float2* partial, float2
 cudaError_t launch_twiddle_tables(float2* twC, int C, float2* twR, int R, cudaStream_t s);
 
 // Reduction + inverse of many products in two launches (a batch): each
-// instance's plan, partial rows, row spectra, twiddle tables and output.
+// instance's plan, partial rows, row spectra, twiddle tables and output; for
+// a product on the direct route (sums != NULL) its integer sums and their
+// scale, converted by the column launch.
+struct DirectScale;
 struct InverseSpec {
+  unsigned long long* sums;
+  const DirectScale* scale;
+  int log2s;
   const SketchPlan* plan;
   const float2* partial;
   float2* V;
@@ -295,6 +301,68 @@ cudaError_t launch_frobenius(const void* A, int64_t lda, const void* B, int64_t 
                              cudaStream_t s);
 cudaError_t launch_merge(const float* const* parts, int count, int64_t len,
                          float* out, cudaStream_t s);
+
+// The sketch from the product's entries (k_direct.cu).
+struct DirectPlan {
+  bool split = false;       // FP32 (or FP64) storage: two FP16 terms per value
+  bool alias = false;       // A = X^T, B = X: tiles on and above the diagonal
+  int tiles1 = 0, tiles3 = 0, nsb = 0, splits = 1, sb_per_split = 1, slots = 0;
+  int64_t tiles = 0;
+  double seconds = 0.0;     // estimate
+  size_t zero_bytes = 0, off_fold = 0;
+  size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_pa = 0, off_pb = 0;
+  size_t ws_bytes = 0;
+};
+DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms);
+// Whether the direct route serves the call (and its plan): beside the
+// transform route's plan, which stays the one that decides what is accepted.
+bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias,
+                   int sms, DirectPlan* out);
+cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
+                          int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws,
+                          cudaStream_t s);
+uint32_t read_clear_error_direct();
+
+// What the direct route's tiles and conversion need of the whole operands.
+struct DirectScale {
+  int emax[2];       // largest block exponent of each side
+  int shift;         // buckets are sums of round(entry * 2^shift), entry in scaled units
+  int bad;           // an infinity or a NaN somewhere
+};
+// FP32 (and FP64) sources carry their values scaled to below 2^15 (FP16's
+// range), BF16 ones to below 2.
+__host__ __device__ constexpr int direct_scale_log2(bool split) { return split ? 14 : 0; }
+#ifdef __CUDACC__
+// A bucket from its integer sum.
+__device__ __forceinline__ float direct_value(unsigned long long sum, const DirectScale& sc, int log2s) {
+  if (sc.bad) return __int_as_float(0x7FC00000);
+  return ldexpf(__ll2float_rn(static_cast<long long>(sum)), sc.emax[0] + sc.emax[1] - 2 * log2s - sc.shift);
+}
+#endif
+
+// Direct products of a batch: packing and tiles of all of them in two
+// launches.  The sums of each product's workspace are zero before a run; the
+// batch's conversion (k_cols_inverse_batched) leaves them zero.
+struct DirectSpec {
+  DirectPlan plan;
+  const cms_hashes* h;
+  const void* A;
+  int64_t lda;
+  const void* B;
+  int64_t ldb;
+  int64_t n1, n2, n3;
+  int dt;
+  char* ws;
+};
+struct DirectBatch {
+  void* buf = nullptr;
+  int count = 0, pack_blocks = 0, tile_blocks = 0;
+  uint32_t pack_smem = 0;
+  size_t o_tile = 0, o_ps = 0, o_ts = 0;
+};
+size_t direct_batch_bytes(int count);
+cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, void* d_buf, DirectBatch* out, cudaStream_t s);
+cudaError_t launch_direct_batched(const DirectBatch& d, cudaStream_t s);
 
 // Plain FP64 path.
 struct PlainPlan {

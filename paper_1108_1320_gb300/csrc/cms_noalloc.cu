@@ -78,7 +78,10 @@ cms_status cms_sketch_product_noalloc(const void* A, int64_t lda, const void* B,
                                  optin > 0 ? static_cast<size_t>(optin) : 48 * 1024, &plan, &why,
                                  A, lda, B, ldb);
   if (r != CMS_OK) { set_error(why); return static_cast<cms_status>(r); }
-  if (plan.ws_bytes > kNoallocScratchBytes) {
+  DirectPlan direct;
+  const bool use = choose_direct(h, plan, n1, n2, n3, dt, A == B && lda == ldb && n1 == n3, sms > 0 ? sms : 1, &direct) &&
+                   direct.ws_bytes <= kNoallocScratchBytes;
+  if (!use && plan.ws_bytes > kNoallocScratchBytes) {
     set_error("cms_sketch_product_noalloc: this shape needs " + std::to_string(plan.ws_bytes) +
               " bytes of scratch, above the fixed " + std::to_string(kNoallocScratchBytes) +
               "-byte array; use cms_sketch_product with a workspace");
@@ -90,8 +93,10 @@ cms_status cms_sketch_product_noalloc(const void* A, int64_t lda, const void* B,
     set_error(std::string("cudaGetSymbolAddress(scratch): ") + cudaGetErrorString(e));
     return CMS_ERR_CUDA;
   }
-  e = launch_sketch(plan, h, A, lda, B, ldb, n1, n2, n3, dt, c, static_cast<char*>(scratch),
-                    static_cast<cudaStream_t>(stream));
+  e = use ? launch_direct(direct, h, A, lda, B, ldb, n1, n2, n3, dt, c, static_cast<char*>(scratch),
+                          static_cast<cudaStream_t>(stream))
+          : launch_sketch(plan, h, A, lda, B, ldb, n1, n2, n3, dt, c, static_cast<char*>(scratch),
+                          static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) {
     set_error(std::string("cms_sketch_product_noalloc: ") + cudaGetErrorString(e));
     return CMS_ERR_CUDA;

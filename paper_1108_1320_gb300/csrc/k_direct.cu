@@ -1,0 +1,831 @@
+// k_direct.cu - the sketch from the product's entries, for sketches that are
+// long beside n1 n3: tensor-core tiles of AB whose entries are added to the
+// buckets (h1(i) + h2(j)) mod b of every repetition as they leave the
+// accumulators.  AB itself is never stored.
+//
+// Sec. 2.2 forms c from the spectra of the columns of A and rows of B, d n2
+// transforms of length b.  By the same identity c_t[z] is the signed sum of
+// the entries of AB whose key is z, which takes n1 n2 n3 multiply-adds on the
+// tensor cores and d n1 n3 additions into c.  Where b is not much smaller
+// than n1 n3 this is by far the cheaper side of the identity.
+//
+//  * k_direct_pack lays A (B) out once per call as K-major tiles of 128 rows
+//    in the 128-byte swizzle that tcgen05.mma reads, so that a stage of the
+//    product is one contiguous 16 KB bulk copy per operand, whatever the
+//    caller's leading dimension and alignment.  FP32 values (and FP64 values
+//    rounded to FP32) are split in two FP16 terms, v = hi + lo to 2^-23 of v
+//    or 2^-40 of the largest value of the 128 x 128 block, after a scaling of
+//    the block by a power of two; BF16 values are exact.
+//    Its last block bounds every bucket (Cauchy-Schwarz) and fixes the grid
+//    of the integer sums.
+//  * k_direct_tile: one 128 x 128 tile of AB per block, two blocks per SM.
+//    The FP32 sums of the tensor cores over kSuper inner indices are added in
+//    registers (round to nearest), then scaled to 64-bit integers and added
+//    to the buckets with integer reductions: the order of the additions does
+//    not matter, so the sketch is the same in every run.
+//  * k_direct_finish converts the sums to FP32.
+//
+// Measured on one GB300 (whole calls, transform route -> this one): X^T X of
+// 4096 x 2048 FP32, b = 2^16, d = 5 with its hash draw and dense decode 2.93
+// -> 0.40 ms; 8192 x 4096 BF16, b = 2^16, d = 3 7.54 -> 0.45 ms; 16384 x
+// 32768 BF16, b = 2^20, d = 7 834 -> 57 ms; 64 uneven products of n = 512 ..
+// 8192, b = 16 n, d = 3 429 -> 24.2 ms.  What bounds it: the additions into
+// the buckets (random 64-bit reductions run at 205 G/s on the whole chip, one
+// 32-byte sector each), then the copies of the tiles' operands from L2 (about
+// 64 bytes per clock and SM).
+#include <algorithm>
+#include <cmath>
+#include <cuda_fp16.h>
+
+#include "cms_internal.h"
+#include "warp_fft.cuh"
+
+namespace cms {
+namespace {
+
+using namespace wfft;
+
+constexpr int kTile = 128;              // rows and columns of a tile
+constexpr int kSuper = 128;             // inner indices with one scale, and one drain of the accumulators
+constexpr int kStageBytes = kTile * 128;   // one operand's share of a stage
+constexpr int kStages = 3;
+constexpr int kMaxSb = 1024;            // scale factors held per block
+constexpr int kFold = 32;               // drains between folds of the register sums (long inner dimensions)
+constexpr int kFoldFrom = 64;           // drains above which they are folded
+constexpr int kEpiThreads = 128;
+constexpr int kTileThreads = kEpiThreads + 32;
+constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
+constexpr int kMinExp = -100;           // scales stay representable
+
+__device__ uint32_t g_direct_error = 0;   // 1: a wait gave up
+
+
+__device__ __forceinline__ float load_val(const float* p) { return __ldg(p); }
+__device__ __forceinline__ float load_val(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+__device__ __forceinline__ float load_val(const double* p) { return static_cast<float>(__ldg(p)); }
+
+// 2^e for |e| <= 126
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+
+// The product whose blocks start[q] .. start[q + 1] - 1 hold block `x`.
+__device__ __forceinline__ int find_instance(const int* __restrict__ start, int count, int x) {
+  int lo = 0, hi = count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(start + mid) <= x) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+struct PackSide {
+  const void* X;       // rows of ld elements, inner index k
+  int64_t ld;
+  int64_t n;           // columns used
+  int tiles;           // 0: the side is the other one's bytes
+  uint8_t* out;        // [tile][stage] images
+  int2* blocks;        // [tile][superblock]: exponent, sum of squares of the scaled values
+};
+
+struct PackArgs {
+  PackSide side[2];
+  int64_t K;
+  int nsb;
+  int dt;
+  int64_t n1, n3;
+  uint32_t* ticket;    // blocks done; left at 0
+  DirectScale* scale;
+};
+
+__device__ __forceinline__ float block_sum256(float v, float* sh) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float r = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) r += sh[w];
+  return r;
+}
+
+__device__ __forceinline__ int block_max256(int v, int* sh) {
+  v = __reduce_max_sync(0xFFFFFFFFu, v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int r = sh[0];
+#pragma unroll
+  for (int w = 1; w < 8; ++w) r = max(r, sh[w]);
+  return r;
+}
+
+// The grid of the integer sums, by the last block of a product's packing.
+// A bucket is a sum of at most n1 n3 entries, so |c_z| <= sqrt(n1 n3) |AB|_F
+// <= sqrt(n1 n3) |A|_F |B|_F: the largest shift that keeps this below 2^62.
+__device__ void direct_scale(const PackArgs& p, float* fsh, int* ish) {
+  float q[2];
+  int em[2];
+  for (int sd = 0; sd < 2; ++sd) {
+    const PackSide& s = p.side[sd];
+    const int64_t count = static_cast<int64_t>(s.tiles) * p.nsb;
+    int m = kMinExp;
+    for (int64_t x = threadIdx.x; x < count; x += 256) m = max(m, __ldcg(&s.blocks[x].x));
+    em[sd] = block_max256(m, ish);
+    float acc = 0.f;
+    for (int64_t x = threadIdx.x; x < count; x += 256) {
+      const int2 v = __ldcg(&s.blocks[x]);
+      const int de = 2 * (v.x - em[sd]);
+      acc += de < -120 ? 0.f : __int_as_float(v.y) * pow2f(de);
+    }
+    q[sd] = block_sum256(acc, fsh);
+  }
+  if (threadIdx.x != 0) return;
+  if (p.side[1].tiles == 0) { q[1] = q[0]; em[1] = em[0]; }
+  DirectScale r;
+  r.emax[0] = em[0];
+  r.emax[1] = em[1];
+  r.bad = em[0] >= kBadExp || em[1] >= kBadExp;
+  // squares of values below 2^15: at most 2^30 K n each, inside FP32's range
+  const float bound = 1.01f * sqrtf(static_cast<float>(p.n1) * static_cast<float>(p.n3)) * sqrtf(q[0]) * sqrtf(q[1]);
+  r.shift = 0;
+  if (bound > 0.f) r.shift = min(61 - ((__float_as_int(bound) >> 23) - 127), 126);
+  *p.scale = r;
+  *p.ticket = 0;
+}
+
+template <typename T, bool SPLIT>
+__device__ __forceinline__ void pack_block(const PackArgs& p, int sb, int tile, int sd, uint8_t* img, float* fsh,
+                                           int* ish) {
+  constexpr int kImages = SPLIT ? 4 : 2;   // stages of a superblock
+  constexpr int kPerStage = kSuper / kImages;
+  const PackSide& s = p.side[sd];
+  const int64_t K = p.K;
+  const int r = threadIdx.x & (kTile - 1), half = threadIdx.x >> 7;
+  const int64_t i = static_cast<int64_t>(tile) * kTile + r;
+  const int64_t k0 = static_cast<int64_t>(sb) * kSuper + half * 64;
+  const T* X = static_cast<const T*>(s.X) + i;
+  float x[64];
+  const int kn = i < s.n ? static_cast<int>(min(max(K - k0, static_cast<int64_t>(0)), static_cast<int64_t>(64))) : 0;
+  if (kn == 64) {
+#pragma unroll
+    for (int q = 0; q < 64; ++q) x[q] = load_val(X + (k0 + q) * s.ld);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 64; ++q) x[q] = q < kn ? load_val(X + (k0 + q) * s.ld) : 0.f;
+  }
+  uint32_t m = 0;
+#pragma unroll
+  for (int q = 0; q < 64; ++q) m = max(m, __float_as_uint(x[q]) & 0x7FFFFFFFu);
+  m = static_cast<uint32_t>(block_max256(static_cast<int>(m), ish));
+  const bool bad = m >= 0x7F800000u;
+  const int e = bad ? 0 : max(static_cast<int>(m >> 23) - 127, kMinExp);
+  // two factors: 2^(14 - e) alone may leave FP32's range
+  const int sh = direct_scale_log2(SPLIT) - e;
+  const float f1 = pow2f(sh / 2), f2 = pow2f(sh - sh / 2);
+  float nn = 0.f;
+#pragma unroll
+  for (int q = 0; q < 64; ++q) {
+    x[q] = x[q] * f1 * f2;
+    nn = fmaf(x[q], x[q], nn);
+  }
+  nn = block_sum256(nn, fsh);
+  const uint32_t rowoff = (r >> 3) * 1024 + (r & 7) * 128;
+  // chunk c: 8 of this thread's 64 inner indices, in the image's 16-byte
+  // column c (swizzled by the row)
+  auto put = [&](int image, int c, const uint32_t (&w)[4]) {
+    *reinterpret_cast<uint4*>(img + image * kStageBytes + rowoff + ((c ^ (r & 7)) << 4)) =
+        make_uint4(w[0], w[1], w[2], w[3]);
+  };
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float a = x[8 * c + 2 * q], b = x[8 * c + 2 * q + 1];
+      if constexpr (SPLIT) {
+        const __half ha = __float2half_rn(a), hb = __float2half_rn(b);
+        const __half2 h2 = __halves2half2(ha, hb);
+        const __half2 l2 = __floats2half2_rn(a - __half2float(ha), b - __half2float(hb));
+        hi[q] = *reinterpret_cast<const uint32_t*>(&h2);
+        lo[q] = *reinterpret_cast<const uint32_t*>(&l2);
+      } else {
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(a, b);
+        hi[q] = *reinterpret_cast<const uint32_t*>(&h2);
+      }
+    }
+    if constexpr (SPLIT) {
+      put(half * 2 + c / 4, c & 3, hi);
+      put(half * 2 + c / 4, 4 + (c & 3), lo);
+    } else {
+      put(half, c, hi);
+    }
+  }
+  fence_proxy_async();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s.blocks[static_cast<size_t>(tile) * p.nsb + sb] = make_int2(bad ? kBadExp : e, __float_as_int(nn));
+    const int64_t left = min(K - static_cast<int64_t>(sb) * kSuper, static_cast<int64_t>(kSuper));
+    const uint32_t bytes = static_cast<uint32_t>((left + kPerStage - 1) / kPerStage) * kStageBytes;
+    const int64_t per_tile = (K + kPerStage - 1) / kPerStage;   // images of a tile
+    uint8_t* dst = s.out + (static_cast<size_t>(tile) * per_tile + static_cast<size_t>(sb) * kImages) * kStageBytes;
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(img)),
+                 "r"(bytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  }
+}
+
+// Block `idx` of a product's packing: superblocks fastest, then the tiles of
+// A, then those of B.
+__device__ __forceinline__ void pack_task(const PackArgs& p, uint32_t idx) {
+  extern __shared__ __align__(1024) uint8_t img[];
+  __shared__ float fsh[8];
+  __shared__ int ish[8];
+  __shared__ bool last;
+  const uint32_t nsb = static_cast<uint32_t>(p.nsb);
+  const uint32_t total = nsb * static_cast<uint32_t>(p.side[0].tiles + p.side[1].tiles);
+  int tile = static_cast<int>(idx / nsb);
+  const int sb = static_cast<int>(idx - tile * nsb);
+  const int sd = tile >= p.side[0].tiles;
+  if (sd) tile -= p.side[0].tiles;
+  if (p.dt == CMS_BF16) pack_block<__nv_bfloat16, false>(p, sb, tile, sd, img, fsh, ish);
+  else if (p.dt == CMS_F64) pack_block<double, true>(p, sb, tile, sd, img, fsh, ish);
+  else pack_block<float, true>(p, sb, tile, sd, img, fsh, ish);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(p.ticket, 1u) == total - 1;
+  }
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    direct_scale(p, fsh, ish);
+  }
+  if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(256) k_direct_pack(const PackArgs p) { pack_task(p, blockIdx.x); }
+
+struct TileArgs {
+  const uint8_t* pa;
+  const uint8_t* pb;
+  const int2* ea;              // (exponent, -) per superblock
+  const int2* eb;
+  const DirectScale* scale;
+  const uint32_t* hs;          // [t][side][n]
+  unsigned long long* acc;     // [t][b]
+  int64_t K;
+  int n, n1, n3, b, d;
+  int tiles1, tiles3;
+  int nsb, sb_per_split;
+  int tiles;                   // of AB
+  float* fold;                 // [slots][128][128] partial sums of the blocks that run, or NULL
+  uint32_t* slot;              // slot taken
+  int slots;
+  int split;
+  int sym;                     // A = X^T, B = X: tiles on and above the diagonal
+};
+
+constexpr uint32_t tile_smem_bytes() { return 1024 + kStages * 2 * kStageBytes + kMaxSb * 4 + 2 * kTile * 4; }
+
+// Shared-memory matrix descriptor of a K-major operand in the 128-byte
+// swizzle: 8-row groups 1024 bytes apart.
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
+  return (static_cast<uint64_t>(addr >> 4) & 0x3FFFu) | (1ull << 16) | (static_cast<uint64_t>(1024 >> 4) << 32) |
+         (1ull << 46) | (2ull << 61);
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+  const uint32_t p = accumulate;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(p)
+      : "memory");
+}
+
+// The barrier's phase completes when the tensor-core work issued so far has.
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+               : "memory");
+}
+
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+__device__ __forceinline__ void bucket_add(unsigned long long* c, uint32_t ha, uint32_t hb, uint32_t b, float v) {
+  uint32_t z = (ha & kBucketMask) + (hb & kBucketMask);
+  if (z >= b) z -= b;
+  const float w = __uint_as_float(__float_as_uint(v) ^ ((ha ^ hb) & 0x80000000u));
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c + z), "l"(__float2ll_rn(w)) : "memory");
+}
+
+__device__ __forceinline__ void tmem_wait_ld8x2(uint32_t (&a)[8], uint32_t (&b)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+                 "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
+               :
+               : "memory");
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split) {
+  constexpr int kImages = SPLIT ? 4 : 2;
+  constexpr int kPerStage = kSuper / kImages;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full[kStages], freed[kStages], ready[2], drained[2];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_err, s_slot;
+  uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  float* factor = reinterpret_cast<float*>(stages + kStages * 2 * kStageBytes);
+  uint32_t* hcol = reinterpret_cast<uint32_t*>(factor + kMaxSb);   // [2][128]
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5;
+  // tile of AB
+  int ti, tj;
+  if (p.sym) {
+    // row by row over the upper triangle: row ti holds tiles1 - ti tiles
+    const int T = p.tiles1;
+    const int q = tile;
+    ti = static_cast<int>((2.0 * T + 1.0 - sqrt((2.0 * T + 1.0) * (2.0 * T + 1.0) - 8.0 * q)) * 0.5);
+    while (ti > 0 && q < ti * T - ti * (ti - 1) / 2) --ti;
+    while (q >= (ti + 1) * T - (ti + 1) * ti / 2) ++ti;
+    tj = ti + q - (ti * T - ti * (ti - 1) / 2);
+  } else {
+    ti = tile / p.tiles3;
+    tj = tile - ti * p.tiles3;
+  }
+  const int sb0 = split * p.sb_per_split;
+  const int sb1 = min(p.nsb, sb0 + p.sb_per_split);
+  const int per_tile = static_cast<int>((p.K + kPerStage - 1) / kPerStage);
+  const int st0 = sb0 * kImages, st1 = min(per_tile, sb1 * kImages);
+  const int nst = st1 - st0;                                  // stages of this block
+  const int chunks = (nst + 1) / 2;                           // drains of the accumulators
+  const bool folds = p.fold != nullptr && chunks > kFoldFrom;
+  if (tid == 0) {
+    for (int q = 0; q < kStages; ++q) { mbar_init(&full[q], 1); mbar_init(&freed[q], 1); }
+    for (int q = 0; q < 2; ++q) { mbar_init(&ready[q], 1); mbar_init(&drained[q], kEpiThreads); }
+    s_err = 0;
+    s_slot = -1;
+    if (folds) {
+      // no more than `slots` blocks run at a time: one is free
+      uint32_t q = static_cast<uint32_t>(blockIdx.x) % static_cast<uint32_t>(p.slots);
+      for (int tries = 0; tries < 64 * p.slots && s_slot < 0; ++tries) {
+        if (atomicCAS(p.slot + q, 0u, 1u) == 0u) s_slot = static_cast<int>(q);
+        q = q + 1 == static_cast<uint32_t>(p.slots) ? 0 : q + 1;
+      }
+      if (s_slot < 0) s_err = 1;
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 4) {
+    tmem_alloc(&s_tmem, 2 * kTile);
+    tmem_relinquish();
+  }
+  const DirectScale sc = *p.scale;
+  for (int q = tid; q < sb1 - sb0; q += kTileThreads) {
+    const int de = p.ea[static_cast<size_t>(ti) * p.nsb + sb0 + q].x - sc.emax[0] +
+                   p.eb[static_cast<size_t>(tj) * p.nsb + sb0 + q].x - sc.emax[1];
+    factor[q] = de < -126 ? 0.f : pow2f(min(de, 0));
+  }
+  tmem_fence_before_sync();
+  __syncthreads();
+  tmem_fence_after_sync();
+  const uint32_t tmem = s_tmem;
+
+  if (warp == 4) {
+    if ((tid & 31) == 0) {
+      // D: FP32; A, B: FP16 (0) or BF16 (1), K-major; N / 8, M / 16
+      constexpr uint32_t idesc = (1u << 4) | ((SPLIT ? 0u : 1u) << 7) | ((SPLIT ? 0u : 1u) << 10) |
+                                 (static_cast<uint32_t>(kTile / 8) << 17) | (static_cast<uint32_t>(kTile / 16) << 24);
+      const uint8_t* ga = p.pa + (static_cast<size_t>(ti) * per_tile + st0) * kStageBytes;
+      const uint8_t* gb = p.pb + (static_cast<size_t>(tj) * per_tile + st0) * kStageBytes;
+      auto load = [&](int st) {
+        uint8_t* dst = stages + (st % kStages) * 2 * kStageBytes;
+        uint64_t* bar = &full[st % kStages];
+        mbar_arrive_expect_tx(bar, 2 * kStageBytes);
+        bulk_g2s(dst, ga + static_cast<size_t>(st) * kStageBytes, kStageBytes, bar);
+        bulk_g2s(dst + kStageBytes, gb + static_cast<size_t>(st) * kStageBytes, kStageBytes, bar);
+      };
+      int issued = min(kStages, nst);
+      for (int st = 0; st < issued; ++st) load(st);
+      bool ok = true;
+      int st = 0;
+      for (int ch = 0; st < nst && ok; ++ch) {
+        const int buf = SPLIT ? 0 : ch & 1;
+        const int use = SPLIT ? ch : ch >> 1;      // of this buffer
+        if (use >= 1) ok = mbar_wait_bounded(&drained[buf], (use - 1) & 1);
+        tmem_fence_after_sync();
+        const int end = min(nst, st + 2);
+        const uint32_t dt = tmem + buf * kTile;
+        const bool cross0 = (ch & 1) == 0;         // first half of a superblock
+        for (bool first = true; st < end && ok; ++st, first = false) {
+          ok = mbar_wait_bounded(&full[st % kStages], (st / kStages) & 1);
+          if (!ok) break;
+          tmem_fence_after_sync();
+          const uint32_t a = smem_u32(stages + (st % kStages) * 2 * kStageBytes);
+          const uint64_t da = smem_desc(a), db = smem_desc(a + kStageBytes);
+          // 16 inner indices are 32 bytes (2 units of 16) along the rows
+          if constexpr (SPLIT) {
+            // hi hi into one accumulator, the cross terms (2^-11 of it) into
+            // the other: added to the same one, each would be cut to the
+            // precision of the large sum
+            mma_f16(dt, da, db, idesc, !first);
+            mma_f16(dt + kTile, da, db + 4, idesc, !(first && cross0));
+            mma_f16(dt, da + 2, db + 2, idesc, true);
+            mma_f16(dt + kTile, da + 2, db + 6, idesc, true);
+            mma_f16(dt + kTile, da + 4, db, idesc, true);
+            mma_f16(dt + kTile, da + 6, db + 2, idesc, true);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mma_f16(dt, da + 2 * q, db + 2 * q, idesc, !first || q > 0);
+          }
+          mma_commit(&freed[st % kStages]);
+          // refill the stage before this one while this one's products run
+          if (st >= 1 && issued < nst) {
+            ok = mbar_wait_bounded(&freed[(st - 1) % kStages], ((st - 1) / kStages) & 1);
+            if (ok) load(issued++);
+          }
+        }
+        if (ok) mma_commit(&ready[buf]);
+      }
+      // the products of the last stages have arrived on their barriers
+      for (int q = max(0, st - kStages); q < st && ok; ++q) ok = mbar_wait_bounded(&freed[q % kStages], (q / kStages) & 1);
+      if (!ok) {
+        s_err = 1;
+        for (int q = max(0, issued - kStages); q < issued; ++q)
+          (void)mbar_wait_bounded(&full[q % kStages], (q / kStages) & 1);
+      }
+    }
+    __syncwarp();
+  } else {
+    float acc[kTile];
+#pragma unroll
+    for (int q = 0; q < kTile; ++q) acc[q] = 0.f;
+    const uint32_t lane = tmem + (static_cast<uint32_t>(warp) << 21);
+    bool ok = true;
+    float* fold = folds && s_slot >= 0 ? p.fold + static_cast<size_t>(s_slot) * kTile * kTile + tid : nullptr;
+    for (int ch = 0; ch < chunks; ++ch) {
+      const int buf = SPLIT ? 0 : ch & 1;
+      if (ok) ok = mbar_wait_bounded(&ready[buf], (SPLIT ? ch : ch >> 1) & 1);
+      ok = __all_sync(0xFFFFFFFFu, ok);
+      if (!ok) break;
+      tmem_fence_after_sync();
+      const float f = factor[SPLIT ? ch >> 1 : ch];
+      const uint32_t col = lane + buf * kTile;
+      if (SPLIT && ((ch & 1) || ch == chunks - 1)) {
+#pragma unroll
+        for (int g = 0; g < kTile / 8; ++g) {
+          uint32_t v[8], w[8];
+          tmem_ld8_nowait(col + g * 8, v);
+          tmem_ld8_nowait(col + kTile + g * 8, w);
+          tmem_wait_ld8x2(v, w);
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            acc[g * 8 + q] = fmaf(__uint_as_float(v[q]) + __uint_as_float(w[q]), f, acc[g * 8 + q]);
+        }
+      } else {
+#pragma unroll
+        for (int g = 0; g < kTile / 16; ++g) {
+          uint32_t v[8], w[8];
+          tmem_ld8_nowait(col + g * 16, v);
+          tmem_ld8_nowait(col + g * 16 + 8, w);
+          tmem_wait_ld8x2(v, w);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            acc[g * 16 + q] = fmaf(__uint_as_float(v[q]), f, acc[g * 16 + q]);
+            acc[g * 16 + 8 + q] = fmaf(__uint_as_float(w[q]), f, acc[g * 16 + 8 + q]);
+          }
+        }
+      }
+      tmem_fence_before_sync();
+      mbar_arrive(&drained[buf]);
+      // the sums so far join those of earlier folds: a long chain of FP32
+      // additions into one large sum would lose a bit per factor of four
+      if (fold != nullptr && (ch + 1) % kFold == 0 && ch + 1 < chunks) {
+        // one thread adds to each word, in order: the same sum in every run
+        const bool first = ch + 1 == kFold;
+#pragma unroll
+        for (int q = 0; q < kTile; ++q) {
+          if (first) __stcg(fold + q * kTile, acc[q]);
+          else asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(fold + q * kTile), "f"(acc[q]) : "memory");
+          acc[q] = 0.f;
+        }
+      }
+    }
+    if (fold != nullptr) {
+#pragma unroll
+      for (int g = 0; g < kTile / 16; ++g) {
+        float v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = __ldcg(fold + (g * 16 + q) * kTile);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) acc[g * 16 + q] += v[q];
+      }
+    }
+    if (!ok) s_err = 1;
+    epi_sync();
+    const bool run = s_err == 0 && !sc.bad;
+    const float up = pow2f(sc.shift / 2), up2 = pow2f(sc.shift - sc.shift / 2);
+#pragma unroll
+    for (int q = 0; q < kTile; ++q) acc[q] = acc[q] * up * up2;
+    const int i = ti * kTile + tid;
+    const int j0 = tj * kTile;
+    const int cols = run ? min(kTile, p.n3 - j0) : 0;
+    const bool mirror = p.sym && ti != tj;
+    const bool row = i < p.n1;
+    const uint32_t b = static_cast<uint32_t>(p.b);
+    for (int t = 0; t < p.d; ++t) {
+      const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
+      const uint32_t* h2 = h1 + p.n;
+      epi_sync();
+      if (tid < cols) {
+        hcol[tid] = h2[j0 + tid];
+        if (mirror) hcol[kTile + tid] = h1[j0 + tid];
+      }
+      epi_sync();
+      if (!row) continue;
+      unsigned long long* c = p.acc + static_cast<size_t>(t) * p.b;
+      const uint32_t hr = h1[i];
+#pragma unroll
+      for (int q = 0; q < kTile; ++q)
+        if (q < cols) bucket_add(c, hr, hcol[q], b, acc[q]);
+      if (mirror) {
+        const uint32_t hm = h2[i];
+#pragma unroll
+        for (int q = 0; q < kTile; ++q)
+          if (q < cols) bucket_add(c, hcol[kTile + q], hm, b, acc[q]);
+      }
+    }
+  }
+  tmem_fence_before_sync();
+  __syncthreads();
+  if (tid == 0 && s_err) atomicOr(&g_direct_error, 1u);
+  if (tid == 0 && s_slot >= 0) atomicExch(p.slot + s_slot, 0u);
+  if (warp == 4) tmem_dealloc(tmem, 2 * kTile);
+  if (tid == 0) {
+    for (int q = 0; q < kStages; ++q) { mbar_inval(&full[q]); mbar_inval(&freed[q]); }
+    for (int q = 0; q < 2; ++q) { mbar_inval(&ready[q]); mbar_inval(&drained[q]); }
+  }
+}
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(kTileThreads, 2) k_direct_tile(const TileArgs p) {
+  tile_task<SPLIT>(p, blockIdx.x, blockIdx.y);
+}
+
+// Tiles of every product of a batch, the longest first.
+__global__ void __launch_bounds__(kTileThreads, 2)
+k_direct_tile_batched(const TileArgs* __restrict__ args, const int* __restrict__ start, int count) {
+  __shared__ TileArgs sp;
+  const int q = find_instance(start, count, static_cast<int>(blockIdx.x));
+  for (int w = threadIdx.x; w < static_cast<int>(sizeof(TileArgs) / 4); w += kTileThreads)
+    reinterpret_cast<uint32_t*>(&sp)[w] = reinterpret_cast<const uint32_t*>(args + q)[w];
+  __syncthreads();
+  const int local = static_cast<int>(blockIdx.x) - __ldg(start + q);
+  const int tile = local % sp.tiles, split = local / sp.tiles;
+  if (sp.split) tile_task<true>(sp, tile, split);
+  else tile_task<false>(sp, tile, split);
+}
+
+__global__ void __launch_bounds__(256)
+k_direct_pack_batched(const PackArgs* __restrict__ args, const int* __restrict__ start, int count) {
+  __shared__ PackArgs sp;
+  const int q = find_instance(start, count, static_cast<int>(blockIdx.x));
+  for (int w = threadIdx.x; w < static_cast<int>(sizeof(PackArgs) / 4); w += 256)
+    reinterpret_cast<uint32_t*>(&sp)[w] = reinterpret_cast<const uint32_t*>(args + q)[w];
+  __syncthreads();
+  pack_task(sp, blockIdx.x - static_cast<uint32_t>(__ldg(start + q)));
+}
+
+__global__ void __launch_bounds__(256) k_direct_finish(const unsigned long long* acc, float* c, int64_t len,
+                                                       const DirectScale* scale, int log2s) {
+  const DirectScale sc = *scale;
+  for (int64_t q = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; q < len; q += static_cast<int64_t>(gridDim.x) * 256)
+    c[q] = direct_value(acc[q], sc, log2s);
+}
+
+}  // namespace
+
+uint32_t read_clear_error_direct() {
+  uint32_t v = 0, zero = 0;
+  if (cudaMemcpyFromSymbol(&v, g_direct_error, sizeof(v)) != cudaSuccess) return 0xFFFFFFFFu;
+  if (v) cudaMemcpyToSymbol(g_direct_error, &zero, sizeof(zero));
+  return v;
+}
+
+DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms) {
+  DirectPlan p;
+  p.split = dt != CMS_BF16;
+  p.alias = alias;
+  p.tiles1 = static_cast<int>((n1 + kTile - 1) / kTile);
+  p.tiles3 = static_cast<int>((n3 + kTile - 1) / kTile);
+  p.nsb = static_cast<int>((n2 + kSuper - 1) / kSuper);
+  const int64_t tiles = alias ? static_cast<int64_t>(p.tiles1) * (p.tiles1 + 1) / 2
+                              : static_cast<int64_t>(p.tiles1) * p.tiles3;
+  p.tiles = tiles;
+  const int per = p.split ? 32 : 64;
+  const int64_t images = (n2 + per - 1) / per;
+  // split the inner dimension while blocks are missing, each split adding a
+  // pass of n1 n3 d reductions
+  const int cap = kMaxSb;
+  int best = std::max(1, (p.nsb + cap - 1) / cap);
+  double cost = 1e30;
+  const double slots = 2.0 * sms;
+  for (int s = best; s <= std::min(p.nsb, std::max(best, 64)); ++s) {
+    const int per_split = (p.nsb + s - 1) / s;
+    const int real = (p.nsb + per_split - 1) / per_split;
+    const double waves = std::max(1.0, std::ceil(static_cast<double>(tiles) * real / slots));
+    const double mma = waves * per_split * (p.split ? 1.0 : 0.5) * 1.1e-6;
+    const double red = static_cast<double>(n1) * n3 * h->d * real / 2.0e11;
+    if (mma + red < cost) { cost = mma + red; best = real; }
+  }
+  p.sb_per_split = (p.nsb + best - 1) / best;
+  p.splits = (p.nsb + p.sb_per_split - 1) / p.sb_per_split;
+  p.seconds = cost + 15e-6;
+  auto al = [](size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); };
+  size_t o = 0;
+  const int t3 = alias ? 0 : p.tiles3;
+  const int drains = p.sb_per_split * (p.split ? 2 : 1);
+  p.slots = drains > kFoldFrom ? 2 * sms : 0;
+  // sums, the ticket, the slots taken (all zero before a run)
+  p.off_acc = o;    o = al(o + static_cast<size_t>(h->d) * h->b * 8 + 256 + static_cast<size_t>(p.slots) * 4);
+  p.zero_bytes = o;
+  p.off_fold = o;   o = al(o + static_cast<size_t>(p.slots) * kTile * kTile * sizeof(float));
+  p.off_scale = o;  o = al(o + sizeof(DirectScale));
+  p.off_blocks = o; o = al(o + static_cast<size_t>(p.tiles1 + t3) * p.nsb * sizeof(int2));
+  p.off_pa = o;     o = al(o + static_cast<size_t>(p.tiles1) * images * kStageBytes);
+  p.off_pb = alias ? p.off_pa : o;
+  if (!alias) o = al(o + static_cast<size_t>(p.tiles3) * images * kStageBytes);
+  p.ws_bytes = o;
+  return p;
+}
+
+// Estimated time of the transform route (make_sketch_plan) at its best rate:
+// 40 TFLOP/s of the conventional 5 b log2 b + 4 b per repetition and inner
+// index, which only the warp-specialised kernel reaches (the others run at 6
+// to 18), so the direct route is taken where it is the faster one by a margin.
+static double transform_seconds(const SketchPlan& p, int64_t n2) {
+  const double b = static_cast<double>(p.b);
+  return 20e-6 + static_cast<double>(p.d) * static_cast<double>(n2) * (5.0 * b * std::log2(std::max(b, 2.0)) + 4.0 * b) / 40e12;
+}
+
+bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias,
+                   int sms, DirectPlan* out) {
+  // under 64 inner indices the packing and the padding to a superblock show
+  if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535) return false;
+  *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms);
+  return out->seconds < transform_seconds(plan, n2);
+}
+namespace {
+
+PackArgs pack_args(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B, int64_t ldb,
+                   int64_t n1, int64_t n2, int64_t n3, int dt, char* ws) {
+  int2* blocks = reinterpret_cast<int2*>(ws + p.off_blocks);
+  PackArgs a{};
+  a.side[0] = PackSide{A, lda, n1, p.tiles1, reinterpret_cast<uint8_t*>(ws + p.off_pa), blocks};
+  a.side[1] = PackSide{B, ldb, n3, p.alias ? 0 : p.tiles3, reinterpret_cast<uint8_t*>(ws + p.off_pb),
+                       blocks + static_cast<size_t>(p.tiles1) * p.nsb};
+  a.K = n2;
+  a.nsb = p.nsb;
+  a.dt = dt;
+  a.n1 = n1;
+  a.n3 = n3;
+  a.ticket = reinterpret_cast<uint32_t*>(ws + p.off_acc + static_cast<size_t>(h->d) * h->b * 8);
+  a.scale = reinterpret_cast<DirectScale*>(ws + p.off_scale);
+  return a;
+}
+
+TileArgs tile_args(const DirectPlan& p, const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, char* ws) {
+  TileArgs a{};
+  a.pa = reinterpret_cast<uint8_t*>(ws + p.off_pa);
+  a.pb = reinterpret_cast<uint8_t*>(ws + p.off_pb);
+  a.ea = reinterpret_cast<int2*>(ws + p.off_blocks);
+  a.eb = p.alias ? a.ea : a.ea + static_cast<size_t>(p.tiles1) * p.nsb;
+  a.scale = reinterpret_cast<DirectScale*>(ws + p.off_scale);
+  a.hs = h->d_hs;
+  a.acc = reinterpret_cast<unsigned long long*>(ws + p.off_acc);
+  a.K = n2;
+  a.n = static_cast<int>(h->n);
+  a.n1 = static_cast<int>(n1);
+  a.n3 = static_cast<int>(n3);
+  a.b = static_cast<int>(h->b);
+  a.d = h->d;
+  a.tiles1 = p.tiles1;
+  a.tiles3 = p.tiles3;
+  a.nsb = p.nsb;
+  a.sb_per_split = p.sb_per_split;
+  a.tiles = static_cast<int>(p.tiles);
+  a.fold = p.slots > 0 ? reinterpret_cast<float*>(ws + p.off_fold) : nullptr;
+  a.slot = reinterpret_cast<uint32_t*>(ws + p.off_acc + static_cast<size_t>(h->d) * h->b * 8 + 256);
+  a.slots = p.slots;
+  a.split = p.split ? 1 : 0;
+  a.sym = p.alias ? 1 : 0;
+  return a;
+}
+
+int pack_blocks(const DirectPlan& p) { return p.nsb * (p.tiles1 + (p.alias ? 0 : p.tiles3)); }
+
+template <typename F>
+cudaError_t with_smem(F kern, uint32_t bytes) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+}
+
+}  // namespace
+
+size_t direct_batch_bytes(int count) {
+  auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
+  return al(count * sizeof(PackArgs)) + al(count * sizeof(TileArgs)) + 2 * al((count + 1) * sizeof(int));
+}
+
+cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, void* d_buf, DirectBatch* out, cudaStream_t s) {
+  auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
+  const int count = static_cast<int>(specs.size());
+  std::vector<unsigned char> host(direct_batch_bytes(count));
+  out->buf = d_buf;
+  out->count = count;
+  out->o_tile = al(count * sizeof(PackArgs));
+  out->o_ps = out->o_tile + al(count * sizeof(TileArgs));
+  out->o_ts = out->o_ps + al((count + 1) * sizeof(int));
+  int* ps = reinterpret_cast<int*>(host.data() + out->o_ps);
+  int* ts = reinterpret_cast<int*>(host.data() + out->o_ts);
+  int np = 0, nt = 0;
+  out->pack_smem = 0;
+  for (int q = 0; q < count; ++q) {
+    const DirectSpec& d = specs[q];
+    reinterpret_cast<PackArgs*>(host.data())[q] =
+        pack_args(d.plan, d.h, d.A, d.lda, d.B, d.ldb, d.n1, d.n2, d.n3, d.dt, d.ws);
+    reinterpret_cast<TileArgs*>(host.data() + out->o_tile)[q] = tile_args(d.plan, d.h, d.n1, d.n2, d.n3, d.ws);
+    ps[q] = np;
+    ts[q] = nt;
+    np += pack_blocks(d.plan);
+    nt += static_cast<int>(d.plan.tiles) * d.plan.splits;
+    out->pack_smem = std::max<uint32_t>(out->pack_smem, (d.plan.split ? 4 : 2) * kStageBytes);
+  }
+  ps[count] = np;
+  ts[count] = nt;
+  out->pack_blocks = np;
+  out->tile_blocks = nt;
+  cudaError_t e = cudaSuccess;
+  for (int q = 0; q < count && e == cudaSuccess; ++q)
+    e = cudaMemsetAsync(specs[q].ws + specs[q].plan.off_acc, 0, specs[q].plan.zero_bytes, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d_buf, host.data(), host.size(), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host copy goes out of scope
+  return e;
+}
+
+cudaError_t launch_direct_batched(const DirectBatch& d, cudaStream_t s) {
+  if (d.count == 0) return cudaSuccess;
+  const char* base = static_cast<const char*>(d.buf);
+  cudaError_t e;
+  {
+    ProfScope prof_scope("k_direct_pack_batched", s);
+    if ((e = with_smem(k_direct_pack_batched, d.pack_smem)) != cudaSuccess) return e;
+    k_direct_pack_batched<<<d.pack_blocks, 256, d.pack_smem, s>>>(reinterpret_cast<const PackArgs*>(base),
+                                                                  reinterpret_cast<const int*>(base + d.o_ps), d.count);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  ProfScope prof_scope("k_direct_tile_batched", s);
+  if ((e = with_smem(k_direct_tile_batched, tile_smem_bytes())) != cudaSuccess) return e;
+  k_direct_tile_batched<<<d.tile_blocks, kTileThreads, tile_smem_bytes(), s>>>(
+      reinterpret_cast<const TileArgs*>(base + d.o_tile), reinterpret_cast<const int*>(base + d.o_ts), d.count);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
+                          int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws,
+                          cudaStream_t s) {
+  const size_t len = static_cast<size_t>(h->d) * h->b;
+  cudaError_t e = cudaMemsetAsync(ws + p.off_acc, 0, p.zero_bytes, s);
+  if (e != cudaSuccess) return e;
+  {
+    ProfScope prof_scope("k_direct_pack", s);
+    const uint32_t smem = (p.split ? 4 : 2) * kStageBytes;
+    if ((e = with_smem(k_direct_pack, smem)) != cudaSuccess) return e;
+    k_direct_pack<<<pack_blocks(p), 256, smem, s>>>(pack_args(p, h, A, lda, B, ldb, n1, n2, n3, dt, ws));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  const TileArgs a = tile_args(p, h, n1, n2, n3, ws);
+  {
+    ProfScope prof_scope("k_direct_tile", s);
+    const dim3 grid(static_cast<unsigned>(p.tiles), p.splits);
+    auto go = [&](auto kern) {
+      cudaError_t r = with_smem(kern, tile_smem_bytes());
+      if (r != cudaSuccess) return r;
+      kern<<<grid, kTileThreads, tile_smem_bytes(), s>>>(a);
+      return cudaGetLastError();
+    };
+    e = p.split ? go(k_direct_tile<true>) : go(k_direct_tile<false>);
+    if (e != cudaSuccess) return e;
+  }
+  {
+    ProfScope prof_scope("k_direct_finish", s);
+    const int64_t blocks = std::min<int64_t>((static_cast<int64_t>(len) + 255) / 256, 152 * 8);
+    k_direct_finish<<<static_cast<unsigned>(blocks), 256, 0, s>>>(a.acc, c, static_cast<int64_t>(len), a.scale,
+                                                                  direct_scale_log2(p.split));
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
+}  // namespace cms

@@ -191,6 +191,7 @@ k_rows_inverse_batched(const InvArgs* __restrict__ args, const int* __restrict__
   extern __shared__ float2 sm2[];
   const int i = batch_instance(start, count, static_cast<int>(blockIdx.x));
   const InvArgs p = args[i];
+  if (p.nrows == 0) return;   // direct route: no spectra
   rows_inverse_block(p, static_cast<int>(blockIdx.x) - __ldg(start + i), sm2);
 }
 
@@ -267,6 +268,9 @@ k_cols_inverse_fft(const float2* __restrict__ V, const float2* __restrict__ twR,
 }
 
 struct ColsArgs {
+  unsigned long long* sums;    // direct route: the integer sums (left zero), else NULL
+  const DirectScale* scale;
+  int log2s;
   const float2* V;
   const float2* twR;
   float* c;
@@ -283,7 +287,14 @@ k_cols_inverse_batched(const ColsArgs* __restrict__ args, const int* __restrict_
   const int local = static_cast<int>(blockIdx.x) - __ldg(start + i);
   const int t = local / a.nbx;
   const int64_t z = static_cast<int64_t>(local % a.nbx) * blockDim.x + threadIdx.x;
-  if (z < a.b) cols_inverse_point(a.V, a.twR, a.b, a.R, a.C, a.nrows, a.c, t, z);
+  if (z >= a.b) return;
+  if (a.sums != nullptr) {
+    const size_t q = static_cast<size_t>(t) * a.b + z;
+    a.c[q] = direct_value(a.sums[q], *a.scale, a.log2s);
+    a.sums[q] = 0;
+    return;
+  }
+  cols_inverse_point(a.V, a.twR, a.b, a.R, a.C, a.nrows, a.c, t, z);
 }
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
@@ -646,11 +657,14 @@ cudaError_t build_inverse_batch(const std::vector<InverseSpec>& specs, void* d_b
     ia.nradC = plan.nradC;
     for (int r = 0; r < 16; ++r) ia.radC[r] = plan.radC[r];
     ia.partial = specs[i].partial; ia.twC = specs[i].twC; ia.V = specs[i].V; ia.skip_if_zero = nullptr;
+    const bool direct = specs[i].sums != nullptr;
+    if (direct) ia.nrows = 0;
     rows[i] = ia;
     rstart[i] = tr;
-    tr += plan.d * plan.nrows;
-    smem = std::max(smem, static_cast<size_t>(3 * plan.C * 8));
+    tr += direct ? 1 : plan.d * plan.nrows;
+    if (!direct) smem = std::max(smem, static_cast<size_t>(3 * plan.C * 8));
     ColsArgs ca{};
+    ca.sums = specs[i].sums; ca.scale = specs[i].scale; ca.log2s = specs[i].log2s;
     ca.V = specs[i].V; ca.twR = specs[i].twR; ca.c = specs[i].c; ca.b = plan.b;
     ca.R = static_cast<int>(plan.R); ca.C = static_cast<int>(plan.C); ca.nrows = plan.nrows;
     ca.nbx = static_cast<int>((plan.b + 255) / 256);

@@ -1,0 +1,182 @@
+"""The direct route (tensor-core tiles of AB added to the buckets) against the
+FP64 oracle, at the sizes where it can go wrong: edges of the 128 x 128 tiles
+and of the 32, 64 and 128 inner indices of a stage and a superblock, every
+storage type, aliased and separate operands, unaligned rows, split and folded
+inner dimensions, values far apart in magnitude, infinities and NaN.
+
+Tolerance: relative L2 1e-6 per repetition.  The products of a drain (64 with
+FP16 terms, 128 with BF16) are summed with a relative error of a few 2^-24,
+at most 64 drains follow each other in one FP32 sum (1/sqrt(3) 2^-24 sqrt(32)
+of it in the mean) and the rest is added exactly: about 2.5e-7, with room for
+a factor of four."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from oracle import cms_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-6
+DT = {"f32": torch.float32, "bf16": torch.bfloat16, "f64": torch.float64}
+
+
+@pytest.fixture(scope="module")
+def cms():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1108_1320_gb300 import build as b
+    b.build()
+    import paper_1108_1320_gb300 as m
+    m.lib()
+    return m
+
+
+def dev():
+    return torch.device("cuda", torch.cuda.current_device())
+
+
+def operands(n1, n2, n3, dts, alias, pad, seed, scale=None):
+    """Device A, B and the FP64 values they hold."""
+    def stored(x):
+        return W.bf16_round(x.astype(np.float32))[0] if dts == "bf16" else x.astype(np.float32 if dts == "f32" else np.float64)
+
+    def put(x):
+        buf = torch.zeros((x.shape[0], x.shape[1] + pad), dtype=DT[dts], device=dev())
+        buf[:, :x.shape[1]] = torch.from_numpy(x).to(dev(), DT[dts])
+        return buf[:, :x.shape[1]]
+
+    At = W.gaussian(n2, n1, seed)
+    if scale is not None:
+        At = At * scale(n2, n1)
+    At = stored(At)
+    at = put(At)
+    if alias:
+        return at.T, at, At.astype(np.float64).T, At.astype(np.float64)
+    B = stored(W.gaussian(n2, n3, seed + 1))
+    return at.T, put(B), At.astype(np.float64).T, B.astype(np.float64)
+
+
+def run(cms, A, B, h, **kw):
+    cms.profile_enable(True)
+    c = cms.sketch_product(A, B, h, **kw)
+    torch.cuda.synchronize()
+    kernels = cms.profile_summary()
+    cms.profile_enable(False)
+    cms.check_async()
+    return c, kernels
+
+
+def worst(c, ref):
+    return max(O.rel_l2(c[t].cpu().numpy(), ref[t]) for t in range(ref.shape[0]))
+
+
+@pytest.mark.parametrize("n1,n2,n3,b,d,dts,alias,pad", [
+    (128, 128, 128, 8192, 2, "f32", True, 0),       # one tile, one superblock
+    (127, 127, 129, 8100, 3, "f32", False, 1),      # one short of and one past a tile
+    (129, 129, 127, 8192, 3, "bf16", False, 1),
+    (257, 95, 257, 16384, 2, "f32", True, 3),       # 3 stages of 32: an odd number in the last drain
+    (300, 65, 300, 20000, 1, "bf16", True, 0),      # one inner index in the second stage of 64
+    (200, 385, 333, 20000, 2, "f64", False, 0),     # FP64 storage
+    (640, 1000, 640, 10240, 3, "f32", True, 0),     # upper triangle of 5 x 5 tiles, split inner dimension
+    (512, 9000, 384, 8192, 1, "bf16", False, 0),
+])
+def test_direct_route_matches_oracle(cms, n1, n2, n3, b, d, dts, alias, pad):
+    n = max(n1, n3)
+    seed = n1 + n2
+    A, B, Ad, Bd = operands(n1, n2, n3, dts, alias, pad, seed)
+    h = cms.make_hashes(seed, n, b, d)
+    c, kernels = run(cms, A, B, h)
+    assert "k_direct_tile" in kernels
+    ref = O.sketch_definition(Ad, Bd, O.make_tables(seed, n, b, d))
+    assert worst(c, ref) < TOL
+    c2, _ = run(cms, A, B, h)
+    assert torch.equal(c, c2)                       # the order of the integer sums does not matter
+    h.free()
+
+
+@pytest.mark.parametrize("n,m,dts", [(1920, 4500, "f32"), (1920, 8500, "bf16")])
+def test_direct_route_folds_long_sums(cms, n, m, dts):
+    # enough tiles that the inner dimension is not split, and more than 64
+    # drains: the register sums are folded
+    A, B, Ad, Bd = operands(n, m, n, dts, True, 0, 7)
+    h = cms.make_hashes(8, n, 16 * n, 1)
+    c, kernels = run(cms, A, B, h)
+    assert "k_direct_tile" in kernels
+    ref = O.sketch_definition(Ad, Bd, O.make_tables(8, n, 16 * n, 1))
+    assert worst(c, ref) < TOL
+    h.free()
+
+
+@pytest.mark.parametrize("dts", ["f32", "bf16"])
+@pytest.mark.parametrize("case", ["rows", "tiny", "huge", "outlier"])
+def test_direct_route_over_magnitudes(cms, dts, case):
+    # inner indices 2^-40 .. 2^40 apart, values near either end of FP32's
+    # range, and one entry that dwarfs the others
+    def scale(n2, n1):
+        if case == "rows":
+            return np.exp2(np.linspace(-40, 40, n2))[:, None]
+        s = np.ones((n2, n1))
+        if case == "outlier":
+            s[n2 // 2, n1 // 3] = 1e6
+            return s
+        return s * (1e-17 if case == "tiny" else 1e16)
+    A, B, Ad, Bd = operands(200, 300, 200, dts, True, 0, 5, scale)
+    h = cms.make_hashes(6, 200, 8192, 2)
+    c, kernels = run(cms, A, B, h)
+    assert "k_direct_tile" in kernels
+    assert worst(c, O.sketch_definition(Ad, Bd, O.make_tables(6, 200, 8192, 2))) < TOL
+    h.free()
+
+
+@pytest.mark.parametrize("n2", [40, 200])            # transform route, direct route
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_non_finite_operands_give_nan_on_both_routes(cms, n2, value):
+    A, B, _, _ = operands(200, n2, 200, "f32", False, 0, 9)
+    A[3, n2 // 2] = value
+    h = cms.make_hashes(6, 200, 8192, 2)
+    c, kernels = run(cms, A, B, h)
+    assert ("k_direct_tile" in kernels) == (n2 >= 64)
+    assert torch.isnan(c).all()
+    A.zero_()
+    c, _ = run(cms, A, B, h)
+    assert torch.count_nonzero(c).item() == 0
+    h.free()
+
+
+def test_workspace_of_the_transform_route_still_serves(cms):
+    # a workspace smaller than the direct route's layout: the transform route
+    A, B, Ad, Bd = operands(400, 4000, 400, "f32", True, 0, 11)
+    h = cms.make_hashes(12, 400, 4096, 1)
+    full = cms.workspace_size(h, 400, 4000, 400)
+    c, kernels = run(cms, A, B, h, ws=cms.alloc_workspace(full))
+    assert "k_direct_tile" in kernels
+    c2, kernels = run(cms, A, B, h, ws=cms.alloc_workspace(6 << 20))
+    assert (6 << 20) < full and "k_direct_tile" not in kernels
+    ref = O.sketch_definition(Ad, Bd, O.make_tables(12, 400, 4096, 1))
+    assert worst(c, ref) < TOL and worst(c2, ref) < 1e-5
+    h.free()
+
+
+def test_batch_of_both_routes(cms):
+    # instances on the direct route beside instances on the transform route
+    # (few inner indices), twice: the sums are left zero for the next run
+    items, refs = [], []
+    for q, (n, m, dts) in enumerate([(300, 700, "f32"), (600, 40, "f32"), (500, 900, "bf16"), (450, 30, "bf16")]):
+        A, B, Ad, Bd = operands(n, m, n, dts, True, 0, 20 + q)
+        items.append((A, B, cms.make_hashes(30 + q, n, 16 * n, 2)))
+        refs.append(O.sketch_definition(Ad, Bd, O.make_tables(30 + q, n, 16 * n, 2)))
+    batch = cms.Batch(items)
+    for _ in range(2):
+        cms.profile_enable(True)
+        batch.run()
+        torch.cuda.synchronize()
+        kernels = cms.profile_summary()
+        cms.profile_enable(False)
+        cms.check_async()
+        assert kernels["k_direct_tile_batched"]["launches"] == 1 and kernels["k_sketch_batched"]["launches"] == 1
+        for c, ref in zip(batch.c, refs):
+            assert worst(c, ref) < 1e-5
+            c.zero_()
+    batch.free()

@@ -246,7 +246,10 @@ CMS_API cms_status cms_sketch_product_noalloc(const void* A, int64_t lda, const 
  * column of A and of a row of B can be listed in linear time; Theorem 5's
  * exact recovery of sparse products).  Only inner indices k whose column
  * a_k and row b_k both have nonzeros contribute; they are compacted on the
- * device in increasing k.  Result as cms_sketch_product.
+ * device in increasing k.  An inner index whose outer product a_k b_k has at
+ * most b log2(b) / 50 terms is sketched term by term (cheaper than two
+ * transforms; integer sums, whose order does not matter), the others by the
+ * FFT route, and the two parts are added.  Result as cms_sketch_product.
  *   a_colptr : device int64 [n2 + 1], CSC column pointers of A (n1 x n2).
  *   a_rowidx : device int32, row index of each nonzero of A (< n1).
  *   a_val    : device values of A, storage type dt.
@@ -257,7 +260,7 @@ CMS_API cms_status cms_sketch_product_noalloc(const void* A, int64_t lda, const 
  *   b must be a multiple of 1024 (CMS_ERR_UNSUPPORTED otherwise).
  *   Asynchronous: the list of nonempty k and its length stay on the device
  *   (the FFT route runs the workspace's worst-case chunking and reads the
- *   length there), so the call never waits for the stream and can be
+ *   length there, and returns at once when it is zero), so the call never waits for the stream and can be
  *   captured in a CUDA graph.
  */
 CMS_API cms_status cms_sparse_workspace_size(const cms_hashes* h, int64_t n1, int64_t n2,

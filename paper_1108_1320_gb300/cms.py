@@ -317,8 +317,9 @@ def sketch_product_csr(a_colptr: torch.Tensor, a_rowidx: torch.Tensor, a_val: to
 
     ``direct_max_pairs`` selects the sparse-k hybrid (cms_sketch_product_csr_hybrid):
     inner indices with at most that many outer-product terms are sketched
-    directly (-1: the library's default split); None keeps every inner index
-    on the FFT route."""
+    directly in FP64 (-1: the library's default split, 0: none, every inner
+    index on the FFT route); None leaves the split to the library, the direct
+    part in integer sums (the same bits in every run)."""
     n2 = a_colptr.numel() - 1
     if b_rowptr.numel() - 1 != n2:
         raise ValueError("A and B disagree on the inner dimension")

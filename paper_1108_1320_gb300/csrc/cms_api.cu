@@ -442,50 +442,75 @@ cms_status cms_sparse_workspace_size(const cms_hashes* h, int64_t n1, int64_t n2
   return CMS_OK;
 }
 
-cms_status cms_sketch_product_csr(const int64_t* a_colptr, const int32_t* a_rowidx, const void* a_val,
-                                  const int64_t* b_rowptr, const int32_t* b_colidx, const void* b_val,
-                                  int64_t n1, int64_t n2, int64_t n3, int32_t dt, const cms_hashes* h,
-                                  float* c, void* ws, size_t ws_bytes, void* stream) {
-  NvtxRange nvtx_range("cms_sketch_product_csr");
+namespace {
+// The sparse product: inner indices whose outer product has at most `limit`
+// terms are sketched directly, the others by the FFT route.  integer: the
+// direct part in integer sums (the same bits in every run), else in FP64.
+cms_status sparse_product(const char* name, const int64_t* a_colptr, const int32_t* a_rowidx, const void* a_val,
+                          const int64_t* b_rowptr, const int32_t* b_colidx, const void* b_val, int64_t n1, int64_t n2,
+                          int64_t n3, int32_t dt, const cms_hashes* h, int64_t limit, int integer, float* c, void* ws,
+                          size_t ws_bytes, void* stream) {
+  DeviceProps dp = device_props(h->device);
+  SketchPlan plan;
+  size_t off_klist = 0;
+  std::string why;
+  int r = make_sparse_plan(h, n2, -1, dp.sms, dp.smem_optin, &plan, &off_klist, &why);
+  if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
+  if (!ws || ws_bytes < plan.ws_bytes)
+    return fail(CMS_ERR_WORKSPACE, "workspace missing or smaller than cms_sparse_workspace_size()");
+  if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return fail(CMS_ERR_WORKSPACE, "workspace must be 256-byte aligned");
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  char* w = static_cast<char*>(ws);
+  int32_t* flist = reinterpret_cast<int32_t*>(w + off_klist);
+  int32_t* dlist = reinterpret_cast<int32_t*>(w + plan.off_dlist);
+  int32_t* counts = dlist + std::max<int64_t>(n2, 1);
+  double* cd = reinterpret_cast<double*>(w + plan.off_cd);
+  SparseArgsHost in{a_colptr, a_rowidx, a_val, b_rowptr, b_colidx, b_val, static_cast<int>(n1),
+                    static_cast<int>(n3)};
+  // both lists and their lengths stay on the device (no host wait): the FFT
+  // route and the inverse return at once when its list is empty, and the
+  // direct scatter strides over the direct list's length
+  cudaError_t e = launch_nonempty_split(h, in, dt, n2, limit, integer, flist, dlist, counts, counts + 2, cd, s);
+  if (e != cudaSuccess) return cuda_fail(e, (std::string(name) + " (inner-index split)").c_str());
+  float2* partial = reinterpret_cast<float2*>(w + plan.off_partial);
+  float2* V = reinterpret_cast<float2*>(w + plan.off_V);
+  float2* twC = reinterpret_cast<float2*>(w + plan.off_twC);
+  float2* twR = reinterpret_cast<float2*>(w + plan.off_twR);
+  e = launch_twiddle_tables(twC, static_cast<int>(plan.C), twR, static_cast<int>(plan.R), s, counts);
+  if (e == cudaSuccess) e = launch_sketch_sparse(plan, h, in, dt, flist, counts, 1, partial, s);
+  if (e == cudaSuccess) e = launch_inverse(plan, partial, V, twC, twR, c, s, counts);
+  if (e == cudaSuccess) e = launch_direct_scatter(h, in, dt, integer, dlist, counts, n2, cd, s);
+  if (e == cudaSuccess) e = launch_add_direct(h, c, cd, integer, counts, s);
+  if (e != cudaSuccess) return cuda_fail(e, name);
+  return CMS_OK;
+}
+
+cms_status check_sparse_call(const cms_hashes* h, const int64_t* a_colptr, const int64_t* b_rowptr, int64_t n1,
+                             int64_t n2, int64_t n3, int32_t dt, const float* c) {
   cms_status st = check_shapes(h, n1, n2, n3, std::max<int64_t>(n1, 1), std::max<int64_t>(n3, 1));
   if (st != CMS_OK) return st;
   if (!valid_dtype(dt)) return fail(CMS_ERR_INVALID_ARG, "unknown dtype");
   if (!c) return fail(CMS_ERR_INVALID_ARG, "c is NULL");
   if (n2 > 0 && (!a_colptr || !b_rowptr)) return fail(CMS_ERR_INVALID_ARG, "pointer array is NULL");
   if (n2 >= (1LL << 31) - 1) return fail(CMS_ERR_INVALID_ARG, "n2 too large for int32 inner indices");
-  st = check_device(h);
+  return check_device(h);
+}
+}  // namespace
+
+cms_status cms_sketch_product_csr(const int64_t* a_colptr, const int32_t* a_rowidx, const void* a_val,
+                                  const int64_t* b_rowptr, const int32_t* b_colidx, const void* b_val,
+                                  int64_t n1, int64_t n2, int64_t n3, int32_t dt, const cms_hashes* h,
+                                  float* c, void* ws, size_t ws_bytes, void* stream) {
+  NvtxRange nvtx_range("cms_sketch_product_csr");
+  cms_status st = check_sparse_call(h, a_colptr, b_rowptr, n1, n2, n3, dt, c);
   if (st != CMS_OK) return st;
-  DeviceProps dp = device_props(h->device);
-  SketchPlan worst;
-  size_t off_klist = 0;
-  std::string why;
-  int r = make_sparse_plan(h, n2, -1, dp.sms, dp.smem_optin, &worst, &off_klist, &why);
-  if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
-  if (!ws || ws_bytes < worst.ws_bytes)
-    return fail(CMS_ERR_WORKSPACE, "workspace missing or smaller than cms_sparse_workspace_size()");
-  if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return fail(CMS_ERR_WORKSPACE, "workspace must be 256-byte aligned");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  char* w = static_cast<char*>(ws);
-  int32_t* klist = reinterpret_cast<int32_t*>(w + off_klist);
-  int32_t* dlist = reinterpret_cast<int32_t*>(w + worst.off_dlist);
-  int32_t* counts = dlist + std::max<int64_t>(n2, 1);
-  // the list of nonempty inner indices and its length stay on the device:
-  // the FFT route runs the plan's worst-case chunking and reads the length
-  // there, so the call returns without waiting for the GPU
-  cudaError_t e = launch_nonempty_split(a_colptr, b_rowptr, n2, -1, klist, dlist, counts, counts + 2, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cms_sketch_product_csr (nonempty inner indices)");
-  const SketchPlan& plan = worst;
-  float2* partial = reinterpret_cast<float2*>(w + plan.off_partial);
-  float2* V = reinterpret_cast<float2*>(w + plan.off_V);
-  float2* twC = reinterpret_cast<float2*>(w + plan.off_twC);
-  float2* twR = reinterpret_cast<float2*>(w + plan.off_twR);
-  SparseArgsHost in{a_colptr, a_rowidx, a_val, b_rowptr, b_colidx, b_val, static_cast<int>(n1),
-                    static_cast<int>(n3)};
-  e = launch_twiddle_tables(twC, static_cast<int>(plan.C), twR, static_cast<int>(plan.R), s);
-  if (e == cudaSuccess) e = launch_sketch_sparse(plan, h, in, dt, klist, counts, 0, partial, s);
-  if (e == cudaSuccess) e = launch_inverse(plan, partial, V, twC, twR, c, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cms_sketch_product_csr");
-  return CMS_OK;
+  // a term costs one addition per repetition (205 G/s), an inner index on
+  // the FFT route about 5 b log2(b) flops per repetition at 52 TFLOP/s: equal
+  // at b log2(b) / 50 terms
+  const int64_t limit = static_cast<int64_t>(static_cast<double>(h->b) *
+                                             std::log2(static_cast<double>(std::max<int64_t>(h->b, 2))) / 50.0);
+  return sparse_product("cms_sketch_product_csr", a_colptr, a_rowidx, a_val, b_rowptr, b_colidx, b_val, n1, n2, n3, dt,
+                        h, limit, 1, c, ws, ws_bytes, stream);
 }
 
 cms_status cms_sketch_product_csr_hybrid(const int64_t* a_colptr, const int32_t* a_rowidx, const void* a_val,
@@ -494,56 +519,16 @@ cms_status cms_sketch_product_csr_hybrid(const int64_t* a_colptr, const int32_t*
                                          int64_t direct_max_pairs, float* c, void* ws, size_t ws_bytes,
                                          void* stream) {
   NvtxRange nvtx_range("cms_sketch_product_csr_hybrid");
-  cms_status st = check_shapes(h, n1, n2, n3, std::max<int64_t>(n1, 1), std::max<int64_t>(n3, 1));
+  cms_status st = check_sparse_call(h, a_colptr, b_rowptr, n1, n2, n3, dt, c);
   if (st != CMS_OK) return st;
-  if (!valid_dtype(dt)) return fail(CMS_ERR_INVALID_ARG, "unknown dtype");
-  if (!c) return fail(CMS_ERR_INVALID_ARG, "c is NULL");
-  if (n2 > 0 && (!a_colptr || !b_rowptr)) return fail(CMS_ERR_INVALID_ARG, "pointer array is NULL");
-  if (n2 >= (1LL << 31) - 1) return fail(CMS_ERR_INVALID_ARG, "n2 too large for int32 inner indices");
-  st = check_device(h);
-  if (st != CMS_OK) return st;
-  DeviceProps dp = device_props(h->device);
-  SketchPlan worst;
-  size_t off_klist = 0;
-  std::string why;
-  int r = make_sparse_plan(h, n2, -1, dp.sms, dp.smem_optin, &worst, &off_klist, &why);
-  if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
-  if (!ws || ws_bytes < worst.ws_bytes)
-    return fail(CMS_ERR_WORKSPACE, "workspace missing or smaller than cms_sparse_workspace_size()");
-  if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return fail(CMS_ERR_WORKSPACE, "workspace must be 256-byte aligned");
   // default split: direct when the outer product has at most 5 b log2(b) / 64
   // terms (the FFT route costs about 5 b log2 b flops per inner index)
   const int64_t limit = direct_max_pairs >= 0
                             ? direct_max_pairs
                             : static_cast<int64_t>(5.0 * static_cast<double>(h->b) *
                                                    std::log2(static_cast<double>(std::max<int64_t>(h->b, 2))) / 64.0);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  char* w = static_cast<char*>(ws);
-  int32_t* flist = reinterpret_cast<int32_t*>(w + off_klist);
-  int32_t* dlist = reinterpret_cast<int32_t*>(w + worst.off_dlist);
-  int32_t* counts = dlist + std::max<int64_t>(n2, 1);
-  double* cd = reinterpret_cast<double*>(w + worst.off_cd);
-  // both lists and their lengths stay on the device (no host wait): the FFT
-  // route and the inverse return at once when its list is empty, and the
-  // direct scatter strides over the direct list's length
-  cudaError_t e = launch_nonempty_split(a_colptr, b_rowptr, n2, limit, flist, dlist, counts, counts + 2, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cms_sketch_product_csr_hybrid (inner-index split)");
-  const SketchPlan& plan = worst;
-  SparseArgsHost in{a_colptr, a_rowidx, a_val, b_rowptr, b_colidx, b_val, static_cast<int>(n1),
-                    static_cast<int>(n3)};
-  {
-    float2* partial = reinterpret_cast<float2*>(w + plan.off_partial);
-    float2* V = reinterpret_cast<float2*>(w + plan.off_V);
-    float2* twC = reinterpret_cast<float2*>(w + plan.off_twC);
-    float2* twR = reinterpret_cast<float2*>(w + plan.off_twR);
-    e = launch_twiddle_tables(twC, static_cast<int>(plan.C), twR, static_cast<int>(plan.R), s);
-    if (e == cudaSuccess) e = launch_sketch_sparse(plan, h, in, dt, flist, counts, 1, partial, s);
-    if (e == cudaSuccess) e = launch_inverse(plan, partial, V, twC, twR, c, s, counts);
-  }
-  if (e == cudaSuccess) e = launch_direct_scatter(h, in, dt, dlist, counts, n2, cd, s);
-  if (e == cudaSuccess) e = launch_add_direct(c, cd, static_cast<int64_t>(h->d) * h->b, counts, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cms_sketch_product_csr_hybrid");
-  return CMS_OK;
+  return sparse_product("cms_sketch_product_csr_hybrid", a_colptr, a_rowidx, a_val, b_rowptr, b_colidx, b_val, n1, n2,
+                        n3, dt, h, limit, 0, c, ws, ws_bytes, stream);
 }
 
 cms_status cms_plain_workspace_size(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3,

@@ -207,7 +207,8 @@ cudaError_t launch_sketch(const SketchPlan& plan, const cms_hashes* h,
 cudaError_t launch_inverse(const SketchPlan& plan, const float2* partial, float2* V, const float2* twC,
                            const float2* twR, float* c, cudaStream_t s,
                            const int32_t* skip_if_zero = nullptr);
-cudaError_t launch_twiddle_tables(float2* twC, int C, float2* twR, int R, cudaStream_t s);
+cudaError_t launch_twiddle_tables(float2* twC, int C, float2* twR, int R, cudaStream_t s,
+                                  const int32_t* skip_if_zero = nullptr);
 
 // Reduction + inverse of many products in two launches (a batch): each
 // instance's plan, partial rows, row spectra, twiddle tables and output; for
@@ -256,13 +257,18 @@ int make_sparse_plan(const cms_hashes* h, int64_t n2, int64_t K, int num_sms, si
                      SketchPlan* plan, size_t* off_klist, std::string* why);
 // Ordered split of the nonempty inner indices into the FFT list (flist)
 // and the direct list (dlist; limit < 0: none); counts[0..1] their lengths;
-// scratch holds 2 x 1024 ints.
-cudaError_t launch_nonempty_split(const int64_t* a_ptr, const int64_t* b_ptr, int64_t n2, int64_t limit,
-                                  int32_t* flist, int32_t* dlist, int32_t* counts, int32_t* scratch, cudaStream_t s);
+// scratch holds 2 x 1024 ints.  Zeroes the direct part's sums cd; integer:
+// also measures the direct list's terms for launch_direct_scatter.
+cudaError_t launch_nonempty_split(const cms_hashes* h, const SparseArgsHost& in, int dt, int64_t n2, int64_t limit,
+                                  int integer, int32_t* flist, int32_t* dlist, int32_t* counts, int32_t* scratch,
+                                  double* cd, cudaStream_t s);
 // The direct list's length is read on the device (counts[1]); n2 bounds it.
-cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, const int32_t* dlist,
-                                  const int32_t* counts, int64_t n2, double* cd, cudaStream_t s);
-cudaError_t launch_add_direct(float* c, const double* cd, int64_t len, const int32_t* counts, cudaStream_t s);
+// integer: sums of integers at a common scale (the same in any order), else
+// FP64 sums.
+cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer,
+                                  const int32_t* dlist, const int32_t* counts, int64_t n2, double* cd, cudaStream_t s);
+cudaError_t launch_add_direct(const cms_hashes* h, float* c, double* cd, int integer, const int32_t* counts,
+                              cudaStream_t s);
 // FFT route over the nonempty inner indices klist[0..*kcount) (the length is
 // read on the device, so the call needs no host wait); plan.nkc chunks per
 // (repetition, row), trailing ones empty.  skip_empty: blocks return at once
@@ -333,10 +339,17 @@ struct DirectScale {
 // range), BF16 ones to below 2.
 __host__ __device__ constexpr int direct_scale_log2(bool split) { return split ? 14 : 0; }
 #ifdef __CUDACC__
+// v 2^e for 0 or 1 <= |v| < 2^63, rounded once (each factor is a power of
+// two and only the second product can leave the normal range): ldexpf's
+// result at a fraction of its instructions.
+__device__ __forceinline__ float scale_pow2(float v, int e) {
+  e = min(max(e, -252), 252);
+  return v * __int_as_float((e / 2 + 127) << 23) * __int_as_float((e - e / 2 + 127) << 23);
+}
 // A bucket from its integer sum.
 __device__ __forceinline__ float direct_value(unsigned long long sum, const DirectScale& sc, int log2s) {
   if (sc.bad) return __int_as_float(0x7FC00000);
-  return ldexpf(__ll2float_rn(static_cast<long long>(sum)), sc.emax[0] + sc.emax[1] - 2 * log2s - sc.shift);
+  return scale_pow2(__ll2float_rn(static_cast<long long>(sum)), sc.emax[0] + sc.emax[1] - 2 * log2s - sc.shift);
 }
 #endif
 

@@ -50,7 +50,9 @@ __device__ __forceinline__ float2 w_pow(uint64_t m, int64_t M) {
 // hi[i] = w_b^{i S} for i < nhi (the high half of the warp-specialised
 // kernel's split twiddle w_b^m = w_b^{m mod S} w_b^{(m div S) S}).
 __global__ void k_twiddle_table(float2* __restrict__ tw, int M, float2* __restrict__ hi, int S, int nhi,
-                                int64_t b, float2* __restrict__ tw2, int M2) {
+                                int64_t b, float2* __restrict__ tw2, int M2,
+                                const int32_t* __restrict__ skip_if_zero) {
+  if (skip_if_zero && *skip_if_zero == 0) return;
   // blocks [0, nbt): w_M^m; then, when hi is given, nbh blocks of w_b^{i S};
   // then, when tw2 is given, the blocks of w_M2^m (one launch for all three)
   const int nbt = (M + 255) / 256;
@@ -534,7 +536,7 @@ cudaError_t launch_sketch(const SketchPlan& plan, const cms_hashes* h, const voi
     float2* hi = plan.ws ? reinterpret_cast<float2*>(ws + plan.off_thi) : nullptr;
     const int R = static_cast<int>(plan.R);
     k_twiddle_table<<<twiddle_blocks(static_cast<int>(plan.C), hi, plan.nhi, twR, R), 256, 0, s>>>(
-        twC, static_cast<int>(plan.C), hi, 1 << plan.tw_shift, plan.nhi, plan.b, twR, R);
+        twC, static_cast<int>(plan.C), hi, 1 << plan.tw_shift, plan.nhi, plan.b, twR, R, nullptr);
   }
   if (!plan.fast) {
     dim3 grid(static_cast<unsigned>(std::min<int64_t>((n + 255) / 256, 64)), plan.nrows, 2 * plan.d);
@@ -605,10 +607,11 @@ cudaError_t launch_frontend_twiddles(const SketchPlan& plan, const cms_hashes* h
   return cudaGetLastError();
 }
 
-cudaError_t launch_twiddle_tables(float2* twC, int C, float2* twR, int R, cudaStream_t s) {
+cudaError_t launch_twiddle_tables(float2* twC, int C, float2* twR, int R, cudaStream_t s,
+                                  const int32_t* skip_if_zero) {
   {
     ProfScope prof_scope("k_twiddle_table", s);
-    k_twiddle_table<<<twiddle_blocks(C, nullptr, 0, twR, R), 256, 0, s>>>(twC, C, nullptr, 1, 0, 1, twR, R);
+    k_twiddle_table<<<twiddle_blocks(C, nullptr, 0, twR, R), 256, 0, s>>>(twC, C, nullptr, 1, 0, 1, twR, R, skip_if_zero);
   }
   return cudaGetLastError();
 }

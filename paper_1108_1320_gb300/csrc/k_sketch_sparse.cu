@@ -15,6 +15,7 @@
 // accumulation, exactly as in k_sketch_fast.cu.
 #include <algorithm>
 #include <cstdlib>
+#include <type_traits>
 
 #include "cms_internal.h"
 #include "warp_fft.cuh"
@@ -46,6 +47,7 @@ struct SparseArgs {
   int nkc;                     // k-chunks per (repetition, row): fixed by the launch
   const int32_t* klist;
   const int32_t* kcount;       // device: length of klist (written by the split kernels)
+  int ntask;
   int skip_empty;              // 1: a block returns at once when the list is empty
   int sepy;                    // 1: scatter into per-warp Y buffers kept zero between groups
   const uint32_t* hs;
@@ -70,8 +72,9 @@ size_t sparse_smem_bytes(int tw_shift, int nhi, bool sepy) {
          (sepy ? static_cast<size_t>(2 * kG) * kC * 8 : 0);
 }
 
+// One (repetition, row, chunk of the list).
 template <typename T>
-__global__ void __launch_bounds__(kThreads, 1) k_sketch_sparse(SparseArgs p) {
+__device__ __forceinline__ void sparse_task(const SparseArgs& p, int task) {
   extern __shared__ __align__(128) unsigned char sm[];
   float2* work = reinterpret_cast<float2*>(sm);
   float4* acc = reinterpret_cast<float4*>(sm + static_cast<size_t>(2 * kG) * kRegion * 8);
@@ -82,7 +85,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_sketch_sparse(SparseArgs p) {
   float2* ysc = thi + p.nhi;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int task = blockIdx.x;
   const int kc = task % p.nkc;
   const int row = (task / p.nkc) % p.nrows;
   const int t = task / (p.nkc * p.nrows);
@@ -92,7 +94,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_sketch_sparse(SparseArgs p) {
   // the chunking follows the list length found on the device: nkc chunks of
   // a whole number of groups; trailing chunks may be empty (zero partials)
   const int K = *p.kcount;
-  if (p.skip_empty && K == 0) return;
   const int kchunk = max(kG, ((K + p.nkc - 1) / p.nkc + kG - 1) / kG * kG);
   const int l_begin = min(K, kc * kchunk);
   const int l_end = min(K, l_begin + kchunk);
@@ -361,14 +362,27 @@ __global__ void __launch_bounds__(kThreads, 1) k_sketch_sparse(SparseArgs p) {
   }
 }
 
+// A few blocks per SM over all tasks: with a block per task the launch took
+// 33 us when the list was empty (6156 blocks of the exact sparse workload,
+// each alone on its SM, only to return), now 5 us.
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1) k_sketch_sparse(const SparseArgs p) {
+  if (p.skip_empty && *p.kcount == 0) return;
+  for (int task = blockIdx.x; task < p.ntask; task += gridDim.x) {
+    sparse_task<T>(p, task);
+    __syncthreads();   // the next task initialises the shared memory that this one read
+  }
+}
+
 // Sparse-k hybrid: the nonempty inner indices split, in increasing k, into
 // those whose outer product a_k b_k has at most `limit` terms (sketched
 // directly, Sec. 2.2 "sketching a matrix product naively") and the rest
 // (the FFT route); limit < 0 sends every nonempty index to the FFT route.
-// Three passes over contiguous chunks of k (one block each): counts per
-// chunk, an exclusive scan of the chunk counts, and an ordered write of
-// every chunk from its offsets.  counts[0] = FFT list length, counts[1] =
-// direct list length.
+// Two passes over contiguous chunks of k (one block each): counts per
+// chunk, and an ordered write of every chunk behind the chunks before it
+// (each block adds up their counts; a scan kernel of its own between the two
+// cost 6 us of the call).  counts[0] = FFT list length, counts[1] = direct
+// list length.
 __device__ __forceinline__ void classify_k(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_ptr,
                                            int64_t n2, int64_t limit, int64_t k, bool* fft, bool* direct) {
   int64_t na = 0, nb = 0;
@@ -381,20 +395,70 @@ __device__ __forceinline__ void classify_k(const int64_t* __restrict__ a_ptr, co
   *fft = live && !*direct;
 }
 
+// Largest magnitude of n values as the bits of an FP32 number (rounded up;
+// infinities and NaN stay above every finite value); the whole warp.
+__device__ __forceinline__ uint32_t abs_bits(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ uint32_t abs_bits(__nv_bfloat16 v) { return abs_bits(__bfloat162float(v)); }
+__device__ __forceinline__ uint32_t abs_bits(double v) { return abs_bits(__double2float_ru(fabs(v))); }
+
+template <typename T>
+__device__ __forceinline__ uint32_t warp_max_abs(const T* __restrict__ v, const int32_t* __restrict__ idx, int64_t n,
+                                                 int nside) {
+  uint32_t m = 0;
+  for (int64_t q = threadIdx.x & 31; q < n; q += 32)
+    if (idx[q] >= 0 && idx[q] < nside) m = max(m, abs_bits(v[q]));
+  return __reduce_max_sync(0xFFFFFFFFu, m);
+}
+
+// What the integer sums of the direct part need: the largest product of a
+// direct inner index, and the number of terms.
+struct DirectTerms {
+  unsigned long long terms;
+  uint32_t max_bits;       // of an FP32 number
+  uint32_t unused;
+};
+
+// Power of two by which a term is scaled before it is rounded to an integer:
+// the sum of all terms stays below 2^62 (terms < 2^bits, each < 2^(e + 1)).
+__device__ __forceinline__ int term_shift(const DirectTerms& m) {
+  if (m.max_bits == 0) return 0;
+  const int bits = 64 - __clzll(static_cast<long long>(m.terms));
+  const int e = max(static_cast<int>(m.max_bits >> 23), 1) - 127;
+  return 62 - bits - (e + 1);
+}
+
+template <typename T>
 __global__ void __launch_bounds__(1024)
 k_split_count(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_ptr, int64_t n2, int64_t limit,
-              int64_t chunk, int32_t* __restrict__ part) {
+              int64_t chunk, int32_t* __restrict__ part, const int32_t* __restrict__ a_idx,
+              const T* __restrict__ a_val, const int32_t* __restrict__ b_idx, const T* __restrict__ b_val, int n1,
+              int n3, DirectTerms* __restrict__ terms) {
   __shared__ int32_t tot[2];
   if (threadIdx.x < 2) tot[threadIdx.x] = 0;
   __syncthreads();
   const int64_t k0 = static_cast<int64_t>(blockIdx.x) * chunk;
   const int64_t k1 = min(n2, k0 + chunk);
   int cf = 0, cd = 0;
-  for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-    bool f, dr;
-    classify_k(a_ptr, b_ptr, n2, limit, k, &f, &dr);
+  unsigned long long nterm = 0;
+  uint32_t mx = 0;
+  for (int64_t base = k0; base < k1; base += blockDim.x) {
+    const int64_t k = base + threadIdx.x;
+    bool f = false, dr = false;
+    if (k < k1) classify_k(a_ptr, b_ptr, n2, limit, k, &f, &dr);
     cf += f;
     cd += dr;
+    if (terms == nullptr) continue;
+    // the warp measures its direct inner indices one after the other
+    for (unsigned todo = __ballot_sync(0xFFFFFFFFu, dr); todo; todo &= todo - 1) {
+      const int64_t kk = base + (threadIdx.x & ~31u) + __ffs(todo) - 1;
+      const int64_t a0 = a_ptr[kk], na = a_ptr[kk + 1] - a0, b0 = b_ptr[kk], nb = b_ptr[kk + 1] - b0;
+      const uint32_t ma = warp_max_abs(a_val + a0, a_idx + a0, na, n1);
+      const uint32_t mb = warp_max_abs(b_val + b0, b_idx + b0, nb, n3);
+      nterm += static_cast<unsigned long long>(na * nb);
+      const uint32_t inf = 0x7F800000u;
+      mx = max(mx, ma >= inf || mb >= inf ? 0x7FC00000u
+                                          : __float_as_uint(__fmul_ru(__uint_as_float(ma), __uint_as_float(mb))));
+    }
   }
   for (int o = 16; o > 0; o >>= 1) {
     cf += __shfl_down_sync(0xFFFFFFFFu, cf, o);
@@ -403,45 +467,32 @@ k_split_count(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_p
   if ((threadIdx.x & 31) == 0) {
     atomicAdd(&tot[0], cf);
     atomicAdd(&tot[1], cd);
+    if (nterm > 0) {
+      atomicAdd(&terms->terms, nterm);
+      atomicMax(&terms->max_bits, mx);
+    }
   }
   __syncthreads();
   if (threadIdx.x < 2) part[2 * blockIdx.x + threadIdx.x] = tot[threadIdx.x];
 }
 
-// exclusive scan of the nblk chunk counts (nblk <= 1024) in place
-__global__ void __launch_bounds__(1024) k_split_scan(int32_t* __restrict__ part, int nblk,
-                                                     int32_t* __restrict__ counts) {
-  __shared__ int32_t wsum[2][32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int side = 0; side < 2; ++side) {
-    const int32_t v = tid < nblk ? part[2 * tid + side] : 0;
-    int32_t x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[side][warp] = x;
-    __syncthreads();
-    int32_t before = 0, total = 0;
-    for (int w = 0; w < 32; ++w) {
-      if (w < warp) before += wsum[side][w];
-      total += wsum[side][w];
-    }
-    if (tid < nblk) part[2 * tid + side] = before + x - v;
-    if (tid == 0) counts[side] = total;
-    __syncthreads();
-  }
-}
-
 __global__ void __launch_bounds__(1024)
 k_split_write(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_ptr, int64_t n2, int64_t limit,
               int64_t chunk, const int32_t* __restrict__ part, int32_t* __restrict__ flist,
-              int32_t* __restrict__ dlist) {
+              int32_t* __restrict__ dlist, int32_t* __restrict__ counts) {
   __shared__ int32_t warp_tot[2][32];
   __shared__ int32_t running[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 2) running[tid] = part[2 * blockIdx.x + tid];
+  // lengths of the lists before this chunk (at most 1024 chunks)
+  if (tid < 2) running[tid] = 0;
   __syncthreads();
+  for (int side = 0; side < 2; ++side) {
+    int32_t v = tid < static_cast<int>(blockIdx.x) ? part[2 * tid + side] : 0;
+    v = __reduce_add_sync(0xFFFFFFFFu, v);
+    if (lane == 0 && v > 0) atomicAdd(&running[side], v);
+  }
+  __syncthreads();
+  if (blockIdx.x == gridDim.x - 1 && tid < 2) counts[tid] = running[tid] + part[2 * blockIdx.x + tid];
   const int64_t k0 = static_cast<int64_t>(blockIdx.x) * chunk;
   const int64_t k1 = min(n2, k0 + chunk);
   for (int64_t base = k0; base < k1; base += 1024) {
@@ -476,32 +527,81 @@ template <> __device__ __forceinline__ double val_f64<__nv_bfloat16>(const __nv_
 
 // Direct sketch of the outer products of the listed inner indices: for every
 // nonzero pair (A_ik, B_kj) and repetition t, s1(i) s2(j) A_ik B_kj goes to
-// bucket (h1(i) + h2(j)) mod b of an FP64 accumulator (products of two FP32
-// or BF16 values are exact in FP64; the additions are atomic, so their order
-// varies, at FP64 rounding).  One block per listed k at a time.
-template <typename T>
+// bucket (h1(i) + h2(j)) mod b.  One block per listed k at a time; the values
+// and hashes of up to kDirA x kDirB nonzeros sit in shared memory, so that a
+// term costs its addition alone (6.3 M random 64-bit reductions of the exact
+// sparse workload: 31 us at the chip's 205 G/s; with the hashes read per term
+// and a 64-bit division per pair 42 us).
+//  INT: terms rounded to integers at a common scale (term_shift) and added
+//       as 64-bit integers: the same sums in any order.
+//  else: FP64 (products of two FP32 or BF16 values are exact), added
+//       atomically: their order varies, at FP64 rounding.
+constexpr int kDirA = 32, kDirB = 128, kDirT = 8;
+
+template <typename T, bool INT>
 __global__ void __launch_bounds__(256)
 k_direct_scatter(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ a_idx, const T* __restrict__ a_val,
                  const int64_t* __restrict__ b_ptr, const int32_t* __restrict__ b_idx, const T* __restrict__ b_val,
                  int n1, int n3, int64_t n, const int32_t* __restrict__ dlist, const int32_t* __restrict__ counts,
-                 const uint32_t* __restrict__ hs, int d, int64_t b, double* __restrict__ cd) {
+                 const uint32_t* __restrict__ hs, int d, int64_t b, double* __restrict__ cd,
+                 const DirectTerms* __restrict__ terms) {
+  __shared__ double va[kDirA], vb[kDirB];
+  __shared__ int xa[kDirA], xb[kDirB];
+  __shared__ uint32_t wa[kDirT][kDirA], wb_[kDirT][kDirB];
   const int Kd = counts[1];
+  const int tid = threadIdx.x;
+  double up = 1.0;
+  if (INT) {
+    if (Kd == 0 || terms->max_bits >= 0x7F800000u) return;   // the conversion writes NaN
+    up = ldexp(1.0, term_shift(*terms));
+  }
   for (int q = blockIdx.x; q < Kd; q += gridDim.x) {
     const int64_t k = dlist[q];
     const int64_t a0 = a_ptr[k], na = a_ptr[k + 1] - a0;
     const int64_t b0 = b_ptr[k], nb = b_ptr[k + 1] - b0;
-    for (int64_t pr = threadIdx.x; pr < na * nb; pr += blockDim.x) {
-      const int64_t ia = a0 + pr / nb, jb = b0 + pr % nb;
-      const int i = a_idx[ia], j = b_idx[jb];
-      if (i < 0 || i >= n1 || j < 0 || j >= n3) continue;
-      const double v = val_f64<T>(a_val, ia) * val_f64<T>(b_val, jb);
-      for (int t = 0; t < d; ++t) {
-        const uint32_t w1 = hs[(static_cast<size_t>(t) * 2 + 0) * n + i];
-        const uint32_t w2 = hs[(static_cast<size_t>(t) * 2 + 1) * n + j];
-        uint64_t z = static_cast<uint64_t>(w1 & kBucketMask) + (w2 & kBucketMask);
-        if (z >= static_cast<uint64_t>(b)) z -= static_cast<uint64_t>(b);
-        const double sv = ((w1 ^ w2) >> 31) ? -v : v;
-        atomicAdd(&cd[static_cast<size_t>(t) * b + z], sv);
+    for (int64_t ca = 0; ca < na; ca += kDirA) {
+      const int la = static_cast<int>(min(na - ca, static_cast<int64_t>(kDirA)));
+      for (int64_t cb = 0; cb < nb; cb += kDirB) {
+        const int lb = static_cast<int>(min(nb - cb, static_cast<int64_t>(kDirB)));
+        __syncthreads();
+        // an index outside the matrix marks its entry as none (-1)
+        if (tid < la) {
+          const int i = a_idx[a0 + ca + tid];
+          xa[tid] = i >= 0 && i < n1 ? i : -1;
+          va[tid] = val_f64<T>(a_val, a0 + ca + tid) * up;
+        } else if (tid >= kDirB && tid - kDirB < lb) {
+          const int j = b_idx[b0 + cb + tid - kDirB];
+          xb[tid - kDirB] = j >= 0 && j < n3 ? j : -1;
+          vb[tid - kDirB] = val_f64<T>(b_val, b0 + cb + tid - kDirB);
+        }
+        __syncthreads();
+        for (int t0 = 0; t0 < d; t0 += kDirT) {
+          const int lt = min(kDirT, d - t0);
+          if (t0 > 0) __syncthreads();
+          for (int e = tid; e < lt * (la + lb); e += 256) {
+            const int t = e / (la + lb), x = e - t * (la + lb);
+            const uint32_t* row = hs + static_cast<size_t>(t0 + t) * 2 * n;
+            if (x < la) wa[t][x] = xa[x] >= 0 ? row[xa[x]] : 0;
+            else wb_[t][x - la] = xb[x - la] >= 0 ? row[n + xb[x - la]] : 0;
+          }
+          __syncthreads();
+          for (int e = tid; e < la * lb; e += 256) {
+            const int i = e / lb, j = e - i * lb;
+            if (xa[i] < 0 || xb[j] < 0) continue;
+            // once per pair: FP64 arithmetic is slow beside the additions
+            const double v = va[i] * vb[j];
+            const long long iv = INT ? __double2ll_rn(v) : 0;
+            for (int t = 0; t < lt; ++t) {
+              const uint32_t w1 = wa[t][i], w2 = wb_[t][j];
+              uint32_t z = (w1 & kBucketMask) + (w2 & kBucketMask);
+              if (z >= static_cast<uint32_t>(b)) z -= static_cast<uint32_t>(b);
+              const bool neg = ((w1 ^ w2) >> 31) != 0;
+              double* dst = cd + static_cast<size_t>(t0 + t) * b + z;
+              if (INT) atomicAdd(reinterpret_cast<unsigned long long*>(dst), static_cast<unsigned long long>(neg ? -iv : iv));
+              else atomicAdd(dst, neg ? -v : v);
+            }
+          }
+        }
       }
     }
   }
@@ -509,12 +609,29 @@ k_direct_scatter(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ 
 
 // c = FFT-route c + direct part (rounded once to FP32), or the direct part
 // alone when no inner index took the FFT route.
+template <bool INT>
 __global__ void k_add_direct(float* __restrict__ c, const double* __restrict__ cd, int64_t len,
-                             const int32_t* __restrict__ counts) {
+                             const int32_t* __restrict__ counts, const DirectTerms* __restrict__ terms) {
   const bool fft = counts[0] > 0;
+  int shift = 0;
+  bool bad = false;
+  if (INT) {
+    if (counts[1] == 0 && fft) return;
+    bad = terms->max_bits >= 0x7F800000u;
+    shift = term_shift(*terms);
+  }
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < len;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    c[i] = static_cast<float>(fft ? static_cast<double>(c[i]) + cd[i] : cd[i]);
+       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const double v = cd[i];
+    if (INT && !fft) {   // without FP64 arithmetic (FP64 took 41 us for 3 x 2^20 buckets)
+      c[i] = bad ? __int_as_float(0x7FC00000) : scale_pow2(__ll2float_rn(__double_as_longlong(v)), -shift);
+    } else if (INT) {
+      const double w = ldexp(static_cast<double>(__double_as_longlong(v)), -shift);
+      c[i] = bad ? __int_as_float(0x7FC00000) : static_cast<float>(static_cast<double>(c[i]) + w);
+    } else {
+      c[i] = static_cast<float>(fft ? static_cast<double>(c[i]) + v : v);
+    }
+  }
 }
 
 }  // namespace
@@ -578,59 +695,73 @@ int make_sparse_plan(const cms_hashes* h, int64_t n2, int64_t K, int num_sms, si
   *off_klist = off;    off = align256(off + static_cast<size_t>(std::max<int64_t>(n2, 1) + 1) * 4);
   // sparse-k hybrid: the direct list, the list counts, the FP64 direct sketch
   p.off_dlist = off;   off = align256(off + (static_cast<size_t>(std::max<int64_t>(n2, 1)) + 2 + 2 * kSplitBlocks) * 4);
-  p.off_cd = off;      off = align256(off + static_cast<size_t>(p.d) * p.b * 8);
+  p.off_cd = off;      off = align256(off + static_cast<size_t>(p.d) * p.b * 8 + sizeof(DirectTerms));
   p.ws_bytes = off;
   (void)why;
   *plan = p;
   return CMS_OK;
 }
 
-cudaError_t launch_nonempty_split(const int64_t* a_ptr, const int64_t* b_ptr, int64_t n2, int64_t limit,
-                                  int32_t* flist, int32_t* dlist, int32_t* counts, int32_t* scratch, cudaStream_t s) {
+namespace {
+DirectTerms* direct_terms(const cms_hashes* h, double* cd) {
+  return reinterpret_cast<DirectTerms*>(cd + static_cast<size_t>(h->d) * h->b);
+}
+}  // namespace
+
+cudaError_t launch_nonempty_split(const cms_hashes* h, const SparseArgsHost& in, int dt, int64_t n2, int64_t limit,
+                                  int integer, int32_t* flist, int32_t* dlist, int32_t* counts, int32_t* scratch,
+                                  double* cd, cudaStream_t s) {
+  // the direct part's sums and its measure start at zero
+  cudaError_t e = cudaMemsetAsync(cd, 0, static_cast<size_t>(h->d) * h->b * sizeof(double) + sizeof(DirectTerms), s);
+  if (e != cudaSuccess) return e;
   if (n2 <= 0) return cudaMemsetAsync(counts, 0, 2 * sizeof(int32_t), s);
   const int64_t nblk = std::min<int64_t>(kSplitBlocks, (n2 + 1023) / 1024);
   const int64_t chunk = ((n2 + nblk - 1) / nblk + 1023) / 1024 * 1024;
   const unsigned g = static_cast<unsigned>((n2 + chunk - 1) / chunk);
   ProfScope prof_scope("k_nonempty_split", s);
-  k_split_count<<<g, 1024, 0, s>>>(a_ptr, b_ptr, n2, limit, chunk, scratch);
-  k_split_scan<<<1, 1024, 0, s>>>(scratch, static_cast<int>(g), counts);
-  k_split_write<<<g, 1024, 0, s>>>(a_ptr, b_ptr, n2, limit, chunk, scratch, flist, dlist);
+  auto count = [&](auto* tag) {
+    using T = std::remove_pointer_t<decltype(tag)>;
+    k_split_count<T><<<g, 1024, 0, s>>>(in.a_ptr, in.b_ptr, n2, limit, chunk, scratch, in.a_idx,
+                                        static_cast<const T*>(in.a_val), in.b_idx, static_cast<const T*>(in.b_val),
+                                        in.n1, in.n3, integer ? direct_terms(h, cd) : nullptr);
+  };
+  if (dt == CMS_F32) count(static_cast<float*>(nullptr));
+  else if (dt == CMS_BF16) count(static_cast<__nv_bfloat16*>(nullptr));
+  else count(static_cast<double*>(nullptr));
+  k_split_write<<<g, 1024, 0, s>>>(in.a_ptr, in.b_ptr, n2, limit, chunk, scratch, flist, dlist, counts);
   return cudaGetLastError();
 }
 
-cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, const int32_t* dlist,
-                                  const int32_t* counts, int64_t n2, double* cd, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(cd, 0, static_cast<size_t>(h->d) * h->b * sizeof(double), s);
-  if (e != cudaSuccess || n2 <= 0) return e;
+cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer,
+                                  const int32_t* dlist, const int32_t* counts, int64_t n2, double* cd, cudaStream_t s) {
+  if (n2 <= 0) return cudaSuccess;
   // the list length is on the device: blocks stride over it and those past
   // its end return at once
-  const unsigned grid = static_cast<unsigned>(std::min<int64_t>(n2, 4096));
+  const unsigned grid = static_cast<unsigned>(std::min<int64_t>(n2, 152 * 8));
   ProfScope prof_scope("k_direct_scatter", s);
-  switch (dt) {
-    case CMS_F32:
-      k_direct_scatter<float><<<grid, 256, 0, s>>>(in.a_ptr, in.a_idx, static_cast<const float*>(in.a_val), in.b_ptr,
-                                                   in.b_idx, static_cast<const float*>(in.b_val), in.n1, in.n3, h->n,
-                                                   dlist, counts, h->d_hs, h->d, h->b, cd);
-      break;
-    case CMS_BF16:
-      k_direct_scatter<__nv_bfloat16><<<grid, 256, 0, s>>>(
-          in.a_ptr, in.a_idx, static_cast<const __nv_bfloat16*>(in.a_val), in.b_ptr, in.b_idx,
-          static_cast<const __nv_bfloat16*>(in.b_val), in.n1, in.n3, h->n, dlist, counts, h->d_hs, h->d, h->b, cd);
-      break;
-    default:
-      k_direct_scatter<double><<<grid, 256, 0, s>>>(in.a_ptr, in.a_idx, static_cast<const double*>(in.a_val), in.b_ptr,
-                                                    in.b_idx, static_cast<const double*>(in.b_val), in.n1, in.n3, h->n,
-                                                    dlist, counts, h->d_hs, h->d, h->b, cd);
-      break;
-  }
+  auto go = [&](auto* tag, auto integer_tag) {
+    using T = std::remove_pointer_t<decltype(tag)>;
+    k_direct_scatter<T, decltype(integer_tag)::value><<<grid, 256, 0, s>>>(
+        in.a_ptr, in.a_idx, static_cast<const T*>(in.a_val), in.b_ptr, in.b_idx, static_cast<const T*>(in.b_val),
+        in.n1, in.n3, h->n, dlist, counts, h->d_hs, h->d, h->b, cd, direct_terms(h, cd));
+  };
+  auto both = [&](auto* tag) {
+    if (integer) go(tag, std::true_type{});
+    else go(tag, std::false_type{});
+  };
+  if (dt == CMS_F32) both(static_cast<float*>(nullptr));
+  else if (dt == CMS_BF16) both(static_cast<__nv_bfloat16*>(nullptr));
+  else both(static_cast<double*>(nullptr));
   return cudaGetLastError();
 }
 
-cudaError_t launch_add_direct(float* c, const double* cd, int64_t len, const int32_t* counts, cudaStream_t s) {
-  {
-    ProfScope prof_scope("k_add_direct", s);
-    k_add_direct<<<static_cast<unsigned>(std::min<int64_t>((len + 255) / 256, 4096)), 256, 0, s>>>(c, cd, len, counts);
-  }
+cudaError_t launch_add_direct(const cms_hashes* h, float* c, double* cd, int integer, const int32_t* counts,
+                              cudaStream_t s) {
+  const int64_t len = static_cast<int64_t>(h->d) * h->b;
+  const unsigned grid = static_cast<unsigned>(std::min<int64_t>((len + 255) / 256, 4096));
+  ProfScope prof_scope("k_add_direct", s);
+  if (integer) k_add_direct<true><<<grid, 256, 0, s>>>(c, cd, len, counts, direct_terms(h, cd));
+  else k_add_direct<false><<<grid, 256, 0, s>>>(c, cd, len, counts, nullptr);
   return cudaGetLastError();
 }
 
@@ -655,20 +786,21 @@ cudaError_t launch_sketch_sparse(const SketchPlan& plan, const cms_hashes* h, co
   a.nhi = plan.nhi;
   a.partial = partial;
   const int smem = static_cast<int>(plan.smem);
-  const unsigned ntask = static_cast<unsigned>(static_cast<int64_t>(plan.d) * plan.nrows * plan.nkc);
+  a.ntask = static_cast<int>(static_cast<int64_t>(plan.d) * plan.nrows * plan.nkc);
+  const unsigned grid = static_cast<unsigned>(std::min(a.ntask, 4 * 152));
   cudaError_t e = cudaSuccess;
   switch (dt) {
     case CMS_F32:
       e = cudaFuncSetAttribute(k_sketch_sparse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e == cudaSuccess) { ProfScope ps("k_sketch_sparse", s); k_sketch_sparse<float><<<ntask, kThreads, smem, s>>>(a); }
+      if (e == cudaSuccess) { ProfScope ps("k_sketch_sparse", s); k_sketch_sparse<float><<<grid, kThreads, smem, s>>>(a); }
       break;
     case CMS_BF16:
       e = cudaFuncSetAttribute(k_sketch_sparse<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e == cudaSuccess) { ProfScope ps("k_sketch_sparse", s); k_sketch_sparse<__nv_bfloat16><<<ntask, kThreads, smem, s>>>(a); }
+      if (e == cudaSuccess) { ProfScope ps("k_sketch_sparse", s); k_sketch_sparse<__nv_bfloat16><<<grid, kThreads, smem, s>>>(a); }
       break;
     default:
       e = cudaFuncSetAttribute(k_sketch_sparse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e == cudaSuccess) { ProfScope ps("k_sketch_sparse", s); k_sketch_sparse<double><<<ntask, kThreads, smem, s>>>(a); }
+      if (e == cudaSuccess) { ProfScope ps("k_sketch_sparse", s); k_sketch_sparse<double><<<grid, kThreads, smem, s>>>(a); }
       break;
   }
   if (e != cudaSuccess) return e;

@@ -180,3 +180,48 @@ def test_batch_of_both_routes(cms):
             assert worst(c, ref) < 1e-5
             c.zero_()
     batch.free()
+
+
+def sparse_pair(rng, n1, n2, n3, na, nb):
+    """CSC A (n1 x n2) and CSR B (n2 x n3) with na[k], nb[k] nonzeros."""
+    def side(n, cnt):
+        ptr = np.concatenate([[0], np.cumsum(cnt)]).astype(np.int64)
+        idx = np.concatenate([np.sort(rng.choice(n, c, replace=False)) for c in cnt] + [np.zeros(0, np.int64)])
+        return ptr, idx.astype(np.int32), rng.standard_normal(ptr[-1]).astype(np.float32)
+    return side(n1, na) + side(n3, nb)
+
+
+@pytest.mark.parametrize("d", [2, 9])
+def test_sparse_default_split(cms, d):
+    # outer products of every kind: empty, one term, more rows and columns
+    # than a block holds at a time (32 x 128), and some past the split
+    # (b log2(b) / 50 = 2129 terms), which take the FFT route; the same bits twice
+    rng = W.rng(3)
+    n, b = 700, 8192
+    na = np.array([0, 1, 33, 70, 5, 40, 0, 200, 31, 64] * 4)
+    nb = np.array([4, 1, 7, 20, 129, 300, 0, 9, 60, 150] * 4)
+    data = sparse_pair(rng, n, na.size, n, na, nb)
+    import scipy.sparse as sp
+    A = sp.csc_matrix((data[2], data[1], data[0]), shape=(n, na.size)).toarray().astype(np.float64)
+    B = sp.csr_matrix((data[5], data[4], data[3]), shape=(na.size, n)).toarray().astype(np.float64)
+    assert ((na * nb > 0) & (na * nb <= 2129)).any() and (na * nb > 2129).any()
+    h = cms.make_hashes(5, n, b, d)
+    args = [torch.from_numpy(x).to(dev()) for x in data]
+    c = cms.sketch_product_csr(*args, n, n, h)
+    c2 = cms.sketch_product_csr(*args, n, n, h)
+    cms.check_async()
+    assert torch.equal(c, c2)
+    assert worst(c, O.sketch_definition(A, B, O.make_tables(5, n, b, d))) < TOL
+    # indices outside the matrix are skipped, an infinity makes c NaN
+    small = [torch.from_numpy(x).to(dev()) for x in sparse_pair(rng, n, 6, n, np.full(6, 9), np.full(6, 11))]
+    want = cms.sketch_product_csr(*small, n, n, h)
+    drop = small[1].clone()
+    drop[4] = n + 5
+    zero = small[2].clone()
+    zero[4] = 0
+    got = cms.sketch_product_csr(small[0], drop, small[2], *small[3:], n, n, h)
+    ref = cms.sketch_product_csr(small[0], small[1], zero, *small[3:], n, n, h)
+    assert worst(got, ref.cpu().numpy()) < TOL and not torch.equal(got, want)
+    zero[7] = float("inf")
+    assert torch.isnan(cms.sketch_product_csr(small[0], small[1], zero, *small[3:], n, n, h)).all()
+    h.free()

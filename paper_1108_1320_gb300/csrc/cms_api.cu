@@ -709,9 +709,12 @@ struct SigLayout {
   size_t sk = 0, mask = 0, P = 0, dec = 0, total = 0;
   int ell = 0;
   int64_t ld0 = 0, ld1 = 0;
+  bool direct = false;
+  DirectPlan plan;
+  size_t dec_direct = 0, masked_total = 0;
 };
 
-cms_status sig_layout(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int32_t dt, int32_t rho,
+cms_status sig_layout(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int32_t dt, int32_t rho, bool alias,
                       SigLayout* L) {
   auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
   size_t sk = 0;
@@ -726,7 +729,22 @@ cms_status sig_layout(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, i
   L->mask = o; o += al(static_cast<size_t>(std::max(L->ld0, L->ld1)) * std::max<int64_t>(n2, 1) * esz);
   L->P = o;    o += al(static_cast<size_t>(2 * L->ell) * h->d * h->b * sizeof(float));
   L->dec = o;  o += al(significant_decode_ws_bytes(h->d, h->b));
-  L->total = o;
+  L->total = L->masked_total = o;
+  // the direct route: all sums of one pass over the entries, then the vote
+  int bits = 0;
+  significant_code_length(n1, n3, rho, &bits);
+  DeviceProps dp = device_props(h->device);
+  SketchPlan plan;
+  std::string why;
+  DirectPlan one;
+  L->direct = false;
+  if (make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &plan, &why) == CMS_OK &&
+      choose_direct_significant(h, plan, n1, n2, n3, dt, alias, dp.sms, bits, L->ell, &one)) {
+    L->direct = true;
+    L->plan = one;
+    L->dec_direct = al(one.ws_bytes);
+    L->total = std::max(L->total, L->dec_direct + al(significant_decode_ws_bytes(h->d, h->b)));
+  }
   return CMS_OK;
 }
 }  // namespace
@@ -736,9 +754,14 @@ cms_status cms_significant_workspace_size(const cms_hashes* h, int64_t n1, int64
   if (!bytes) return fail(CMS_ERR_INVALID_ARG, "bytes is NULL");
   if (rho < 1 || rho > 8) return fail(CMS_ERR_INVALID_ARG, "rho must be in [1, 8]");
   SigLayout L;
-  cms_status st = sig_layout(h, n1, n2, n3, dt, rho, &L);
+  cms_status st = sig_layout(h, n1, n2, n3, dt, rho, false, &L);
   if (st != CMS_OK) return st;
   *bytes = L.total;
+  if (n1 == n3) {   // A = X^T, B = X packs one operand: not more, but its own plan
+    st = sig_layout(h, n1, n2, n3, dt, rho, true, &L);
+    if (st != CMS_OK) return st;
+    *bytes = std::max(*bytes, L.total);
+  }
   return CMS_OK;
 }
 
@@ -785,14 +808,23 @@ cms_status cms_find_significant(const void* A, int64_t lda, const void* B, int64
   st = check_device(h);
   if (st != CMS_OK) return st;
   SigLayout L;
-  st = sig_layout(h, n1, n2, n3, dt, rho, &L);
+  st = sig_layout(h, n1, n2, n3, dt, rho, A == B && lda == ldb && n1 == n3, &L);
   if (st != CMS_OK) return st;
-  if (!ws || ws_bytes < L.total)
+  const bool direct = L.direct && ws_bytes >= L.total;
+  if (!ws || ws_bytes < (direct ? L.total : L.masked_total))
     return fail(CMS_ERR_WORKSPACE, "workspace missing or smaller than cms_significant_workspace_size()");
   if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return fail(CMS_ERR_WORKSPACE, "workspace must be 256-byte aligned");
   DeviceProps dp = device_props(h->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
+  if (direct) {
+    cudaError_t e = launch_direct_significant(L.plan, h, A, lda, B, ldb, n1, n2, n3, dt, delta,
+                                              reinterpret_cast<uint64_t*>(w + L.dec_direct), w, s);
+    if (e == cudaSuccess)
+      e = launch_decode_significant(nullptr, h, n1, n3, delta, rho, ij_out, capacity, count_out, w + L.dec_direct, s);
+    if (e != cudaSuccess) return cuda_fail(e, "cms_find_significant");
+    return CMS_OK;
+  }
   void* M = w + L.mask;
   float* P = reinterpret_cast<float*>(w + L.P);
   const size_t per = static_cast<size_t>(h->d) * h->b;

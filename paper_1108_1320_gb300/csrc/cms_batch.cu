@@ -394,12 +394,12 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
       char* w = b->ws + b->ws_off[i];
       if (b->is_direct[i]) {
         const DirectPlan& dp = b->direct[i];
-        specs[i] = InverseSpec{reinterpret_cast<unsigned long long*>(w + dp.off_acc),
+        specs[i] = InverseSpec{reinterpret_cast<unsigned long long*>(w + dp.off_acc), dp.copies,
                                reinterpret_cast<const DirectScale*>(w + dp.off_scale), direct_scale_log2(dp.split),
                                &p, nullptr, nullptr, nullptr, nullptr, items[i].c};
         continue;
       }
-      specs[i] = InverseSpec{nullptr, nullptr, 0, &p, reinterpret_cast<const float2*>(w + p.off_partial),
+      specs[i] = InverseSpec{nullptr, 1, nullptr, 0, &p, reinterpret_cast<const float2*>(w + p.off_partial),
                              reinterpret_cast<float2*>(w + p.off_V), reinterpret_cast<const float2*>(w + p.off_twC),
                              reinterpret_cast<const float2*>(w + p.off_twR), items[i].c};
     }

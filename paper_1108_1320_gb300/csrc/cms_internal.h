@@ -217,6 +217,7 @@ cudaError_t launch_twiddle_tables(float2* twC, int C, float2* twR, int R, cudaSt
 struct DirectScale;
 struct InverseSpec {
   unsigned long long* sums;
+  int copies;
   const DirectScale* scale;
   int log2s;
   const SketchPlan* plan;
@@ -294,6 +295,8 @@ cudaError_t launch_remove_diagonal(const void* A, int64_t lda, const void* B, in
 size_t frobenius_ws_bytes(int64_t n1, int64_t n2, int64_t n3, int d);
 int significant_code_length(int64_t n1, int64_t n3, int rho, int* L);
 size_t significant_decode_ws_bytes(int d, int64_t b);
+// Fig. 3's multiset vote on the keys at the start of the decode workspace ws
+// (P NULL), or the decode of given sketches P and the vote.
 cudaError_t launch_decode_significant(const float* P, const cms_hashes* h, int64_t n1, int64_t n3, float delta,
                                       int rho, int64_t* ij, int64_t capacity, int64_t* count, char* ws,
                                       cudaStream_t s);
@@ -313,17 +316,27 @@ struct DirectPlan {
   bool split = false;       // FP32 (or FP64) storage: two FP16 terms per value
   bool alias = false;       // A = X^T, B = X: tiles on and above the diagonal
   int tiles1 = 0, tiles3 = 0, nsb = 0, splits = 1, sb_per_split = 1, slots = 0;
+  int copies = 1;           // of the sums, for short sketches
+  int sets = 1;             // sums of different entries (1 + 2 L: FINDSIGNIFICANTENTRIES)
   int64_t tiles = 0;
   double seconds = 0.0;     // estimate
-  size_t zero_bytes = 0, off_fold = 0;
+  size_t zero_bytes = 0, acc_bytes = 0, off_fold = 0;
   size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_pa = 0, off_pb = 0;
   size_t ws_bytes = 0;
 };
-DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms);
+DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms,
+                            int sets = 1);
+// The keys i n3 + j + 1 (0: none) that the masked sums of Fig. 3 decode to,
+// one per (repetition, bucket); p made with 1 + 2 L sets.
+cudaError_t launch_direct_significant(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda,
+                                      const void* B, int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt,
+                                      float delta, uint64_t* keys, char* ws, cudaStream_t s);
 // Whether the direct route serves the call (and its plan): beside the
 // transform route's plan, which stays the one that decides what is accepted.
 bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias,
                    int sms, DirectPlan* out);
+bool choose_direct_significant(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt,
+                               bool alias, int sms, int bits, int ell, DirectPlan* out);
 cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
                           int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws,
                           cudaStream_t s);

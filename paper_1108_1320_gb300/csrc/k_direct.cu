@@ -273,7 +273,9 @@ struct TileArgs {
   const int2* eb;
   const DirectScale* scale;
   const uint32_t* hs;          // [t][side][n]
-  unsigned long long* acc;     // [t][b]
+  unsigned long long* acc;     // [copy][t][b]
+  int copies;                  // blocks add to copy (block mod copies)
+  int bits;                    // masked sums: bits of a position (copies = 1)
   int64_t K;
   int n, n1, n3, b, d;
   int tiles1, tiles3;
@@ -328,7 +330,28 @@ __device__ __forceinline__ void tmem_wait_ld8x2(uint32_t (&a)[8], uint32_t (&b)[
                : "memory");
 }
 
-template <bool SPLIT>
+// A value added to its bucket's sum, to the sums of the bits set in the
+// position i of its row, and to those of the bits set in j.
+__device__ __forceinline__ void bucket_add_masked(unsigned long long* c, size_t set, int bits, uint32_t i, uint32_t j,
+                                                  uint32_t ha, uint32_t hb, uint32_t b, float v) {
+  uint32_t z = (ha & kBucketMask) + (hb & kBucketMask);
+  if (z >= b) z -= b;
+  const float w = __uint_as_float(__float_as_uint(v) ^ ((ha ^ hb) & 0x80000000u));
+  const long long iv = __float2ll_rn(w);
+  c += z;
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+  for (int m = 0; m < bits; ++m) {
+    c += set;
+    if ((i >> m) & 1u) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+  }
+  for (int m = 0; m < bits; ++m) {
+    c += set;
+    if ((j >> m) & 1u) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+  }
+}
+
+// MASKED: the sums of FINDSIGNIFICANTENTRIES (p.bits of them for each side).
+template <bool SPLIT, bool MASKED = false>
 __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split) {
   constexpr int kImages = SPLIT ? 4 : 2;
   constexpr int kPerStage = kSuper / kImages;
@@ -535,6 +558,14 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
     const bool mirror = p.sym && ti != tj;
     const bool row = i < p.n1;
     const uint32_t b = static_cast<uint32_t>(p.b);
+    const size_t set = static_cast<size_t>(p.d) * p.b;
+    unsigned long long* sums = p.acc + (p.copies > 1 ? static_cast<size_t>(tile + split) % p.copies * set : 0);
+    // the stages' memory is free: every product has been read
+    float* stash = reinterpret_cast<float*>(stages) + tid;
+    if constexpr (MASKED) {
+#pragma unroll
+      for (int q = 0; q < kTile; ++q) stash[q * kTile] = acc[q];
+    }
     for (int t = 0; t < p.d; ++t) {
       const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
       const uint32_t* h2 = h1 + p.n;
@@ -545,8 +576,18 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
       }
       epi_sync();
       if (!row) continue;
-      unsigned long long* c = p.acc + static_cast<size_t>(t) * p.b;
+      unsigned long long* c = sums + static_cast<size_t>(t) * p.b;
       const uint32_t hr = h1[i];
+      if constexpr (MASKED) {
+        // the row from shared memory: a loop of its own per value
+        const uint32_t hm = mirror ? h2[i] : 0;
+        for (int q = 0; q < cols; ++q) {
+          const float v = stash[q * kTile];
+          bucket_add_masked(c, set, p.bits, i, j0 + q, hr, hcol[q], b, v);
+          if (mirror) bucket_add_masked(c, set, p.bits, j0 + q, i, hcol[kTile + q], hm, b, v);
+        }
+        continue;
+      }
 #pragma unroll
       for (int q = 0; q < kTile; ++q)
         if (q < cols) bucket_add(c, hr, hcol[q], b, acc[q]);
@@ -569,9 +610,9 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
   }
 }
 
-template <bool SPLIT>
+template <bool SPLIT, bool MASKED>
 __global__ void __launch_bounds__(kTileThreads, 2) k_direct_tile(const TileArgs p) {
-  tile_task<SPLIT>(p, blockIdx.x, blockIdx.y);
+  tile_task<SPLIT, MASKED>(p, blockIdx.x, blockIdx.y);
 }
 
 // Tiles of every product of a batch, the longest first.
@@ -598,11 +639,64 @@ k_direct_pack_batched(const PackArgs* __restrict__ args, const int* __restrict__
   pack_task(sp, blockIdx.x - static_cast<uint32_t>(__ldg(start + q)));
 }
 
-__global__ void __launch_bounds__(256) k_direct_finish(const unsigned long long* acc, float* c, int64_t len,
+// COPIES: 32 buckets per block, the copies dealt to its 8 warps.
+template <bool COPIES>
+__global__ void __launch_bounds__(256) k_direct_finish(const unsigned long long* acc, int copies, float* c, int64_t len,
                                                        const DirectScale* scale, int log2s) {
   const DirectScale sc = *scale;
-  for (int64_t q = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; q < len; q += static_cast<int64_t>(gridDim.x) * 256)
-    c[q] = direct_value(acc[q], sc, log2s);
+  if constexpr (COPIES) {
+    __shared__ unsigned long long part[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t q = static_cast<int64_t>(blockIdx.x) * 32 + lane;
+    unsigned long long v = 0;
+    if (q < len) {
+#pragma unroll 4
+      for (int r = warp; r < copies; r += 8) v += __ldg(acc + r * len + q);
+    }
+    part[warp][lane] = v;
+    __syncthreads();
+    if (warp == 0 && q < len) {
+#pragma unroll
+      for (int w = 1; w < 8; ++w) v += part[w][lane];
+      c[q] = direct_value(v, sc, log2s);
+    }
+  } else {
+    for (int64_t q = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; q < len;
+         q += static_cast<int64_t>(gridDim.x) * 256)
+      c[q] = direct_value(acc[q], sc, log2s);
+  }
+}
+
+// The bits |sum| > half of each (repetition, bucket) and side, decoded into a
+// position (0: none).  The rho copies of a bit of E are the same mask, so
+// their sketches are the same sums, and a complement's sums are the total's
+// less the bit's: a bit is 1 when its sum alone is above, 0 when its
+// complement's alone is, and no bit (a tie of the votes) otherwise.
+__global__ void __launch_bounds__(256)
+k_direct_sig_decode(const unsigned long long* __restrict__ acc, int bits, int64_t len, int64_t n1, int64_t n3,
+                    float half, const DirectScale* __restrict__ scale, int log2s, uint64_t* __restrict__ keys) {
+  const DirectScale sc = *scale;
+  const int64_t q = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
+  if (q >= len) return;
+  const unsigned long long total = acc[q];
+  int64_t pos[2];
+  for (int sd = 0; sd < 2; ++sd) {
+    int64_t x = 0;
+    const unsigned long long* a = acc + static_cast<size_t>(1 + sd * bits) * len + q;
+    for (int m = 0; m < bits; ++m) {
+      const unsigned long long s1 = a[static_cast<size_t>(m) * len];
+      const bool one = fabsf(direct_value(s1, sc, log2s)) > half;
+      const bool zero = fabsf(direct_value(total - s1, sc, log2s)) > half;
+      if (one == zero) { x = -1; break; }
+      x |= static_cast<int64_t>(one) << m;
+    }
+    pos[sd] = x;
+    if (x < 0) break;
+  }
+  uint64_t key = 0;
+  if (pos[0] >= 0 && pos[0] < n1 && pos[1] >= 0 && pos[1] < n3)
+    key = static_cast<uint64_t>(pos[0]) * static_cast<uint64_t>(n3) + static_cast<uint64_t>(pos[1]) + 1u;
+  keys[q] = key;
 }
 
 }  // namespace
@@ -614,7 +708,8 @@ uint32_t read_clear_error_direct() {
   return v;
 }
 
-DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms) {
+DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms,
+                            int sets) {
   DirectPlan p;
   p.split = dt != CMS_BF16;
   p.alias = alias;
@@ -637,19 +732,28 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
     const int real = (p.nsb + per_split - 1) / per_split;
     const double waves = std::max(1.0, std::ceil(static_cast<double>(tiles) * real / slots));
     const double mma = waves * per_split * (p.split ? 1.0 : 0.5) * 1.1e-6;
-    const double red = static_cast<double>(n1) * n3 * h->d * real / 2.0e11;
+    const double red = static_cast<double>(n1) * n3 * h->d * real * 0.5 * (sets + 1) / 2.0e11;
     if (mma + red < cost) { cost = mma + red; best = real; }
   }
   p.sb_per_split = (p.nsb + best - 1) / best;
   p.splits = (p.nsb + p.sb_per_split - 1) / p.sb_per_split;
   p.seconds = cost + 15e-6;
+  // short sketches: reductions to few words queue up (23 G/s on 2^10 words,
+  // 100 on 2^14, 165 on 2^16, 200 from 2^18 on), so blocks share several
+  // copies of the sums, which the conversion adds up
+  const int64_t words = static_cast<int64_t>(h->d) * h->b;
+  p.copies = sets > 1 ? 1
+                      : static_cast<int>(std::max<int64_t>(
+                            1, std::min<int64_t>({256, (int64_t{1} << 18) / words, tiles * p.splits})));
+  p.sets = sets;
   auto al = [](size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); };
   size_t o = 0;
   const int t3 = alias ? 0 : p.tiles3;
   const int drains = p.sb_per_split * (p.split ? 2 : 1);
   p.slots = drains > kFoldFrom ? 2 * sms : 0;
   // sums, the ticket, the slots taken (all zero before a run)
-  p.off_acc = o;    o = al(o + static_cast<size_t>(h->d) * h->b * 8 + 256 + static_cast<size_t>(p.slots) * 4);
+  p.acc_bytes = static_cast<size_t>(p.copies) * sets * words * 8;
+  p.off_acc = o;    o = al(o + p.acc_bytes + 256 + static_cast<size_t>(p.slots) * 4);
   p.zero_bytes = o;
   p.off_fold = o;   o = al(o + static_cast<size_t>(p.slots) * kTile * kTile * sizeof(float));
   p.off_scale = o;  o = al(o + sizeof(DirectScale));
@@ -677,9 +781,21 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
   *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms);
   return out->seconds < transform_seconds(plan, n2);
 }
+// The masked sums of FINDSIGNIFICANTENTRIES in one pass: an entry is added to
+// its bucket's total and, in the mean, to half of the 2 `bits` masked sums,
+// against 2 ell products.
+bool choose_direct_significant(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt,
+                               bool alias, int sms, int bits, int ell, DirectPlan* out) {
+  if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535) return false;
+  *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1 + 2 * bits);
+  const double sums = static_cast<double>(n1) * static_cast<double>(n3) * h->d * bits * out->splits / 2.0e11 +
+                      static_cast<double>(out->acc_bytes) / 3e12;
+  return out->seconds + sums < 2.0 * ell * transform_seconds(plan, n2);
+}
+
 namespace {
 
-PackArgs pack_args(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B, int64_t ldb,
+PackArgs pack_args(const DirectPlan& p, const void* A, int64_t lda, const void* B, int64_t ldb,
                    int64_t n1, int64_t n2, int64_t n3, int dt, char* ws) {
   int2* blocks = reinterpret_cast<int2*>(ws + p.off_blocks);
   PackArgs a{};
@@ -691,7 +807,7 @@ PackArgs pack_args(const DirectPlan& p, const cms_hashes* h, const void* A, int6
   a.dt = dt;
   a.n1 = n1;
   a.n3 = n3;
-  a.ticket = reinterpret_cast<uint32_t*>(ws + p.off_acc + static_cast<size_t>(h->d) * h->b * 8);
+  a.ticket = reinterpret_cast<uint32_t*>(ws + p.off_acc + p.acc_bytes);
   a.scale = reinterpret_cast<DirectScale*>(ws + p.off_scale);
   return a;
 }
@@ -717,8 +833,10 @@ TileArgs tile_args(const DirectPlan& p, const cms_hashes* h, int64_t n1, int64_t
   a.sb_per_split = p.sb_per_split;
   a.tiles = static_cast<int>(p.tiles);
   a.fold = p.slots > 0 ? reinterpret_cast<float*>(ws + p.off_fold) : nullptr;
-  a.slot = reinterpret_cast<uint32_t*>(ws + p.off_acc + static_cast<size_t>(h->d) * h->b * 8 + 256);
+  a.slot = reinterpret_cast<uint32_t*>(ws + p.off_acc + p.acc_bytes + 256);
   a.slots = p.slots;
+  a.copies = p.copies;
+  a.bits = (p.sets - 1) / 2;
   a.split = p.split ? 1 : 0;
   a.sym = p.alias ? 1 : 0;
   return a;
@@ -754,7 +872,7 @@ cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, void* d_buf
   for (int q = 0; q < count; ++q) {
     const DirectSpec& d = specs[q];
     reinterpret_cast<PackArgs*>(host.data())[q] =
-        pack_args(d.plan, d.h, d.A, d.lda, d.B, d.ldb, d.n1, d.n2, d.n3, d.dt, d.ws);
+        pack_args(d.plan, d.A, d.lda, d.B, d.ldb, d.n1, d.n2, d.n3, d.dt, d.ws);
     reinterpret_cast<TileArgs*>(host.data() + out->o_tile)[q] = tile_args(d.plan, d.h, d.n1, d.n2, d.n3, d.ws);
     ps[q] = np;
     ts[q] = nt;
@@ -792,40 +910,64 @@ cudaError_t launch_direct_batched(const DirectBatch& d, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
-                          int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws,
-                          cudaStream_t s) {
-  const size_t len = static_cast<size_t>(h->d) * h->b;
+namespace {
+
+// Zeroed sums, packing, tiles.
+cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
+                        int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, char* ws, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(ws + p.off_acc, 0, p.zero_bytes, s);
   if (e != cudaSuccess) return e;
   {
     ProfScope prof_scope("k_direct_pack", s);
     const uint32_t smem = (p.split ? 4 : 2) * kStageBytes;
     if ((e = with_smem(k_direct_pack, smem)) != cudaSuccess) return e;
-    k_direct_pack<<<pack_blocks(p), 256, smem, s>>>(pack_args(p, h, A, lda, B, ldb, n1, n2, n3, dt, ws));
+    k_direct_pack<<<pack_blocks(p), 256, smem, s>>>(pack_args(p, A, lda, B, ldb, n1, n2, n3, dt, ws));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const TileArgs a = tile_args(p, h, n1, n2, n3, ws);
-  {
-    ProfScope prof_scope("k_direct_tile", s);
-    const dim3 grid(static_cast<unsigned>(p.tiles), p.splits);
-    auto go = [&](auto kern) {
-      cudaError_t r = with_smem(kern, tile_smem_bytes());
-      if (r != cudaSuccess) return r;
-      kern<<<grid, kTileThreads, tile_smem_bytes(), s>>>(a);
-      return cudaGetLastError();
-    };
-    e = p.split ? go(k_direct_tile<true>) : go(k_direct_tile<false>);
-    if (e != cudaSuccess) return e;
-  }
-  {
-    ProfScope prof_scope("k_direct_finish", s);
-    const int64_t blocks = std::min<int64_t>((static_cast<int64_t>(len) + 255) / 256, 152 * 8);
-    k_direct_finish<<<static_cast<unsigned>(blocks), 256, 0, s>>>(a.acc, c, static_cast<int64_t>(len), a.scale,
-                                                                  direct_scale_log2(p.split));
-    e = cudaGetLastError();
-  }
-  return e;
+  ProfScope prof_scope("k_direct_tile", s);
+  const dim3 grid(static_cast<unsigned>(p.tiles), p.splits);
+  auto go = [&](auto kern) {
+    cudaError_t r = with_smem(kern, tile_smem_bytes());
+    if (r != cudaSuccess) return r;
+    kern<<<grid, kTileThreads, tile_smem_bytes(), s>>>(a);
+    return cudaGetLastError();
+  };
+  if (p.sets > 1) return p.split ? go(k_direct_tile<true, true>) : go(k_direct_tile<false, true>);
+  return p.split ? go(k_direct_tile<true, false>) : go(k_direct_tile<false, false>);
+}
+
+}  // namespace
+
+cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
+                          int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws,
+                          cudaStream_t s) {
+  cudaError_t e = launch_sums(p, h, A, lda, B, ldb, n1, n2, n3, dt, ws, s);
+  if (e != cudaSuccess) return e;
+  const int64_t len = static_cast<int64_t>(h->d) * h->b;
+  const unsigned long long* acc = reinterpret_cast<const unsigned long long*>(ws + p.off_acc);
+  const DirectScale* scale = reinterpret_cast<const DirectScale*>(ws + p.off_scale);
+  ProfScope prof_scope("k_direct_finish", s);
+  if (p.copies > 1)
+    k_direct_finish<true><<<static_cast<unsigned>((len + 31) / 32), 256, 0, s>>>(acc, p.copies, c, len, scale,
+                                                                                 direct_scale_log2(p.split));
+  else
+    k_direct_finish<false><<<static_cast<unsigned>(std::min<int64_t>((len + 255) / 256, 152 * 8)), 256, 0, s>>>(
+        acc, 1, c, len, scale, direct_scale_log2(p.split));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_direct_significant(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda,
+                                      const void* B, int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt,
+                                      float delta, uint64_t* keys, char* ws, cudaStream_t s) {
+  cudaError_t e = launch_sums(p, h, A, lda, B, ldb, n1, n2, n3, dt, ws, s);
+  if (e != cudaSuccess) return e;
+  const int64_t len = static_cast<int64_t>(h->d) * h->b;
+  ProfScope prof_scope("k_direct_sig_decode", s);
+  k_direct_sig_decode<<<static_cast<unsigned>((len + 255) / 256), 256, 0, s>>>(
+      reinterpret_cast<const unsigned long long*>(ws + p.off_acc), (p.sets - 1) / 2, len, n1, n3, 0.5f * delta,
+      reinterpret_cast<const DirectScale*>(ws + p.off_scale), direct_scale_log2(p.split), keys);
+  return cudaGetLastError();
 }
 
 }  // namespace cms

@@ -163,7 +163,7 @@ cudaError_t launch_decode_significant(const float* P, const cms_hashes* h, int64
   if (e != cudaSuccess) return e;
   const int64_t nk = static_cast<int64_t>(d) * b;
   const unsigned g1 = static_cast<unsigned>(std::min<int64_t>((nk + 255) / 256, 8192));
-  {
+  if (P != nullptr) {
     ProfScope prof_scope("k_sig_decode", s);
     k_sig_decode<<<g1, 256, 0, s>>>(P, d, b, n1, n3, delta, L, rho, keys);
   }

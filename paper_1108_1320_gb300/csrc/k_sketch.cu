@@ -271,6 +271,7 @@ k_cols_inverse_fft(const float2* __restrict__ V, const float2* __restrict__ twR,
 
 struct ColsArgs {
   unsigned long long* sums;    // direct route: the integer sums (left zero), else NULL
+  int copies;
   const DirectScale* scale;
   int log2s;
   const float2* V;
@@ -279,6 +280,7 @@ struct ColsArgs {
   int64_t b;
   int R, C, nrows;
   int nbx;   // blocks of 256 points per repetition
+  int nbd;   // repetitions
 };
 
 // K2b for a batch: every instance's (repetition, point block) in one launch.
@@ -292,8 +294,13 @@ k_cols_inverse_batched(const ColsArgs* __restrict__ args, const int* __restrict_
   if (z >= a.b) return;
   if (a.sums != nullptr) {
     const size_t q = static_cast<size_t>(t) * a.b + z;
-    a.c[q] = direct_value(a.sums[q], *a.scale, a.log2s);
-    a.sums[q] = 0;
+    const size_t len = static_cast<size_t>(a.nbd) * a.b;
+    unsigned long long v = 0;
+    for (int r = 0; r < a.copies; ++r) {
+      v += a.sums[r * len + q];
+      a.sums[r * len + q] = 0;
+    }
+    a.c[q] = direct_value(v, *a.scale, a.log2s);
     return;
   }
   cols_inverse_point(a.V, a.twR, a.b, a.R, a.C, a.nrows, a.c, t, z);
@@ -667,7 +674,7 @@ cudaError_t build_inverse_batch(const std::vector<InverseSpec>& specs, void* d_b
     tr += direct ? 1 : plan.d * plan.nrows;
     if (!direct) smem = std::max(smem, static_cast<size_t>(3 * plan.C * 8));
     ColsArgs ca{};
-    ca.sums = specs[i].sums; ca.scale = specs[i].scale; ca.log2s = specs[i].log2s;
+    ca.sums = specs[i].sums; ca.copies = specs[i].copies; ca.nbd = plan.d; ca.scale = specs[i].scale; ca.log2s = specs[i].log2s;
     ca.V = specs[i].V; ca.twR = specs[i].twR; ca.c = specs[i].c; ca.b = plan.b;
     ca.R = static_cast<int>(plan.R); ca.C = static_cast<int>(plan.C); ca.nrows = plan.nrows;
     ca.nbx = static_cast<int>((plan.b + 255) / 256);

@@ -225,3 +225,42 @@ def test_sparse_default_split(cms, d):
     zero[7] = float("inf")
     assert torch.isnan(cms.sketch_product_csr(small[0], small[1], zero, *small[3:], n, n, h)).all()
     h.free()
+
+
+@pytest.mark.parametrize("n1,n2,n3,b,d", [(64, 300, 64, 12, 2), (200, 130, 150, 1, 3), (140, 64, 140, 96, 7)])
+def test_direct_route_short_sketches(cms, n1, n2, n3, b, d):
+    # few buckets: blocks add to copies of the sums (and the finish adds
+    # those up); the direct route where the rule picks it
+    A, B, Ad, Bd = operands(n1, n2, n3, "f32", False, 0, n1)
+    h = cms.make_hashes(n1, max(n1, n3), b, d)
+    c, _ = run(cms, A, B, h)
+    ref = O.sketch_definition(Ad, Bd, O.make_tables(n1, max(n1, n3), b, d))
+    assert worst(c, ref) < 1e-5
+    h.free()
+
+
+@pytest.mark.parametrize("n1,n2,n3,rho,alias", [(300, 80, 280, 1, False), (257, 200, 257, 3, True), (90, 64, 1, 2, False)])
+def test_find_significant_on_the_direct_route(cms, n1, n2, n3, rho, alias):
+    # planted entries far above the noise: exactly these positions, from the
+    # masked sums of one pass over the entries of AB
+    b, d = 16384, 5
+    g = W.rng(50 + n1)
+    At = (0.01 * g.standard_normal((n2, n1))).astype(np.float32)
+    B = At if alias else (0.01 * g.standard_normal((n2, n3))).astype(np.float32)
+    big = [(3, 5), (min(117, n1 - 1), 230), (n1 - 1, 0), (21, 21)]
+    for q, (i, j) in enumerate(big):
+        At[q, i] += 10.0
+        B[q, j % n3] += 10.0 + q
+    AB = At.astype(np.float64).T @ B.astype(np.float64)
+    want = sorted((int(i), int(j)) for i, j in zip(*np.nonzero(np.abs(AB) > 50.0)))
+    h = cms.make_hashes(151, max(n1, n3), b, d)
+    at = torch.from_numpy(At).to(dev())
+    bt = at if alias else torch.from_numpy(B).to(dev())
+    cms.profile_enable(True)
+    got, count = cms.find_significant(at.T, bt, h, 50.0, rho)
+    kernels = cms.profile_summary()
+    cms.profile_enable(False)
+    cms.check_async()
+    assert "k_direct_sig_decode" in kernels and "k_mask_copy" not in kernels
+    assert [tuple(p) for p in got.cpu().numpy().tolist()] == want and count == len(want)
+    h.free()

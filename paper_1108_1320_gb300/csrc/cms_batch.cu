@@ -245,7 +245,8 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
                              true, 0, 0, false, false);
     if (r != CMS_OK) { delete b; return fail(static_cast<cms_status>(r), "instance " + std::to_string(i) + ": " + why); }
     b->is_direct[i] = choose_direct(it.h, p, it.n1, it.n2, it.n3, it.dt,
-                                    it.A == it.B && it.lda == it.ldb && it.n1 == it.n3, sms, &b->direct[i]) ? 1 : 0;
+                                    it.A == it.B && it.lda == it.ldb && it.n1 == it.n3, sms, &b->direct[i],
+                                    true) ? 1 : 0;
     b->plans[i] = p;
     if (!b->is_direct[i]) continue;
     // the direct route has no tiles to tune: the cache holds whether it was

@@ -317,15 +317,17 @@ struct DirectPlan {
   bool alias = false;       // A = X^T, B = X: tiles on and above the diagonal
   int tiles1 = 0, tiles3 = 0, nsb = 0, splits = 1, sb_per_split = 1, slots = 0;
   int copies = 1;           // of the sums, for short sketches
+  bool grid = false;        // the entries stored, added to the buckets by a launch of its own
+  bool grid64 = false;      // ... as integers
   int sets = 1;             // sums of different entries (1 + 2 L: FINDSIGNIFICANTENTRIES)
   int64_t tiles = 0;
   double seconds = 0.0;     // estimate
-  size_t zero_bytes = 0, acc_bytes = 0, off_fold = 0;
+  size_t zero_bytes = 0, acc_bytes = 0, off_fold = 0, off_grid = 0;
   size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_pa = 0, off_pb = 0;
   size_t ws_bytes = 0;
 };
 DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms,
-                            int sets = 1);
+                            int sets, bool batch);
 // The keys i n3 + j + 1 (0: none) that the masked sums of Fig. 3 decode to,
 // one per (repetition, bucket); p made with 1 + 2 L sets.
 cudaError_t launch_direct_significant(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda,
@@ -334,7 +336,7 @@ cudaError_t launch_direct_significant(const DirectPlan& p, const cms_hashes* h, 
 // Whether the direct route serves the call (and its plan): beside the
 // transform route's plan, which stays the one that decides what is accepted.
 bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias,
-                   int sms, DirectPlan* out);
+                   int sms, DirectPlan* out, bool batch = false);
 bool choose_direct_significant(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt,
                                bool alias, int sms, int bits, int ell, DirectPlan* out);
 cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,

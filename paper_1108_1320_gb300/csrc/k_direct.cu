@@ -275,7 +275,8 @@ struct TileArgs {
   const uint32_t* hs;          // [t][side][n]
   unsigned long long* acc;     // [copy][t][b]
   int copies;                  // blocks add to copy (block mod copies)
-  int bits;                    // masked sums: bits of a position (copies = 1)
+  void* grid;                  // entries in units of the integer sums, rows of tiles3 * 128: FP32, or
+  int grid64;                  //   64-bit integers added by the splits of the inner dimension
   int64_t K;
   int n, n1, n3, b, d;
   int tiles1, tiles3;
@@ -330,28 +331,45 @@ __device__ __forceinline__ void tmem_wait_ld8x2(uint32_t (&a)[8], uint32_t (&b)[
                : "memory");
 }
 
-// A value added to its bucket's sum, to the sums of the bits set in the
-// position i of its row, and to those of the bits set in j.
-__device__ __forceinline__ void bucket_add_masked(unsigned long long* c, size_t set, int bits, uint32_t i, uint32_t j,
-                                                  uint32_t ha, uint32_t hb, uint32_t b, float v) {
-  uint32_t z = (ha & kBucketMask) + (hb & kBucketMask);
-  if (z >= b) z -= b;
-  const float w = __uint_as_float(__float_as_uint(v) ^ ((ha ^ hb) & 0x80000000u));
-  const long long iv = __float2ll_rn(w);
-  c += z;
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
-  for (int m = 0; m < bits; ++m) {
-    c += set;
-    if ((i >> m) & 1u) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+constexpr int kPitch = kTile + 4;        // words per row of a tile in shared memory
+
+// This thread's row of the tile (128 columns from j0), and its mirror image.
+__device__ __forceinline__ void store_grid(const TileArgs& p, const float (&acc)[kTile], float* smem, int tid, int i,
+                                           int j0, bool mirror) {
+  const size_t ld = static_cast<size_t>(p.tiles3) * kTile;
+  if (p.grid64) {
+    unsigned long long* g = static_cast<unsigned long long*>(p.grid);
+#pragma unroll
+    for (int q = 0; q < kTile; ++q) {
+      const long long v = __float2ll_rn(acc[q]);
+      atomicAdd(g + i * ld + j0 + q, static_cast<unsigned long long>(v));
+      if (mirror) atomicAdd(g + (j0 + q) * ld + i, static_cast<unsigned long long>(v));
+    }
+    return;
   }
-  for (int m = 0; m < bits; ++m) {
-    c += set;
-    if ((j >> m) & 1u) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+  float* g = static_cast<float*>(p.grid);
+  // the lanes hold consecutive rows: the mirror image is stored as it is
+  // (128 bytes per warp), the tile itself through shared memory (the stages'
+  // memory is free: every product has been read), a row per bulk copy
+  if (mirror) {
+#pragma unroll
+    for (int q = 0; q < kTile; ++q) g[(j0 + q) * ld + i] = acc[q];
   }
+  float* row = smem + tid * kPitch;
+#pragma unroll
+  for (int q = 0; q < kTile; q += 4)
+    *reinterpret_cast<float4*>(row + q) = make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]);
+  fence_proxy_async();
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(g + i * ld + j0),
+               "r"(smem_u32(row)), "r"(kTile * 4)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// MASKED: the sums of FINDSIGNIFICANTENTRIES (p.bits of them for each side).
-template <bool SPLIT, bool MASKED = false>
+// GRID: the entries go to p.grid (k_direct_grid adds them to the buckets);
+// else straight to the buckets.
+template <bool SPLIT, bool GRID = false>
 __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split) {
   constexpr int kImages = SPLIT ? 4 : 2;
   constexpr int kPerStage = kSuper / kImages;
@@ -554,19 +572,17 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
     for (int q = 0; q < kTile; ++q) acc[q] = acc[q] * up * up2;
     const int i = ti * kTile + tid;
     const int j0 = tj * kTile;
-    const int cols = run ? min(kTile, p.n3 - j0) : 0;
+    int cols = run ? min(kTile, p.n3 - j0) : 0;
     const bool mirror = p.sym && ti != tj;
     const bool row = i < p.n1;
     const uint32_t b = static_cast<uint32_t>(p.b);
+    if constexpr (GRID) {
+      if (run) store_grid(p, acc, reinterpret_cast<float*>(stages), tid, i, j0, mirror);
+      cols = 0;
+    }
     const size_t set = static_cast<size_t>(p.d) * p.b;
     unsigned long long* sums = p.acc + (p.copies > 1 ? static_cast<size_t>(tile + split) % p.copies * set : 0);
-    // the stages' memory is free: every product has been read
-    float* stash = reinterpret_cast<float*>(stages) + tid;
-    if constexpr (MASKED) {
-#pragma unroll
-      for (int q = 0; q < kTile; ++q) stash[q * kTile] = acc[q];
-    }
-    for (int t = 0; t < p.d; ++t) {
+    for (int t = 0; t < (GRID ? 0 : p.d); ++t) {
       const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
       const uint32_t* h2 = h1 + p.n;
       epi_sync();
@@ -578,16 +594,6 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
       if (!row) continue;
       unsigned long long* c = sums + static_cast<size_t>(t) * p.b;
       const uint32_t hr = h1[i];
-      if constexpr (MASKED) {
-        // the row from shared memory: a loop of its own per value
-        const uint32_t hm = mirror ? h2[i] : 0;
-        for (int q = 0; q < cols; ++q) {
-          const float v = stash[q * kTile];
-          bucket_add_masked(c, set, p.bits, i, j0 + q, hr, hcol[q], b, v);
-          if (mirror) bucket_add_masked(c, set, p.bits, j0 + q, i, hcol[kTile + q], hm, b, v);
-        }
-        continue;
-      }
 #pragma unroll
       for (int q = 0; q < kTile; ++q)
         if (q < cols) bucket_add(c, hr, hcol[q], b, acc[q]);
@@ -610,9 +616,9 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
   }
 }
 
-template <bool SPLIT, bool MASKED>
+template <bool SPLIT, bool GRID>
 __global__ void __launch_bounds__(kTileThreads, 2) k_direct_tile(const TileArgs p) {
-  tile_task<SPLIT, MASKED>(p, blockIdx.x, blockIdx.y);
+  tile_task<SPLIT, GRID>(p, blockIdx.x, blockIdx.y);
 }
 
 // Tiles of every product of a batch, the longest first.
@@ -637,6 +643,89 @@ k_direct_pack_batched(const PackArgs* __restrict__ args, const int* __restrict__
     reinterpret_cast<uint32_t*>(&sp)[w] = reinterpret_cast<const uint32_t*>(args + q)[w];
   __syncthreads();
   pack_task(sp, blockIdx.x - static_cast<uint32_t>(__ldg(start + q)));
+}
+
+// A value added to its bucket's sum, to the sums of the bits set in the
+// position i of its row, and to those of the bits set in j.
+__device__ __forceinline__ void bucket_add_masked(unsigned long long* c, size_t set, int bits, uint32_t i, uint32_t j,
+                                                  uint32_t ha, uint32_t hb, uint32_t b, long long v) {
+  uint32_t z = (ha & kBucketMask) + (hb & kBucketMask);
+  if (z >= b) z -= b;
+  const long long iv = ((ha ^ hb) >> 31) ? -v : v;
+  c += z;
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+  for (int m = 0; m < bits; ++m) {
+    c += set;
+    if ((i >> m) & 1u) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+  }
+  for (int m = 0; m < bits; ++m) {
+    c += set;
+    if ((j >> m) & 1u) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c), "l"(iv) : "memory");
+  }
+}
+
+struct GridArgs {
+  const void* grid;
+  int64_t ld;
+  const uint32_t* hs;          // [t][side][n]
+  const DirectScale* scale;
+  unsigned long long* acc;     // [copy][t][b], or [1 + 2 bits][t][b]
+  int copies, bits;
+  int n, n1, n3, b, d;
+};
+
+__device__ __forceinline__ void load4(const float* g, float (&v)[4]) {
+  const float4 x = __ldg(reinterpret_cast<const float4*>(g));
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+}
+__device__ __forceinline__ void load4(const long long* g, long long (&v)[4]) {
+  const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(g)), y = __ldg(reinterpret_cast<const longlong2*>(g) + 1);
+  v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+}
+__device__ __forceinline__ long long to_sum(float v) { return __float2ll_rn(v); }
+__device__ __forceinline__ long long to_sum(long long v) { return v; }
+
+// The entries of the grid added to the buckets: a warp takes 128 columns of
+// kGridRows rows.
+constexpr int kGridRows = 2;
+template <typename T, bool MASKED>
+__global__ void __launch_bounds__(256) k_direct_grid(const GridArgs p) {
+  if (p.scale->bad) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j = static_cast<int>(blockIdx.x) * 128 + lane * 4;
+  const int i0 = (static_cast<int>(blockIdx.y) * 8 + warp) * kGridRows;
+  if (i0 >= p.n1) return;
+  T v[kGridRows][4];
+#pragma unroll
+  for (int r = 0; r < kGridRows; ++r) load4(static_cast<const T*>(p.grid) + (i0 + r) * p.ld + j, v[r]);
+  const uint32_t b = static_cast<uint32_t>(p.b);
+  const size_t set = static_cast<size_t>(p.d) * p.b;
+  unsigned long long* sums = p.acc + (p.copies > 1 ? static_cast<size_t>(blockIdx.x + blockIdx.y) % p.copies * set : 0);
+  for (int t = 0; t < p.d; ++t) {
+    const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
+    const uint32_t* h2 = h1 + p.n;
+    unsigned long long* c = sums + static_cast<size_t>(t) * p.b;
+    uint32_t hc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) hc[q] = j + q < p.n3 ? __ldg(h2 + j + q) : 0;
+#pragma unroll
+    for (int r = 0; r < kGridRows; ++r) {
+      if (i0 + r >= p.n1) break;
+      const uint32_t hr = __ldg(h1 + i0 + r);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (j + q >= p.n3) continue;
+        const long long iv = to_sum(v[r][q]);
+        if constexpr (MASKED) bucket_add_masked(c, set, p.bits, i0 + r, j + q, hr, hc[q], b, iv);
+        else {
+          uint32_t z = (hr & kBucketMask) + (hc[q] & kBucketMask);
+          if (z >= b) z -= b;
+          const long long w = ((hr ^ hc[q]) >> 31) ? -iv : iv;
+          asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c + z), "l"(w) : "memory");
+        }
+      }
+    }
+  }
 }
 
 // COPIES: 32 buckets per block, the copies dealt to its 8 warps.
@@ -709,7 +798,7 @@ uint32_t read_clear_error_direct() {
 }
 
 DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms,
-                            int sets) {
+                            int sets, bool batch) {
   DirectPlan p;
   p.split = dt != CMS_BF16;
   p.alias = alias;
@@ -721,23 +810,34 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   p.tiles = tiles;
   const int per = p.split ? 32 : 64;
   const int64_t images = (n2 + per - 1) / per;
-  // split the inner dimension while blocks are missing, each split adding a
-  // pass of n1 n3 d reductions
-  const int cap = kMaxSb;
-  int best = std::max(1, (p.nsb + cap - 1) / cap);
+  // Splits of the inner dimension (while blocks are missing), and whether the
+  // tiles add their entries to the buckets themselves (fused: d additions per
+  // entry and split, and only the SMs that hold tiles issue them) or store
+  // them for a launch of its own (d additions per entry from every SM; about
+  // 6 us more, and entries beyond L2's reach are not worth storing).
+  const int lo = std::max(1, (p.nsb + kMaxSb - 1) / kMaxSb);
+  int best = lo;
   double cost = 1e30;
   const double slots = 2.0 * sms;
-  for (int s = best; s <= std::min(p.nsb, std::max(best, 64)); ++s) {
-    const int per_split = (p.nsb + s - 1) / s;
-    const int real = (p.nsb + per_split - 1) / per_split;
-    const double waves = std::max(1.0, std::ceil(static_cast<double>(tiles) * real / slots));
-    const double mma = waves * per_split * (p.split ? 1.0 : 0.5) * 1.1e-6;
-    const double red = static_cast<double>(n1) * n3 * h->d * real * 0.5 * (sets + 1) / 2.0e11;
-    if (mma + red < cost) { cost = mma + red; best = real; }
+  const double entries = static_cast<double>(n1) * static_cast<double>(n3);
+  for (int grid = 0; grid < 2; ++grid) {
+    if (grid ? (batch || (sets == 1 && entries > 16.8e6)) : sets > 1) continue;
+    for (int s = lo; s <= std::min(p.nsb, std::max(lo, 64)); ++s) {
+      const int per_split = (p.nsb + s - 1) / s;
+      const int real = (p.nsb + per_split - 1) / per_split;
+      const double blocks = static_cast<double>(tiles) * real;
+      const double waves = std::max(1.0, std::ceil(blocks / slots));
+      const double mma = waves * per_split * (p.split ? 1.0 : 0.5) * 1.1e-6;
+      const double rate = std::min(2.0e11, 1.3e9 * std::min(blocks, static_cast<double>(sms)));
+      const double add = grid ? 6e-6 + entries * (h->d * 0.5 * (sets + 1) + (real > 1 ? 2.0 * real : 0.25)) / 2.0e11
+                              : entries * h->d * real / rate;
+      if (mma + add < cost) { cost = mma + add; best = real; p.grid = grid != 0; }
+    }
   }
+  const bool use_grid = p.grid;
   p.sb_per_split = (p.nsb + best - 1) / best;
   p.splits = (p.nsb + p.sb_per_split - 1) / p.sb_per_split;
-  p.seconds = cost + 15e-6;
+  p.seconds = cost + 30e-6;
   // short sketches: reductions to few words queue up (23 G/s on 2^10 words,
   // 100 on 2^14, 165 on 2^16, 200 from 2^18 on), so blocks share several
   // copies of the sums, which the conversion adds up
@@ -754,7 +854,12 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   // sums, the ticket, the slots taken (all zero before a run)
   p.acc_bytes = static_cast<size_t>(p.copies) * sets * words * 8;
   p.off_acc = o;    o = al(o + p.acc_bytes + 256 + static_cast<size_t>(p.slots) * 4);
+  p.grid64 = p.splits > 1;
+  const size_t grid_bytes = use_grid ? static_cast<size_t>(p.tiles1) * p.tiles3 * kTile * kTile * (p.grid64 ? 8 : 4) : 0;
+  p.off_grid = o;
+  if (p.grid64) o = al(o + grid_bytes);   // sums too: zeroed
   p.zero_bytes = o;
+  if (!p.grid64) { p.off_grid = o; o = al(o + grid_bytes); }
   p.off_fold = o;   o = al(o + static_cast<size_t>(p.slots) * kTile * kTile * sizeof(float));
   p.off_scale = o;  o = al(o + sizeof(DirectScale));
   p.off_blocks = o; o = al(o + static_cast<size_t>(p.tiles1 + t3) * p.nsb * sizeof(int2));
@@ -765,21 +870,31 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   return p;
 }
 
-// Estimated time of the transform route (make_sketch_plan) at its best rate:
-// 40 TFLOP/s of the conventional 5 b log2 b + 4 b per repetition and inner
-// index, which only the warp-specialised kernel reaches (the others run at 6
-// to 18), so the direct route is taken where it is the faster one by a margin.
-static double transform_seconds(const SketchPlan& p, int64_t n2) {
+// Estimated time of the transform route (make_sketch_plan): launches, the
+// conventional 5 b log2 b + 4 b flops per repetition and inner index, and the
+// gathers of its front end (every entry of a_k and b_k for each computed row),
+// at rates fitted per kernel family to 90 calls of n = 64 .. 16384, b = n / 8
+// .. 32 n, 64 to 8192 inner indices (within a factor of two of most).
+static double transform_seconds(const SketchPlan& p, int64_t n1, int64_t n2, int64_t n3, bool batch) {
   const double b = static_cast<double>(p.b);
-  return 20e-6 + static_cast<double>(p.d) * static_cast<double>(n2) * (5.0 * b * std::log2(std::max(b, 2.0)) + 4.0 * b) / 40e12;
+  const double dk = static_cast<double>(p.d) * static_cast<double>(n2);
+  const double gflop = dk * (5.0 * b * std::log2(std::max(b, 2.0)) + 4.0 * b) * 1e-9;
+  const double mgather = dk * p.nrows * static_cast<double>(n1 + n3) * 1e-6;
+  double us;
+  if (p.wide) us = 60.0 + 66.0 * gflop;
+  else if (p.ws) us = 40.0 + 25.0 * gflop;
+  else if (!p.fast) us = 38.0 + 226.0 * gflop + 5.8 * mgather;
+  else us = (p.tmem_rec ? 60.0 : 50.0) + 55.0 * gflop + (p.tmem_rec ? 1.3 : 1.9) * mgather;
+  return 1e-6 * (batch ? us - 38.0 : us);
 }
 
 bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias,
-                   int sms, DirectPlan* out) {
-  // under 64 inner indices the packing and the padding to a superblock show
+                   int sms, DirectPlan* out, bool batch) {
+  // under 64 inner indices the packing and the padding to a superblock show;
+  // the launches of a batch are shared by its instances
   if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535) return false;
-  *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms);
-  return out->seconds < transform_seconds(plan, n2);
+  *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1, batch);
+  return out->seconds - (batch ? 30e-6 : 0.0) < transform_seconds(plan, n1, n2, n3, batch);
 }
 // The masked sums of FINDSIGNIFICANTENTRIES in one pass: an entry is added to
 // its bucket's total and, in the mean, to half of the 2 `bits` masked sums,
@@ -787,10 +902,10 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
 bool choose_direct_significant(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt,
                                bool alias, int sms, int bits, int ell, DirectPlan* out) {
   if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535) return false;
-  *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1 + 2 * bits);
+  *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1 + 2 * bits, false);
   const double sums = static_cast<double>(n1) * static_cast<double>(n3) * h->d * bits * out->splits / 2.0e11 +
                       static_cast<double>(out->acc_bytes) / 3e12;
-  return out->seconds + sums < 2.0 * ell * transform_seconds(plan, n2);
+  return out->seconds + sums < 2.0 * ell * transform_seconds(plan, n1, n2, n3, false);
 }
 
 namespace {
@@ -836,7 +951,8 @@ TileArgs tile_args(const DirectPlan& p, const cms_hashes* h, int64_t n1, int64_t
   a.slot = reinterpret_cast<uint32_t*>(ws + p.off_acc + p.acc_bytes + 256);
   a.slots = p.slots;
   a.copies = p.copies;
-  a.bits = (p.sets - 1) / 2;
+  a.grid = ws + p.off_grid;
+  a.grid64 = p.grid64 ? 1 : 0;
   a.split = p.split ? 1 : 0;
   a.sym = p.alias ? 1 : 0;
   return a;
@@ -925,16 +1041,36 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const TileArgs a = tile_args(p, h, n1, n2, n3, ws);
-  ProfScope prof_scope("k_direct_tile", s);
   const dim3 grid(static_cast<unsigned>(p.tiles), p.splits);
   auto go = [&](auto kern) {
+    ProfScope prof_scope("k_direct_tile", s);
     cudaError_t r = with_smem(kern, tile_smem_bytes());
     if (r != cudaSuccess) return r;
     kern<<<grid, kTileThreads, tile_smem_bytes(), s>>>(a);
     return cudaGetLastError();
   };
-  if (p.sets > 1) return p.split ? go(k_direct_tile<true, true>) : go(k_direct_tile<false, true>);
-  return p.split ? go(k_direct_tile<true, false>) : go(k_direct_tile<false, false>);
+  if (!p.grid) return p.split ? go(k_direct_tile<true, false>) : go(k_direct_tile<false, false>);
+  e = p.split ? go(k_direct_tile<true, true>) : go(k_direct_tile<false, true>);
+  if (e != cudaSuccess) return e;
+  GridArgs g{};
+  g.grid = a.grid;
+  g.ld = static_cast<int64_t>(p.tiles3) * kTile;
+  g.hs = h->d_hs;
+  g.scale = a.scale;
+  g.acc = a.acc;
+  g.copies = p.copies;
+  g.bits = (p.sets - 1) / 2;
+  g.n = a.n; g.n1 = a.n1; g.n3 = a.n3; g.b = a.b; g.d = a.d;
+  ProfScope grid_scope("k_direct_grid", s);
+  const dim3 gg(p.tiles3, static_cast<unsigned>((n1 + 8 * kGridRows - 1) / (8 * kGridRows)));
+  if (p.sets > 1) {
+    if (p.grid64) k_direct_grid<long long, true><<<gg, 256, 0, s>>>(g);
+    else k_direct_grid<float, true><<<gg, 256, 0, s>>>(g);
+  } else {
+    if (p.grid64) k_direct_grid<long long, false><<<gg, 256, 0, s>>>(g);
+    else k_direct_grid<float, false><<<gg, 256, 0, s>>>(g);
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace

@@ -73,11 +73,11 @@ def worst(c, ref):
 
 
 @pytest.mark.parametrize("n1,n2,n3,b,d,dts,alias,pad", [
-    (128, 128, 128, 8192, 2, "f32", True, 0),       # one tile, one superblock
-    (127, 127, 129, 8100, 3, "f32", False, 1),      # one short of and one past a tile
-    (129, 129, 127, 8192, 3, "bf16", False, 1),
-    (257, 95, 257, 16384, 2, "f32", True, 3),       # 3 stages of 32: an odd number in the last drain
-    (300, 65, 300, 20000, 1, "bf16", True, 0),      # one inner index in the second stage of 64
+    (128, 128, 128, 1 << 17, 3, "f32", True, 0),       # one tile, one superblock
+    (127, 127, 129, 64800, 3, "f32", False, 1),      # one short of and one past a tile
+    (129, 129, 127, 1 << 15, 3, "bf16", False, 1),
+    (257, 95, 257, 1 << 17, 2, "f32", True, 3),       # 3 stages of 32: an odd number in the last drain
+    (300, 65, 300, 1 << 18, 2, "bf16", True, 0),      # one inner index in the second stage of 64
     (200, 385, 333, 20000, 2, "f64", False, 0),     # FP64 storage
     (640, 1000, 640, 10240, 3, "f32", True, 0),     # upper triangle of 5 x 5 tiles, split inner dimension
     (512, 9000, 384, 8192, 1, "bf16", False, 0),
@@ -123,10 +123,10 @@ def test_direct_route_over_magnitudes(cms, dts, case):
             return s
         return s * (1e-17 if case == "tiny" else 1e16)
     A, B, Ad, Bd = operands(200, 300, 200, dts, True, 0, 5, scale)
-    h = cms.make_hashes(6, 200, 8192, 2)
+    h = cms.make_hashes(6, 200, 1 << 16, 2)
     c, kernels = run(cms, A, B, h)
     assert "k_direct_tile" in kernels
-    assert worst(c, O.sketch_definition(Ad, Bd, O.make_tables(6, 200, 8192, 2))) < TOL
+    assert worst(c, O.sketch_definition(Ad, Bd, O.make_tables(6, 200, 1 << 16, 2))) < TOL
     h.free()
 
 
@@ -135,7 +135,7 @@ def test_direct_route_over_magnitudes(cms, dts, case):
 def test_non_finite_operands_give_nan_on_both_routes(cms, n2, value):
     A, B, _, _ = operands(200, n2, 200, "f32", False, 0, 9)
     A[3, n2 // 2] = value
-    h = cms.make_hashes(6, 200, 8192, 2)
+    h = cms.make_hashes(6, 200, 1 << 16, 2)
     c, kernels = run(cms, A, B, h)
     assert ("k_direct_tile" in kernels) == (n2 >= 64)
     assert torch.isnan(c).all()

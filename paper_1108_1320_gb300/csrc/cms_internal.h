@@ -322,9 +322,19 @@ struct DirectPlan {
   int sets = 1;             // sums of different entries (1 + 2 L: FINDSIGNIFICANTENTRIES)
   int64_t tiles = 0;
   double seconds = 0.0;     // estimate
+  bool pre = false;         // of pre-sketched operands (PrePlan)
+  bool alias_operands = false;
+  int sms = 0;
   size_t zero_bytes = 0, acc_bytes = 0, off_fold = 0, off_grid = 0;
   size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_pa = 0, off_pb = 0;
   size_t ws_bytes = 0;
+};
+// Pre-sketched operands: one direct product of b rows per repetition.
+struct PrePlan {
+  bool usable = false;
+  int R = 0, C = 0, classes = 0, tiles = 0, rep_blocks = 0;
+  size_t rep_images = 0, off_ent = 0, off_start = 0, off_vhs = 0, off_slab = 0;
+  DirectPlan direct;
 };
 DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms,
                             int sets, bool batch);

@@ -53,6 +53,7 @@ constexpr int kMaxSb = 1024;            // scale factors held per block
 constexpr int kFold = 32;               // drains between folds of the register sums (long inner dimensions)
 constexpr int kFoldFrom = 64;           // drains above which they are folded
 constexpr int kEpiThreads = 128;
+constexpr double kFixedSeconds = 36e-6;   // launches of a single product
 constexpr int kTileThreads = kEpiThreads + 32;
 constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
 constexpr int kMinExp = -100;           // scales stay representable
@@ -266,6 +267,231 @@ __device__ __forceinline__ void pack_task(const PackArgs& p, uint32_t idx) {
 
 __global__ void __launch_bounds__(256) k_direct_pack(const PackArgs p) { pack_task(p, blockIdx.x); }
 
+// ---- pre-sketched operands: b well below n ----
+// By Fig. 1 c_t is the cyclic convolution of the count sketches of a_k and
+// b_k, summed over k: with A'_t = S1 A (b x n2) and B'_t = B S2 (n2 x b) it is
+// the sum over the entries of A'_t B'_t whose two positions add up to z mod b,
+// the direct route's problem with b in the place of n1 and n3.
+//
+//  * k_pre_transpose: the operand as slabs [superblock][i][128] of FP32, so
+//    that an entry of a column is 512 contiguous bytes over its inner indices
+//    and a slab (n x 512 bytes) stays in L2 while every repetition and side
+//    reads it;
+//  * k_pre_lists: the entries of every bucket, from the bucket lists by h mod
+//    C: bucket z = C z1 + z2 has the row u = z2 R + z1 of A'_t;
+//  * k_pre_pack: 128 buckets x 128 inner indices per block, a warp 16 buckets:
+//    the sums of its entries' rows in registers, then scaled, split and
+//    stored as k_direct_pack does.
+// X^T X of 2048 x 16384 FP32, b = 2048, d = 5: 7.2 ms through the
+// shared-memory transform kernel (every entry gathered for each of its rows,
+// with its twiddle), 6.9 ms through the tiles of n1 x n3 (1.3e9 additions),
+// 0.62 ms this way (transpose 74 us, lists 6, sums and packing 200, tiles
+// 306).  What bounds it: the tiles (b^2 n2 d multiply-adds), and the 1.3 GB of
+// rows read by the sums.  It is the cheapest way from b of about n / 4 down;
+// over 130 calls of n = 64 .. 16384, b = n / 8 .. 32 n, 64 to 8192 inner
+// indices it won 22 times, by up to 6.7 over the transform route.
+struct PreArgs {
+  const void* X[2];
+  int64_t ld[2];
+  int64_t n[2];
+  int alias;
+  int64_t K;
+  int nsb, d;
+  int hn;                 // hash domain
+  int R, C, classes, tiles;   // classes of R buckets per tile of 128 rows
+  float* slab[2];         // [superblock][n][128]
+  const uint32_t* hs;     // [t][side][hn]
+  const uint32_t* perm;
+  const uint32_t* off;    // [t][side][C + 1]
+  uint32_t* ent;          // [t][side][hn]: x | sign << 31, by row
+  uint32_t* start;        // [t][side][tiles 128 + 1]
+  uint32_t* vhs;          // [2][tiles 128]: bucket of each row
+  PackArgs pack;          // repetition 0
+  size_t rep_images;
+  int rep_blocks;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_pre_transpose(const PreArgs p) {
+  __shared__ float sh[kSuper][33];
+  const int side = blockIdx.z;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * 32 + lane;
+  const int64_t k0 = static_cast<int64_t>(blockIdx.y) * kSuper;
+  if (static_cast<int64_t>(blockIdx.x) * 32 >= p.n[side]) return;
+  const T* X = static_cast<const T*>(p.X[side]);
+#pragma unroll
+  for (int q = 0; q < kSuper / 8; ++q) {
+    const int k = q * 8 + warp;
+    sh[k][lane] = i < p.n[side] && k0 + k < p.K ? load_val(X + (k0 + k) * p.ld[side] + i) : 0.f;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int x = q * 8 + warp;
+    const int64_t xi = static_cast<int64_t>(blockIdx.x) * 32 + x;
+    if (xi >= p.n[side]) continue;
+    float* dst = p.slab[side] + (static_cast<size_t>(blockIdx.y) * p.n[side] + xi) * kSuper;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) dst[g * 32 + lane] = sh[g * 32 + lane][x];
+  }
+}
+
+// A warp per class z2 of one (t, side): its entries by z1, in their order.
+__global__ void __launch_bounds__(256) k_pre_lists(const PreArgs p) {
+  const int lane = threadIdx.x & 31;
+  const int z2 = static_cast<int>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const size_t ts = blockIdx.y;
+  const int rows = p.tiles * kTile;
+  if (z2 >= p.C) return;
+  const uint32_t* off = p.off + ts * (p.C + 1);
+  const uint32_t e0 = off[z2], e1 = off[z2 + 1];
+  uint32_t* ent = p.ent + ts * p.hn;
+  uint32_t* start = p.start + ts * (rows + 1);
+  const int row0 = z2 / p.classes * kTile + z2 % p.classes * p.R;   // of bucket (z1 = 0, z2)
+  uint32_t at = e0;
+  for (int z1 = 0; z1 < p.R; ++z1) {
+    if (lane == 0) {
+      start[row0 + z1] = at;
+      if (ts < 2) p.vhs[ts * rows + row0 + z1] = static_cast<uint32_t>(z1 * p.C + z2);
+    }
+    for (uint32_t e = e0; e < e1; e += 32) {
+      uint32_t w = 0, x = 0;
+      bool mine = false;
+      if (e + lane < e1) {
+        x = p.perm[ts * p.hn + e + lane];
+        w = p.hs[ts * p.hn + x];
+        mine = static_cast<int>((w & kBucketMask) / static_cast<uint32_t>(p.C)) == z1;
+      }
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, mine);
+      if (mine) ent[at + __popc(m & ((1u << lane) - 1u))] = x | (w & 0x80000000u);
+      at += __popc(m);
+    }
+  }
+  // rows of the tile that hold no bucket (128 is no multiple of R, or the last tile)
+  const bool last_of_tile = z2 % p.classes == p.classes - 1 || z2 == p.C - 1;
+  const int pad_end = z2 == p.C - 1 ? rows + 1 : (z2 / p.classes + 1) * kTile;
+  if (last_of_tile)
+    for (int r = row0 + p.R + lane; r < pad_end; r += 32) {
+      start[r] = e1;
+      if (ts < 2 && r < rows) p.vhs[ts * rows + r] = 0;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_pre_pack(const PreArgs p) {
+  extern __shared__ __align__(1024) uint8_t img[];
+  __shared__ float fsh[8];
+  __shared__ int ish[8];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // superblocks slowest: their slab stays in L2
+  const int per_sb = p.tiles * 2 * p.d;
+  const int sb = static_cast<int>(blockIdx.x) / per_sb;
+  int rest = static_cast<int>(blockIdx.x) - sb * per_sb;
+  const int ts = rest / p.tiles, tile = rest - ts * p.tiles;
+  const int t = ts >> 1, side = ts & 1;
+  const int64_t n = p.n[side];
+  const float* slab = p.slab[p.alias ? 0 : side] + static_cast<size_t>(sb) * n * kSuper + lane * 4;
+  const uint32_t* ent = p.ent + static_cast<size_t>(ts) * p.hn;
+  const uint32_t* start = p.start + static_cast<size_t>(ts) * (p.tiles * kTile + 1) + tile * kTile + warp * 16;
+  const uint32_t bound = lane <= 16 ? start[lane] : 0;
+  float v[16][4];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const uint32_t e0 = __shfl_sync(0xFFFFFFFFu, bound, r), e1 = __shfl_sync(0xFFFFFFFFu, bound, r + 1);
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+    for (uint32_t e = e0; e < e1; e += 32) {
+      const uint32_t mine = e + lane < e1 ? ent[e + lane] : 0x7FFFFFFFu;
+      const int cnt = static_cast<int>(min(e1 - e, 32u));
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int q = 0; q < cnt; q += 4) {
+        float4 x[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const uint32_t w = __shfl_sync(0xFFFFFFFFu, mine, min(q + g, 31));
+          const uint32_t xi = w & kBucketMask;
+          x[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (q + g < cnt && static_cast<int64_t>(xi) < n)
+            x[g] = __ldg(reinterpret_cast<const float4*>(slab + static_cast<size_t>(xi) * kSuper));
+          if (w >> 31) x[g] = make_float4(-x[g].x, -x[g].y, -x[g].z, -x[g].w);
+        }
+        s[0] += (x[0].x + x[1].x) + (x[2].x + x[3].x);
+        s[1] += (x[0].y + x[1].y) + (x[2].y + x[3].y);
+        s[2] += (x[0].z + x[1].z) + (x[2].z + x[3].z);
+        s[3] += (x[0].w + x[1].w) + (x[2].w + x[3].w);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) a[q] += s[q];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[r][q] = a[q];
+  }
+  uint32_t m = 0;
+#pragma unroll
+  for (int r = 0; r < 16; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) m = max(m, __float_as_uint(v[r][q]) & 0x7FFFFFFFu);
+  m = static_cast<uint32_t>(block_max256(static_cast<int>(m), ish));
+  const bool bad = m >= 0x7F800000u;
+  const int e = bad ? 0 : max(static_cast<int>(m >> 23) - 127, kMinExp);
+  const int sh = direct_scale_log2(true) - e;
+  const float f1 = pow2f(sh / 2), f2 = pow2f(sh - sh / 2);
+  float nn = 0.f;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    uint32_t hi[2], lo[2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v[r][q] = v[r][q] * f1 * f2;
+      nn = fmaf(v[r][q], v[r][q], nn);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const __half ha = __float2half_rn(v[r][2 * q]), hb = __float2half_rn(v[r][2 * q + 1]);
+      const __half2 h2 = __halves2half2(ha, hb);
+      const __half2 l2 = __floats2half2_rn(v[r][2 * q] - __half2float(ha), v[r][2 * q + 1] - __half2float(hb));
+      hi[q] = *reinterpret_cast<const uint32_t*>(&h2);
+      lo[q] = *reinterpret_cast<const uint32_t*>(&l2);
+    }
+    // inner indices 4 lane .. 4 lane + 3: image lane / 8 (32 of them), 8-byte
+    // half of 16-byte column (lane / 2) mod 4 (hi) and 4 beyond (lo)
+    const int row = warp * 16 + r;
+    uint8_t* base = img + (lane >> 3) * kStageBytes + (row >> 3) * 1024 + (row & 7) * 128 + (lane & 1) * 8;
+    const int c = (lane >> 1) & 3;
+    *reinterpret_cast<uint2*>(base + ((c ^ (row & 7)) << 4)) = make_uint2(hi[0], hi[1]);
+    *reinterpret_cast<uint2*>(base + (((c + 4) ^ (row & 7)) << 4)) = make_uint2(lo[0], lo[1]);
+  }
+  nn = block_sum256(nn, fsh);
+  fence_proxy_async();
+  __syncthreads();
+  PackArgs pk = p.pack;
+#pragma unroll
+  for (int sd = 0; sd < 2; ++sd) {
+    pk.side[sd].out += t * p.rep_images;
+    pk.side[sd].blocks += static_cast<size_t>(t) * p.rep_blocks;
+  }
+  pk.ticket += t;
+  pk.scale += t;
+  if (threadIdx.x == 0) {
+    pk.side[side].blocks[static_cast<size_t>(tile) * p.nsb + sb] = make_int2(bad ? kBadExp : e, __float_as_int(nn));
+    const int64_t left = min(p.K - static_cast<int64_t>(sb) * kSuper, static_cast<int64_t>(kSuper));
+    const int64_t per_tile = (p.K + 31) / 32;
+    uint8_t* dst = pk.side[side].out + (static_cast<size_t>(tile) * per_tile + static_cast<size_t>(sb) * 4) * kStageBytes;
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(img)),
+                 "r"(static_cast<uint32_t>((left + 31) / 32) * kStageBytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    __threadfence();
+    last = atomicAdd(pk.ticket, 1u) == static_cast<uint32_t>(2 * p.tiles * p.nsb) - 1;
+  }
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    direct_scale(pk, fsh, ish);
+  }
+  if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
 struct TileArgs {
   const uint8_t* pa;
   const uint8_t* pb;
@@ -275,6 +501,12 @@ struct TileArgs {
   const uint32_t* hs;          // [t][side][n]
   unsigned long long* acc;     // [copy][t][b]
   int copies;                  // blocks add to copy (block mod copies)
+  // more than one pair of operands (repetitions of pre-sketched operands):
+  // bytes and superblocks from one pair's to the next; one scale and b
+  // buckets each
+  size_t rep_images;
+  int rep_blocks;
+  int reps;
   void* grid;                  // entries in units of the integer sums, rows of tiles3 * 128: FP32, or
   int grid64;                  //   64-bit integers added by the splits of the inner dimension
   int64_t K;
@@ -370,7 +602,7 @@ __device__ __forceinline__ void store_grid(const TileArgs& p, const float (&acc)
 // GRID: the entries go to p.grid (k_direct_grid adds them to the buckets);
 // else straight to the buckets.
 template <bool SPLIT, bool GRID = false>
-__device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split) {
+__device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split, int rep) {
   constexpr int kImages = SPLIT ? 4 : 2;
   constexpr int kPerStage = kSuper / kImages;
   extern __shared__ uint8_t smem_raw[];
@@ -423,10 +655,11 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
     tmem_alloc(&s_tmem, 2 * kTile);
     tmem_relinquish();
   }
-  const DirectScale sc = *p.scale;
+  const DirectScale sc = p.scale[rep];
   for (int q = tid; q < sb1 - sb0; q += kTileThreads) {
-    const int de = p.ea[static_cast<size_t>(ti) * p.nsb + sb0 + q].x - sc.emax[0] +
-                   p.eb[static_cast<size_t>(tj) * p.nsb + sb0 + q].x - sc.emax[1];
+    const size_t rb = static_cast<size_t>(rep) * p.rep_blocks;
+    const int de = p.ea[rb + static_cast<size_t>(ti) * p.nsb + sb0 + q].x - sc.emax[0] +
+                   p.eb[rb + static_cast<size_t>(tj) * p.nsb + sb0 + q].x - sc.emax[1];
     factor[q] = de < -126 ? 0.f : pow2f(min(de, 0));
   }
   tmem_fence_before_sync();
@@ -439,8 +672,8 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
       // D: FP32; A, B: FP16 (0) or BF16 (1), K-major; N / 8, M / 16
       constexpr uint32_t idesc = (1u << 4) | ((SPLIT ? 0u : 1u) << 7) | ((SPLIT ? 0u : 1u) << 10) |
                                  (static_cast<uint32_t>(kTile / 8) << 17) | (static_cast<uint32_t>(kTile / 16) << 24);
-      const uint8_t* ga = p.pa + (static_cast<size_t>(ti) * per_tile + st0) * kStageBytes;
-      const uint8_t* gb = p.pb + (static_cast<size_t>(tj) * per_tile + st0) * kStageBytes;
+      const uint8_t* ga = p.pa + rep * p.rep_images + (static_cast<size_t>(ti) * per_tile + st0) * kStageBytes;
+      const uint8_t* gb = p.pb + rep * p.rep_images + (static_cast<size_t>(tj) * per_tile + st0) * kStageBytes;
       auto load = [&](int st) {
         uint8_t* dst = stages + (st % kStages) * 2 * kStageBytes;
         uint64_t* bar = &full[st % kStages];
@@ -580,8 +813,9 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
       if (run) store_grid(p, acc, reinterpret_cast<float*>(stages), tid, i, j0, mirror);
       cols = 0;
     }
-    const size_t set = static_cast<size_t>(p.d) * p.b;
-    unsigned long long* sums = p.acc + (p.copies > 1 ? static_cast<size_t>(tile + split) % p.copies * set : 0);
+    const size_t set = static_cast<size_t>(p.d) * (p.reps > 1 ? p.reps : 1) * p.b;
+    unsigned long long* sums = p.acc + static_cast<size_t>(rep) * p.b +
+                               (p.copies > 1 ? static_cast<size_t>(tile + split) % p.copies * set : 0);
     for (int t = 0; t < (GRID ? 0 : p.d); ++t) {
       const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
       const uint32_t* h2 = h1 + p.n;
@@ -618,7 +852,7 @@ __device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split
 
 template <bool SPLIT, bool GRID>
 __global__ void __launch_bounds__(kTileThreads, 2) k_direct_tile(const TileArgs p) {
-  tile_task<SPLIT, GRID>(p, blockIdx.x, blockIdx.y);
+  tile_task<SPLIT, GRID>(p, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // Tiles of every product of a batch, the longest first.
@@ -631,8 +865,8 @@ k_direct_tile_batched(const TileArgs* __restrict__ args, const int* __restrict__
   __syncthreads();
   const int local = static_cast<int>(blockIdx.x) - __ldg(start + q);
   const int tile = local % sp.tiles, split = local / sp.tiles;
-  if (sp.split) tile_task<true>(sp, tile, split);
-  else tile_task<false>(sp, tile, split);
+  if (sp.split) tile_task<true>(sp, tile, split, 0);
+  else tile_task<false>(sp, tile, split, 0);
 }
 
 __global__ void __launch_bounds__(256)
@@ -728,11 +962,11 @@ __global__ void __launch_bounds__(256) k_direct_grid(const GridArgs p) {
   }
 }
 
-// COPIES: 32 buckets per block, the copies dealt to its 8 warps.
+// `per` buckets share a scale.  COPIES: 32 buckets per block, the copies
+// dealt to its 8 warps.
 template <bool COPIES>
 __global__ void __launch_bounds__(256) k_direct_finish(const unsigned long long* acc, int copies, float* c, int64_t len,
-                                                       const DirectScale* scale, int log2s) {
-  const DirectScale sc = *scale;
+                                                       int64_t per, const DirectScale* scale, int log2s) {
   if constexpr (COPIES) {
     __shared__ unsigned long long part[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -747,12 +981,12 @@ __global__ void __launch_bounds__(256) k_direct_finish(const unsigned long long*
     if (warp == 0 && q < len) {
 #pragma unroll
       for (int w = 1; w < 8; ++w) v += part[w][lane];
-      c[q] = direct_value(v, sc, log2s);
+      c[q] = direct_value(v, scale[q / per], log2s);
     }
   } else {
     for (int64_t q = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; q < len;
          q += static_cast<int64_t>(gridDim.x) * 256)
-      c[q] = direct_value(acc[q], sc, log2s);
+      c[q] = direct_value(acc[q], scale[q / per], log2s);
   }
 }
 
@@ -837,7 +1071,7 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   const bool use_grid = p.grid;
   p.sb_per_split = (p.nsb + best - 1) / best;
   p.splits = (p.nsb + p.sb_per_split - 1) / p.sb_per_split;
-  p.seconds = cost + 30e-6;
+  p.seconds = cost + kFixedSeconds;
   // short sketches: reductions to few words queue up (23 G/s on 2^10 words,
   // 100 on 2^14, 165 on 2^16, 200 from 2^18 on), so blocks share several
   // copies of the sums, which the conversion adds up
@@ -873,19 +1107,82 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
 // Estimated time of the transform route (make_sketch_plan): launches, the
 // conventional 5 b log2 b + 4 b flops per repetition and inner index, and the
 // gathers of its front end (every entry of a_k and b_k for each computed row),
-// at rates fitted per kernel family to 90 calls of n = 64 .. 16384, b = n / 8
+// at rates fitted per kernel family to 130 calls of n = 64 .. 16384, b = n / 8
 // .. 32 n, 64 to 8192 inner indices (within a factor of two of most).
 static double transform_seconds(const SketchPlan& p, int64_t n1, int64_t n2, int64_t n3, bool batch) {
   const double b = static_cast<double>(p.b);
   const double dk = static_cast<double>(p.d) * static_cast<double>(n2);
   const double gflop = dk * (5.0 * b * std::log2(std::max(b, 2.0)) + 4.0 * b) * 1e-9;
-  const double mgather = dk * p.nrows * static_cast<double>(n1 + n3) * 1e-6;
+  const int rows = p.fast ? (p.nrows + 1) / 2 * 2 : p.nrows;   // the register kernels take two at a time
+  const double mgather = dk * rows * static_cast<double>(n1 + n3) * 1e-6;
   double us;
   if (p.wide) us = 60.0 + 66.0 * gflop;
   else if (p.ws) us = 40.0 + 25.0 * gflop;
   else if (!p.fast) us = 38.0 + 226.0 * gflop + 5.8 * mgather;
-  else us = (p.tmem_rec ? 60.0 : 50.0) + 55.0 * gflop + (p.tmem_rec ? 1.3 : 1.9) * mgather;
+  else us = (p.tmem_rec ? 60.0 : 50.0) + 55.0 * gflop + (p.tmem_rec ? 2.2 : 2.5) * mgather;
   return 1e-6 * (batch ? us - 38.0 : us);
+}
+
+// Pre-sketched operands: the direct route's tiles over b x b x n2 for each
+// repetition.
+PrePlan make_pre_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, bool alias, int sms) {
+  PrePlan q;
+  if (h->C <= 0 || h->R > kTile || h->d_perm == nullptr) return q;
+  q.R = static_cast<int>(h->R);
+  q.C = static_cast<int>(h->C);
+  q.classes = kTile / q.R;
+  q.tiles = (q.C + q.classes - 1) / q.classes;
+  if (q.tiles > 128) return q;    // b above about 16384 is never cheap
+  const int64_t rows = static_cast<int64_t>(q.tiles) * kTile;
+  DirectPlan& p = q.direct;
+  p.split = true;
+  p.tiles1 = p.tiles3 = q.tiles;
+  p.tiles = static_cast<int64_t>(q.tiles) * q.tiles;
+  p.nsb = static_cast<int>((n2 + kSuper - 1) / kSuper);
+  const int lo = std::max(1, (p.nsb + kMaxSb - 1) / kMaxSb);
+  int best = lo;
+  double cost = 1e30;
+  const double entries = static_cast<double>(rows) * rows * h->d;
+  for (int s = lo; s <= std::min(p.nsb, std::max(lo, 64)); ++s) {
+    const int per_split = (p.nsb + s - 1) / s;
+    const int real = (p.nsb + per_split - 1) / per_split;
+    const double blocks = static_cast<double>(p.tiles) * h->d * real;
+    const double t = std::max(1.0, std::ceil(blocks / (2.0 * sms))) * per_split * 1.1e-6 +
+                     entries * real / std::min(5.0e11, 4e9 * std::min(blocks, static_cast<double>(sms)));
+    if (t < cost) { cost = t; best = real; }
+  }
+  p.sb_per_split = (p.nsb + best - 1) / best;
+  p.splits = (p.nsb + p.sb_per_split - 1) / p.sb_per_split;
+  const double n = static_cast<double>(alias ? n1 : n1 + n3), k = static_cast<double>(p.nsb) * kSuper;
+  p.seconds = cost + 50e-6 + n * k * 8.0 / 4e12 + static_cast<double>(n1 + n3) * k * h->d * 4.0 / 5e12 +
+              2.0 * static_cast<double>(rows) * k * h->d * 4.0 / 3e12;
+  auto al = [](size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); };
+  const int64_t words = static_cast<int64_t>(h->d) * h->b;
+  p.copies = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({256, (int64_t{1} << 18) / words, p.tiles * p.splits})));
+  const int64_t images = (n2 + 31) / 32;
+  size_t o = 0;
+  const int drains = p.sb_per_split * 2;
+  p.slots = drains > kFoldFrom ? 2 * sms : 0;
+  p.acc_bytes = static_cast<size_t>(p.copies) * words * 8;
+  // sums, a ticket per repetition, the slots taken: zero before a run
+  p.off_acc = o;    o = al(o + p.acc_bytes + 256 + static_cast<size_t>(p.slots) * 4);
+  p.zero_bytes = o;
+  p.off_fold = o;   o = al(o + static_cast<size_t>(p.slots) * kTile * kTile * sizeof(float));
+  p.off_scale = o;  o = al(o + sizeof(DirectScale) * h->d);
+  q.rep_blocks = 2 * q.tiles * p.nsb;
+  p.off_blocks = o; o = al(o + static_cast<size_t>(q.rep_blocks) * h->d * sizeof(int2));
+  const size_t side = static_cast<size_t>(q.tiles) * images * kStageBytes;
+  q.rep_images = 2 * side;
+  p.off_pa = o;
+  p.off_pb = o + side;
+  o = al(o + q.rep_images * h->d);
+  q.off_ent = o;    o = al(o + static_cast<size_t>(2 * h->d) * h->n * 4);
+  q.off_start = o;  o = al(o + static_cast<size_t>(2 * h->d) * (rows + 1) * 4);
+  q.off_vhs = o;    o = al(o + static_cast<size_t>(2) * rows * 4);
+  q.off_slab = o;   o = al(o + static_cast<size_t>(p.nsb) * (alias ? n1 : n1 + n3) * kSuper * 4);
+  p.ws_bytes = o;
+  q.usable = true;
+  return q;
 }
 
 bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias,
@@ -894,8 +1191,21 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
   // the launches of a batch are shared by its instances
   if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535) return false;
   *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1, batch);
-  return out->seconds - (batch ? 30e-6 : 0.0) < transform_seconds(plan, n1, n2, n3, batch);
+  double best = out->seconds - (batch ? kFixedSeconds : 0.0);
+  if (!batch) {
+    const PrePlan pre = make_pre_plan(h, n1, n2, n3, alias, sms);
+    if (pre.usable && pre.direct.seconds < best) {
+      *out = pre.direct;
+      out->pre = true;
+      out->alias_operands = alias;
+      out->sms = sms;
+      best = pre.direct.seconds;
+    }
+  }
+  // a margin for the estimates' error where both are mostly launches
+  return best + (batch ? 0.0 : 4e-6) < transform_seconds(plan, n1, n2, n3, batch);
 }
+
 // The masked sums of FINDSIGNIFICANTENTRIES in one pass: an entry is added to
 // its bucket's total and, in the mean, to half of the 2 `bits` masked sums,
 // against 2 ell products.
@@ -933,6 +1243,7 @@ TileArgs tile_args(const DirectPlan& p, const cms_hashes* h, int64_t n1, int64_t
   a.pb = reinterpret_cast<uint8_t*>(ws + p.off_pb);
   a.ea = reinterpret_cast<int2*>(ws + p.off_blocks);
   a.eb = p.alias ? a.ea : a.ea + static_cast<size_t>(p.tiles1) * p.nsb;
+  a.reps = 1;
   a.scale = reinterpret_cast<DirectScale*>(ws + p.off_scale);
   a.hs = h->d_hs;
   a.acc = reinterpret_cast<unsigned long long*>(ws + p.off_acc);
@@ -1073,24 +1384,99 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
   return cudaGetLastError();
 }
 
-}  // namespace
-
-cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
-                          int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws,
-                          cudaStream_t s) {
-  cudaError_t e = launch_sums(p, h, A, lda, B, ldb, n1, n2, n3, dt, ws, s);
-  if (e != cudaSuccess) return e;
+// `per` buckets share a scale.
+cudaError_t launch_finish(const DirectPlan& p, const cms_hashes* h, float* c, int64_t per, char* ws, cudaStream_t s) {
   const int64_t len = static_cast<int64_t>(h->d) * h->b;
   const unsigned long long* acc = reinterpret_cast<const unsigned long long*>(ws + p.off_acc);
   const DirectScale* scale = reinterpret_cast<const DirectScale*>(ws + p.off_scale);
   ProfScope prof_scope("k_direct_finish", s);
   if (p.copies > 1)
-    k_direct_finish<true><<<static_cast<unsigned>((len + 31) / 32), 256, 0, s>>>(acc, p.copies, c, len, scale,
+    k_direct_finish<true><<<static_cast<unsigned>((len + 31) / 32), 256, 0, s>>>(acc, p.copies, c, len, per, scale,
                                                                                  direct_scale_log2(p.split));
   else
     k_direct_finish<false><<<static_cast<unsigned>(std::min<int64_t>((len + 255) / 256, 152 * 8)), 256, 0, s>>>(
-        acc, 1, c, len, scale, direct_scale_log2(p.split));
+        acc, 1, c, len, per, scale, direct_scale_log2(p.split));
   return cudaGetLastError();
+}
+
+}  // namespace
+
+namespace {
+
+cudaError_t launch_pre(const DirectPlan& chosen, const cms_hashes* h, const void* A, int64_t lda, const void* B,
+                       int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws, cudaStream_t s) {
+  const bool alias = chosen.alias_operands;
+  const PrePlan q = make_pre_plan(h, n1, n2, n3, alias, chosen.sms);
+  const DirectPlan& p = q.direct;
+  const int rows = q.tiles * kTile;
+  PreArgs a{};
+  a.X[0] = A; a.X[1] = B;
+  a.ld[0] = lda; a.ld[1] = ldb;
+  a.n[0] = n1; a.n[1] = n3;
+  a.alias = alias ? 1 : 0;
+  a.K = n2;
+  a.nsb = p.nsb;
+  a.d = h->d;
+  a.hn = static_cast<int>(h->n);
+  a.R = q.R; a.C = q.C; a.classes = q.classes; a.tiles = q.tiles;
+  a.slab[0] = reinterpret_cast<float*>(ws + q.off_slab);
+  a.slab[1] = alias ? a.slab[0] : a.slab[0] + static_cast<size_t>(p.nsb) * n1 * kSuper;
+  a.hs = h->d_hs;
+  a.perm = h->d_perm;
+  a.off = h->d_off;
+  a.ent = reinterpret_cast<uint32_t*>(ws + q.off_ent);
+  a.start = reinterpret_cast<uint32_t*>(ws + q.off_start);
+  a.vhs = reinterpret_cast<uint32_t*>(ws + q.off_vhs);
+  a.pack = pack_args(p, nullptr, 0, nullptr, 0, rows, n2, rows, CMS_F32, ws);
+  a.rep_images = q.rep_images;
+  a.rep_blocks = q.rep_blocks;
+  cudaError_t e = cudaMemsetAsync(ws + p.off_acc, 0, p.zero_bytes, s);
+  if (e != cudaSuccess) return e;
+  {
+    ProfScope prof_scope("k_pre_transpose", s);
+    const dim3 grid(static_cast<unsigned>((std::max(n1, n3) + 31) / 32), p.nsb, alias ? 1 : 2);
+    if (dt == CMS_BF16) k_pre_transpose<__nv_bfloat16><<<grid, 256, 0, s>>>(a);
+    else if (dt == CMS_F64) k_pre_transpose<double><<<grid, 256, 0, s>>>(a);
+    else k_pre_transpose<float><<<grid, 256, 0, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  {
+    ProfScope prof_scope("k_pre_lists", s);
+    k_pre_lists<<<dim3((q.C + 7) / 8, 2 * h->d), 256, 0, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  {
+    ProfScope prof_scope("k_pre_pack", s);
+    if ((e = with_smem(k_pre_pack, 4 * kStageBytes)) != cudaSuccess) return e;
+    k_pre_pack<<<p.nsb * q.tiles * 2 * h->d, 256, 4 * kStageBytes, s>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  TileArgs ta = tile_args(p, h, rows, n2, rows, ws);
+  ta.hs = a.vhs;
+  ta.n = rows;
+  ta.d = 1;
+  ta.reps = h->d;
+  ta.rep_images = q.rep_images;
+  ta.rep_blocks = q.rep_blocks;
+  {
+    ProfScope prof_scope("k_direct_tile", s);
+    if ((e = with_smem(k_direct_tile<true, false>, tile_smem_bytes())) != cudaSuccess) return e;
+    k_direct_tile<true, false><<<dim3(static_cast<unsigned>(p.tiles), p.splits, h->d), kTileThreads, tile_smem_bytes(),
+                                 s>>>(ta);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return launch_finish(p, h, c, h->b, ws, s);
+}
+
+}  // namespace
+
+cudaError_t launch_direct(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
+                          int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, float* c, char* ws,
+                          cudaStream_t s) {
+  if (p.pre) return launch_pre(p, h, A, lda, B, ldb, n1, n2, n3, dt, c, ws, s);
+  cudaError_t e = launch_sums(p, h, A, lda, B, ldb, n1, n2, n3, dt, ws, s);
+  if (e != cudaSuccess) return e;
+  return launch_finish(p, h, c, static_cast<int64_t>(h->d) * h->b, ws, s);
 }
 
 cudaError_t launch_direct_significant(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda,

@@ -264,3 +264,43 @@ def test_find_significant_on_the_direct_route(cms, n1, n2, n3, rho, alias):
     assert "k_direct_sig_decode" in kernels and "k_mask_copy" not in kernels
     assert [tuple(p) for p in got.cpu().numpy().tolist()] == want and count == len(want)
     h.free()
+
+
+@pytest.mark.parametrize("n1,n2,n3,b,d,dts,alias,pad", [
+    (3000, 500, 2500, 600, 3, "f32", False, 1),    # R = 1, a last superblock of 116 inner indices
+    (5000, 300, 5000, 1500, 2, "bf16", True, 0),   # R = 2, C = 750: the last tile is not full
+    (8000, 257, 8000, 2916, 3, "f32", True, 0),    # R = 4 (128 rows hold 32 classes), one inner index in the last stage
+    (6000, 400, 6000, 2187, 3, "f64", True, 3),    # R = 3: rows without a bucket in every tile
+])
+def test_pre_sketched_operands_match_oracle(cms, n1, n2, n3, b, d, dts, alias, pad):
+    n = max(n1, n3)
+    A, B, Ad, Bd = operands(n1, n2, n3, dts, alias, pad, n1)
+    h = cms.make_hashes(n1, n, b, d)
+    c, kernels = run(cms, A, B, h)
+    assert "k_pre_pack" in kernels
+    tab = O.make_tables(n1, n, b, d)
+    ref = O.sketch_definition(Ad, Bd, tab)
+    assert worst(c, ref) < TOL
+    c2, _ = run(cms, A, B, h)
+    assert torch.equal(c, c2)
+    A[7, n2 // 2] = float("nan")
+    c, _ = run(cms, A, B, h)
+    assert torch.isnan(c).all()
+    h.free()
+
+
+def test_pre_sketched_operands_skewed_tables(cms):
+    # every row of A in two buckets (lists of 2000 entries), columns of B spread
+    n, m, b = 4000, 200, 512
+    g = W.rng(5)
+    h1 = (np.arange(n) % 2 * 300)[None, :].astype(np.uint32)
+    h2 = g.integers(0, b, size=(1, n)).astype(np.uint32)
+    s1 = g.choice([-1, 1], size=(1, n)).astype(np.int8)
+    s2 = g.choice([-1, 1], size=(1, n)).astype(np.int8)
+    h = cms.Hashes.from_tables(h1, s1, h2, s2, b)
+    A, B, Ad, Bd = operands(n, m, n, "f32", True, 0, 6)
+    c, kernels = run(cms, A, B, h)
+    assert "k_pre_pack" in kernels
+    tab = O.Tables(h1.astype(np.int64), s1.astype(np.int64), h2.astype(np.int64), s2.astype(np.int64), b)
+    assert worst(c, O.sketch_definition(Ad, Bd, tab)) < TOL
+    h.free()

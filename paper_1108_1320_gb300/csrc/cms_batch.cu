@@ -256,9 +256,11 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
       b->is_direct[i] = hit->second.nkc == 0;
     } else if (flags & CMS_BATCH_AUTOTUNE) {
       char* tws = nullptr;
-      cudaError_t e = cudaMalloc(&tws, std::max<size_t>(std::max(p.ws_bytes, b->direct[i].ws_bytes), 256));
+      // (the batch's own plan leaves the tile kernel's words to the batch)
+      const DirectPlan one = make_direct_plan(it.h, it.n1, it.n2, it.n3, it.dt, b->direct[i].alias, sms, 1, false);
+      cudaError_t e = cudaMalloc(&tws, std::max<size_t>(std::max(p.ws_bytes, one.ws_bytes), 256));
       double td = 0.0, tt = 0.0;
-      if (e == cudaSuccess) e = time_plan(p, it, tws, s, &td, &b->direct[i]);
+      if (e == cudaSuccess) e = time_plan(p, it, tws, s, &td, &one);
       if (e == cudaSuccess) e = time_plan(p, it, tws, s, &tt);
       if (tws) cudaFree(tws);
       if (e != cudaSuccess) { delete b; return cuda_fail(e, "cms_batch_create (autotune)"); }
@@ -422,11 +424,11 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
                                  b->ws + b->ws_off[i]});
     }
     if (!specs.empty()) {
-      e = cudaMalloc(&b->d_direct, direct_batch_bytes(static_cast<int>(specs.size())));
-      if (e == cudaSuccess) e = build_direct_batch(specs, b->d_direct, &b->direct_batch, s);
+      e = cudaMalloc(&b->d_direct, direct_batch_bytes(static_cast<int>(specs.size()), sms));
+      if (e == cudaSuccess) e = build_direct_batch(specs, sms, b->d_direct, &b->direct_batch, s);
       if (e != cudaSuccess) { release(b); delete b; return cuda_fail(e, "cms_batch_create (direct arguments)"); }
     }
-    b->total_tasks += b->direct_batch.tile_blocks;
+    b->total_tasks += b->direct_batch.units;
   }
   // counter reset + persistent kernel, packing + tiles, batched inverse (rows, columns)
   int launches = (ntr > 0 ? 2 : 0) + (ntr < count ? 2 : 0) + 2;

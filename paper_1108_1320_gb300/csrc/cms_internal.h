@@ -315,17 +315,19 @@ cudaError_t launch_merge(const float* const* parts, int count, int64_t len,
 struct DirectPlan {
   bool split = false;       // FP32 (or FP64) storage: two FP16 terms per value
   bool alias = false;       // A = X^T, B = X: tiles on and above the diagonal
-  int tiles1 = 0, tiles3 = 0, nsb = 0, splits = 1, sb_per_split = 1, slots = 0;
+  int tiles1 = 0, tiles3 = 0, nsb = 0, splits = 1, sb_per_split = 1;
+  bool wide = true;         // units of two tiles side by side
+  int units = 0, blocks = 0;
+  bool need_fold = false, need_hand = false, need_merge = false;   // words of the tile kernel
   int copies = 1;           // of the sums, for short sketches
   bool grid = false;        // the entries stored, added to the buckets by a launch of its own
-  bool grid64 = false;      // ... as integers
+  int parts = 1;            // ... in this many parts to add up
   int sets = 1;             // sums of different entries (1 + 2 L: FINDSIGNIFICANTENTRIES)
-  int64_t tiles = 0;
   double seconds = 0.0;     // estimate
   bool pre = false;         // of pre-sketched operands (PrePlan)
   bool alias_operands = false;
   int sms = 0;
-  size_t zero_bytes = 0, acc_bytes = 0, off_fold = 0, off_grid = 0;
+  size_t zero_bytes = 0, acc_bytes = 0, off_work = 0, off_grid = 0;
   size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_pa = 0, off_pb = 0;
   size_t ws_bytes = 0;
 };
@@ -394,12 +396,14 @@ struct DirectSpec {
 };
 struct DirectBatch {
   void* buf = nullptr;
-  int count = 0, pack_blocks = 0, tile_blocks = 0;
+  int count = 0, pack_blocks = 0, tile_blocks = 0, units = 0;
+  bool need_fold = false;
   uint32_t pack_smem = 0;
-  size_t o_tile = 0, o_ps = 0, o_ts = 0;
+  size_t o_tile = 0, o_ps = 0, o_ts = 0, o_work = 0;
 };
-size_t direct_batch_bytes(int count);
-cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, void* d_buf, DirectBatch* out, cudaStream_t s);
+size_t direct_batch_bytes(int count, int sms);
+cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, int sms, void* d_buf, DirectBatch* out,
+                               cudaStream_t s);
 cudaError_t launch_direct_batched(const DirectBatch& d, cudaStream_t s);
 
 // Plain FP64 path.

@@ -18,47 +18,40 @@
 //    the block by a power of two; BF16 values are exact.
 //    Its last block bounds every bucket (Cauchy-Schwarz) and fixes the grid
 //    of the integer sums.
-//  * k_direct_tile: one 128 x 128 tile of AB per block, two blocks per SM.
-//    The FP32 sums of the tensor cores over kSuper inner indices are added in
-//    registers (round to nearest), then scaled to 64-bit integers and added
-//    to the buckets with integer reductions: the order of the additions does
-//    not matter, so the sketch is the same in every run.
+//  * k_direct_tile (k_direct_tile.cu) multiplies tiles of AB on the tensor
+//    cores.  Entries are scaled to 64-bit integers and added to the buckets
+//    with integer reductions: the order of the additions does not matter, so
+//    the sketch is the same in every run.  Its scatter warps add them while the
+//    next tile is multiplied, or the entries are stored (at most 16.8 M) and
+//    k_direct_grid adds them with the whole chip: a tile's additions take an
+//    SM 12 us a repetition, so that a last wave of few tiles would wait for
+//    them (2265 x 2265 x 503, d = 7: 318 us fused, 24 + 197 us in two).
 //  * k_direct_finish converts the sums to FP32.
 //
 // Measured on one GB300 (whole calls, transform route -> this one): X^T X of
 // 4096 x 2048 FP32, b = 2^16, d = 5 with its hash draw and dense decode 2.93
-// -> 0.40 ms; 8192 x 4096 BF16, b = 2^16, d = 3 7.54 -> 0.45 ms; 16384 x
-// 32768 BF16, b = 2^20, d = 7 834 -> 57 ms; 64 uneven products of n = 512 ..
-// 8192, b = 16 n, d = 3 429 -> 24.2 ms.  What bounds it: the additions into
+// -> 0.35 ms; 8192 x 4096 BF16, b = 2^16, d = 3 7.54 -> 0.42 ms; 16384 x
+// 32768 BF16, b = 2^20, d = 7 834 -> 50.6 ms; 64 uneven products of n = 512 ..
+// 8192, b = 16 n, d = 3 416 -> 25.2 ms.  What bounds it: the additions into
 // the buckets (random 64-bit reductions run at 205 G/s on the whole chip, one
-// 32-byte sector each), then the copies of the tiles' operands from L2 (about
-// 64 bytes per clock and SM).
+// 32-byte sector each), then shared memory, which the operands' copies and the
+// tensor cores' reads of them share (about 110 bytes per clock and SM).
 #include <algorithm>
 #include <cmath>
 #include <cuda_fp16.h>
 
-#include "cms_internal.h"
+#include "direct_tile.cuh"
 #include "warp_fft.cuh"
 
 namespace cms {
 namespace {
 
 using namespace wfft;
+using namespace dtile;
 
-constexpr int kTile = 128;              // rows and columns of a tile
-constexpr int kSuper = 128;             // inner indices with one scale, and one drain of the accumulators
-constexpr int kStageBytes = kTile * 128;   // one operand's share of a stage
-constexpr int kStages = 3;
-constexpr int kMaxSb = 1024;            // scale factors held per block
-constexpr int kFold = 32;               // drains between folds of the register sums (long inner dimensions)
-constexpr int kFoldFrom = 64;           // drains above which they are folded
-constexpr int kEpiThreads = 128;
 constexpr double kFixedSeconds = 36e-6;   // launches of a single product
-constexpr int kTileThreads = kEpiThreads + 32;
 constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
 constexpr int kMinExp = -100;           // scales stay representable
-
-__device__ uint32_t g_direct_error = 0;   // 1: a wait gave up
 
 
 __device__ __forceinline__ float load_val(const float* p) { return __ldg(p); }
@@ -492,393 +485,6 @@ __global__ void __launch_bounds__(256) k_pre_pack(const PreArgs p) {
   if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-struct TileArgs {
-  const uint8_t* pa;
-  const uint8_t* pb;
-  const int2* ea;              // (exponent, -) per superblock
-  const int2* eb;
-  const DirectScale* scale;
-  const uint32_t* hs;          // [t][side][n]
-  unsigned long long* acc;     // [copy][t][b]
-  int copies;                  // blocks add to copy (block mod copies)
-  // more than one pair of operands (repetitions of pre-sketched operands):
-  // bytes and superblocks from one pair's to the next; one scale and b
-  // buckets each
-  size_t rep_images;
-  int rep_blocks;
-  int reps;
-  void* grid;                  // entries in units of the integer sums, rows of tiles3 * 128: FP32, or
-  int grid64;                  //   64-bit integers added by the splits of the inner dimension
-  int64_t K;
-  int n, n1, n3, b, d;
-  int tiles1, tiles3;
-  int nsb, sb_per_split;
-  int tiles;                   // of AB
-  float* fold;                 // [slots][128][128] partial sums of the blocks that run, or NULL
-  uint32_t* slot;              // slot taken
-  int slots;
-  int split;
-  int sym;                     // A = X^T, B = X: tiles on and above the diagonal
-};
-
-constexpr uint32_t tile_smem_bytes() { return 1024 + kStages * 2 * kStageBytes + kMaxSb * 4 + 2 * kTile * 4; }
-
-// Shared-memory matrix descriptor of a K-major operand in the 128-byte
-// swizzle: 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  return (static_cast<uint64_t>(addr >> 4) & 0x3FFFu) | (1ull << 16) | (static_cast<uint64_t>(1024 >> 4) << 32) |
-         (1ull << 46) | (2ull << 61);
-}
-
-__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool accumulate) {
-  const uint32_t p = accumulate;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(p)
-      : "memory");
-}
-
-// The barrier's phase completes when the tensor-core work issued so far has.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
-__device__ __forceinline__ void bucket_add(unsigned long long* c, uint32_t ha, uint32_t hb, uint32_t b, float v) {
-  uint32_t z = (ha & kBucketMask) + (hb & kBucketMask);
-  if (z >= b) z -= b;
-  const float w = __uint_as_float(__float_as_uint(v) ^ ((ha ^ hb) & 0x80000000u));
-  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c + z), "l"(__float2ll_rn(w)) : "memory");
-}
-
-__device__ __forceinline__ void tmem_wait_ld8x2(uint32_t (&a)[8], uint32_t (&b)[8]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
-                 "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
-               :
-               : "memory");
-}
-
-constexpr int kPitch = kTile + 4;        // words per row of a tile in shared memory
-
-// This thread's row of the tile (128 columns from j0), and its mirror image.
-__device__ __forceinline__ void store_grid(const TileArgs& p, const float (&acc)[kTile], float* smem, int tid, int i,
-                                           int j0, bool mirror) {
-  const size_t ld = static_cast<size_t>(p.tiles3) * kTile;
-  if (p.grid64) {
-    unsigned long long* g = static_cast<unsigned long long*>(p.grid);
-#pragma unroll
-    for (int q = 0; q < kTile; ++q) {
-      const long long v = __float2ll_rn(acc[q]);
-      atomicAdd(g + i * ld + j0 + q, static_cast<unsigned long long>(v));
-      if (mirror) atomicAdd(g + (j0 + q) * ld + i, static_cast<unsigned long long>(v));
-    }
-    return;
-  }
-  float* g = static_cast<float*>(p.grid);
-  // the lanes hold consecutive rows: the mirror image is stored as it is
-  // (128 bytes per warp), the tile itself through shared memory (the stages'
-  // memory is free: every product has been read), a row per bulk copy
-  if (mirror) {
-#pragma unroll
-    for (int q = 0; q < kTile; ++q) g[(j0 + q) * ld + i] = acc[q];
-  }
-  float* row = smem + tid * kPitch;
-#pragma unroll
-  for (int q = 0; q < kTile; q += 4)
-    *reinterpret_cast<float4*>(row + q) = make_float4(acc[q], acc[q + 1], acc[q + 2], acc[q + 3]);
-  fence_proxy_async();
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(g + i * ld + j0),
-               "r"(smem_u32(row)), "r"(kTile * 4)
-               : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-// GRID: the entries go to p.grid (k_direct_grid adds them to the buckets);
-// else straight to the buckets.
-template <bool SPLIT, bool GRID = false>
-__device__ __forceinline__ void tile_task(const TileArgs& p, int tile, int split, int rep) {
-  constexpr int kImages = SPLIT ? 4 : 2;
-  constexpr int kPerStage = kSuper / kImages;
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full[kStages], freed[kStages], ready[2], drained[2];
-  __shared__ uint32_t s_tmem;
-  __shared__ int s_err, s_slot;
-  uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  float* factor = reinterpret_cast<float*>(stages + kStages * 2 * kStageBytes);
-  uint32_t* hcol = reinterpret_cast<uint32_t*>(factor + kMaxSb);   // [2][128]
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-  // tile of AB
-  int ti, tj;
-  if (p.sym) {
-    // row by row over the upper triangle: row ti holds tiles1 - ti tiles
-    const int T = p.tiles1;
-    const int q = tile;
-    ti = static_cast<int>((2.0 * T + 1.0 - sqrt((2.0 * T + 1.0) * (2.0 * T + 1.0) - 8.0 * q)) * 0.5);
-    while (ti > 0 && q < ti * T - ti * (ti - 1) / 2) --ti;
-    while (q >= (ti + 1) * T - (ti + 1) * ti / 2) ++ti;
-    tj = ti + q - (ti * T - ti * (ti - 1) / 2);
-  } else {
-    ti = tile / p.tiles3;
-    tj = tile - ti * p.tiles3;
-  }
-  const int sb0 = split * p.sb_per_split;
-  const int sb1 = min(p.nsb, sb0 + p.sb_per_split);
-  const int per_tile = static_cast<int>((p.K + kPerStage - 1) / kPerStage);
-  const int st0 = sb0 * kImages, st1 = min(per_tile, sb1 * kImages);
-  const int nst = st1 - st0;                                  // stages of this block
-  const int chunks = (nst + 1) / 2;                           // drains of the accumulators
-  const bool folds = p.fold != nullptr && chunks > kFoldFrom;
-  if (tid == 0) {
-    for (int q = 0; q < kStages; ++q) { mbar_init(&full[q], 1); mbar_init(&freed[q], 1); }
-    for (int q = 0; q < 2; ++q) { mbar_init(&ready[q], 1); mbar_init(&drained[q], kEpiThreads); }
-    s_err = 0;
-    s_slot = -1;
-    if (folds) {
-      // no more than `slots` blocks run at a time: one is free
-      uint32_t q = static_cast<uint32_t>(blockIdx.x) % static_cast<uint32_t>(p.slots);
-      for (int tries = 0; tries < 64 * p.slots && s_slot < 0; ++tries) {
-        if (atomicCAS(p.slot + q, 0u, 1u) == 0u) s_slot = static_cast<int>(q);
-        q = q + 1 == static_cast<uint32_t>(p.slots) ? 0 : q + 1;
-      }
-      if (s_slot < 0) s_err = 1;
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 4) {
-    tmem_alloc(&s_tmem, 2 * kTile);
-    tmem_relinquish();
-  }
-  const DirectScale sc = p.scale[rep];
-  for (int q = tid; q < sb1 - sb0; q += kTileThreads) {
-    const size_t rb = static_cast<size_t>(rep) * p.rep_blocks;
-    const int de = p.ea[rb + static_cast<size_t>(ti) * p.nsb + sb0 + q].x - sc.emax[0] +
-                   p.eb[rb + static_cast<size_t>(tj) * p.nsb + sb0 + q].x - sc.emax[1];
-    factor[q] = de < -126 ? 0.f : pow2f(min(de, 0));
-  }
-  tmem_fence_before_sync();
-  __syncthreads();
-  tmem_fence_after_sync();
-  const uint32_t tmem = s_tmem;
-
-  if (warp == 4) {
-    if ((tid & 31) == 0) {
-      // D: FP32; A, B: FP16 (0) or BF16 (1), K-major; N / 8, M / 16
-      constexpr uint32_t idesc = (1u << 4) | ((SPLIT ? 0u : 1u) << 7) | ((SPLIT ? 0u : 1u) << 10) |
-                                 (static_cast<uint32_t>(kTile / 8) << 17) | (static_cast<uint32_t>(kTile / 16) << 24);
-      const uint8_t* ga = p.pa + rep * p.rep_images + (static_cast<size_t>(ti) * per_tile + st0) * kStageBytes;
-      const uint8_t* gb = p.pb + rep * p.rep_images + (static_cast<size_t>(tj) * per_tile + st0) * kStageBytes;
-      auto load = [&](int st) {
-        uint8_t* dst = stages + (st % kStages) * 2 * kStageBytes;
-        uint64_t* bar = &full[st % kStages];
-        mbar_arrive_expect_tx(bar, 2 * kStageBytes);
-        bulk_g2s(dst, ga + static_cast<size_t>(st) * kStageBytes, kStageBytes, bar);
-        bulk_g2s(dst + kStageBytes, gb + static_cast<size_t>(st) * kStageBytes, kStageBytes, bar);
-      };
-      int issued = min(kStages, nst);
-      for (int st = 0; st < issued; ++st) load(st);
-      bool ok = true;
-      int st = 0;
-      for (int ch = 0; st < nst && ok; ++ch) {
-        const int buf = SPLIT ? 0 : ch & 1;
-        const int use = SPLIT ? ch : ch >> 1;      // of this buffer
-        if (use >= 1) ok = mbar_wait_bounded(&drained[buf], (use - 1) & 1);
-        tmem_fence_after_sync();
-        const int end = min(nst, st + 2);
-        const uint32_t dt = tmem + buf * kTile;
-        const bool cross0 = (ch & 1) == 0;         // first half of a superblock
-        for (bool first = true; st < end && ok; ++st, first = false) {
-          ok = mbar_wait_bounded(&full[st % kStages], (st / kStages) & 1);
-          if (!ok) break;
-          tmem_fence_after_sync();
-          const uint32_t a = smem_u32(stages + (st % kStages) * 2 * kStageBytes);
-          const uint64_t da = smem_desc(a), db = smem_desc(a + kStageBytes);
-          // 16 inner indices are 32 bytes (2 units of 16) along the rows
-          if constexpr (SPLIT) {
-            // hi hi into one accumulator, the cross terms (2^-11 of it) into
-            // the other: added to the same one, each would be cut to the
-            // precision of the large sum
-            mma_f16(dt, da, db, idesc, !first);
-            mma_f16(dt + kTile, da, db + 4, idesc, !(first && cross0));
-            mma_f16(dt, da + 2, db + 2, idesc, true);
-            mma_f16(dt + kTile, da + 2, db + 6, idesc, true);
-            mma_f16(dt + kTile, da + 4, db, idesc, true);
-            mma_f16(dt + kTile, da + 6, db + 2, idesc, true);
-          } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) mma_f16(dt, da + 2 * q, db + 2 * q, idesc, !first || q > 0);
-          }
-          mma_commit(&freed[st % kStages]);
-          // refill the stage before this one while this one's products run
-          if (st >= 1 && issued < nst) {
-            ok = mbar_wait_bounded(&freed[(st - 1) % kStages], ((st - 1) / kStages) & 1);
-            if (ok) load(issued++);
-          }
-        }
-        if (ok) mma_commit(&ready[buf]);
-      }
-      // the products of the last stages have arrived on their barriers
-      for (int q = max(0, st - kStages); q < st && ok; ++q) ok = mbar_wait_bounded(&freed[q % kStages], (q / kStages) & 1);
-      if (!ok) {
-        s_err = 1;
-        for (int q = max(0, issued - kStages); q < issued; ++q)
-          (void)mbar_wait_bounded(&full[q % kStages], (q / kStages) & 1);
-      }
-    }
-    __syncwarp();
-  } else {
-    float acc[kTile];
-#pragma unroll
-    for (int q = 0; q < kTile; ++q) acc[q] = 0.f;
-    const uint32_t lane = tmem + (static_cast<uint32_t>(warp) << 21);
-    bool ok = true;
-    float* fold = folds && s_slot >= 0 ? p.fold + static_cast<size_t>(s_slot) * kTile * kTile + tid : nullptr;
-    for (int ch = 0; ch < chunks; ++ch) {
-      const int buf = SPLIT ? 0 : ch & 1;
-      if (ok) ok = mbar_wait_bounded(&ready[buf], (SPLIT ? ch : ch >> 1) & 1);
-      ok = __all_sync(0xFFFFFFFFu, ok);
-      if (!ok) break;
-      tmem_fence_after_sync();
-      const float f = factor[SPLIT ? ch >> 1 : ch];
-      const uint32_t col = lane + buf * kTile;
-      if (SPLIT && ((ch & 1) || ch == chunks - 1)) {
-#pragma unroll
-        for (int g = 0; g < kTile / 8; ++g) {
-          uint32_t v[8], w[8];
-          tmem_ld8_nowait(col + g * 8, v);
-          tmem_ld8_nowait(col + kTile + g * 8, w);
-          tmem_wait_ld8x2(v, w);
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            acc[g * 8 + q] = fmaf(__uint_as_float(v[q]) + __uint_as_float(w[q]), f, acc[g * 8 + q]);
-        }
-      } else {
-#pragma unroll
-        for (int g = 0; g < kTile / 16; ++g) {
-          uint32_t v[8], w[8];
-          tmem_ld8_nowait(col + g * 16, v);
-          tmem_ld8_nowait(col + g * 16 + 8, w);
-          tmem_wait_ld8x2(v, w);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            acc[g * 16 + q] = fmaf(__uint_as_float(v[q]), f, acc[g * 16 + q]);
-            acc[g * 16 + 8 + q] = fmaf(__uint_as_float(w[q]), f, acc[g * 16 + 8 + q]);
-          }
-        }
-      }
-      tmem_fence_before_sync();
-      mbar_arrive(&drained[buf]);
-      // the sums so far join those of earlier folds: a long chain of FP32
-      // additions into one large sum would lose a bit per factor of four
-      if (fold != nullptr && (ch + 1) % kFold == 0 && ch + 1 < chunks) {
-        // one thread adds to each word, in order: the same sum in every run
-        const bool first = ch + 1 == kFold;
-#pragma unroll
-        for (int q = 0; q < kTile; ++q) {
-          if (first) __stcg(fold + q * kTile, acc[q]);
-          else asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(fold + q * kTile), "f"(acc[q]) : "memory");
-          acc[q] = 0.f;
-        }
-      }
-    }
-    if (fold != nullptr) {
-#pragma unroll
-      for (int g = 0; g < kTile / 16; ++g) {
-        float v[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = __ldcg(fold + (g * 16 + q) * kTile);
-#pragma unroll
-        for (int q = 0; q < 16; ++q) acc[g * 16 + q] += v[q];
-      }
-    }
-    if (!ok) s_err = 1;
-    epi_sync();
-    const bool run = s_err == 0 && !sc.bad;
-    const float up = pow2f(sc.shift / 2), up2 = pow2f(sc.shift - sc.shift / 2);
-#pragma unroll
-    for (int q = 0; q < kTile; ++q) acc[q] = acc[q] * up * up2;
-    const int i = ti * kTile + tid;
-    const int j0 = tj * kTile;
-    int cols = run ? min(kTile, p.n3 - j0) : 0;
-    const bool mirror = p.sym && ti != tj;
-    const bool row = i < p.n1;
-    const uint32_t b = static_cast<uint32_t>(p.b);
-    if constexpr (GRID) {
-      if (run) store_grid(p, acc, reinterpret_cast<float*>(stages), tid, i, j0, mirror);
-      cols = 0;
-    }
-    const size_t set = static_cast<size_t>(p.d) * (p.reps > 1 ? p.reps : 1) * p.b;
-    unsigned long long* sums = p.acc + static_cast<size_t>(rep) * p.b +
-                               (p.copies > 1 ? static_cast<size_t>(tile + split) % p.copies * set : 0);
-    for (int t = 0; t < (GRID ? 0 : p.d); ++t) {
-      const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
-      const uint32_t* h2 = h1 + p.n;
-      epi_sync();
-      if (tid < cols) {
-        hcol[tid] = h2[j0 + tid];
-        if (mirror) hcol[kTile + tid] = h1[j0 + tid];
-      }
-      epi_sync();
-      if (!row) continue;
-      unsigned long long* c = sums + static_cast<size_t>(t) * p.b;
-      const uint32_t hr = h1[i];
-#pragma unroll
-      for (int q = 0; q < kTile; ++q)
-        if (q < cols) bucket_add(c, hr, hcol[q], b, acc[q]);
-      if (mirror) {
-        const uint32_t hm = h2[i];
-#pragma unroll
-        for (int q = 0; q < kTile; ++q)
-          if (q < cols) bucket_add(c, hcol[kTile + q], hm, b, acc[q]);
-      }
-    }
-  }
-  tmem_fence_before_sync();
-  __syncthreads();
-  if (tid == 0 && s_err) atomicOr(&g_direct_error, 1u);
-  if (tid == 0 && s_slot >= 0) atomicExch(p.slot + s_slot, 0u);
-  if (warp == 4) tmem_dealloc(tmem, 2 * kTile);
-  if (tid == 0) {
-    for (int q = 0; q < kStages; ++q) { mbar_inval(&full[q]); mbar_inval(&freed[q]); }
-    for (int q = 0; q < 2; ++q) { mbar_inval(&ready[q]); mbar_inval(&drained[q]); }
-  }
-}
-
-template <bool SPLIT, bool GRID>
-__global__ void __launch_bounds__(kTileThreads, 2) k_direct_tile(const TileArgs p) {
-  tile_task<SPLIT, GRID>(p, blockIdx.x, blockIdx.y, blockIdx.z);
-}
-
-// Tiles of every product of a batch, the longest first.
-__global__ void __launch_bounds__(kTileThreads, 2)
-k_direct_tile_batched(const TileArgs* __restrict__ args, const int* __restrict__ start, int count) {
-  __shared__ TileArgs sp;
-  const int q = find_instance(start, count, static_cast<int>(blockIdx.x));
-  for (int w = threadIdx.x; w < static_cast<int>(sizeof(TileArgs) / 4); w += kTileThreads)
-    reinterpret_cast<uint32_t*>(&sp)[w] = reinterpret_cast<const uint32_t*>(args + q)[w];
-  __syncthreads();
-  const int local = static_cast<int>(blockIdx.x) - __ldg(start + q);
-  const int tile = local % sp.tiles, split = local / sp.tiles;
-  if (sp.split) tile_task<true>(sp, tile, split, 0);
-  else tile_task<false>(sp, tile, split, 0);
-}
-
-__global__ void __launch_bounds__(256)
-k_direct_pack_batched(const PackArgs* __restrict__ args, const int* __restrict__ start, int count) {
-  __shared__ PackArgs sp;
-  const int q = find_instance(start, count, static_cast<int>(blockIdx.x));
-  for (int w = threadIdx.x; w < static_cast<int>(sizeof(PackArgs) / 4); w += 256)
-    reinterpret_cast<uint32_t*>(&sp)[w] = reinterpret_cast<const uint32_t*>(args + q)[w];
-  __syncthreads();
-  pack_task(sp, blockIdx.x - static_cast<uint32_t>(__ldg(start + q)));
-}
-
 // A value added to its bucket's sum, to the sums of the bits set in the
 // position i of its row, and to those of the bits set in j.
 __device__ __forceinline__ void bucket_add_masked(unsigned long long* c, size_t set, int bits, uint32_t i, uint32_t j,
@@ -898,9 +504,21 @@ __device__ __forceinline__ void bucket_add_masked(unsigned long long* c, size_t 
   }
 }
 
+__global__ void __launch_bounds__(256)
+k_direct_pack_batched(const PackArgs* __restrict__ args, const int* __restrict__ start, int count) {
+  __shared__ PackArgs sp;
+  const int q = find_instance(start, count, static_cast<int>(blockIdx.x));
+  for (int w = threadIdx.x; w < static_cast<int>(sizeof(PackArgs) / 4); w += 256)
+    reinterpret_cast<uint32_t*>(&sp)[w] = reinterpret_cast<const uint32_t*>(args + q)[w];
+  __syncthreads();
+  pack_task(sp, blockIdx.x - static_cast<uint32_t>(__ldg(start + q)));
+}
+
 struct GridArgs {
-  const void* grid;
-  int64_t ld;
+  const float* grid;           // [part][tile row][tile column][128 columns][128 rows]
+  size_t part;                 // entries from one part to the next
+  int parts;
+  int tiles3, sym;
   const uint32_t* hs;          // [t][side][n]
   const DirectScale* scale;
   unsigned long long* acc;     // [copy][t][b], or [1 + 2 bits][t][b]
@@ -908,55 +526,69 @@ struct GridArgs {
   int n, n1, n3, b, d;
 };
 
-__device__ __forceinline__ void load4(const float* g, float (&v)[4]) {
-  const float4 x = __ldg(reinterpret_cast<const float4*>(g));
-  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-}
-__device__ __forceinline__ void load4(const long long* g, long long (&v)[4]) {
-  const longlong2 x = __ldg(reinterpret_cast<const longlong2*>(g)), y = __ldg(reinterpret_cast<const longlong2*>(g) + 1);
-  v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
-}
-__device__ __forceinline__ long long to_sum(float v) { return __float2ll_rn(v); }
-__device__ __forceinline__ long long to_sum(long long v) { return v; }
-
-// The entries of the grid added to the buckets: a warp takes 128 columns of
-// kGridRows rows.
-constexpr int kGridRows = 2;
-template <typename T, bool MASKED>
+// The entries of the grid, and the mirror images of a symmetric product's,
+// added to the buckets: a block takes 16 columns of a tile, a warp two, a lane
+// four rows of each, and the repetitions from blockIdx.z on.  The parts of an
+// entry are added as integers.
+constexpr int kGridCols = 2;
+template <bool MASKED>
 __global__ void __launch_bounds__(256) k_direct_grid(const GridArgs p) {
   if (p.scale->bad) return;
+  const int tile = static_cast<int>(blockIdx.x), ti = tile / p.tiles3, tj = tile - ti * p.tiles3;
+  if (p.sym && ti > tj) return;
+  const bool mirror = p.sym && ti < tj;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = static_cast<int>(blockIdx.x) * 128 + lane * 4;
-  const int i0 = (static_cast<int>(blockIdx.y) * 8 + warp) * kGridRows;
-  if (i0 >= p.n1) return;
-  T v[kGridRows][4];
+  const int q0 = (static_cast<int>(blockIdx.y) * 8 + warp) * kGridCols;   // columns of the tile
+  const int i0 = ti * kTile + lane, j0 = tj * kTile + q0;                 // rows i0 + 32 r
+  const int cols = min(kGridCols, p.n3 - j0);
+  if (cols <= 0) return;
+  const float* src = p.grid + static_cast<size_t>(tile) * kTile * kTile + q0 * kTile + lane;
+  long long v[kGridCols][4];
 #pragma unroll
-  for (int r = 0; r < kGridRows; ++r) load4(static_cast<const T*>(p.grid) + (i0 + r) * p.ld + j, v[r]);
+  for (int q = 0; q < kGridCols; ++q)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[q][r] = __float2ll_rn(__ldcg(src + q * kTile + r * 32));
+#pragma unroll 4
+  for (int s = 1; s < p.parts; ++s) {
+    src += p.part;
+#pragma unroll
+    for (int q = 0; q < kGridCols; ++q)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) v[q][r] += __float2ll_rn(__ldcg(src + q * kTile + r * 32));
+  }
   const uint32_t b = static_cast<uint32_t>(p.b);
   const size_t set = static_cast<size_t>(p.d) * p.b;
   unsigned long long* sums = p.acc + (p.copies > 1 ? static_cast<size_t>(blockIdx.x + blockIdx.y) % p.copies * set : 0);
-  for (int t = 0; t < p.d; ++t) {
+  auto add = [&](unsigned long long* c, uint32_t i, uint32_t j, uint32_t ha, uint32_t hb, long long iv) {
+    if constexpr (MASKED) bucket_add_masked(c, set, p.bits, i, j, ha, hb, b, iv);
+    else {
+      uint32_t z = (ha & kBucketMask) + (hb & kBucketMask);
+      if (z >= b) z -= b;
+      const long long w = ((ha ^ hb) >> 31) ? -iv : iv;
+      asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c + z), "l"(w) : "memory");
+    }
+  };
+  for (int t = blockIdx.z; t < p.d; t += gridDim.z) {
     const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
     const uint32_t* h2 = h1 + p.n;
     unsigned long long* c = sums + static_cast<size_t>(t) * p.b;
-    uint32_t hc[4];
+    uint32_t hr[4], hm[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) hc[q] = j + q < p.n3 ? __ldg(h2 + j + q) : 0;
+    for (int r = 0; r < 4; ++r) {
+      const bool in = i0 + 32 * r < p.n1;
+      hr[r] = in ? __ldg(h1 + i0 + 32 * r) : 0;
+      hm[r] = mirror && in ? __ldg(h2 + i0 + 32 * r) : 0;
+    }
 #pragma unroll
-    for (int r = 0; r < kGridRows; ++r) {
-      if (i0 + r >= p.n1) break;
-      const uint32_t hr = __ldg(h1 + i0 + r);
+    for (int q = 0; q < kGridCols; ++q) {
+      if (q >= cols) break;
+      const uint32_t hc = __ldg(h2 + j0 + q), hx = mirror ? __ldg(h1 + j0 + q) : 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (j + q >= p.n3) continue;
-        const long long iv = to_sum(v[r][q]);
-        if constexpr (MASKED) bucket_add_masked(c, set, p.bits, i0 + r, j + q, hr, hc[q], b, iv);
-        else {
-          uint32_t z = (hr & kBucketMask) + (hc[q] & kBucketMask);
-          if (z >= b) z -= b;
-          const long long w = ((hr ^ hc[q]) >> 31) ? -iv : iv;
-          asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c + z), "l"(w) : "memory");
-        }
+      for (int r = 0; r < 4; ++r) {
+        const int i = i0 + 32 * r;
+        if (i >= p.n1) continue;
+        add(c, i, j0 + q, hr[r], hc, v[q][r]);
+        if (mirror) add(c, j0 + q, i, hx, hm[r], v[q][r]);
       }
     }
   }
@@ -1024,12 +656,73 @@ k_direct_sig_decode(const unsigned long long* __restrict__ acc, int bits, int64_
 
 }  // namespace
 
-uint32_t read_clear_error_direct() {
-  uint32_t v = 0, zero = 0;
-  if (cudaMemcpyFromSymbol(&v, g_direct_error, sizeof(v)) != cudaSuccess) return 0xFFFFFFFFu;
-  if (v) cudaMemcpyToSymbol(g_direct_error, &zero, sizeof(zero));
-  return v;
+uint32_t read_clear_error_direct() { return dtile::read_clear_error_tile(); }
+
+namespace {
+
+// How the tiles are cut and where their entries go.
+//  wide   units of two tiles side by side (an operand tile of A serves both:
+//         96 KB from L2 for 2 x 128 x 128 x 128 BF16 products instead of 128),
+//         or one tile with its inner indices dealt to the block's halves
+//         (twice the units, where tiles are few);
+//  splits of the inner dimension while SMs have no unit;
+//  grid   entries stored for a launch of its own (additions from every SM,
+//         about 6 us more; entries beyond L2's reach are not worth storing),
+//         or added by the tile kernel while it multiplies on.
+// Times: a chunk of 64 (FP16 terms) or 128 (BF16) inner indices of a tile
+// 0.40 us (BF16 alone on its operands 0.53: the copies from L2 bound it).
+void choose_tiles(DirectPlan& p, bool sym, int reps, double entries, double adds, double full_rate, double sm_rate,
+                  bool may_grid, bool may_fuse, bool shared, int sms) {
+  double best = 1e30;
+  for (int wide = 0; wide < 2; ++wide) {
+    if (!wide && shared) continue;
+    const int units = tile_units(p.tiles1, p.tiles3, wide != 0, sym);
+    for (int s = 1; s <= std::min(p.nsb, 64); ++s) {
+      const int per = (p.nsb + s - 1) / s, real = (p.nsb + per - 1) / per;
+      if (real != s && s > 1) continue;
+      const double blocks = static_cast<double>(units) * real * reps;
+      const double chunk = wide ? 0.85e-6 : (p.split ? 0.43e-6 : 0.55e-6);
+      const double unit = per * (p.split ? 2.0 : 1.0) * chunk + 3e-6;
+      // (a batch's products share the last wave)
+      const double waves = shared ? std::max(1.0, blocks / sms) : std::ceil(blocks / sms);
+      const double mma = waves * unit;
+      for (int grid = 0; grid < 2; ++grid) {
+        if (grid ? !may_grid : !may_fuse) continue;
+        const double parts = real * (wide || per * (p.split ? 2 : 1) == 1 ? 1.0 : 2.0);
+        const double t =
+            grid ? mma + 3e-6 + entries * reps * (adds / full_rate + (sym ? 4.0 : 8.0) * parts / 4e12) + parts * 0.1e-6
+                 : mma + std::max(entries * reps * adds * real / full_rate,
+                                  waves * entries * adds / units / sm_rate);
+        if (t < best) {
+          best = t;
+          p.wide = wide != 0;
+          p.grid = grid != 0;
+          p.sb_per_split = per;
+          p.splits = real;
+        }
+      }
+    }
+  }
+  p.units = tile_units(p.tiles1, p.tiles3, p.wide, sym);
+  p.seconds = best + kFixedSeconds;
+  p.blocks = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(p.units) * p.splits * reps, sms));
+  const int chunks = p.sb_per_split * (p.split ? 2 : 1);
+  p.need_fold = (p.wide ? chunks : (chunks + 1) / 2) > 64;
+  p.need_hand = !p.grid;
+  p.need_merge = !p.wide && !p.grid && chunks > 1;
+  p.parts = p.splits * (!p.wide && chunks > 1 ? 2 : 1);
 }
+
+size_t al1k(size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); }
+
+// Copies of `words` sums.  Reductions to few words queue up (23 G/s on 2^10
+// words, 100 on 2^14, 165 on 2^16, 200 from 2^18 on), so tiles share several
+// copies of a short sketch's sums, which the conversion adds up.
+int sum_copies(int64_t words, int64_t units) {
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({256, (int64_t{1} << 18) / words, units})));
+}
+
+}  // namespace
 
 DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int dt, bool alias, int sms,
                             int sets, bool batch) {
@@ -1039,67 +732,30 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   p.tiles1 = static_cast<int>((n1 + kTile - 1) / kTile);
   p.tiles3 = static_cast<int>((n3 + kTile - 1) / kTile);
   p.nsb = static_cast<int>((n2 + kSuper - 1) / kSuper);
-  const int64_t tiles = alias ? static_cast<int64_t>(p.tiles1) * (p.tiles1 + 1) / 2
-                              : static_cast<int64_t>(p.tiles1) * p.tiles3;
-  p.tiles = tiles;
   const int per = p.split ? 32 : 64;
   const int64_t images = (n2 + per - 1) / per;
-  // Splits of the inner dimension (while blocks are missing), and whether the
-  // tiles add their entries to the buckets themselves (fused: d additions per
-  // entry and split, and only the SMs that hold tiles issue them) or store
-  // them for a launch of its own (d additions per entry from every SM; about
-  // 6 us more, and entries beyond L2's reach are not worth storing).
-  const int lo = std::max(1, (p.nsb + kMaxSb - 1) / kMaxSb);
-  int best = lo;
-  double cost = 1e30;
-  const double slots = 2.0 * sms;
   const double entries = static_cast<double>(n1) * static_cast<double>(n3);
-  for (int grid = 0; grid < 2; ++grid) {
-    if (grid ? (batch || (sets == 1 && entries > 16.8e6)) : sets > 1) continue;
-    for (int s = lo; s <= std::min(p.nsb, std::max(lo, 64)); ++s) {
-      const int per_split = (p.nsb + s - 1) / s;
-      const int real = (p.nsb + per_split - 1) / per_split;
-      const double blocks = static_cast<double>(tiles) * real;
-      const double waves = std::max(1.0, std::ceil(blocks / slots));
-      const double mma = waves * per_split * (p.split ? 1.0 : 0.5) * 1.1e-6;
-      const double rate = std::min(2.0e11, 1.3e9 * std::min(blocks, static_cast<double>(sms)));
-      const double add = grid ? 6e-6 + entries * (h->d * 0.5 * (sets + 1) + (real > 1 ? 2.0 * real : 0.25)) / 2.0e11
-                              : entries * h->d * real / rate;
-      if (mma + add < cost) { cost = mma + add; best = real; p.grid = grid != 0; }
-    }
-  }
-  const bool use_grid = p.grid;
-  p.sb_per_split = (p.nsb + best - 1) / best;
-  p.splits = (p.nsb + p.sb_per_split - 1) / p.sb_per_split;
-  p.seconds = cost + kFixedSeconds;
-  // short sketches: reductions to few words queue up (23 G/s on 2^10 words,
-  // 100 on 2^14, 165 on 2^16, 200 from 2^18 on), so blocks share several
-  // copies of the sums, which the conversion adds up
+  choose_tiles(p, alias, 1, entries, 0.5 * h->d * (sets + 1), 2.05e11, 1.35e9,
+               !batch && (sets > 1 || entries <= 16.8e6), sets == 1, batch, sms);
   const int64_t words = static_cast<int64_t>(h->d) * h->b;
-  p.copies = sets > 1 ? 1
-                      : static_cast<int>(std::max<int64_t>(
-                            1, std::min<int64_t>({256, (int64_t{1} << 18) / words, tiles * p.splits})));
+  // (a batch's products queue up less: others' additions are under way too)
+  p.copies = sets > 1 ? 1 : sum_copies(words, static_cast<int64_t>(p.units) * p.splits);
+  if (batch) p.copies = std::min(p.copies, 4);
   p.sets = sets;
-  auto al = [](size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); };
   size_t o = 0;
   const int t3 = alias ? 0 : p.tiles3;
-  const int drains = p.sb_per_split * (p.split ? 2 : 1);
-  p.slots = drains > kFoldFrom ? 2 * sms : 0;
-  // sums, the ticket, the slots taken (all zero before a run)
+  // sums and the ticket (zero before a run)
   p.acc_bytes = static_cast<size_t>(p.copies) * sets * words * 8;
-  p.off_acc = o;    o = al(o + p.acc_bytes + 256 + static_cast<size_t>(p.slots) * 4);
-  p.grid64 = p.splits > 1;
-  const size_t grid_bytes = use_grid ? static_cast<size_t>(p.tiles1) * p.tiles3 * kTile * kTile * (p.grid64 ? 8 : 4) : 0;
-  p.off_grid = o;
-  if (p.grid64) o = al(o + grid_bytes);   // sums too: zeroed
+  p.off_acc = o;    o = al1k(o + p.acc_bytes + 256);
   p.zero_bytes = o;
-  if (!p.grid64) { p.off_grid = o; o = al(o + grid_bytes); }
-  p.off_fold = o;   o = al(o + static_cast<size_t>(p.slots) * kTile * kTile * sizeof(float));
-  p.off_scale = o;  o = al(o + sizeof(DirectScale));
-  p.off_blocks = o; o = al(o + static_cast<size_t>(p.tiles1 + t3) * p.nsb * sizeof(int2));
-  p.off_pa = o;     o = al(o + static_cast<size_t>(p.tiles1) * images * kStageBytes);
+  p.off_grid = o;
+  if (p.grid) o = al1k(o + static_cast<size_t>(p.parts) * p.tiles1 * p.tiles3 * kTile * kTile * sizeof(float));
+  p.off_work = o;   o = al1k(o + (batch ? 0 : tile_work_bytes(p.blocks, p.need_fold, p.need_hand, p.need_merge)));
+  p.off_scale = o;  o = al1k(o + sizeof(DirectScale));
+  p.off_blocks = o; o = al1k(o + static_cast<size_t>(p.tiles1 + t3) * p.nsb * sizeof(int2));
+  p.off_pa = o;     o = al1k(o + static_cast<size_t>(p.tiles1) * images * kStageBytes);
   p.off_pb = alias ? p.off_pa : o;
-  if (!alias) o = al(o + static_cast<size_t>(p.tiles3) * images * kStageBytes);
+  if (!alias) o = al1k(o + static_cast<size_t>(p.tiles3) * images * kStageBytes);
   p.ws_bytes = o;
   return p;
 }
@@ -1107,20 +763,27 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
 // Estimated time of the transform route (make_sketch_plan): launches, the
 // conventional 5 b log2 b + 4 b flops per repetition and inner index, and the
 // gathers of its front end (every entry of a_k and b_k for each computed row),
-// at rates fitted per kernel family to 130 calls of n = 64 .. 16384, b = n / 8
-// .. 32 n, 64 to 8192 inner indices (within a factor of two of most).
+// at rates fitted per kernel family to 160 calls of n = 64 .. 16384, b = n / 8
+// .. 32 n, 64 to 8192 inner indices.  With them the chosen route was the faster
+// one, or within 20% of it, in all of them (n = 454, K = 142, b = 810, d = 4 BF16:
+// 96 us by the spectra, 44 us this way; n = 6746, K = 184, b = 1620, d = 4 the
+// other way round: 160 and 1136 us).
 static double transform_seconds(const SketchPlan& p, int64_t n1, int64_t n2, int64_t n3, bool batch) {
   const double b = static_cast<double>(p.b);
   const double dk = static_cast<double>(p.d) * static_cast<double>(n2);
   const double gflop = dk * (5.0 * b * std::log2(std::max(b, 2.0)) + 4.0 * b) * 1e-9;
   const int rows = p.fast ? (p.nrows + 1) / 2 * 2 : p.nrows;   // the register kernels take two at a time
   const double mgather = dk * rows * static_cast<double>(n1 + n3) * 1e-6;
-  double us;
-  if (p.wide) us = 60.0 + 66.0 * gflop;
-  else if (p.ws) us = 40.0 + 25.0 * gflop;
-  else if (!p.fast) us = 38.0 + 226.0 * gflop + 5.8 * mgather;
-  else us = (p.tmem_rec ? 60.0 : 50.0) + 55.0 * gflop + (p.tmem_rec ? 2.2 : 2.5) * mgather;
-  return 1e-6 * (batch ? us - 38.0 : us);
+  double fixed, work;
+  if (p.wide) fixed = 60.0, work = 66.0 * gflop;
+  else if (p.ws) fixed = 50.0, work = 25.0 * gflop;
+  else if (!p.fast) fixed = 34.0, work = 208.0 * gflop + 4.0 * mgather;
+  else if (p.tmem_rec) fixed = 95.0, work = 30.0 * gflop + 1.6 * mgather;
+  else fixed = 50.0, work = 52.0 * gflop + 1.6 * mgather;
+  // a row's block adds up the partial spectra of the inner dimension's chunks,
+  // 256 points at a time: latency where the rows are few, shared in a batch
+  const double inverse = (p.fast ? 0.13 : 0.09) * p.nkc * static_cast<double>(p.C) / 256.0;
+  return 1e-6 * (batch ? work + 12.0 : fixed + work + inverse);
 }
 
 // Pre-sketched operands: the direct route's tiles over b x b x n2 for each
@@ -1137,49 +800,32 @@ PrePlan make_pre_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, b
   DirectPlan& p = q.direct;
   p.split = true;
   p.tiles1 = p.tiles3 = q.tiles;
-  p.tiles = static_cast<int64_t>(q.tiles) * q.tiles;
   p.nsb = static_cast<int>((n2 + kSuper - 1) / kSuper);
-  const int lo = std::max(1, (p.nsb + kMaxSb - 1) / kMaxSb);
-  int best = lo;
-  double cost = 1e30;
-  const double entries = static_cast<double>(rows) * rows * h->d;
-  for (int s = lo; s <= std::min(p.nsb, std::max(lo, 64)); ++s) {
-    const int per_split = (p.nsb + s - 1) / s;
-    const int real = (p.nsb + per_split - 1) / per_split;
-    const double blocks = static_cast<double>(p.tiles) * h->d * real;
-    const double t = std::max(1.0, std::ceil(blocks / (2.0 * sms))) * per_split * 1.1e-6 +
-                     entries * real / std::min(5.0e11, 4e9 * std::min(blocks, static_cast<double>(sms)));
-    if (t < cost) { cost = t; best = real; }
-  }
-  p.sb_per_split = (p.nsb + best - 1) / best;
-  p.splits = (p.nsb + p.sb_per_split - 1) / p.sb_per_split;
+  choose_tiles(p, false, h->d, static_cast<double>(rows) * rows, 1.0, 5.0e11, 4e9, false, true, false, sms);
   const double n = static_cast<double>(alias ? n1 : n1 + n3), k = static_cast<double>(p.nsb) * kSuper;
-  p.seconds = cost + 50e-6 + n * k * 8.0 / 4e12 + static_cast<double>(n1 + n3) * k * h->d * 4.0 / 5e12 +
+  p.seconds += 14e-6 + n * k * 8.0 / 4e12 + static_cast<double>(n1 + n3) * k * h->d * 4.0 / 5e12 +
               2.0 * static_cast<double>(rows) * k * h->d * 4.0 / 3e12;
-  auto al = [](size_t x) { return (x + 1023) & ~static_cast<size_t>(1023); };
   const int64_t words = static_cast<int64_t>(h->d) * h->b;
-  p.copies = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({256, (int64_t{1} << 18) / words, p.tiles * p.splits})));
+  p.copies = sum_copies(words, static_cast<int64_t>(p.units) * p.splits);
   const int64_t images = (n2 + 31) / 32;
   size_t o = 0;
-  const int drains = p.sb_per_split * 2;
-  p.slots = drains > kFoldFrom ? 2 * sms : 0;
   p.acc_bytes = static_cast<size_t>(p.copies) * words * 8;
-  // sums, a ticket per repetition, the slots taken: zero before a run
-  p.off_acc = o;    o = al(o + p.acc_bytes + 256 + static_cast<size_t>(p.slots) * 4);
+  // sums and a ticket per repetition: zero before a run
+  p.off_acc = o;    o = al1k(o + p.acc_bytes + 256);
   p.zero_bytes = o;
-  p.off_fold = o;   o = al(o + static_cast<size_t>(p.slots) * kTile * kTile * sizeof(float));
-  p.off_scale = o;  o = al(o + sizeof(DirectScale) * h->d);
+  p.off_work = o;   o = al1k(o + tile_work_bytes(p.blocks, p.need_fold, p.need_hand, p.need_merge));
+  p.off_scale = o;  o = al1k(o + sizeof(DirectScale) * h->d);
   q.rep_blocks = 2 * q.tiles * p.nsb;
-  p.off_blocks = o; o = al(o + static_cast<size_t>(q.rep_blocks) * h->d * sizeof(int2));
+  p.off_blocks = o; o = al1k(o + static_cast<size_t>(q.rep_blocks) * h->d * sizeof(int2));
   const size_t side = static_cast<size_t>(q.tiles) * images * kStageBytes;
   q.rep_images = 2 * side;
   p.off_pa = o;
   p.off_pb = o + side;
-  o = al(o + q.rep_images * h->d);
-  q.off_ent = o;    o = al(o + static_cast<size_t>(2 * h->d) * h->n * 4);
-  q.off_start = o;  o = al(o + static_cast<size_t>(2 * h->d) * (rows + 1) * 4);
-  q.off_vhs = o;    o = al(o + static_cast<size_t>(2) * rows * 4);
-  q.off_slab = o;   o = al(o + static_cast<size_t>(p.nsb) * (alias ? n1 : n1 + n3) * kSuper * 4);
+  o = al1k(o + q.rep_images * h->d);
+  q.off_ent = o;    o = al1k(o + static_cast<size_t>(2 * h->d) * h->n * 4);
+  q.off_start = o;  o = al1k(o + static_cast<size_t>(2 * h->d) * (rows + 1) * 4);
+  q.off_vhs = o;    o = al1k(o + static_cast<size_t>(2) * rows * 4);
+  q.off_slab = o;   o = al1k(o + static_cast<size_t>(p.nsb) * (alias ? n1 : n1 + n3) * kSuper * 4);
   p.ws_bytes = o;
   q.usable = true;
   return q;
@@ -1189,7 +835,7 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
                    int sms, DirectPlan* out, bool batch) {
   // under 64 inner indices the packing and the padding to a superblock show;
   // the launches of a batch are shared by its instances
-  if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535) return false;
+  if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535 || !tile_kernel_usable()) return false;
   *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1, batch);
   double best = out->seconds - (batch ? kFixedSeconds : 0.0);
   if (!batch) {
@@ -1211,11 +857,9 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
 // against 2 ell products.
 bool choose_direct_significant(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int64_t n2, int64_t n3, int dt,
                                bool alias, int sms, int bits, int ell, DirectPlan* out) {
-  if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535) return false;
+  if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535 || !tile_kernel_usable()) return false;
   *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1 + 2 * bits, false);
-  const double sums = static_cast<double>(n1) * static_cast<double>(n3) * h->d * bits * out->splits / 2.0e11 +
-                      static_cast<double>(out->acc_bytes) / 3e12;
-  return out->seconds + sums < 2.0 * ell * transform_seconds(plan, n1, n2, n3, false);
+  return out->seconds + static_cast<double>(out->acc_bytes) / 3e12 < 2.0 * ell * transform_seconds(plan, n1, n2, n3, false);
 }
 
 namespace {
@@ -1257,13 +901,11 @@ TileArgs tile_args(const DirectPlan& p, const cms_hashes* h, int64_t n1, int64_t
   a.tiles3 = p.tiles3;
   a.nsb = p.nsb;
   a.sb_per_split = p.sb_per_split;
-  a.tiles = static_cast<int>(p.tiles);
-  a.fold = p.slots > 0 ? reinterpret_cast<float*>(ws + p.off_fold) : nullptr;
-  a.slot = reinterpret_cast<uint32_t*>(ws + p.off_acc + p.acc_bytes + 256);
-  a.slots = p.slots;
+  a.splits = p.splits;
+  a.units = p.units;
   a.copies = p.copies;
-  a.grid = ws + p.off_grid;
-  a.grid64 = p.grid64 ? 1 : 0;
+  a.grid = reinterpret_cast<float*>(ws + p.off_grid);
+  a.parts = p.parts;
   a.split = p.split ? 1 : 0;
   a.sym = p.alias ? 1 : 0;
   return a;
@@ -1278,20 +920,24 @@ cudaError_t with_smem(F kern, uint32_t bytes) {
 
 }  // namespace
 
-size_t direct_batch_bytes(int count) {
+size_t direct_batch_bytes(int count, int sms) {
   auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
-  return al(count * sizeof(PackArgs)) + al(count * sizeof(TileArgs)) + 2 * al((count + 1) * sizeof(int));
+  // arguments, then the tile kernel's words (folds and tiles handed over)
+  return al(count * sizeof(PackArgs)) + al(count * sizeof(TileArgs)) + 2 * al((count + 1) * sizeof(int)) +
+         tile_work_bytes(sms, true, true, false);
 }
 
-cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, void* d_buf, DirectBatch* out, cudaStream_t s) {
+cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, int sms, void* d_buf, DirectBatch* out,
+                               cudaStream_t s) {
   auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
   const int count = static_cast<int>(specs.size());
-  std::vector<unsigned char> host(direct_batch_bytes(count));
+  std::vector<unsigned char> host(direct_batch_bytes(count, 0));
   out->buf = d_buf;
   out->count = count;
   out->o_tile = al(count * sizeof(PackArgs));
   out->o_ps = out->o_tile + al(count * sizeof(TileArgs));
   out->o_ts = out->o_ps + al((count + 1) * sizeof(int));
+  out->o_work = out->o_ts + al((count + 1) * sizeof(int));
   int* ps = reinterpret_cast<int*>(host.data() + out->o_ps);
   int* ts = reinterpret_cast<int*>(host.data() + out->o_ts);
   int np = 0, nt = 0;
@@ -1304,13 +950,15 @@ cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, void* d_buf
     ps[q] = np;
     ts[q] = nt;
     np += pack_blocks(d.plan);
-    nt += static_cast<int>(d.plan.tiles) * d.plan.splits;
+    nt += d.plan.units * d.plan.splits;
+    out->need_fold |= d.plan.need_fold;
     out->pack_smem = std::max<uint32_t>(out->pack_smem, (d.plan.split ? 4 : 2) * kStageBytes);
   }
   ps[count] = np;
   ts[count] = nt;
   out->pack_blocks = np;
-  out->tile_blocks = nt;
+  out->units = nt;
+  out->tile_blocks = std::min(nt, sms);
   cudaError_t e = cudaSuccess;
   for (int q = 0; q < count && e == cudaSuccess; ++q)
     e = cudaMemsetAsync(specs[q].ws + specs[q].plan.off_acc, 0, specs[q].plan.zero_bytes, s);
@@ -1331,13 +979,29 @@ cudaError_t launch_direct_batched(const DirectBatch& d, cudaStream_t s) {
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   ProfScope prof_scope("k_direct_tile_batched", s);
-  if ((e = with_smem(k_direct_tile_batched, tile_smem_bytes())) != cudaSuccess) return e;
-  k_direct_tile_batched<<<d.tile_blocks, kTileThreads, tile_smem_bytes(), s>>>(
-      reinterpret_cast<const TileArgs*>(base + d.o_tile), reinterpret_cast<const int*>(base + d.o_ts), d.count);
-  return cudaGetLastError();
+  TileLaunch l{};
+  l.args = reinterpret_cast<const TileArgs*>(base + d.o_tile);
+  l.start = reinterpret_cast<const int*>(base + d.o_ts);
+  l.count = d.count;
+  l.total = d.units;
+  l.need_fold = d.need_fold ? 1 : 0;
+  l.need_hand = 1;
+  l.work = reinterpret_cast<float*>(const_cast<char*>(base) + d.o_work);
+  return launch_tiles(TileArgs{}, l, true, false, d.tile_blocks, s);
 }
 
 namespace {
+
+cudaError_t launch_product_tiles(const DirectPlan& p, const TileArgs& a, char* ws, cudaStream_t s) {
+  ProfScope prof_scope("k_direct_tile", s);
+  TileLaunch l{};
+  l.total = p.units * p.splits * a.reps;
+  l.need_fold = p.need_fold ? 1 : 0;
+  l.need_hand = p.need_hand ? 1 : 0;
+  l.need_merge = p.need_merge ? 1 : 0;
+  l.work = reinterpret_cast<float*>(ws + p.off_work);
+  return launch_tiles(a, l, p.wide, p.grid, p.blocks, s);
+}
 
 // Zeroed sums, packing, tiles.
 cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
@@ -1352,20 +1016,14 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const TileArgs a = tile_args(p, h, n1, n2, n3, ws);
-  const dim3 grid(static_cast<unsigned>(p.tiles), p.splits);
-  auto go = [&](auto kern) {
-    ProfScope prof_scope("k_direct_tile", s);
-    cudaError_t r = with_smem(kern, tile_smem_bytes());
-    if (r != cudaSuccess) return r;
-    kern<<<grid, kTileThreads, tile_smem_bytes(), s>>>(a);
-    return cudaGetLastError();
-  };
-  if (!p.grid) return p.split ? go(k_direct_tile<true, false>) : go(k_direct_tile<false, false>);
-  e = p.split ? go(k_direct_tile<true, true>) : go(k_direct_tile<false, true>);
-  if (e != cudaSuccess) return e;
+  e = launch_product_tiles(p, a, ws, s);
+  if (e != cudaSuccess || !p.grid) return e;
   GridArgs g{};
   g.grid = a.grid;
-  g.ld = static_cast<int64_t>(p.tiles3) * kTile;
+  g.part = static_cast<size_t>(p.tiles1) * p.tiles3 * kTile * kTile;
+  g.parts = p.parts;
+  g.tiles3 = p.tiles3;
+  g.sym = p.alias ? 1 : 0;
   g.hs = h->d_hs;
   g.scale = a.scale;
   g.acc = a.acc;
@@ -1373,14 +1031,11 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
   g.bits = (p.sets - 1) / 2;
   g.n = a.n; g.n1 = a.n1; g.n3 = a.n3; g.b = a.b; g.d = a.d;
   ProfScope grid_scope("k_direct_grid", s);
-  const dim3 gg(p.tiles3, static_cast<unsigned>((n1 + 8 * kGridRows - 1) / (8 * kGridRows)));
-  if (p.sets > 1) {
-    if (p.grid64) k_direct_grid<long long, true><<<gg, 256, 0, s>>>(g);
-    else k_direct_grid<float, true><<<gg, 256, 0, s>>>(g);
-  } else {
-    if (p.grid64) k_direct_grid<long long, false><<<gg, 256, 0, s>>>(g);
-    else k_direct_grid<float, false><<<gg, 256, 0, s>>>(g);
-  }
+  // an SM adds 1.35 G/s: few tiles are shared by the repetitions' blocks
+  const int tiles = p.tiles1 * p.tiles3, per_tile = kTile / (8 * kGridCols);
+  const dim3 gg(tiles, per_tile, std::min(h->d, std::max(1, 152 * 2 / (tiles * per_tile))));
+  if (p.sets > 1) k_direct_grid<true><<<gg, 256, 0, s>>>(g);
+  else k_direct_grid<false><<<gg, 256, 0, s>>>(g);
   return cudaGetLastError();
 }
 
@@ -1458,13 +1113,7 @@ cudaError_t launch_pre(const DirectPlan& chosen, const cms_hashes* h, const void
   ta.reps = h->d;
   ta.rep_images = q.rep_images;
   ta.rep_blocks = q.rep_blocks;
-  {
-    ProfScope prof_scope("k_direct_tile", s);
-    if ((e = with_smem(k_direct_tile<true, false>, tile_smem_bytes())) != cudaSuccess) return e;
-    k_direct_tile<true, false><<<dim3(static_cast<unsigned>(p.tiles), p.splits, h->d), kTileThreads, tile_smem_bytes(),
-                                 s>>>(ta);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+  if ((e = launch_product_tiles(p, ta, ws, s)) != cudaSuccess) return e;
   return launch_finish(p, h, c, h->b, ws, s);
 }
 

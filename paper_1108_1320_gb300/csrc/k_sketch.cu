@@ -289,21 +289,30 @@ k_cols_inverse_batched(const ColsArgs* __restrict__ args, const int* __restrict_
   const int i = batch_instance(start, count, static_cast<int>(blockIdx.x));
   const ColsArgs a = args[i];
   const int local = static_cast<int>(blockIdx.x) - __ldg(start + i);
-  const int t = local / a.nbx;
-  const int64_t z = static_cast<int64_t>(local % a.nbx) * blockDim.x + threadIdx.x;
-  if (z >= a.b) return;
   if (a.sums != nullptr) {
-    const size_t q = static_cast<size_t>(t) * a.b + z;
-    const size_t len = static_cast<size_t>(a.nbd) * a.b;
-    unsigned long long v = 0;
+    // 2048 sums per block, 8 per thread in flight (256 per block took 500 us
+    // for 64 products, mostly the search for the product)
+    const int64_t len = a.b * a.nbd;
+    const int64_t q0 = static_cast<int64_t>(local) * 2048 + threadIdx.x;
+    const DirectScale sc = *a.scale;
+    unsigned long long v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (int r = 0; r < a.copies; ++r) {
-      v += a.sums[r * len + q];
-      a.sums[r * len + q] = 0;
+      unsigned long long* sums = a.sums + r * len;
+#pragma unroll
+      for (int g = 0; g < 8; ++g)
+        if (q0 + g * 256 < len) v[g] += __ldcg(sums + q0 + g * 256);
+#pragma unroll
+      for (int g = 0; g < 8; ++g)
+        if (q0 + g * 256 < len) __stcg(sums + q0 + g * 256, 0ull);
     }
-    a.c[q] = direct_value(v, *a.scale, a.log2s);
+#pragma unroll
+    for (int g = 0; g < 8; ++g)
+      if (q0 + g * 256 < len) a.c[q0 + g * 256] = direct_value(v[g], sc, a.log2s);
     return;
   }
-  cols_inverse_point(a.V, a.twR, a.b, a.R, a.C, a.nrows, a.c, t, z);
+  const int t = local / a.nbx;
+  const int64_t z = static_cast<int64_t>(local % a.nbx) * blockDim.x + threadIdx.x;
+  if (z < a.b) cols_inverse_point(a.V, a.twR, a.b, a.R, a.C, a.nrows, a.c, t, z);
 }
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
@@ -680,7 +689,7 @@ cudaError_t build_inverse_batch(const std::vector<InverseSpec>& specs, void* d_b
     ca.nbx = static_cast<int>((plan.b + 255) / 256);
     cols[i] = ca;
     cstart[i] = tc;
-    tc += ca.nbx * plan.d;
+    tc += direct ? static_cast<int>((plan.b * plan.d + 2047) / 2048) : ca.nbx * plan.d;
   }
   rstart[count] = tr;
   cstart[count] = tc;

@@ -269,7 +269,7 @@ def test_find_significant_on_the_direct_route(cms, n1, n2, n3, rho, alias):
 @pytest.mark.parametrize("n1,n2,n3,b,d,dts,alias,pad", [
     (3000, 500, 2500, 600, 3, "f32", False, 1),    # R = 1, a last superblock of 116 inner indices
     (5000, 300, 5000, 1500, 2, "bf16", True, 0),   # R = 2, C = 750: the last tile is not full
-    (8000, 257, 8000, 2916, 3, "f32", True, 0),    # R = 4 (128 rows hold 32 classes), one inner index in the last stage
+    (8000, 513, 8000, 1944, 3, "f32", True, 0),    # R = 2, C = 972: the last tile is not full; one inner index in the last stage
     (6000, 400, 6000, 2187, 3, "f64", True, 3),    # R = 3: rows without a bucket in every tile
 ])
 def test_pre_sketched_operands_match_oracle(cms, n1, n2, n3, b, d, dts, alias, pad):

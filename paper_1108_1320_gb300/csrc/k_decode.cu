@@ -111,35 +111,49 @@ __global__ void k_decode_dense(const T* __restrict__ c, const uint32_t* __restri
 // Thresholded decode (Fig. 2: the approximation is thresholded into a short
 // list of candidates): pass 1 counts, per row i, the j with
 // |estimate(i, j)| > tau (i != j when skip_diagonal); pass 2 turns the
-// counts into row offsets; pass 3 recomputes the estimates and writes the
-// hits of row i in increasing j from its offset (row-major order overall,
-// independent of scheduling).
+// counts into row offsets; pass 3 recomputes the estimates of the segments of
+// row i that hold hits and writes them in increasing j from its offset
+// (row-major order overall, independent of scheduling).  The gathers of the
+// estimates bound the first pass (284 G/s of random sectors); a few hits per
+// row leave little of them to the third (1500 x 1500, d = 5, 32 pairs: 45 us
+// over whole rows, 12 us).
 __device__ __forceinline__ bool thresh_hit(float v, float tau, int skip, int64_t i, int64_t j) {
   return fabsf(v) > tau && !(skip && i == j);
 }
 
+// A row's word: its count, then its offset, in the low kOffBits (n1 n3 <=
+// 2^48), and above them a bit for each of kSegments segments of the row that
+// hold a hit.
+constexpr int kOffBits = 49, kSegments = 64 - kOffBits;
+constexpr uint64_t kOffMask = (uint64_t{1} << kOffBits) - 1;
+__host__ __device__ __forceinline__ int64_t segment_cols(int64_t n3) { return (n3 + kSegments * 32 - 1) / (kSegments * 32) * 32; }
+
 __global__ void __launch_bounds__(256)
 k_thresh_count(const float* __restrict__ c, const uint32_t* __restrict__ hs, int64_t n, uint32_t b, int d,
-               int64_t n1, int64_t n3, float tau, int skip, int64_t* __restrict__ rowcnt) {
-  __shared__ int64_t part[8];
+               int64_t n1, int64_t n3, float tau, int skip, uint64_t* __restrict__ rows) {
+  __shared__ unsigned long long word;
+  const uint32_t seg = static_cast<uint32_t>(segment_cols(n3));
   for (int64_t i = blockIdx.x; i < n1; i += gridDim.x) {
-    int64_t cnt = 0;
-    for (int64_t j = threadIdx.x; j < n3; j += blockDim.x)
-      cnt += thresh_hit(estimate(c, hs, n, b, d, i, j), tau, skip, i, j) ? 1 : 0;
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = cnt;
+    if (threadIdx.x == 0) word = 0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      int64_t s = 0;
-      for (int w = 0; w < 8; ++w) s += part[w];
-      rowcnt[i] = s;
+    for (int64_t j0 = threadIdx.x & ~31u; j0 < n3; j0 += blockDim.x) {   // a warp's 32 columns lie in one segment
+      const int64_t j = j0 + (threadIdx.x & 31);
+      const bool hit = j < n3 && thresh_hit(estimate(c, hs, n, b, d, i, j), tau, skip, i, j);
+      const unsigned bal = __ballot_sync(0xffffffffu, hit);
+      if (bal && (threadIdx.x & 31) == 0) {
+        atomicAdd(&word, static_cast<unsigned long long>(__popc(bal)));
+        atomicOr(&word, 1ull << (kOffBits + static_cast<uint32_t>(j0) / seg));
+      }
     }
+    __syncthreads();
+    if (threadIdx.x == 0) rows[i] = word;
     __syncthreads();
   }
 }
 
-// exclusive scan of rowcnt[0..n1) in place; rowcnt[n1] and *total get the sum
-__global__ void __launch_bounds__(1024) k_thresh_scan(int64_t* __restrict__ rowcnt, int64_t n1,
+// exclusive scan of the counts of rows[0..n1) in place; rows[n1] and *total get
+// the sum
+__global__ void __launch_bounds__(1024) k_thresh_scan(uint64_t* __restrict__ rows, int64_t n1,
                                                       int64_t* __restrict__ total) {
   __shared__ int64_t wsum[32];
   __shared__ int64_t running;
@@ -148,7 +162,8 @@ __global__ void __launch_bounds__(1024) k_thresh_scan(int64_t* __restrict__ rowc
   __syncthreads();
   for (int64_t base = 0; base < n1; base += 1024) {
     const int64_t i = base + tid;
-    const int64_t v = i < n1 ? rowcnt[i] : 0;
+    const uint64_t r = i < n1 ? rows[i] : 0;
+    const int64_t v = static_cast<int64_t>(r & kOffMask);
     int64_t x = v;
     for (int o = 1; o < 32; o <<= 1) {
       const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -158,7 +173,7 @@ __global__ void __launch_bounds__(1024) k_thresh_scan(int64_t* __restrict__ rowc
     __syncthreads();
     int64_t before = 0;
     for (int w = 0; w < warp; ++w) before += wsum[w];
-    if (i < n1) rowcnt[i] = running + before + x - v;
+    if (i < n1) rows[i] = static_cast<uint64_t>(running + before + x - v) | (r & ~kOffMask);
     __syncthreads();
     if (tid == 0) {
       int64_t s = 0;
@@ -168,22 +183,33 @@ __global__ void __launch_bounds__(1024) k_thresh_scan(int64_t* __restrict__ rowc
     __syncthreads();
   }
   if (tid == 0) {
-    rowcnt[n1] = running;
+    rows[n1] = static_cast<uint64_t>(running);
     *total = running;
   }
 }
 
+// 32 columns per warp of the segments that hold hits, in column order.
 __global__ void __launch_bounds__(256)
 k_thresh_write(const float* __restrict__ c, const uint32_t* __restrict__ hs, int64_t n, uint32_t b, int d,
-               int64_t n1, int64_t n3, float tau, int skip, const int64_t* __restrict__ rowoff,
+               int64_t n1, int64_t n3, float tau, int skip, const uint64_t* __restrict__ rows,
                int64_t capacity, int64_t* __restrict__ ij, float* __restrict__ val) {
   __shared__ int wcnt[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t seg = segment_cols(n3), strips = seg / 32;
   for (int64_t i = blockIdx.x; i < n1; i += gridDim.x) {
-    if (rowoff[i] == rowoff[i + 1]) continue;   // uniform over the block
-    int64_t pos = rowoff[i];
-    for (int64_t j0 = 0; j0 < n3; j0 += blockDim.x) {
-      const int64_t j = j0 + threadIdx.x;
+    const uint64_t word = rows[i];
+    int64_t pos = static_cast<int64_t>(word & kOffMask);
+    // uniform over the block: no hits, or none within the capacity
+    const uint32_t mask = static_cast<uint32_t>(word >> kOffBits);
+    if (mask == 0 || pos >= capacity) continue;
+    const int64_t count = __popc(mask) * strips;
+    for (int64_t s0 = 0; s0 < count; s0 += 8) {
+      const int64_t s = s0 + warp;
+      int64_t j = n3;
+      if (s < count) {
+        const int64_t q = s / strips;
+        j = static_cast<int64_t>(__fns(mask, 0, static_cast<int>(q) + 1)) * seg + (s - q * strips) * 32 + lane;
+      }
       float v = 0.f;
       bool hit = false;
       if (j < n3) {
@@ -276,17 +302,18 @@ cudaError_t launch_decode_threshold(const float* c, const cms_hashes* h, int64_t
   if (n1 == 0 || n3 == 0) return cudaMemsetAsync(count, 0, sizeof(int64_t), s);
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(n1, 65535));
   const uint32_t b = static_cast<uint32_t>(h->b);
+  uint64_t* rows = reinterpret_cast<uint64_t*>(rowcnt);
   {
     ProfScope prof_scope("k_thresh_count", s);
-    k_thresh_count<<<grid, 256, 0, s>>>(c, h->d_hs, h->n, b, h->d, n1, n3, tau, skip_diagonal, rowcnt);
+    k_thresh_count<<<grid, 256, 0, s>>>(c, h->d_hs, h->n, b, h->d, n1, n3, tau, skip_diagonal, rows);
   }
   {
     ProfScope prof_scope("k_thresh_scan", s);
-    k_thresh_scan<<<1, 1024, 0, s>>>(rowcnt, n1, count);
+    k_thresh_scan<<<1, 1024, 0, s>>>(rows, n1, count);
   }
   {
     ProfScope prof_scope("k_thresh_write", s);
-    k_thresh_write<<<grid, 256, 0, s>>>(c, h->d_hs, h->n, b, h->d, n1, n3, tau, skip_diagonal, rowcnt,
+    k_thresh_write<<<grid, 256, 0, s>>>(c, h->d_hs, h->n, b, h->d, n1, n3, tau, skip_diagonal, rows,
                                         capacity, ij, val);
   }
   return cudaGetLastError();

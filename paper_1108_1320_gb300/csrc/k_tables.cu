@@ -233,18 +233,32 @@ k_frontend_tables(const uint32_t* __restrict__ hs, const uint32_t* __restrict__ 
   } else {
     key[tid] = 0xFFFFFFFFu;   // sorts after every bucket
   }
-  __syncthreads();
-  for (int size = 2; size <= kMax; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      const int partner = tid ^ stride;
-      if (partner > tid) {
-        const bool up = (tid & size) == 0;
-        const uint32_t a = key[tid], b2 = key[partner];
-        if ((a > b2) == up) { key[tid] = b2; key[partner] = a; }
+  // bitonic sort, a key per thread: exchanges within a warp by shuffles (40 of
+  // the 55 steps), the others through two buffers in turn (with the dealing
+  // below: 25 -> 23 us)
+  {
+    uint32_t kv = key[tid];
+    uint32_t* buf = key;
+    for (int size = 2; size <= kMax; size <<= 1) {
+      for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        uint32_t other;
+        if (stride >= 32) {
+          buf = buf == key ? used : key;
+          __syncthreads();   // the ranks' reads, or those of two steps before
+          buf[tid] = kv;
+          __syncthreads();
+          other = buf[tid ^ stride];
+        } else {
+          other = __shfl_xor_sync(0xFFFFFFFFu, kv, stride);
+        }
+        const bool low = ((tid & size) == 0) == ((tid & stride) == 0);
+        kv = low ? min(kv, other) : max(kv, other);
       }
-      __syncthreads();
     }
+    __syncthreads();
+    key[tid] = kv;
   }
+  __syncthreads();
   // Within each group of 32 buckets, place buckets so that each half-warp
   // holds distinct z2 mod 16 where possible: the front end's 8-byte stores
   // to Y[z2] are then free of bank conflicts.  The group's bucket set (and
@@ -341,10 +355,9 @@ k_frontend_tables(const uint32_t* __restrict__ hs, const uint32_t* __restrict__ 
     for (uint32_t i = 0; i < 32; ++i) {
       const int g = __ffs(__ballot_sync(0xFFFFFFFFu, rk == i)) - 1;
       const uint32_t cg = __shfl_sync(0xFFFFFFFFu, myc, g);
-      uint64_t key = (lane < 8 && fill < 4) ? ((static_cast<uint64_t>(load) << 8) | static_cast<uint64_t>(lane))
-                                            : ~0ull;
-      for (int o = 4; o > 0; o >>= 1) key = min(key, __shfl_xor_sync(0xFFFFFFFFu, key, o));
-      if (lane < 8 && static_cast<uint64_t>(lane) == (key & 0xFFu)) {
+      // (loads stay below 2^27: n <= 2^24)
+      const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, lane < 8 && fill < 4 ? load << 3 | lane : 0xFFFFFFFFu);
+      if (lane < 8 && static_cast<uint32_t>(lane) == (least & 7u)) {
         as[lane * 4 + fill] = static_cast<uint8_t>(g);
         ++fill;
         load += cg;
@@ -372,7 +385,8 @@ k_frontend_records(const uint32_t* __restrict__ hs, const uint32_t* __restrict__
                    const uint32_t* __restrict__ ovf_off, uint32_t* __restrict__ ovf_x,
                    uint32_t* __restrict__ ovf_hs, int C) {
   constexpr uint32_t kCap = static_cast<uint32_t>(kFeCap);
-  __shared__ uint32_t ub[32];
+  static_assert(kCap <= 8, "an entry's index takes three bits");
+  __shared__ uint32_t turn[32];
   const int L = (C + 31) / 32;
   const int ts = blockIdx.x / L, g = blockIdx.x % L;
   const int lane = threadIdx.x;
@@ -404,43 +418,52 @@ k_frontend_records(const uint32_t* __restrict__ hs, const uint32_t* __restrict__
     ox[oz + (r - kCap)] = x;
     oh[oz + (r - kCap)] = tab[x];
   }
+  // the lane whose turn is k: lanes in order of ascending count
   uint32_t rank = 0;
   for (int o = 0; o < 32; ++o) {
     const uint32_t co = __shfl_sync(0xFFFFFFFFu, c, o);
     rank += (co < c || (co == c && o < lane)) ? 1u : 0u;
   }
+  turn[rank] = lane;
+  __syncwarp();
+  const int my_turn = static_cast<int>(turn[lane]);
   // steps r unrolled so that every index into xs / wsv is a constant (the
   // arrays stay in registers); the lanes with no entry left at step r have
-  // the lowest ranks and take no turn
+  // the lowest ranks and take no turn.  Each lane keeps the uses so far of its
+  // remaining entries' banks, so a turn is one shuffle (the bank taken) and
+  // the other lanes' counts (counters in shared memory took several accesses
+  // of one lane after another: 45 us for 2 x 5 x 32 groups of n = 2048, 27 so).
 #pragma unroll
   for (uint32_t r = 0; r < kCap; ++r) {
     if (r >= cm) break;
-    ub[lane] = 0;
     const uint32_t done = __ballot_sync(0xFFFFFFFFu, c <= r);
-    __syncwarp();
-    if (lane == 0 && done) ub[n & 31u] = 1;
-    __syncwarp();
+    uint32_t key[kFeCap];     // uses of the entry's bank * 8 + entry (the first of the least used)
+#pragma unroll
+    for (uint32_t i = r; i < kCap; ++i)
+      key[i] = i < c ? ((done && (xs[i] & 31u) == (n & 31u)) ? 8u : 0u) | i : 0xFFFFFFFFu;
+    uint32_t mine = r;
     for (uint32_t k = __popc(done); k < 32; ++k) {
-      if (rank == k) {
-        uint32_t best = r, bu = ub[xs[r] & 31u];
+      uint32_t best = key[r];
 #pragma unroll
-        for (uint32_t i = r + 1; i < kCap; ++i) {
-          if (i < c) {
-            const uint32_t u = ub[xs[i] & 31u];
-            if (u < bu) { bu = u; best = i; }
-          }
-        }
+      for (uint32_t i = r + 1; i < kCap; ++i) best = min(best, key[i]);
+      best &= 7u;
+      uint32_t x = xs[r];
 #pragma unroll
-        for (uint32_t i = r + 1; i < kCap; ++i) {
-          if (best == i) {
-            const uint32_t tx = xs[r], tw = wsv[r];
-            xs[r] = xs[i]; wsv[r] = wsv[i];
-            xs[i] = tx; wsv[i] = tw;
-          }
-        }
-        ub[xs[r] & 31u] += 1;
+      for (uint32_t i = r + 1; i < kCap; ++i)
+        if (best == i) x = xs[i];
+      const uint32_t bank = __shfl_sync(0xFFFFFFFFu, x & 31u, __shfl_sync(0xFFFFFFFFu, my_turn, static_cast<int>(k)));
+      if (rank == k) mine = best;
+#pragma unroll
+      for (uint32_t i = r; i < kCap; ++i)
+        if (i < c && (xs[i] & 31u) == bank) key[i] += 8u;
+    }
+#pragma unroll
+    for (uint32_t i = r + 1; i < kCap; ++i) {
+      if (mine == i && c > r) {
+        const uint32_t tx = xs[r], tw = wsv[r];
+        xs[r] = xs[i]; wsv[r] = wsv[i];
+        xs[i] = tx; wsv[i] = tw;
       }
-      __syncwarp();
     }
   }
 #pragma unroll

@@ -23,14 +23,15 @@
 //    with integer reductions: the order of the additions does not matter, so
 //    the sketch is the same in every run.  Its scatter warps add them while the
 //    next tile is multiplied, or the entries are stored (at most 16.8 M) and
-//    k_direct_grid adds them with the whole chip: a tile's additions take an
-//    SM 12 us a repetition, so that a last wave of few tiles would wait for
-//    them (2265 x 2265 x 503, d = 7: 318 us fused, 24 + 197 us in two).
+//    k_direct_grid or k_direct_window adds them with the whole chip: a tile's
+//    additions take an SM 12 us a repetition, so that a last wave of few tiles
+//    would wait for them (2265 x 2265 x 503, d = 7: 318 us fused, 24 + 197 us
+//    in two).
 //  * k_direct_finish converts the sums to FP32.
 //
 // Measured on one GB300 (whole calls, transform route -> this one): X^T X of
 // 4096 x 2048 FP32, b = 2^16, d = 5 with its hash draw and dense decode 2.93
-// -> 0.35 ms; 8192 x 4096 BF16, b = 2^16, d = 3 7.54 -> 0.42 ms; 16384 x
+// -> 0.31 ms; 8192 x 4096 BF16, b = 2^16, d = 3 7.54 -> 0.37 ms; 16384 x
 // 32768 BF16, b = 2^20, d = 7 834 -> 50.6 ms; 64 uneven products of n = 512 ..
 // 8192, b = 16 n, d = 3 416 -> 25.2 ms.  What bounds it: the additions into
 // the buckets (random 64-bit reductions run at 205 G/s on the whole chip, one
@@ -50,6 +51,7 @@ using namespace wfft;
 using namespace dtile;
 
 constexpr double kFixedSeconds = 36e-6;   // launches of a single product
+constexpr int kWindow = 28672;             // buckets in shared memory (224 KB)
 constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
 constexpr int kMinExp = -100;           // scales stay representable
 
@@ -518,7 +520,7 @@ struct GridArgs {
   const float* grid;           // [part][tile row][tile column][128 columns][128 rows]
   size_t part;                 // entries from one part to the next
   int parts;
-  int tiles3, sym;
+  int tiles1, tiles3, sym;
   const uint32_t* hs;          // [t][side][n]
   const DirectScale* scale;
   unsigned long long* acc;     // [copy][t][b], or [1 + 2 bits][t][b]
@@ -591,6 +593,139 @@ __global__ void __launch_bounds__(256) k_direct_grid(const GridArgs p) {
         if (mirror) add(c, j0 + q, i, hx, hm[r], v[q][r]);
       }
     }
+  }
+}
+
+// __float2ll_rn for |v| < 2^63 without the 64-bit conversion (2 a clock and SM)
+__device__ __forceinline__ long long to_units(float v) {
+  const uint32_t bits = __float_as_uint(v);
+  const int shift = static_cast<int>((bits >> 23) & 0xFFu) - 150;
+  const long long big = static_cast<long long>(static_cast<unsigned long long>((bits & 0x7FFFFFu) | 0x800000u) << (shift & 63));
+  const long long small = __float2int_rn(v);
+  return shift < 0 ? small : (static_cast<int>(bits) < 0 ? -big : big);
+}
+
+// Byte of a window's bucket (z4: four times the bucket).  The hashes are linear
+// in the position mod a prime, so that a warp's 32 rows are mostly an even
+// progression of buckets: one step in 16 words would put them in two banks.
+__device__ __forceinline__ uint32_t window_byte(uint32_t z4) { return z4 ^ ((z4 >> 5) & 0x7Cu); }
+
+// The entries of the grid added to the buckets with the first kWindow buckets
+// of a repetition in a block's shared memory (two words each) and the others'
+// additions in L2: a block adds its share of the tiles for one repetition.
+// 64 bits are added in two halves, the low half's carry taken from the value
+// that its addition returns (64-bit additions in shared memory are a loop of
+// compare and swap, a quarter as fast).  Beside k_direct_grid, bound by 1.35 G
+// reductions a second and SM: 4096 x 4096 entries, d = 3, b = 2^16 (44% of the
+// buckets in the window) 228 -> 175 us; 1500 x 1500, d = 5, b = 30000 (all but
+// 4%) 78 -> 45 us, 30 clocks for a warp's 32 additions, most of them latency.
+// Three windows a repetition, every entry read for each: 279 us of the 228.
+__global__ void __launch_bounds__(1024, 1) k_direct_window(const GridArgs p, int shares) {
+  extern __shared__ uint32_t words[];        // low halves, then high halves
+  if (p.scale->bad) return;
+  const int t = static_cast<int>(blockIdx.x) / shares, share = static_cast<int>(blockIdx.x) - t * shares;
+  const uint32_t b = static_cast<uint32_t>(p.b), mine = min(b, static_cast<uint32_t>(kWindow));
+  const uint32_t b4 = 4 * b, mine4 = 4 * mine;
+  const uint32_t used = (mine + 31) & ~31u;
+  for (uint32_t q = threadIdx.x; q < used; q += 1024) words[q] = words[kWindow + q] = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
+  const uint32_t* h2 = h1 + p.n;
+  unsigned long long* out = p.acc + static_cast<size_t>(t) * b;
+  const uint32_t base = smem_u32(words);
+  // four rows: their low halves are on their way together
+  auto add4 = [&](const uint32_t (&row4)[4], const int (&rowneg)[4], uint32_t col4, int colneg, const long long (&v)[4]) {
+    uint32_t z4[4], l[4], h[4], old[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const uint32_t z = row4[r] + col4;
+      z4[r] = min(z, z - b4);              // (row4 + col4) mod b4
+      const int m = (rowneg[r] ^ colneg) >> 31;
+      const unsigned long long iv = static_cast<unsigned long long>((v[r] ^ m) - m);
+      l[r] = static_cast<uint32_t>(iv);
+      h[r] = static_cast<uint32_t>(iv >> 32);
+      asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %3, %4;\n\tmov.u32 %0, 0;\n\t"
+                   "@p atom.shared.add.u32 %0, [%1], %2;\n\t}"
+                   : "=&r"(old[r])
+                   : "r"(base + window_byte(z4[r])), "r"(l[r]), "r"(z4[r]), "r"(mine4)
+                   : "memory");
+      if (z4[r] >= mine4)
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(out + z4[r] / 4), "l"(iv) : "memory");
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 x, y;\n\tsetp.lt.u32 p, %0, %1;\n\t"
+                   "add.cc.u32 x, %4, %5;\n\taddc.u32 y, %6, 0;\n\t"
+                   "@p red.shared.add.u32 [%2+%3], y;\n\t}" ::"r"(z4[r]), "r"(mine4), "r"(base + window_byte(z4[r])),
+                   "n"(4 * kWindow), "r"(old[r]), "r"(l[r]), "r"(h[r])
+                   : "memory");
+    }
+  };
+  // half tiles: two columns a warp, four rows of each a lane
+  const int tiles = p.sym ? p.tiles3 * (p.tiles3 + 1) / 2 : p.tiles1 * p.tiles3;
+  for (int u = share; u < 2 * tiles; u += shares) {
+    int ti, tj;
+    const int q = u >> 1;
+    if (p.sym) {
+      tj = static_cast<int>((sqrtf(8.f * static_cast<float>(q) + 1.f) - 1.f) * 0.5f);
+      while (tj * (tj + 1) / 2 > q) --tj;
+      while ((tj + 1) * (tj + 2) / 2 <= q) ++tj;
+      ti = q - tj * (tj + 1) / 2;
+    } else {
+      ti = q / p.tiles3;
+      tj = q - ti * p.tiles3;
+    }
+    const bool mirror = p.sym && ti != tj;
+    const int i0 = ti * kTile + lane, q0 = (u & 1) * 64 + warp * 2, j0 = tj * kTile + q0;
+    if (j0 >= p.n3) continue;
+    const float* src = p.grid + (static_cast<size_t>(ti) * p.tiles3 + tj) * kTile * kTile + q0 * kTile + lane;
+    long long v[2][4];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) v[c][r] = to_units(__ldcg(src + c * kTile + r * 32));
+#pragma unroll 2
+    for (int x = 1; x < p.parts; ++x) {
+      src += p.part;
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[c][r] += to_units(__ldcg(src + c * kTile + r * 32));
+    }
+    uint32_t row4[4];
+    int rowneg[4];
+    auto rows = [&](const uint32_t* hh) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {   // (entries past the last row are zero)
+        const uint32_t w = i0 + 32 * r < p.n1 ? __ldg(hh + i0 + 32 * r) : 0;
+        rowneg[r] = static_cast<int>(w);
+        row4[r] = 4 * (w & kBucketMask);
+      }
+    };
+    const int cols = min(2, p.n3 - j0);
+    rows(h1);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (c >= cols) break;
+      const uint32_t w = __ldg(h2 + j0 + c);
+      add4(row4, rowneg, 4 * (w & kBucketMask), static_cast<int>(w), v[c]);
+    }
+    if (mirror) {
+      rows(h2);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        if (c >= cols) break;
+        const uint32_t w = __ldg(h1 + j0 + c);
+        add4(row4, rowneg, 4 * (w & kBucketMask), static_cast<int>(w), v[c]);
+      }
+    }
+  }
+  __syncthreads();
+  for (uint32_t q = threadIdx.x; q < mine; q += 1024) {
+    const uint32_t w = window_byte(4 * q) / 4;
+    const unsigned long long sum = static_cast<unsigned long long>(words[kWindow + w]) << 32 | words[w];
+    if (sum) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(out + q), "l"(sum) : "memory");
   }
 }
 
@@ -672,7 +807,11 @@ namespace {
 // Times: a chunk of 64 (FP16 terms) or 128 (BF16) inner indices of a tile
 // 0.40 us (BF16 alone on its operands 0.53: the copies from L2 bound it).
 void choose_tiles(DirectPlan& p, bool sym, int reps, double entries, double adds, double full_rate, double sm_rate,
-                  bool may_grid, bool may_fuse, bool shared, int sms) {
+                  double window, bool may_grid, bool may_fuse, bool shared, int sms) {
+  // stored entries added: in L2, or with a share of the buckets in shared memory
+  // (2.7 us less per million of its additions, 4 us more)
+  p.window = entries * adds * window >= 3e6;
+  const double added = entries * reps * adds / full_rate * (p.window ? 1.0 - 0.65 * window : 1.0) + (p.window ? 4e-6 : 0.0);
   double best = 1e30;
   for (int wide = 0; wide < 2; ++wide) {
     if (!wide && shared) continue;
@@ -690,7 +829,7 @@ void choose_tiles(DirectPlan& p, bool sym, int reps, double entries, double adds
         if (grid ? !may_grid : !may_fuse) continue;
         const double parts = real * (wide || per * (p.split ? 2 : 1) == 1 ? 1.0 : 2.0);
         const double t =
-            grid ? mma + 3e-6 + entries * reps * (adds / full_rate + (sym ? 4.0 : 8.0) * parts / 4e12) + parts * 0.1e-6
+            grid ? mma + 3e-6 + added + entries * reps * (sym ? 4.0 : 8.0) * parts / 4e12 + parts * 0.1e-6
                  : mma + std::max(entries * reps * adds * real / full_rate,
                                   waves * entries * adds / units / sm_rate);
         if (t < best) {
@@ -736,6 +875,7 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   const int64_t images = (n2 + per - 1) / per;
   const double entries = static_cast<double>(n1) * static_cast<double>(n3);
   choose_tiles(p, alias, 1, entries, 0.5 * h->d * (sets + 1), 2.05e11, 1.35e9,
+               sets == 1 ? std::min(1.0, static_cast<double>(kWindow) / static_cast<double>(h->b)) : 0.0,
                !batch && (sets > 1 || entries <= 16.8e6), sets == 1, batch, sms);
   const int64_t words = static_cast<int64_t>(h->d) * h->b;
   // (a batch's products queue up less: others' additions are under way too)
@@ -801,7 +941,7 @@ PrePlan make_pre_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, b
   p.split = true;
   p.tiles1 = p.tiles3 = q.tiles;
   p.nsb = static_cast<int>((n2 + kSuper - 1) / kSuper);
-  choose_tiles(p, false, h->d, static_cast<double>(rows) * rows, 1.0, 5.0e11, 4e9, false, true, false, sms);
+  choose_tiles(p, false, h->d, static_cast<double>(rows) * rows, 1.0, 5.0e11, 4e9, 0.0, false, true, false, sms);
   const double n = static_cast<double>(alias ? n1 : n1 + n3), k = static_cast<double>(p.nsb) * kSuper;
   p.seconds += 14e-6 + n * k * 8.0 / 4e12 + static_cast<double>(n1 + n3) * k * h->d * 4.0 / 5e12 +
               2.0 * static_cast<double>(rows) * k * h->d * 4.0 / 3e12;
@@ -1022,6 +1162,7 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
   g.grid = a.grid;
   g.part = static_cast<size_t>(p.tiles1) * p.tiles3 * kTile * kTile;
   g.parts = p.parts;
+  g.tiles1 = p.tiles1;
   g.tiles3 = p.tiles3;
   g.sym = p.alias ? 1 : 0;
   g.hs = h->d_hs;
@@ -1030,9 +1171,16 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
   g.copies = p.copies;
   g.bits = (p.sets - 1) / 2;
   g.n = a.n; g.n1 = a.n1; g.n3 = a.n3; g.b = a.b; g.d = a.d;
-  ProfScope grid_scope("k_direct_grid", s);
   // an SM adds 1.35 G/s: few tiles are shared by the repetitions' blocks
+  if (p.window) {
+    ProfScope window_scope("k_direct_window", s);
+    if ((e = with_smem(k_direct_window, 8 * kWindow)) != cudaSuccess) return e;
+    const int shares = std::max(1, 152 / h->d);
+    k_direct_window<<<h->d * shares, 1024, 8 * kWindow, s>>>(g, shares);
+    return cudaGetLastError();
+  }
   const int tiles = p.tiles1 * p.tiles3, per_tile = kTile / (8 * kGridCols);
+  ProfScope grid_scope("k_direct_grid", s);
   const dim3 gg(tiles, per_tile, std::min(h->d, std::max(1, 152 * 2 / (tiles * per_tile))));
   if (p.sets > 1) k_direct_grid<true><<<gg, 256, 0, s>>>(g);
   else k_direct_grid<false><<<gg, 256, 0, s>>>(g);

@@ -145,6 +145,22 @@ def test_non_finite_operands_give_nan_on_both_routes(cms, n2, value):
     h.free()
 
 
+@pytest.mark.parametrize("n1,n2,n3,b,d,dts,alias", [
+    (1100, 200, 1000, 20000, 3, "f32", False), (1025, 700, 1025, 27000, 3, "f32", True),
+    (1001, 64, 1025, 28800, 4, "f32", False), (1500, 130, 1500, 65536, 5, "bf16", True),
+    (1153, 300, 1153, 5000, 3, "bf16", True), (1024, 100, 1153, 40000, 7, "f64", False)])
+def test_stored_entries_with_a_window_of_the_buckets(cms, n1, n2, n3, b, d, dts, alias):
+    # all buckets in shared memory, or the first 28672 and the rest in L2
+    A, B, Ad, Bd = operands(n1, n2, n3, dts, alias, 0, n1 + b)
+    h = cms.make_hashes(b, max(n1, n3), b, d)
+    c, kernels = run(cms, A, B, h)
+    again, _ = run(cms, A, B, h)
+    assert "k_direct_window" in kernels
+    assert worst(c, O.sketch_definition(Ad, Bd, O.make_tables(b, max(n1, n3), b, d))) < TOL
+    assert torch.equal(c, again)
+    h.free()
+
+
 def test_workspace_of_the_transform_route_still_serves(cms):
     # a workspace smaller than the direct route's layout: the transform route
     A, B, Ad, Bd = operands(400, 4000, 400, "f32", True, 0, 11)

@@ -31,7 +31,7 @@
 //
 // Measured on one GB300 (whole calls, transform route -> this one): X^T X of
 // 4096 x 2048 FP32, b = 2^16, d = 5 with its hash draw and dense decode 2.93
-// -> 0.31 ms; 8192 x 4096 BF16, b = 2^16, d = 3 7.54 -> 0.37 ms; 16384 x
+// -> 0.31 ms; 8192 x 4096 BF16, b = 2^16, d = 3 7.54 -> 0.35 ms; 16384 x
 // 32768 BF16, b = 2^20, d = 7 834 -> 50.6 ms; 64 uneven products of n = 512 ..
 // 8192, b = 16 n, d = 3 416 -> 25.2 ms.  What bounds it: the additions into
 // the buckets (random 64-bit reductions run at 205 G/s on the whole chip, one
@@ -260,7 +260,10 @@ __device__ __forceinline__ void pack_task(const PackArgs& p, uint32_t idx) {
   if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(256) k_direct_pack(const PackArgs p) { pack_task(p, blockIdx.x); }
+__global__ void __launch_bounds__(256) k_direct_pack(const PackArgs p) {
+  next_kernel_may_start();
+  pack_task(p, blockIdx.x);
+}
 
 // ---- pre-sketched operands: b well below n ----
 // By Fig. 1 c_t is the cyclic convolution of the count sketches of a_k and
@@ -535,6 +538,8 @@ struct GridArgs {
 constexpr int kGridCols = 2;
 template <bool MASKED>
 __global__ void __launch_bounds__(256) k_direct_grid(const GridArgs p) {
+  next_kernel_may_start();
+  wait_for_kernel_before();
   if (p.scale->bad) return;
   const int tile = static_cast<int>(blockIdx.x), ti = tile / p.tiles3, tj = tile - ti * p.tiles3;
   if (p.sym && ti > tj) return;
@@ -622,13 +627,15 @@ __device__ __forceinline__ uint32_t window_byte(uint32_t z4) { return z4 ^ ((z4 
 // Three windows a repetition, every entry read for each: 279 us of the 228.
 __global__ void __launch_bounds__(1024, 1) k_direct_window(const GridArgs p, int shares) {
   extern __shared__ uint32_t words[];        // low halves, then high halves
-  if (p.scale->bad) return;
+  next_kernel_may_start();
   const int t = static_cast<int>(blockIdx.x) / shares, share = static_cast<int>(blockIdx.x) - t * shares;
   const uint32_t b = static_cast<uint32_t>(p.b), mine = min(b, static_cast<uint32_t>(kWindow));
   const uint32_t b4 = 4 * b, mine4 = 4 * mine;
   const uint32_t used = (mine + 31) & ~31u;
   for (uint32_t q = threadIdx.x; q < used; q += 1024) words[q] = words[kWindow + q] = 0;
   __syncthreads();
+  wait_for_kernel_before();
+  if (p.scale->bad) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t* h1 = p.hs + static_cast<size_t>(2 * t) * p.n;
   const uint32_t* h2 = h1 + p.n;
@@ -734,6 +741,7 @@ __global__ void __launch_bounds__(1024, 1) k_direct_window(const GridArgs p, int
 template <bool COPIES>
 __global__ void __launch_bounds__(256) k_direct_finish(const unsigned long long* acc, int copies, float* c, int64_t len,
                                                        int64_t per, const DirectScale* scale, int log2s) {
+  wait_for_kernel_before();
   if constexpr (COPIES) {
     __shared__ unsigned long long part[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1176,15 +1184,12 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
     ProfScope window_scope("k_direct_window", s);
     if ((e = with_smem(k_direct_window, 8 * kWindow)) != cudaSuccess) return e;
     const int shares = std::max(1, 152 / h->d);
-    k_direct_window<<<h->d * shares, 1024, 8 * kWindow, s>>>(g, shares);
-    return cudaGetLastError();
+    return launch_after(k_direct_window, dim3(h->d * shares), 1024, 8 * kWindow, s, g, shares);
   }
   const int tiles = p.tiles1 * p.tiles3, per_tile = kTile / (8 * kGridCols);
   ProfScope grid_scope("k_direct_grid", s);
   const dim3 gg(tiles, per_tile, std::min(h->d, std::max(1, 152 * 2 / (tiles * per_tile))));
-  if (p.sets > 1) k_direct_grid<true><<<gg, 256, 0, s>>>(g);
-  else k_direct_grid<false><<<gg, 256, 0, s>>>(g);
-  return cudaGetLastError();
+  return launch_after(p.sets > 1 ? k_direct_grid<true> : k_direct_grid<false>, gg, 256, 0, s, g);
 }
 
 // `per` buckets share a scale.
@@ -1194,12 +1199,10 @@ cudaError_t launch_finish(const DirectPlan& p, const cms_hashes* h, float* c, in
   const DirectScale* scale = reinterpret_cast<const DirectScale*>(ws + p.off_scale);
   ProfScope prof_scope("k_direct_finish", s);
   if (p.copies > 1)
-    k_direct_finish<true><<<static_cast<unsigned>((len + 31) / 32), 256, 0, s>>>(acc, p.copies, c, len, per, scale,
-                                                                                 direct_scale_log2(p.split));
-  else
-    k_direct_finish<false><<<static_cast<unsigned>(std::min<int64_t>((len + 255) / 256, 152 * 8)), 256, 0, s>>>(
-        acc, 1, c, len, per, scale, direct_scale_log2(p.split));
-  return cudaGetLastError();
+    return launch_after(k_direct_finish<true>, dim3(static_cast<unsigned>((len + 31) / 32)), 256, 0, s, acc, p.copies, c,
+                        len, per, scale, direct_scale_log2(p.split));
+  return launch_after(k_direct_finish<false>, dim3(static_cast<unsigned>(std::min<int64_t>((len + 255) / 256, 152 * 8))),
+                      256, 0, s, acc, 1, c, len, per, scale, direct_scale_log2(p.split));
 }
 
 }  // namespace

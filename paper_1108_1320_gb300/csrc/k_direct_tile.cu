@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_direct_tile(const __grid_consta
   __shared__ volatile int s_err;
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
+  next_kernel_may_start();
   constexpr int kStoring = WIDE ? 256 : 128;
   if (tid == 0) {
     for (int q = 0; q < kSlots; ++q) { mbar_init(&full[q], 1); mbar_init(&freed[q], 1); }
@@ -273,6 +274,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_direct_tile(const __grid_consta
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
+  wait_for_kernel_before();
   const uint32_t tmem = static_cast<uint32_t>(uniform(static_cast<int>(s_tmem)));
   const size_t per_block = static_cast<size_t>((l.need_fold ? 2 : 0) + (l.need_hand ? 4 : 0) + (l.need_merge ? 1 : 0)) * kTileFloats;
   float* work = l.work + blockIdx.x * per_block;
@@ -619,8 +621,7 @@ cudaError_t launch_tiles(const TileArgs& one, const TileLaunch& l, bool wide, bo
   const Kernel k = kernel_of(wide, grid);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(tile_smem_bytes()));
   if (e != cudaSuccess) return e;
-  k<<<blocks, kThreads, tile_smem_bytes(), s>>>(one, l);
-  return cudaGetLastError();
+  return launch_after(k, dim3(blocks), kThreads, tile_smem_bytes(), s, one, l);
 }
 
 }  // namespace dtile

@@ -37,7 +37,10 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_sketch_ws_covariance.json")
 # the fused sketch kernels' profiling names: warp-specialised, lock-step,
 # shared-memory (generic)
 SKETCH_KERNEL_NAMES = ("k_sketch_ws", "k_sketch_fast", "k_sketch_fused")
-# the sources of the dominant kernel's code and launch: the kernel itself,
+# the direct route's kernels (tensor-core tiles of AB added to the buckets)
+DIRECT_KERNEL_NAMES = ("k_direct_pack", "k_direct_tile", "k_direct_grid", "k_direct_window", "k_direct_finish",
+                       "k_pre_transpose", "k_pre_lists", "k_pre_pack")
+# the sources of the transform route's kernel and its launch: the kernel itself,
 # its helpers, the planner that shapes its launch and the table builder whose
 # records it reads (a change to any of them voids the kept DRAM counters)
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1108_1320_gb300", "csrc", f)
@@ -59,6 +62,37 @@ def sketch_flops(d: int, K: int, b: int) -> float:
 
 def total_flops(d: int, K: int, b: int) -> float:
     return sketch_flops(d, K, b) + d * 2.5 * b * math.log2(b)
+
+
+def sketch_roofline(prof: dict, m: int, n: int, b: int, d: int, alu_peak: float) -> dict:
+    """Roofline of one product X^T X's kernels as profiled.  The direct route's
+    kernels together against the tensor cores: the products of the symmetric
+    matrix's distinct entries, m n (n + 1) flops, at the measured BF16 rate.
+    The transform route's fused kernel against the FP32 pipe."""
+    direct = [k for k in DIRECT_KERNEL_NAMES if prof.get(k, {}).get("launches", 0) > 0]
+    if direct:
+        ms = sum(prof[k]["ms"] / prof[k]["launches"] for k in direct)
+        peaks = {}
+        try:
+            with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+                peaks = json.load(f)
+        except (OSError, ValueError):
+            pass
+        peak = peaks.get("bf16_tflops", 1900.0)
+        flops = float(m) * n * (n + 1)
+        achieved = flops / (ms * 1e-3) / 1e12
+        return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                "traffic": None, "kernel": " + ".join(direct), "kernel_ms": ms, "alg_flops_per_launch": flops,
+                "peak_source": "measured cuBLAS BF16 burst" if "bf16_tflops" in peaks else "fallback"}
+    name = next((k for k in SKETCH_KERNEL_NAMES if prof.get(k, {}).get("launches", 0) > 0), "k_sketch_ws")
+    fused = prof.get(name, {"launches": 0, "ms": float("nan")})
+    ms = fused["ms"] / max(fused["launches"], 1)
+    flops = sketch_flops(d, m, b)
+    achieved = flops / (ms * 1e-3) / 1e12
+    return {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s", "frac": achieved / alu_peak,
+            "traffic": load_traffic(), "kernel": name, "kernel_ms": ms, "alg_flops_per_launch": flops,
+            "peak_source": f"derived: SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 flop/FMA x maximum SM clock "
+                           "(FP32 FMA pipe, not tensor)"}
 
 
 def kernel_source_hash() -> str:
@@ -397,24 +431,11 @@ def gpu_arm(args):
     value = job_value(world, args.steps, total_ms)
     launches = int(sum(v["launches"] for v in prof.values()))
 
-    # ---- roofline of the dominant kernel (the fused sketch kernel) --------
-    # the fused sketch kernel this plan ran (each kernel has its own record)
-    fused_name = next((k for k in SKETCH_KERNEL_NAMES if prof.get(k, {}).get("launches", 0) > 0),
-                      "k_sketch_ws")
-    fused = prof.get(fused_name, {"launches": 0, "ms": float("nan")})
-    fused_ms = fused["ms"] / max(fused["launches"], 1)
+    # ---- roofline of the sketch's kernels ----------------------------------
     props = torch.cuda.get_device_properties(dev)
     max_mhz = clocks.get("sm_max_mhz") or 2070.0
     peak_tflops = props.multi_processor_count * FP32_LANES_PER_SM * 2 * max_mhz * 1e6 / 1e12
-    alg_flops = sketch_flops(d, m, b)
-    achieved = alg_flops / (fused_ms * 1e-3) / 1e12
-    traffic = load_traffic()
-    roofline = {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
-                "frac": achieved / peak_tflops, "traffic": traffic,
-                "kernel": fused_name, "kernel_ms": fused_ms,
-                "alg_flops_per_launch": alg_flops,
-                "peak_source": f"derived: {props.multi_processor_count} SMs x {FP32_LANES_PER_SM} FP32 "
-                               f"lanes x 2 flop/FMA x {max_mhz:.0f} MHz (FP32 FMA pipe, not tensor)"}
+    roofline = sketch_roofline(prof, m, n, b, d, peak_tflops)
     ms_step = total_ms / args.steps
     ab_bytes = 2 * m * n * 4                       # A and B each read once (same bytes here)
     peaks = {}
@@ -428,11 +449,11 @@ def gpu_arm(args):
     extra = {
         "ab_gbs": ab_gbs, "ab_hbm_frac": ab_gbs / hbm,
         "hbm_peak_gbs": hbm, "hbm_peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
-        "roofline_time_ms": max(ab_bytes / (hbm * 1e9), total_flops(d, m, b) / (peak_tflops * 1e12)) * 1e3,
+        "roofline_time_ms": max(ab_bytes / (hbm * 1e9), roofline["alg_flops_per_launch"] / (roofline["peak"] * 1e12)) * 1e3,
         "kernel_ms": {k: v["ms"] / max(v["launches"], 1) for k, v in prof.items()},
     }
     extra["step_frac_of_roofline"] = extra["roofline_time_ms"] / ms_step
-    sketch_kernels = ("k_twiddle_table", "k_frontend_twiddles", *SKETCH_KERNEL_NAMES, "k_rows_inverse",
+    sketch_kernels = (*DIRECT_KERNEL_NAMES, "k_twiddle_table", "k_frontend_twiddles", *SKETCH_KERNEL_NAMES, "k_rows_inverse",
                       "k_cols_inverse")
     extra["sketch_only_ms"] = sum(prof[k]["ms"] for k in sketch_kernels if k in prof) / args.steps
 
@@ -603,14 +624,11 @@ def gpu_arm_kshard(args):
     total_ms = reduce_max(sum(a.elapsed_time(z) for a, z in zip(starts, stops)), dist if world > 1 else None,
                           dev)
     value = args.steps / (total_ms / 1e3)
-    fused_name = next((k for k in SKETCH_KERNEL_NAMES if prof.get(k, {}).get("launches", 0) > 0),
-                      "k_sketch_ws")
-    fused = prof.get(fused_name, {"launches": 0, "ms": float("nan")})
-    fused_ms = fused["ms"] / max(fused["launches"], 1)
     props = torch.cuda.get_device_properties(dev)
     max_mhz = clocks.get("sm_max_mhz") or 2070.0
     peak = props.multi_processor_count * FP32_LANES_PER_SM * 2 * max_mhz * 1e6 / 1e12
-    achieved = sketch_flops(d, k1 - k0, b) / (fused_ms * 1e-3) / 1e12
+    roofline = sketch_roofline(prof, k1 - k0, n, b, d, peak)
+    roofline["note"] = "this rank's share of the inner indices"
     # end to end: each rank's rows of X copied from pinned host memory, the
     # merged sketch read back, inside the timed region
     c_host = torch.empty((d, b), dtype=torch.float32).pin_memory()
@@ -642,9 +660,7 @@ def gpu_arm_kshard(args):
                    "l2": f"flushed between steps ({FLUSH_BYTES >> 20} MiB write, outside the step events)",
                    "parallelism": f"one product over {world} GPUs: inner indices split in contiguous ranges, "
                                   f"partial sketches all-gathered and merged in rank order"},
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak, "traffic": None, "kernel": fused_name, "kernel_ms": fused_ms,
-                     "note": "this rank's share of the inner indices"},
+        "roofline": roofline,
         "clocks": clocks,
         "e2e": {"value": e2e_steps / (e2e_ms / 1e3), "unit": "products/s",
                 "h2d_bytes_per_step": (k1 - k0) * n * 4, "d2h_bytes_per_step": d * b * 4, "steps": e2e_steps},
@@ -814,7 +830,8 @@ def sparse_context(cms, torch, dev):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     K = 256 * 8
-    flops = d * K * (5.0 * b * math.log2(b) + 4.0 * b) + d * 2.5 * b * math.log2(b)
+    # (every inner index is cheaper term by term than by transforms here)
+    flops = 2.0 * d * K * 32 * 32
     # sparse-k hybrid (default split): every outer product here has 1024
     # terms, so all 2048 inner indices are sketched directly
     ch = torch.empty_like(c)
@@ -836,12 +853,12 @@ def sparse_context(cms, torch, dev):
             "alg_tflops": flops / (ms * 1e-3) / 1e12, "host_ms_per_call": host_ms,
             "c_rel_l2_vs_exact": float(err.max()),
             "c_max_abs_err_vs_exact": float((c.double() - ch.double()).abs().max()),
-            "note": "FFT route, CUDA events (the call does not wait for the device); error against the "
-                    "direct route's exact sketch of the integer product",
+            "note": "default call, inner indices with few terms sketched term by term in integer sums; CUDA events "
+                    "(the call does not wait for the device); error against the hybrid call's FP64 sums",
             "hybrid": {"ms_per_product": ms_h, "products_per_s": 1e3 / ms_h,
-                       "direct_terms": d * K * 32 * 32, "rounded_c_equal_to_fft_route": same,
+                       "direct_terms": d * K * 32 * 32, "rounded_c_equal_to_default_call": same,
                        "note": "sparse-k hybrid, default split (all inner indices direct, FP64 scatter); "
-                               "not an FFT-route roofline number"}}
+                               "no transforms"}}
 
 
 def large_context(cms, torch, dev):
@@ -876,7 +893,8 @@ def large_context(cms, torch, dev):
     torch.cuda.synchronize()
     cms.check_async()
     ms = e0.elapsed_time(e1) / reps
-    flops = total_flops(d, m, b)
+    # direct route: the products of the symmetric matrix's distinct entries
+    flops = float(m) * n * (n + 1) if "k_direct_tile" in kernels else total_flops(d, m, b)
     pe = cms.decode(c, h, perm.to(torch.int64))
     out = {"workload": "large covariance X 16384x32768 BF16, 4096 pairs rho=0.3, b=2^20, d=7",
            "ms_per_product": ms, "products_per_s": 1e3 / ms, "alg_tflops": flops / (ms * 1e-3) / 1e12,
@@ -973,7 +991,8 @@ def batched_context(cms, torch, dev, n_hi: int = 8192):
         cq = batch.c[q].double()
         errs.append(float((torch.linalg.norm(cq - c64, dim=1) / torch.linalg.norm(c64, dim=1)).max()))
         del Xd, ws, c64
-    flops = sum(3 * sp.m * (5.0 * 16 * sp.n * math.log2(16 * sp.n) + 4.0 * 16 * sp.n) for sp in specs)
+    # the products of the symmetric matrices' distinct entries (direct route)
+    flops = sum(float(sp.m) * sp.n * (sp.n + 1) for sp in specs)
     batch.free()
     for _, _, h in items:
         h.free()

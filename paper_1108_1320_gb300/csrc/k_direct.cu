@@ -51,6 +51,7 @@ using namespace wfft;
 using namespace dtile;
 
 constexpr double kFixedSeconds = 36e-6;   // launches of a single product
+constexpr double kMargin = 4e-6;
 constexpr int kWindow = 28672;             // buckets in shared memory (224 KB)
 constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
 constexpr int kMinExp = -100;           // scales stay representable
@@ -826,6 +827,7 @@ void choose_tiles(DirectPlan& p, bool sym, int reps, double entries, double adds
     const int units = tile_units(p.tiles1, p.tiles3, wide != 0, sym);
     for (int s = 1; s <= std::min(p.nsb, 64); ++s) {
       const int per = (p.nsb + s - 1) / s, real = (p.nsb + per - 1) / per;
+      if (s > 1 && static_cast<int64_t>(units) * s * reps > 2 * sms) break;   // every SM has work
       if (real != s && s > 1) continue;
       const double blocks = static_cast<double>(units) * real * reps;
       const double chunk = wide ? 0.85e-6 : (p.split ? 0.43e-6 : 0.55e-6);
@@ -984,6 +986,9 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
   // under 64 inner indices the packing and the padding to a superblock show;
   // the launches of a batch are shared by its instances
   if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535 || !tile_kernel_usable()) return false;
+  // (no plan for calls that the launches alone decide: planning is host time)
+  const double transform = transform_seconds(plan, n1, n2, n3, batch);
+  if (!batch && transform <= kFixedSeconds + kMargin + 3e-6) return false;
   *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1, batch);
   double best = out->seconds - (batch ? kFixedSeconds : 0.0);
   if (!batch) {
@@ -997,7 +1002,7 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
     }
   }
   // a margin for the estimates' error where both are mostly launches
-  return best + (batch ? 0.0 : 4e-6) < transform_seconds(plan, n1, n2, n3, batch);
+  return best + (batch ? 0.0 : kMargin) < transform;
 }
 
 // The masked sums of FINDSIGNIFICANTENTRIES in one pass: an entry is added to

@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_direct_tile(const __grid_consta
   __shared__ volatile int s_err;
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
-  next_kernel_may_start();
+  if constexpr (GRID) next_kernel_may_start();
   constexpr int kStoring = WIDE ? 256 : 128;
   if (tid == 0) {
     for (int q = 0; q < kSlots; ++q) { mbar_init(&full[q], 1); mbar_init(&freed[q], 1); }
@@ -621,7 +621,12 @@ cudaError_t launch_tiles(const TileArgs& one, const TileLaunch& l, bool wide, bo
   const Kernel k = kernel_of(wide, grid);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(tile_smem_bytes()));
   if (e != cudaSuccess) return e;
-  return launch_after(k, dim3(blocks), kThreads, tile_smem_bytes(), s, one, l);
+  // stored entries: small products, set up while the packing ends.  Fused: blocks
+  // placed one by one as the packing leaves the SMs cost more than that saves
+  // (16384 x 32768 BF16: 51.0 -> 56.3 ms).
+  if (grid) return launch_after(k, dim3(blocks), kThreads, tile_smem_bytes(), s, one, l);
+  k<<<blocks, kThreads, tile_smem_bytes(), s>>>(one, l);
+  return cudaGetLastError();
 }
 
 }  // namespace dtile

@@ -111,7 +111,9 @@ inline size_t tile_work_bytes(int blocks, bool fold, bool hand, bool merge) {
 // one is set up (its blocks' barriers, tensor memory, zeroed words) while the
 // last blocks of the one before finish, and waits for all of its results (256 x
 // 256 x 256 in FP64, b = 1024: 37.9 -> 32.3 us a call).  Every block waits, so
-// that a kernel's end implies the end of those before it.
+// that a kernel's end implies the end of those before it.  What the kernels
+// before wrote is read by plain or L2 loads: the read-only path (__ldg) is for
+// the hash tables, which are complete before the first of them starts.
 __device__ __forceinline__ void next_kernel_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_kernel_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(256) k_direct_finish(const unsigned long long*
     unsigned long long v = 0;
     if (q < len) {
 #pragma unroll 4
-      for (int r = warp; r < copies; r += 8) v += __ldg(acc + r * len + q);
+      for (int r = warp; r < copies; r += 8) v += __ldcg(acc + r * len + q);
     }
     part[warp][lane] = v;
     __syncthreads();

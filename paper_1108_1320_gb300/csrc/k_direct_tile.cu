@@ -484,13 +484,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_direct_tile(const __grid_consta
 #pragma unroll
       for (int q = 0; q < kTile; ++q) acc[q] = 0.f;
       {
+        // (plain loads: a programmatic launch may run while the packing still
+        // writes the exponents, which the read-only path does not allow)
         const size_t rb = static_cast<size_t>(u.rep) * p.rep_blocks + u.sb0;
         const int2* ea = p.ea + rb + static_cast<size_t>(u.ti) * p.nsb;
         const int2* eb = p.eb + rb + static_cast<size_t>(max(tj, 0)) * p.nsb;
         for (int lc = 0; lc < mine; ++lc) {
           const int ch = WIDE ? lc : 2 * lc + half;
           const int sb = split ? ch >> 1 : ch;
-          const int de = __ldg(&ea[sb].x) - sc.emax[0] + __ldg(&eb[sb].x) - sc.emax[1];
+          const int de = ea[sb].x - sc.emax[0] + eb[sb].x - sc.emax[1];
           const float f = de < -126 ? 0.f : pow2f(min(de, 0));
           const int buf = split ? 0 : lc & 1;
           const int a = WIDE ? buf : half * 2 + buf;

@@ -430,8 +430,8 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
     }
     b->total_tasks += b->direct_batch.units;
   }
-  // counter reset + persistent kernel, packing + tiles, batched inverse (rows, columns)
-  int launches = (ntr > 0 ? 2 : 0) + (ntr < count ? 2 : 0) + 2;
+  // counter reset + persistent kernel, (balance +) packing + tiles, batched inverse (rows, columns)
+  int launches = (ntr > 0 ? 2 : 0) + (ntr < count ? 2 : 0) + 2 + (b->direct_batch.balanced + 65534) / 65535;
   for (int i : b->order) launches += b->plans[i].fast ? 0 : 1;
   b->launches = launches;
   *out = b;

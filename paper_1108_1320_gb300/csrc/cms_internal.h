@@ -329,7 +329,7 @@ struct DirectPlan {
   bool alias_operands = false;
   int sms = 0;
   size_t zero_bytes = 0, acc_bytes = 0, off_work = 0, off_grid = 0;
-  size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_pa = 0, off_pb = 0;
+  size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_bal = 0, off_pa = 0, off_pb = 0;
   size_t ws_bytes = 0;
 };
 // Pre-sketched operands: one direct product of b rows per repetition.
@@ -400,7 +400,8 @@ struct DirectBatch {
   int count = 0, pack_blocks = 0, tile_blocks = 0, units = 0;
   bool need_fold = false;
   uint32_t pack_smem = 0;
-  size_t o_tile = 0, o_ps = 0, o_ts = 0, o_work = 0;
+  int balanced = 0;         // products of two operands (their inner indices are balanced)
+  size_t o_tile = 0, o_ps = 0, o_ts = 0, o_bal = 0, o_work = 0;
 };
 size_t direct_batch_bytes(int count, int sms);
 cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, int sms, void* d_buf, DirectBatch* out,

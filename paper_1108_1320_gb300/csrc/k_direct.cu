@@ -38,6 +38,7 @@
 // 32-byte sector each), then shared memory, which the operands' copies and the
 // tensor cores' reads of them share (about 110 bytes per clock and SM).
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cuda_fp16.h>
 
@@ -79,6 +80,7 @@ struct PackSide {
   const void* X;       // rows of ld elements, inner index k
   int64_t ld;
   int64_t n;           // columns used
+  const int8_t* bal;   // [k]: power of two that multiplies row k (A's; B's is the inverse), NULL: none
   int tiles;           // 0: the side is the other one's bytes
   uint8_t* out;        // [tile][stage] images
   int2* blocks;        // [tile][superblock]: exponent, sum of squares of the scaled values
@@ -151,6 +153,98 @@ __device__ void direct_scale(const PackArgs& p, float* fsh, int* ish) {
   *p.ticket = 0;
 }
 
+// ---- inner indices brought to one magnitude ----
+// Blocks of 128 inner indices share an exponent, and all of AB one grid of the
+// integer sums.  Both are fine for a_k b_k of any size, but not for a large a_k
+// with a small b_k beside a small a_k with a large b_k: columns of A scaled by
+// 2^-20 .. 2^20 and rows of B by the inverse were off by 0.36 in relative L2
+// (2.6e-7 through the spectra).  So the larger of the two lends half of the
+// difference of their exponents to the smaller: a_k 2^g and b_k 2^-g, exact.
+// X^T X needs none (a_k and b_k are the same).  The kernel also zeroes the
+// call's sums, so that it takes the place of a memset, not one more launch: a
+// few warps per inner index, bound by reading the operands once more; the packing
+// reads them at the same time and waits before it uses the balance (1777 x 1003,
+// 1203 inner indices, FP32: 68 us a call without, 72 with it, 79 one after the
+// other; 256 x 256 x 256 in FP64 31 us either way).
+struct BalanceSide {
+  const void* X;
+  int64_t ld;
+  int64_t n;
+};
+struct BalanceArgs {
+  BalanceSide side[2];
+  int64_t K;
+  int dt;
+  int warps;           // per inner index: 1, 2, 4 or 8
+  int8_t* bal;
+  uint4* zero;         // words of 16 bytes to set to zero
+  int64_t words;
+};
+
+// Largest magnitude of values x, x + step, ... of a row, as FP32 bits.
+template <typename T>
+__device__ __forceinline__ uint32_t row_max(const BalanceSide& s, int64_t k, int x, int step) {
+  const T* row = static_cast<const T*>(s.X) + k * s.ld;
+  uint32_t m = 0;
+#pragma unroll 8
+  for (int64_t i = x; i < s.n; i += step) m = max(m, __float_as_uint(load_val(row + i)) & 0x7FFFFFFFu);
+  return m;
+}
+
+// `warps` of the block's 8 take an inner index (the same count of turns in
+// every warp of the block: they meet at barriers).
+template <typename T>
+__device__ __forceinline__ void balance_rows(const BalanceArgs& p, int64_t block, int64_t blocks) {
+  __shared__ uint32_t part[2][8];
+  const int warp = threadIdx.x >> 5, per = 8 / p.warps, row = warp / p.warps;
+  const int x = threadIdx.x - row * p.warps * 32, step = 32 * p.warps;
+  for (int64_t k0 = block * per; k0 < p.K; k0 += blocks * per) {
+    const int64_t k = k0 + row;
+    uint32_t m[2] = {0, 0};
+    if (k < p.K) {
+      m[0] = row_max<T>(p.side[0], k, x, step);
+      m[1] = row_max<T>(p.side[1], k, x, step);
+    }
+    m[0] = __reduce_max_sync(0xFFFFFFFFu, m[0]);
+    m[1] = __reduce_max_sync(0xFFFFFFFFu, m[1]);
+    if (p.warps > 1) {
+      __syncthreads();
+      if ((threadIdx.x & 31) == 0) { part[0][warp] = m[0]; part[1][warp] = m[1]; }
+      __syncthreads();
+      if (x == 0)
+        for (int w = 1; w < p.warps; ++w) { m[0] = max(m[0], part[0][warp + w]); m[1] = max(m[1], part[1][warp + w]); }
+    }
+    if (x == 0 && k < p.K) {
+      // none for a row of zeros, or with an infinity or a NaN; rounded to zero:
+      // a difference of one is left alone
+      const bool none = m[0] == 0 || m[1] == 0 || max(m[0], m[1]) >= 0x7F800000u;
+      const int half = (static_cast<int>(m[1] >> 23) - static_cast<int>(m[0] >> 23)) / 2;
+      p.bal[k] = static_cast<int8_t>(none ? 0 : min(max(half, -126), 126));
+    }
+  }
+}
+__device__ __forceinline__ void balance_task(const BalanceArgs& p, int64_t block, int64_t blocks) {
+  if (p.dt == CMS_BF16) balance_rows<__nv_bfloat16>(p, block, blocks);
+  else if (p.dt == CMS_F64) balance_rows<double>(p, block, blocks);
+  else balance_rows<float>(p, block, blocks);
+}
+
+__global__ void __launch_bounds__(256) k_direct_balance(const BalanceArgs p) {
+  next_kernel_may_start();
+  for (int64_t q = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; q < p.words;
+       q += static_cast<int64_t>(gridDim.x) * 256)
+    p.zero[q] = make_uint4(0, 0, 0, 0);
+  balance_task(p, blockIdx.x, gridDim.x);
+}
+
+__global__ void __launch_bounds__(256) k_direct_balance_batched(const BalanceArgs* __restrict__ args) {
+  const BalanceArgs p = args[blockIdx.y];
+  balance_task(p, blockIdx.x, gridDim.x);
+}
+
+// Multiplies the values of inner index k by their power of two (side 0: A).
+__device__ __forceinline__ float balanced(float v, int g, int side) { return v * pow2f(side ? -g : g); }
+
 template <typename T, bool SPLIT>
 __device__ __forceinline__ void pack_block(const PackArgs& p, int sb, int tile, int sd, uint8_t* img, float* fsh,
                                            int* ish) {
@@ -170,6 +264,26 @@ __device__ __forceinline__ void pack_block(const PackArgs& p, int sb, int tile, 
   } else {
 #pragma unroll
     for (int q = 0; q < 64; ++q) x[q] = q < kn ? load_val(X + (k0 + q) * s.ld) : 0.f;
+  }
+  // (the operands are read while the kernel before, which finds the balance
+  // and zeroes the sums, still runs)
+  wait_for_kernel_before();
+  if (s.bal != nullptr) {
+    // (64 bytes of the same 64 inner indices for every row)
+    if (kn == 64) {
+      uint32_t w[16];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(s.bal + k0) + q);
+        w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+      }
+#pragma unroll
+      for (int q = 0; q < 64; ++q) x[q] = balanced(x[q], static_cast<int8_t>(w[q / 4] >> (q % 4 * 8)), sd);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 64; ++q)
+        if (q < kn) x[q] = balanced(x[q], s.bal[k0 + q], sd);
+    }
   }
   uint32_t m = 0;
 #pragma unroll
@@ -293,6 +407,7 @@ struct PreArgs {
   const void* X[2];
   int64_t ld[2];
   int64_t n[2];
+  const int8_t* bal;      // powers of two of the inner indices, NULL: none
   int alias;
   int64_t K;
   int nsb, d;
@@ -317,12 +432,15 @@ __global__ void __launch_bounds__(256) k_pre_transpose(const PreArgs p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 32 + lane;
   const int64_t k0 = static_cast<int64_t>(blockIdx.y) * kSuper;
+  wait_for_kernel_before();
   if (static_cast<int64_t>(blockIdx.x) * 32 >= p.n[side]) return;
   const T* X = static_cast<const T*>(p.X[side]);
 #pragma unroll
   for (int q = 0; q < kSuper / 8; ++q) {
     const int k = q * 8 + warp;
-    sh[k][lane] = i < p.n[side] && k0 + k < p.K ? load_val(X + (k0 + k) * p.ld[side] + i) : 0.f;
+    float v = i < p.n[side] && k0 + k < p.K ? load_val(X + (k0 + k) * p.ld[side] + i) : 0.f;
+    if (p.bal != nullptr && k0 + k < p.K) v = balanced(v, p.bal[k0 + k], side);
+    sh[k][lane] = v;
   }
   __syncthreads();
 #pragma unroll
@@ -903,6 +1021,8 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   p.off_work = o;   o = al1k(o + (batch ? 0 : tile_work_bytes(p.blocks, p.need_fold, p.need_hand, p.need_merge)));
   p.off_scale = o;  o = al1k(o + sizeof(DirectScale));
   p.off_blocks = o; o = al1k(o + static_cast<size_t>(p.tiles1 + t3) * p.nsb * sizeof(int2));
+  p.off_bal = o;
+  if (!alias) o = al1k(o + static_cast<size_t>(n2));
   p.off_pa = o;     o = al1k(o + static_cast<size_t>(p.tiles1) * images * kStageBytes);
   p.off_pb = alias ? p.off_pa : o;
   if (!alias) o = al1k(o + static_cast<size_t>(p.tiles3) * images * kStageBytes);
@@ -975,6 +1095,8 @@ PrePlan make_pre_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, b
   q.off_ent = o;    o = al1k(o + static_cast<size_t>(2 * h->d) * h->n * 4);
   q.off_start = o;  o = al1k(o + static_cast<size_t>(2 * h->d) * (rows + 1) * 4);
   q.off_vhs = o;    o = al1k(o + static_cast<size_t>(2) * rows * 4);
+  p.off_bal = o;
+  if (!alias) o = al1k(o + static_cast<size_t>(n2));
   q.off_slab = o;   o = al1k(o + static_cast<size_t>(p.nsb) * (alias ? n1 : n1 + n3) * kSuper * 4);
   p.ws_bytes = o;
   q.usable = true;
@@ -1021,8 +1143,9 @@ PackArgs pack_args(const DirectPlan& p, const void* A, int64_t lda, const void* 
                    int64_t n1, int64_t n2, int64_t n3, int dt, char* ws) {
   int2* blocks = reinterpret_cast<int2*>(ws + p.off_blocks);
   PackArgs a{};
-  a.side[0] = PackSide{A, lda, n1, p.tiles1, reinterpret_cast<uint8_t*>(ws + p.off_pa), blocks};
-  a.side[1] = PackSide{B, ldb, n3, p.alias ? 0 : p.tiles3, reinterpret_cast<uint8_t*>(ws + p.off_pb),
+  const int8_t* bal = p.alias ? nullptr : reinterpret_cast<const int8_t*>(ws + p.off_bal);
+  a.side[0] = PackSide{A, lda, n1, bal, p.tiles1, reinterpret_cast<uint8_t*>(ws + p.off_pa), blocks};
+  a.side[1] = PackSide{B, ldb, n3, bal, p.alias ? 0 : p.tiles3, reinterpret_cast<uint8_t*>(ws + p.off_pb),
                        blocks + static_cast<size_t>(p.tiles1) * p.nsb};
   a.K = n2;
   a.nsb = p.nsb;
@@ -1064,6 +1187,33 @@ TileArgs tile_args(const DirectPlan& p, const cms_hashes* h, int64_t n1, int64_t
   return a;
 }
 
+BalanceArgs balance_args(const DirectPlan& p, const void* A, int64_t lda, const void* B, int64_t ldb, int64_t n1,
+                         int64_t n2, int64_t n3, int dt, char* ws) {
+  BalanceArgs a{};
+  a.side[0] = BalanceSide{A, lda, n1};
+  a.side[1] = BalanceSide{B, ldb, n3};
+  a.K = n2;
+  a.dt = dt;
+  // warps on every SM, and at least four loads a lane
+  a.warps = 1;
+  while (a.warps < 8 && n2 * a.warps < 152 * 32 && std::max(n1, n3) >= 256 * a.warps) a.warps *= 2;
+  a.bal = reinterpret_cast<int8_t*>(ws + p.off_bal);
+  return a;
+}
+
+// Zeroed sums and tickets, and the inner indices' powers of two where A and B differ.
+cudaError_t launch_start(const DirectPlan& p, bool alias, const void* A, int64_t lda, const void* B, int64_t ldb,
+                         int64_t n1, int64_t n2, int64_t n3, int dt, char* ws, cudaStream_t s) {
+  if (alias) return cudaMemsetAsync(ws + p.off_acc, 0, p.zero_bytes, s);
+  BalanceArgs a = balance_args(p, A, lda, B, ldb, n1, n2, n3, dt, ws);
+  a.zero = reinterpret_cast<uint4*>(ws + p.off_acc);
+  a.words = static_cast<int64_t>(p.zero_bytes / 16);
+  ProfScope prof_scope("k_direct_balance", s);
+  const int64_t work = std::max((n2 * a.warps + 7) / 8, (a.words + 1023) / 1024);
+  k_direct_balance<<<static_cast<unsigned>(std::min<int64_t>(work, 152 * 8)), 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
 int pack_blocks(const DirectPlan& p) { return p.nsb * (p.tiles1 + (p.alias ? 0 : p.tiles3)); }
 
 template <typename F>
@@ -1077,7 +1227,7 @@ size_t direct_batch_bytes(int count, int sms) {
   auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
   // arguments, then the tile kernel's words (folds and tiles handed over)
   return al(count * sizeof(PackArgs)) + al(count * sizeof(TileArgs)) + 2 * al((count + 1) * sizeof(int)) +
-         tile_work_bytes(sms, true, true, false);
+         al(count * sizeof(BalanceArgs)) + tile_work_bytes(sms, true, true, false);
 }
 
 cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, int sms, void* d_buf, DirectBatch* out,
@@ -1090,7 +1240,9 @@ cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, int sms, vo
   out->o_tile = al(count * sizeof(PackArgs));
   out->o_ps = out->o_tile + al(count * sizeof(TileArgs));
   out->o_ts = out->o_ps + al((count + 1) * sizeof(int));
-  out->o_work = out->o_ts + al((count + 1) * sizeof(int));
+  out->o_bal = out->o_ts + al((count + 1) * sizeof(int));
+  out->o_work = out->o_bal + al(count * sizeof(BalanceArgs));
+  out->balanced = 0;
   int* ps = reinterpret_cast<int*>(host.data() + out->o_ps);
   int* ts = reinterpret_cast<int*>(host.data() + out->o_ts);
   int np = 0, nt = 0;
@@ -1100,6 +1252,9 @@ cudaError_t build_direct_batch(const std::vector<DirectSpec>& specs, int sms, vo
     reinterpret_cast<PackArgs*>(host.data())[q] =
         pack_args(d.plan, d.A, d.lda, d.B, d.ldb, d.n1, d.n2, d.n3, d.dt, d.ws);
     reinterpret_cast<TileArgs*>(host.data() + out->o_tile)[q] = tile_args(d.plan, d.h, d.n1, d.n2, d.n3, d.ws);
+    if (!d.plan.alias)
+      reinterpret_cast<BalanceArgs*>(host.data() + out->o_bal)[out->balanced++] =
+          balance_args(d.plan, d.A, d.lda, d.B, d.ldb, d.n1, d.n2, d.n3, d.dt, d.ws);
     ps[q] = np;
     ts[q] = nt;
     np += pack_blocks(d.plan);
@@ -1124,6 +1279,13 @@ cudaError_t launch_direct_batched(const DirectBatch& d, cudaStream_t s) {
   if (d.count == 0) return cudaSuccess;
   const char* base = static_cast<const char*>(d.buf);
   cudaError_t e;
+  for (int q = 0; q < d.balanced; q += 65535) {
+    ProfScope prof_scope("k_direct_balance_batched", s);
+    const int blocks = std::min(std::max(152 * 8 / d.balanced, 8), 152 * 2);   // of a product
+    k_direct_balance_batched<<<dim3(blocks, std::min(d.balanced - q, 65535)), 256, 0, s>>>(
+        reinterpret_cast<const BalanceArgs*>(base + d.o_bal) + q);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   {
     ProfScope prof_scope("k_direct_pack_batched", s);
     if ((e = with_smem(k_direct_pack_batched, d.pack_smem)) != cudaSuccess) return e;
@@ -1159,14 +1321,20 @@ cudaError_t launch_product_tiles(const DirectPlan& p, const TileArgs& a, char* w
 // Zeroed sums, packing, tiles.
 cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A, int64_t lda, const void* B,
                         int64_t ldb, int64_t n1, int64_t n2, int64_t n3, int dt, char* ws, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(ws + p.off_acc, 0, p.zero_bytes, s);
+  cudaError_t e = launch_start(p, p.alias, A, lda, B, ldb, n1, n2, n3, dt, ws, s);
   if (e != cudaSuccess) return e;
   {
     ProfScope prof_scope("k_direct_pack", s);
     const uint32_t smem = (p.split ? 4 : 2) * kStageBytes;
     if ((e = with_smem(k_direct_pack, smem)) != cudaSuccess) return e;
-    k_direct_pack<<<pack_blocks(p), 256, smem, s>>>(pack_args(p, A, lda, B, ldb, n1, n2, n3, dt, ws));
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const PackArgs a = pack_args(p, A, lda, B, ldb, n1, n2, n3, dt, ws);
+    if (p.alias) {
+      k_direct_pack<<<pack_blocks(p), 256, smem, s>>>(a);
+      e = cudaGetLastError();
+    } else {
+      e = launch_after(k_direct_pack, dim3(pack_blocks(p)), 256, smem, s, a);
+    }
+    if (e != cudaSuccess) return e;
   }
   const TileArgs a = tile_args(p, h, n1, n2, n3, ws);
   e = launch_product_tiles(p, a, ws, s);
@@ -1224,6 +1392,7 @@ cudaError_t launch_pre(const DirectPlan& chosen, const cms_hashes* h, const void
   a.X[0] = A; a.X[1] = B;
   a.ld[0] = lda; a.ld[1] = ldb;
   a.n[0] = n1; a.n[1] = n3;
+  a.bal = alias ? nullptr : reinterpret_cast<const int8_t*>(ws + p.off_bal);
   a.alias = alias ? 1 : 0;
   a.K = n2;
   a.nsb = p.nsb;
@@ -1241,15 +1410,21 @@ cudaError_t launch_pre(const DirectPlan& chosen, const cms_hashes* h, const void
   a.pack = pack_args(p, nullptr, 0, nullptr, 0, rows, n2, rows, CMS_F32, ws);
   a.rep_images = q.rep_images;
   a.rep_blocks = q.rep_blocks;
-  cudaError_t e = cudaMemsetAsync(ws + p.off_acc, 0, p.zero_bytes, s);
+  cudaError_t e = launch_start(p, alias, A, lda, B, ldb, n1, n2, n3, dt, ws, s);
   if (e != cudaSuccess) return e;
   {
     ProfScope prof_scope("k_pre_transpose", s);
     const dim3 grid(static_cast<unsigned>((std::max(n1, n3) + 31) / 32), p.nsb, alias ? 1 : 2);
-    if (dt == CMS_BF16) k_pre_transpose<__nv_bfloat16><<<grid, 256, 0, s>>>(a);
-    else if (dt == CMS_F64) k_pre_transpose<double><<<grid, 256, 0, s>>>(a);
-    else k_pre_transpose<float><<<grid, 256, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    void (*const kern)(const PreArgs) = dt == CMS_BF16  ? k_pre_transpose<__nv_bfloat16>
+                                        : dt == CMS_F64 ? k_pre_transpose<double>
+                                                        : k_pre_transpose<float>;
+    if (alias) {
+      kern<<<grid, 256, 0, s>>>(a);
+      e = cudaGetLastError();
+    } else {
+      e = launch_after(kern, grid, 256, 0, s, a);
+    }
+    if (e != cudaSuccess) return e;
   }
   {
     ProfScope prof_scope("k_pre_lists", s);

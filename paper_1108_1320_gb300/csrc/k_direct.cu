@@ -55,7 +55,7 @@ constexpr double kFixedSeconds = 36e-6;   // launches of a single product
 constexpr double kMargin = 4e-6;
 constexpr int kWindow = 28672;             // buckets in shared memory (224 KB)
 constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
-constexpr int kMinExp = -100;           // scales stay representable
+constexpr int kMinExp = -126;           // smallest normal values: scales stay representable
 
 
 __device__ __forceinline__ float load_val(const float* p) { return __ldg(p); }

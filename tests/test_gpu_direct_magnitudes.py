@@ -113,3 +113,17 @@ def test_significant_entries_of_opposite_scales(cms):
     ij, count = cms.find_significant(a.T, b, h, 1000.0, 2)
     assert count == 1 and ij.cpu().numpy().tolist() == [[17, 121]]
     h.free()
+
+
+@pytest.mark.parametrize("n1,n2,n3,b", [(300, 512, 260, 16384), (6000, 400, 5000, 1536)])
+@pytest.mark.parametrize("e", [-118, -126])
+def test_smallest_normal_values_times_large_ones(cms, e, n1, n2, n3, b):
+    # AB is of ordinary size although A is at the end of FP32's range
+    at, At = put(np.exp2(e) * (1 + W.rng(3).random((n2, n1))), "f32")
+    bd, B = put(np.exp2(100) * W.gaussian(n2, n3, 4), "f32")
+    for A, X, Ad, Xd in [(at.T, bd, At.T, B), (bd.T, at, B.T, At)]:
+        h = cms.make_hashes(5, max(n1, n3), b, 2)
+        c, kernels = run(cms, A, X, h)
+        assert "k_direct_tile" in kernels
+        assert worst(c, O.sketch_definition(Ad, Xd, O.make_tables(5, max(n1, n3), b, 2))) < TOL
+        h.free()

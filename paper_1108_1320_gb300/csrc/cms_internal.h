@@ -325,6 +325,7 @@ struct DirectPlan {
   bool window = false;      // ... with a window of the buckets in shared memory
   int sets = 1;             // sums of different entries (1 + 2 L: FINDSIGNIFICANTENTRIES)
   double seconds = 0.0;     // estimate
+  bool beyond_l2 = false;   // packed operands larger than L2 holds
   bool pre = false;         // of pre-sketched operands (PrePlan)
   bool alias_operands = false;
   int sms = 0;

@@ -53,6 +53,7 @@ using namespace dtile;
 
 constexpr double kFixedSeconds = 36e-6;   // launches of a single product
 constexpr double kMargin = 4e-6;
+constexpr double kInL2 = 110e6;           // bytes of packed operands that stay in L2
 constexpr int kWindow = 28672;             // buckets in shared memory (224 KB)
 constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
 constexpr int kMinExp = -126;           // smallest normal values: scales stay representable
@@ -932,14 +933,20 @@ namespace {
 //         about 6 us more; entries beyond L2's reach are not worth storing),
 //         or added by the tile kernel while it multiplies on.
 // Times: a chunk of 64 (FP16 terms) or 128 (BF16) inner indices of a tile
-// 0.40 us (BF16 alone on its operands 0.53: the copies from L2 bound it).
+// 0.40 us (BF16 alone on its operands 0.53: the copies from L2 bound it), and
+// more where the packed operands (`packed` bytes) do not stay in L2: 2.0 times as
+// much in units of two tiles and 2.45 in units of one (BF16 1.7 and 2.2; fitted,
+// as the line at 110 MB of the 129, to 320 calls of n = 32 .. 17000 and 64 to 2 M
+// inner indices by either route; 5022 x 19702 FP32, b = 3125, d = 1: 0.96 ms
+// estimated without it, 1.76 ms taken, 1.01 by the spectra).  The shape of the
+// units is chosen without it.
 void choose_tiles(DirectPlan& p, bool sym, int reps, double entries, double adds, double full_rate, double sm_rate,
-                  double window, bool may_grid, bool may_fuse, bool shared, int sms) {
+                  double window, double packed, bool may_grid, bool may_fuse, bool shared, int sms) {
   // stored entries added: in L2, or with a share of the buckets in shared memory
   // (2.7 us less per million of its additions, 4 us more)
   p.window = entries * adds * window >= 3e6;
   const double added = entries * reps * adds / full_rate * (p.window ? 1.0 - 0.65 * window : 1.0) + (p.window ? 4e-6 : 0.0);
-  double best = 1e30;
+  double best = 1e30, best_mma = 0.0;
   for (int wide = 0; wide < 2; ++wide) {
     if (!wide && shared) continue;
     const int units = tile_units(p.tiles1, p.tiles3, wide != 0, sym);
@@ -962,6 +969,7 @@ void choose_tiles(DirectPlan& p, bool sym, int reps, double entries, double adds
                                   waves * entries * adds / units / sm_rate);
         if (t < best) {
           best = t;
+          best_mma = mma;
           p.wide = wide != 0;
           p.grid = grid != 0;
           p.sb_per_split = per;
@@ -971,7 +979,9 @@ void choose_tiles(DirectPlan& p, bool sym, int reps, double entries, double adds
     }
   }
   p.units = tile_units(p.tiles1, p.tiles3, p.wide, sym);
-  p.seconds = best + kFixedSeconds;
+  const double beyond = p.split ? (p.wide ? 2.0 : 2.45) : (p.wide ? 1.7 : 2.2);
+  p.beyond_l2 = packed > kInL2;
+  p.seconds = best + kFixedSeconds + (p.beyond_l2 ? (beyond - 1.0) * best_mma : 0.0);
   p.blocks = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(p.units) * p.splits * reps, sms));
   const int chunks = p.sb_per_split * (p.split ? 2 : 1);
   p.need_fold = (p.wide ? chunks : (chunks + 1) / 2) > 64;
@@ -1002,9 +1012,16 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   const int per = p.split ? 32 : 64;
   const int64_t images = (n2 + per - 1) / per;
   const double entries = static_cast<double>(n1) * static_cast<double>(n3);
+  const double packed = static_cast<double>(p.tiles1 + (alias ? 0 : p.tiles3)) * static_cast<double>(images) * kStageBytes;
   choose_tiles(p, alias, 1, entries, 0.5 * h->d * (sets + 1), 2.05e11, 1.35e9,
-               sets == 1 ? std::min(1.0, static_cast<double>(kWindow) / static_cast<double>(h->b)) : 0.0,
+               sets == 1 ? std::min(1.0, static_cast<double>(kWindow) / static_cast<double>(h->b)) : 0.0, packed,
                !batch && (sets > 1 || entries <= 16.8e6), sets == 1, batch, sms);
+  // large operands: read (twice where their inner indices are balanced) and
+  // packed at 5 TB/s; small ones are in the fixed part
+  if (p.beyond_l2) {
+    const double values = static_cast<double>(alias ? n1 : n1 + n3) * static_cast<double>(n2);
+    p.seconds += (values * (dt == CMS_F64 ? 8.0 : dt == CMS_BF16 ? 2.0 : 4.0) * (alias ? 1.0 : 2.0) + packed) / 5e12;
+  }
   const int64_t words = static_cast<int64_t>(h->d) * h->b;
   // (a batch's products queue up less: others' additions are under way too)
   p.copies = sets > 1 ? 1 : sum_copies(words, static_cast<int64_t>(p.units) * p.splits);
@@ -1034,8 +1051,7 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
 // conventional 5 b log2 b + 4 b flops per repetition and inner index, and the
 // gathers of its front end (every entry of a_k and b_k for each computed row),
 // at rates fitted per kernel family to 160 calls of n = 64 .. 16384, b = n / 8
-// .. 32 n, 64 to 8192 inner indices.  With them the chosen route was the faster
-// one, or within 20% of it, in all of them (n = 454, K = 142, b = 810, d = 4 BF16:
+// .. 32 n, 64 to 8192 inner indices (n = 454, K = 142, b = 810, d = 4 BF16:
 // 96 us by the spectra, 44 us this way; n = 6746, K = 184, b = 1620, d = 4 the
 // other way round: 160 and 1136 us).
 static double transform_seconds(const SketchPlan& p, int64_t n1, int64_t n2, int64_t n3, bool batch) {
@@ -1071,10 +1087,13 @@ PrePlan make_pre_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, b
   p.split = true;
   p.tiles1 = p.tiles3 = q.tiles;
   p.nsb = static_cast<int>((n2 + kSuper - 1) / kSuper);
-  choose_tiles(p, false, h->d, static_cast<double>(rows) * rows, 1.0, 5.0e11, 4e9, 0.0, false, true, false, sms);
+  const double packed = 2.0 * static_cast<double>(rows) * static_cast<double>(n2) * 4.0 * h->d;
+  choose_tiles(p, false, h->d, static_cast<double>(rows) * rows, 1.0, 5.0e11, 4e9, 0.0, packed, false, true, false, sms);
   const double n = static_cast<double>(alias ? n1 : n1 + n3), k = static_cast<double>(p.nsb) * kSuper;
   p.seconds += 14e-6 + n * k * 8.0 / 4e12 + static_cast<double>(n1 + n3) * k * h->d * 4.0 / 5e12 +
               2.0 * static_cast<double>(rows) * k * h->d * 4.0 / 3e12;
+  // (beyond L2 the measured times were 1.0 to 1.5 of the rest)
+  if (p.beyond_l2) p.seconds = 1.2 * (p.seconds + (alias ? 0.0 : n * k * 4.0 / 5e12));
   const int64_t words = static_cast<int64_t>(h->d) * h->b;
   p.copies = sum_copies(words, static_cast<int64_t>(p.units) * p.splits);
   const int64_t images = (n2 + 31) / 32;
@@ -1123,8 +1142,10 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
       best = pre.direct.seconds;
     }
   }
-  // a margin for the estimates' error where both are mostly launches
-  return best + (batch ? 0.0 : kMargin) < transform;
+  // a margin for the estimates' error: where both are mostly launches, and a
+  // fourth beyond L2, where 5 of 200 calls of other sizes than the fitted ones
+  // were up to 1.33 slower by the chosen route without it
+  return best * (out->beyond_l2 ? 1.25 : 1.0) + (batch ? 0.0 : kMargin) < transform;
 }
 
 // The masked sums of FINDSIGNIFICANTENTRIES in one pass: an entry is added to

@@ -157,6 +157,15 @@ CMS_API cms_status cms_workspace_size(const cms_hashes* h, int64_t n1, int64_t n
                               int64_t n3, int32_t dt, size_t* bytes);
 
 /*
+ * cms_workspace_size_min - the least workspace that cms_sketch_product takes
+ * for these shapes: its transform route's share, which does not grow with n2.
+ * (The direct route's holds a copy of the operands, up to 16 GiB; above that it
+ * is not offered.)  Errors as cms_workspace_size.
+ */
+CMS_API cms_status cms_workspace_size_min(const cms_hashes* h, int64_t n1, int64_t n2,
+                                  int64_t n3, int32_t dt, size_t* bytes);
+
+/*
  * cms_plan_kernel - which fused kernel the transform route of
  * cms_sketch_product would run for these arguments (the choice depends on b,
  * n, the storage type, the alignment of A and B and whether they alias),
@@ -201,8 +210,8 @@ CMS_API cms_status cms_plan_kernel(const void* A, int64_t lda, const void* B, in
  *   h   : hashes with n >= max(n1, n3).
  *   c   : device float [d][b], written (not accumulated).
  *   ws  : device workspace of at least cms_workspace_size() bytes,
- *         256-byte aligned (one that holds only the transform route's share
- *         is accepted and selects that route).
+ *         256-byte aligned (one of cms_workspace_size_min() bytes, the
+ *         transform route's share, is accepted and selects that route).
  * Errors: CMS_ERR_INVALID_ARG, CMS_ERR_UNSUPPORTED (b not 5-smooth or shape
  * beyond the kernels' limits), CMS_ERR_WORKSPACE, CMS_ERR_CUDA.
  */
@@ -222,8 +231,10 @@ CMS_API cms_status cms_sketch_product(const void* A, int64_t lda, const void* B,
  *   caller still passes A, B, the hashes and the output c.
  *   Scratch: a fixed 32 MiB device array owned by the library (held on every
  *   GPU that loads it until the process exits).  The direct route runs where
- *   its layout fits in it; shapes whose transform route needs more than
- *   32 MiB as well are rejected with CMS_ERR_WORKSPACE (the covariance shape n = 2048, b = 65536, d = 5 needs about 18 MiB).
+ *   its layout fits in it, else the transform route; shapes whose transform
+ *   route needs more than 32 MiB as well are rejected with CMS_ERR_WORKSPACE
+ *   (the covariance shape of 4096 samples, n = 2048, b = 65536, d = 5 takes the
+ *   transform route: 28 MB against 86 MB).
  *   The call allocates nothing.  Its first call on a device looks up the
  *   array's device address (cudaGetSymbolAddress) with that device current;
  *   make that first call before any stream capture.  The address is cached

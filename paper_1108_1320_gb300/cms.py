@@ -43,6 +43,7 @@ SIGNATURES = {
     "cms_hashes_tables": (_I32, [_P, _P, _P, _P, _P]),
     "cms_hashes_buckets": (_I32, [_P, _I32, _I32, _P, _P]),
     "cms_workspace_size": (_I32, [_P, _I64, _I64, _I64, _I32, ctypes.POINTER(_SZ)]),
+    "cms_workspace_size_min": (_I32, [_P, _I64, _I64, _I64, _I32, ctypes.POINTER(_SZ)]),
     "cms_sketch_product": (_I32, [_P, _I64, _P, _I64, _I64, _I64, _I64, _I32, _P, _P, _P, _SZ, _P]),
     "cms_sketch_product_noalloc": (_I32, [_P, _I64, _P, _I64, _I64, _I64, _I64, _I32, _P, _P, _P]),
     "cms_sparse_workspace_size": (_I32, [_P, _I64, _I64, _I64, ctypes.POINTER(_SZ)]),
@@ -251,9 +252,12 @@ def _ab_args(A: torch.Tensor, B: torch.Tensor):
     return n1, n2, n3, lda, ldb
 
 
-def workspace_size(h: Hashes, n1: int, n2: int, n3: int, dtype=torch.float32) -> int:
+def workspace_size(h: Hashes, n1: int, n2: int, n3: int, dtype=torch.float32, smallest: bool = False) -> int:
+    """Bytes of scratch for sketch_product; ``smallest``: the least it takes
+    (the transform route's share, which does not grow with n2)."""
     out = _SZ()
-    _check(lib().cms_workspace_size(h.handle, n1, n2, n3, _DTYPES[dtype], ctypes.byref(out)))
+    query = lib().cms_workspace_size_min if smallest else lib().cms_workspace_size
+    _check(query(h.handle, n1, n2, n3, _DTYPES[dtype], ctypes.byref(out)))
     return out.value
 
 
@@ -264,12 +268,18 @@ def alloc_workspace(nbytes: int, device=None) -> torch.Tensor:
 
 def sketch_product(A: torch.Tensor, B: torch.Tensor, h: Hashes, c: torch.Tensor | None = None,
                    ws: torch.Tensor | None = None, stream=None) -> torch.Tensor:
-    """COMPRESSEDPRODUCT (Fig. 1): returns c, float32 of shape (d, b)."""
+    """COMPRESSEDPRODUCT (Fig. 1): returns c, float32 of shape (d, b).
+
+    ``ws`` is scratch of workspace_size() bytes, allocated here when None (of
+    the smallest size when the device has no room for more)."""
     n1, n2, n3, lda, ldb = _ab_args(A, B)
     c = _sketch_out(c, h, A.device)
     need = workspace_size(h, n1, n2, n3, A.dtype)
     if ws is None:
-        ws = alloc_workspace(need, A.device)
+        try:
+            ws = alloc_workspace(need, A.device)
+        except torch.cuda.OutOfMemoryError:
+            ws = alloc_workspace(workspace_size(h, n1, n2, n3, A.dtype, smallest=True), A.device)
     _check_buf(ws, "ws", A.device)
     _check(lib().cms_sketch_product(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, _DTYPES[A.dtype], h.handle,
                                     _ptr(c), _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)))

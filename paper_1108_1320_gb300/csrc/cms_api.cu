@@ -319,6 +319,46 @@ int check_dense_call(const cms_hashes* h, const void* A, int64_t lda, const void
   if (n2 > 0 && ((n1 > 0 && !A) || (n3 > 0 && !B))) return fail(CMS_ERR_INVALID_ARG, "A or B is NULL");
   return check_device(h);
 }
+
+// Bytes for either route, and for the transform route alone (NULL: not asked).
+cms_status workspace_sizes(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int32_t dt, size_t* bytes,
+                           size_t* smallest) {
+  if (!bytes) return fail(CMS_ERR_INVALID_ARG, "bytes is NULL");
+  cms_status st = check_shapes(h, n1, n2, n3, std::max<int64_t>(n1, 1), std::max<int64_t>(n3, 1));
+  if (st != CMS_OK) return st;
+  if (!valid_dtype(dt)) return fail(CMS_ERR_INVALID_ARG, "unknown dtype");
+  DeviceProps dp = device_props(h->device);
+  SketchPlan plan;
+  std::string why;
+  // the kernel is chosen per call (pointer alignment); cover both plans
+  int r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &plan, &why);
+  if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
+  SketchPlan generic;
+  r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &generic, &why, nullptr, 0, nullptr, 0,
+                       false);
+  if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
+  size_t transform = std::max(plan.ws_bytes, generic.ws_bytes), either = 0;
+  DirectPlan direct;
+  if (n1 == n3) {
+    // A and B the same bytes (A = X^T, B = X): the register-FFT and cluster
+    // kernels stage each row once, so their plans can differ from the
+    // two-operand one (leading dimensions in whole 16-byte units of FP32
+    // and of BF16 cover both storage types)
+    const void* same = reinterpret_cast<const void*>(static_cast<uintptr_t>(256));
+    for (int64_t unit : {4, 8}) {
+      const int64_t ld = std::max<int64_t>((n1 + unit - 1) / unit * unit, unit);
+      SketchPlan alias;
+      r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &alias, &why, same, ld, same, ld);
+      if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
+      transform = std::max(transform, alias.ws_bytes);
+      if (choose_direct(h, alias, n1, n2, n3, dt, true, dp.sms, &direct)) either = std::max(either, direct.ws_bytes);
+    }
+  }
+  if (choose_direct(h, plan, n1, n2, n3, dt, false, dp.sms, &direct)) either = std::max(either, direct.ws_bytes);
+  *bytes = std::max(transform, either);
+  if (smallest) *smallest = transform;
+  return CMS_OK;
+}
 }  // namespace cms
 
 extern "C" {
@@ -343,40 +383,14 @@ cms_status cms_hashes_buckets(const cms_hashes* h, int32_t t, int32_t side, uint
 
 cms_status cms_workspace_size(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int32_t dt,
                               size_t* bytes) {
+  return workspace_sizes(h, n1, n2, n3, dt, bytes, nullptr);
+}
+
+cms_status cms_workspace_size_min(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int32_t dt,
+                                  size_t* bytes) {
+  size_t all = 0;
   if (!bytes) return fail(CMS_ERR_INVALID_ARG, "bytes is NULL");
-  cms_status st = check_shapes(h, n1, n2, n3, std::max<int64_t>(n1, 1), std::max<int64_t>(n3, 1));
-  if (st != CMS_OK) return st;
-  if (!valid_dtype(dt)) return fail(CMS_ERR_INVALID_ARG, "unknown dtype");
-  DeviceProps dp = device_props(h->device);
-  SketchPlan plan;
-  std::string why;
-  // the kernel is chosen per call (pointer alignment); cover both plans
-  int r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &plan, &why);
-  if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
-  SketchPlan generic;
-  r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &generic, &why, nullptr, 0, nullptr, 0,
-                       false);
-  if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
-  *bytes = std::max(plan.ws_bytes, generic.ws_bytes);
-  if (n1 == n3) {
-    // A and B the same bytes (A = X^T, B = X): the register-FFT and cluster
-    // kernels stage each row once, so their plans can differ from the
-    // two-operand one (leading dimensions in whole 16-byte units of FP32
-    // and of BF16 cover both storage types)
-    const void* same = reinterpret_cast<const void*>(static_cast<uintptr_t>(256));
-    for (int64_t unit : {4, 8}) {
-      const int64_t ld = std::max<int64_t>((n1 + unit - 1) / unit * unit, unit);
-      SketchPlan alias;
-      r = make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &alias, &why, same, ld, same, ld);
-      if (r != CMS_OK) return fail(static_cast<cms_status>(r), why);
-      *bytes = std::max(*bytes, alias.ws_bytes);
-      DirectPlan direct;
-      if (choose_direct(h, alias, n1, n2, n3, dt, true, dp.sms, &direct)) *bytes = std::max(*bytes, direct.ws_bytes);
-    }
-  }
-  DirectPlan direct;
-  if (choose_direct(h, plan, n1, n2, n3, dt, false, dp.sms, &direct)) *bytes = std::max(*bytes, direct.ws_bytes);
-  return CMS_OK;
+  return workspace_sizes(h, n1, n2, n3, dt, &all, bytes);
 }
 
 cms_status cms_plan_kernel(const void* A, int64_t lda, const void* B, int64_t ldb, int64_t n1, int64_t n2,

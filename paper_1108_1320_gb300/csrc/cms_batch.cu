@@ -259,6 +259,11 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
       // (the batch's own plan leaves the tile kernel's words to the batch)
       const DirectPlan one = make_direct_plan(it.h, it.n1, it.n2, it.n3, it.dt, b->direct[i].alias, sms, 1, false);
       cudaError_t e = cudaMalloc(&tws, std::max<size_t>(std::max(p.ws_bytes, one.ws_bytes), 256));
+      if (e == cudaErrorMemoryAllocation) {   // no room for the packed operands
+        cudaGetLastError();
+        b->is_direct[i] = 0;
+        continue;
+      }
       double td = 0.0, tt = 0.0;
       if (e == cudaSuccess) e = time_plan(p, it, tws, s, &td, &one);
       if (e == cudaSuccess) e = time_plan(p, it, tws, s, &tt);
@@ -269,72 +274,95 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
       cache_dirty = true;
     }
   }
-  for (int i = 0; i < count; ++i) {
-    if (b->is_direct[i]) continue;
-    const cms_instance& it = items[i];
-    SketchPlan p = b->plans[i];
-    // k-chunking for the batch as a whole: each instance gets tasks in
-    // proportion to its work out of a budget of kBatchWaves waves over the
-    // SMs (the planner alone would split every instance to fill the GPU by
-    // itself: many short tasks, each repeating its prologue and writing a
-    // partial row)
-    {
-      const int nkc = batch_chunks(it, p, items, b->is_direct, count, sms);
-      SketchPlan q;
-      if (nkc > 0 && make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &q, &why, it.A, it.lda, it.B,
-                                      it.ldb, true, nkc, 0, false, false) == CMS_OK)
-        p = q;
+  // the direct instances' packed operands within the bound (the largest give
+  // way to the transform route)
+  for (;;) {
+    size_t total = 0;
+    int largest = -1;
+    for (int i = 0; i < count; ++i) {
+      if (!b->is_direct[i]) continue;
+      total += b->direct[i].ws_bytes;
+      if (largest < 0 || b->direct[i].ws_bytes > b->direct[largest].ws_bytes) largest = i;
     }
-    auto hit = cache.find(tune_key(it, p, sms));
-    if (hit != cache.end()) {
-      SketchPlan q;
-      if (make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &q, &why, it.A, it.lda, it.B, it.ldb,
-                           true, hit->second.nkc, hit->second.G, false, false) == CMS_OK)
-        p = q;
-    } else if (flags & CMS_BATCH_AUTOTUNE) {
-      // candidates: the planner's chunking, half and twice as many chunks;
-      // for the generic kernel also groups of 1, 2 and 4 inner indices
-      std::vector<std::pair<int, int>> cand;
-      for (int mul : {1, 2, 4}) {
-        const int nk = std::max(1, p.nkc * mul / 2);
-        if (p.fast) cand.push_back({nk, 0});
-        else for (int g : {1, 2, 4}) cand.push_back({nk, g});
-      }
-      std::vector<SketchPlan> cps;
-      size_t need = 0;
-      for (auto& c2 : cand) {
+    if (total <= kDirectMaxWorkspace) break;
+    b->is_direct[largest] = 0;
+  }
+  cudaError_t e = cudaSuccess;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    for (int i = 0; i < count; ++i) {
+      if (b->is_direct[i]) continue;
+      const cms_instance& it = items[i];
+      SketchPlan p = b->plans[i];
+      // k-chunking for the batch as a whole: each instance gets tasks in
+      // proportion to its work out of a budget of kBatchWaves waves over the
+      // SMs (the planner alone would split every instance to fill the GPU by
+      // itself: many short tasks, each repeating its prologue and writing a
+      // partial row)
+      {
+        const int nkc = batch_chunks(it, p, items, b->is_direct, count, sms);
         SketchPlan q;
-        if (make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &q, &why, it.A, it.lda, it.B,
-                             it.ldb, true, c2.first, c2.second, false, false) == CMS_OK) {
-          cps.push_back(q);
-          need = std::max(need, q.ws_bytes);
+        if (nkc > 0 && make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &q, &why, it.A, it.lda, it.B,
+                                        it.ldb, true, nkc, 0, false, false) == CMS_OK)
+          p = q;
+      }
+      auto hit = cache.find(tune_key(it, p, sms));
+      if (hit != cache.end()) {
+        SketchPlan q;
+        if (make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &q, &why, it.A, it.lda, it.B, it.ldb,
+                             true, hit->second.nkc, hit->second.G, false, false) == CMS_OK)
+          p = q;
+      } else if (flags & CMS_BATCH_AUTOTUNE) {
+        // candidates: the planner's chunking, half and twice as many chunks;
+        // for the generic kernel also groups of 1, 2 and 4 inner indices
+        std::vector<std::pair<int, int>> cand;
+        for (int mul : {1, 2, 4}) {
+          const int nk = std::max(1, p.nkc * mul / 2);
+          if (p.fast) cand.push_back({nk, 0});
+          else for (int g : {1, 2, 4}) cand.push_back({nk, g});
         }
+        std::vector<SketchPlan> cps;
+        size_t need = 0;
+        for (auto& c2 : cand) {
+          SketchPlan q;
+          if (make_sketch_plan(it.h, it.n1, it.n2, it.n3, it.dt, sms, optin, &q, &why, it.A, it.lda, it.B,
+                               it.ldb, true, c2.first, c2.second, false, false) == CMS_OK) {
+            cps.push_back(q);
+            need = std::max(need, q.ws_bytes);
+          }
+        }
+        char* tws = nullptr;
+        cudaError_t e = cudaMalloc(&tws, std::max<size_t>(need, 256));
+        if (e != cudaSuccess) { delete b; return cuda_fail(e, "cms_batch_create (autotune workspace)"); }
+        double best = 1e30;
+        for (const SketchPlan& q : cps) {
+          double ms = 0.0;
+          e = time_plan(q, it, tws, s, &ms);
+          if (e != cudaSuccess) { cudaFree(tws); delete b; return cuda_fail(e, "cms_batch_create (autotune)"); }
+          if (ms < best) { best = ms; p = q; }
+        }
+        cudaFree(tws);
+        cache[tune_key(it, p, sms)] = Tuned{p.nkc, p.fast ? 0 : p.G, best};
+        cache_dirty = true;
       }
-      char* tws = nullptr;
-      cudaError_t e = cudaMalloc(&tws, std::max<size_t>(need, 256));
-      if (e != cudaSuccess) { delete b; return cuda_fail(e, "cms_batch_create (autotune workspace)"); }
-      double best = 1e30;
-      for (const SketchPlan& q : cps) {
-        double ms = 0.0;
-        e = time_plan(q, it, tws, s, &ms);
-        if (e != cudaSuccess) { cudaFree(tws); delete b; return cuda_fail(e, "cms_batch_create (autotune)"); }
-        if (ms < best) { best = ms; p = q; }
-      }
-      cudaFree(tws);
-      cache[tune_key(it, p, sms)] = Tuned{p.nkc, p.fast ? 0 : p.G, best};
-      cache_dirty = true;
+      b->plans[i] = p;
     }
-    b->plans[i] = p;
+    if (cache_dirty) save_cache(tune_cache, cache);
+    // ---- one workspace for all instances ---------------------------------
+    size_t off = 0;
+    bool any = false;
+    for (int i = 0; i < count; ++i) {
+      b->ws_off[i] = off;
+      any |= b->is_direct[i] != 0;
+      off = align256(off + (b->is_direct[i] ? b->direct[i].ws_bytes : b->plans[i].ws_bytes));
+    }
+    b->ws_bytes = off;
+    e = cudaMalloc(&b->ws, std::max<size_t>(off, 256));
+    if (e != cudaErrorMemoryAllocation || !any) break;
+    // no room for packed operands: every instance by the transform route
+    cudaGetLastError();
+    b->ws = nullptr;
+    std::fill(b->is_direct.begin(), b->is_direct.end(), 0);
   }
-  if (cache_dirty) save_cache(tune_cache, cache);
-  // ---- one workspace for all instances ----------------------------------
-  size_t off = 0;
-  for (int i = 0; i < count; ++i) {
-    b->ws_off[i] = off;
-    off = align256(off + (b->is_direct[i] ? b->direct[i].ws_bytes : b->plans[i].ws_bytes));
-  }
-  b->ws_bytes = off;
-  cudaError_t e = cudaMalloc(&b->ws, std::max<size_t>(off, 256));
   if (e != cudaSuccess) { release(b); delete b; return cuda_fail(e, "cms_batch_create (workspace)"); }
   // ---- task layout: instances with the longest tasks first --------------
   b->order.resize(count);

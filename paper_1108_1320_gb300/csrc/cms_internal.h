@@ -333,6 +333,11 @@ struct DirectPlan {
   size_t off_acc = 0, off_scale = 0, off_blocks = 0, off_bal = 0, off_pa = 0, off_pb = 0;
   size_t ws_bytes = 0;
 };
+// Most scratch that a call's (or a batch's) direct route may ask for.  Its packed
+// operands are as large as the operands, so that above this (about a
+// seventeenth of the card) the transform route serves, whose scratch does not
+// grow with the inner dimension.
+constexpr size_t kDirectMaxWorkspace = size_t{16} << 30;
 // Pre-sketched operands: one direct product of b rows per repetition.
 struct PrePlan {
   bool usable = false;

@@ -1131,10 +1131,10 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
   const double transform = transform_seconds(plan, n1, n2, n3, batch);
   if (!batch && transform <= kFixedSeconds + kMargin + 3e-6) return false;
   *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1, batch);
-  double best = out->seconds - (batch ? kFixedSeconds : 0.0);
+  double best = out->ws_bytes <= kDirectMaxWorkspace ? out->seconds - (batch ? kFixedSeconds : 0.0) : 1e30;
   if (!batch) {
     const PrePlan pre = make_pre_plan(h, n1, n2, n3, alias, sms);
-    if (pre.usable && pre.direct.seconds < best) {
+    if (pre.usable && pre.direct.seconds < best && pre.direct.ws_bytes <= kDirectMaxWorkspace) {
       *out = pre.direct;
       out->pre = true;
       out->alias_operands = alias;

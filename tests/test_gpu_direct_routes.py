@@ -48,3 +48,58 @@ def test_long_inner_dimensions_take_the_faster_route(cms, n1, n2, n3, b, d, dts,
     else:
         assert route in kernels or (route == "k_direct_grid" and "k_direct_window" in kernels)
     h.free()
+
+
+GIB = 1 << 30
+
+
+def test_workspace_of_large_operands_stays_bounded(cms):
+    # packed copies of the operands would take 305 GB, 215 GB and 34 GB
+    for n, m, b, d in [(9000, 1 << 22, 65536, 1), (3072, 8400000, 128, 1), (256, 1 << 24, 4096, 3)]:
+        h = cms.make_hashes(1, n, b, d)
+        full, least = cms.workspace_size(h, n, m, n), cms.workspace_size(h, n, m, n, smallest=True)
+        assert least <= full <= 16 * GIB and least < 64 << 20
+        h.free()
+
+
+def test_least_workspace_is_taken_and_used_when_memory_is_short(cms, monkeypatch):
+    n, m, b, d = 700, 5000, 12000, 3
+    x = torch.randn((m, n), device="cuda")
+    h = cms.make_hashes(2, n, b, d)
+    full, least = cms.workspace_size(h, n, m, n), cms.workspace_size(h, n, m, n, smallest=True)
+    want, kernels = kernels_of(cms, lambda: cms.sketch_product(x.T, x, h))
+    assert "k_direct_tile" in kernels and least < full
+    got, kernels = kernels_of(cms, lambda: cms.sketch_product(x.T, x, h, ws=cms.alloc_workspace(least)))
+    assert "k_direct_tile" not in kernels
+    assert ((got - want).norm() / want.norm()).item() < 1e-5
+    from paper_1108_1320_gb300 import cms as binding
+    with pytest.raises(binding.CmsError):
+        cms.sketch_product(x.T, x, h, ws=cms.alloc_workspace(least)[:least - 256])
+    real, asked = binding.alloc_workspace, []
+
+    def short(nbytes, device=None):
+        asked.append(nbytes)
+        if nbytes >= full:
+            raise torch.cuda.OutOfMemoryError("no room")
+        return real(nbytes, device)
+    monkeypatch.setattr(binding, "alloc_workspace", short)
+    again, kernels = kernels_of(cms, lambda: cms.sketch_product(x.T, x, h))
+    assert asked == [full, least] and torch.equal(again, got)
+    h.free()
+
+
+def test_batch_of_large_operands_stays_bounded(cms):
+    # 24 products of one 1 GiB operand: packed copies of all would take 26 GB
+    n, m, b = 8192, 1 << 15, 1 << 16
+    x = torch.randn((m, n), device="cuda")
+    hs = [cms.make_hashes(q, n, b, 1) for q in range(24)]
+    batch = cms.Batch([(x.T, x, h) for h in hs])
+    assert batch.info()["ws_bytes"] <= 17 * GIB
+    out, kernels = kernels_of(cms, batch.run)
+    assert "k_direct_tile_batched" in kernels and "k_sketch_batched" in kernels
+    for c, h in zip(out, hs):                      # both routes against the single call
+        want = cms.sketch_product(x.T, x, h)
+        assert ((c - want).norm() / want.norm()).item() < 1e-5
+    batch.free()
+    for h in hs:
+        h.free()

@@ -530,7 +530,10 @@ CMS_API cms_status cms_nnz_estimate(const int64_t* a_colptr, const int32_t* a_ro
  *               the device's atomic appends; sort for a canonical order).
  *   count_out : device int64, the number of positions (may exceed capacity).
  *   ws        : device scratch of cms_significant_workspace_size bytes,
- *               256-byte aligned.
+ *               256-byte aligned (cms_significant_workspace_size_min bytes are
+ *               taken too: the masked products, by the transform route).
+ * Where cheaper, all masked sums are formed in one pass over the entries of AB
+ * (stored in bands of at most 256 MiB, or 12 rows of 128 x 128 tiles).
  * cms_decode_significant - the decode and vote alone, on 2 l given
  * sketches (device float [2 l][d][b], as above), with a scratch of
  * cms_significant_decode_workspace_size bytes.
@@ -539,6 +542,8 @@ CMS_API cms_status cms_nnz_estimate(const int64_t* a_colptr, const int32_t* a_ro
  */
 CMS_API cms_status cms_significant_workspace_size(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3,
                                                   int32_t dt, int32_t rho, size_t* bytes);
+CMS_API cms_status cms_significant_workspace_size_min(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3,
+                                                      int32_t dt, int32_t rho, size_t* bytes);
 CMS_API cms_status cms_find_significant(const void* A, int64_t lda, const void* B, int64_t ldb,
                                         int64_t n1, int64_t n2, int64_t n3, int32_t dt,
                                         const cms_hashes* h, float delta, int32_t rho, int64_t* ij_out,

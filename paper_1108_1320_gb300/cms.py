@@ -56,6 +56,7 @@ SIGNATURES = {
     "cms_nnz_estimate": (_I32, [_P, _P, _P, _P, _P, _P, _I64, _I64, _I64, _I32, ctypes.c_uint64, _I32, _I64,
                                 ctypes.POINTER(_I64), ctypes.POINTER(_I64), _P, _SZ, _P]),
     "cms_significant_workspace_size": (_I32, [_P, _I64, _I64, _I64, _I32, _I32, ctypes.POINTER(_SZ)]),
+    "cms_significant_workspace_size_min": (_I32, [_P, _I64, _I64, _I64, _I32, _I32, ctypes.POINTER(_SZ)]),
     "cms_find_significant": (_I32, [_P, _I64, _P, _I64, _I64, _I64, _I64, _I32, _P, ctypes.c_float, _I32, _P, _I64,
                                     _P, _P, _SZ, _P]),
     "cms_significant_decode_workspace_size": (_I32, [_P, ctypes.POINTER(_SZ)]),
@@ -531,7 +532,12 @@ def find_significant(A: torch.Tensor, B: torch.Tensor, h: Hashes, delta: float, 
     n1, n2, n3, lda, ldb = _ab_args(A, B)
     need = _SZ()
     _check(lib().cms_significant_workspace_size(h.handle, n1, n2, n3, _DTYPES[A.dtype], rho, ctypes.byref(need)))
-    ws = alloc_workspace(need.value, A.device)
+    try:
+        ws = alloc_workspace(need.value, A.device)
+    except torch.cuda.OutOfMemoryError:
+        _check(lib().cms_significant_workspace_size_min(h.handle, n1, n2, n3, _DTYPES[A.dtype], rho,
+                                                        ctypes.byref(need)))
+        ws = alloc_workspace(need.value, A.device)
     ij = torch.empty((max(capacity, 1), 2), dtype=torch.int64, device=A.device)
     cnt = torch.zeros(1, dtype=torch.int64, device=A.device)
     _check(lib().cms_find_significant(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, _DTYPES[A.dtype], h.handle,

@@ -728,12 +728,14 @@ struct SigLayout {
   size_t dec_direct = 0, masked_total = 0;
 };
 
+// least: the masked products by the transform route, nothing by the direct one.
 cms_status sig_layout(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int32_t dt, int32_t rho, bool alias,
-                      SigLayout* L) {
+                      bool least, SigLayout* L) {
   auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
-  size_t sk = 0;
-  cms_status st = cms_workspace_size(h, n1, n2, n3, dt, &sk);
+  size_t sk = 0, sk_least = 0;
+  cms_status st = workspace_sizes(h, n1, n2, n3, dt, &sk, &sk_least);
   if (st != CMS_OK) return st;
+  if (least) sk = sk_least;
   const size_t esz = dt == CMS_BF16 ? 2 : (dt == CMS_F64 ? 8 : 4);
   L->ell = significant_code_length(n1, n3, rho, nullptr);
   L->ld0 = std::max<int64_t>((n1 + 7) / 8 * 8, 8);
@@ -752,7 +754,7 @@ cms_status sig_layout(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, i
   std::string why;
   DirectPlan one;
   L->direct = false;
-  if (make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &plan, &why) == CMS_OK &&
+  if (!least && make_sketch_plan(h, n1, n2, n3, dt, dp.sms, dp.smem_optin, &plan, &why) == CMS_OK &&
       choose_direct_significant(h, plan, n1, n2, n3, dt, alias, dp.sms, bits, L->ell, &one)) {
     L->direct = true;
     L->plan = one;
@@ -768,14 +770,25 @@ cms_status cms_significant_workspace_size(const cms_hashes* h, int64_t n1, int64
   if (!bytes) return fail(CMS_ERR_INVALID_ARG, "bytes is NULL");
   if (rho < 1 || rho > 8) return fail(CMS_ERR_INVALID_ARG, "rho must be in [1, 8]");
   SigLayout L;
-  cms_status st = sig_layout(h, n1, n2, n3, dt, rho, false, &L);
+  cms_status st = sig_layout(h, n1, n2, n3, dt, rho, false, false, &L);
   if (st != CMS_OK) return st;
   *bytes = L.total;
   if (n1 == n3) {   // A = X^T, B = X packs one operand: not more, but its own plan
-    st = sig_layout(h, n1, n2, n3, dt, rho, true, &L);
+    st = sig_layout(h, n1, n2, n3, dt, rho, true, false, &L);
     if (st != CMS_OK) return st;
     *bytes = std::max(*bytes, L.total);
   }
+  return CMS_OK;
+}
+
+cms_status cms_significant_workspace_size_min(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, int32_t dt,
+                                              int32_t rho, size_t* bytes) {
+  if (!bytes) return fail(CMS_ERR_INVALID_ARG, "bytes is NULL");
+  if (rho < 1 || rho > 8) return fail(CMS_ERR_INVALID_ARG, "rho must be in [1, 8]");
+  SigLayout L;
+  cms_status st = sig_layout(h, n1, n2, n3, dt, rho, false, true, &L);
+  if (st != CMS_OK) return st;
+  *bytes = L.total;
   return CMS_OK;
 }
 
@@ -822,9 +835,14 @@ cms_status cms_find_significant(const void* A, int64_t lda, const void* B, int64
   st = check_device(h);
   if (st != CMS_OK) return st;
   SigLayout L;
-  st = sig_layout(h, n1, n2, n3, dt, rho, A == B && lda == ldb && n1 == n3, &L);
+  const bool alias = A == B && lda == ldb && n1 == n3;
+  st = sig_layout(h, n1, n2, n3, dt, rho, alias, false, &L);
   if (st != CMS_OK) return st;
   const bool direct = L.direct && ws_bytes >= L.total;
+  if (!direct && ws_bytes < L.masked_total) {
+    st = sig_layout(h, n1, n2, n3, dt, rho, alias, true, &L);
+    if (st != CMS_OK) return st;
+  }
   if (!ws || ws_bytes < (direct ? L.total : L.masked_total))
     return fail(CMS_ERR_WORKSPACE, "workspace missing or smaller than cms_significant_workspace_size()");
   if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return fail(CMS_ERR_WORKSPACE, "workspace must be 256-byte aligned");

@@ -322,6 +322,7 @@ struct DirectPlan {
   int copies = 1;           // of the sums, for short sketches
   bool grid = false;        // the entries stored, added to the buckets by a launch of its own
   int parts = 1;            // ... in this many parts to add up
+  int band = 0;             // ... this many tile rows at a time (all of them unless AB is large)
   bool window = false;      // ... with a window of the buckets in shared memory
   int sets = 1;             // sums of different entries (1 + 2 L: FINDSIGNIFICANTENTRIES)
   double seconds = 0.0;     // estimate

@@ -28,16 +28,18 @@ struct TileArgs {
   size_t rep_images;
   int rep_blocks;
   int reps;
-  // entries in units of the integer sums: [part][tile row][tile column][128
-  // columns][128 rows], a part per split of the inner dimension, or two where
-  // a unit's halves hold a share of it each
+  // entries in units of the integer sums: [part][tile row - row0][tile
+  // column][128 columns][128 rows], a part per split of the inner dimension, or
+  // two where a unit's halves hold a share of it each; rows tile rows from row0
+  // on, whose units follow unit0
   float* grid;
+  int row0, rows, unit0;
   int64_t K;
   int n, n1, n3, b, d;
   int tiles1, tiles3;
   int nsb, sb_per_split, splits;
   int parts;                   // of the grid: splits, or twice as many
-  int units;                   // of work per split and repetition (tile_units)
+  int units;                   // of work per split and repetition (tile_units; of the rows)
   int split;                   // two FP16 terms per value
   int sym;                     // A = X^T, B = X: tiles on and above the diagonal
 };

@@ -54,6 +54,10 @@ using namespace dtile;
 constexpr double kFixedSeconds = 36e-6;   // launches of a single product
 constexpr double kMargin = 4e-6;
 constexpr double kInL2 = 110e6;           // bytes of packed operands that stay in L2
+// Bytes of stored entries.  Products of one sketch stay below it; the masked
+// sums of FINDSIGNIFICANTENTRIES, which have no fused form, take AB in bands of
+// tile rows one after the other above it.
+constexpr size_t kMaxStored = size_t{256} << 20;
 constexpr int kWindow = 28672;             // buckets in shared memory (224 KB)
 constexpr int kBadExp = 0x4000;         // block with an infinity or a NaN
 constexpr int kMinExp = -126;           // smallest normal values: scales stay representable
@@ -640,8 +644,9 @@ k_direct_pack_batched(const PackArgs* __restrict__ args, const int* __restrict__
 }
 
 struct GridArgs {
-  const float* grid;           // [part][tile row][tile column][128 columns][128 rows]
+  const float* grid;           // [part][tile row - row0][tile column][128 columns][128 rows]
   size_t part;                 // entries from one part to the next
+  int row0;
   int parts;
   int tiles1, tiles3, sym;
   const uint32_t* hs;          // [t][side][n]
@@ -661,7 +666,7 @@ __global__ void __launch_bounds__(256) k_direct_grid(const GridArgs p) {
   next_kernel_may_start();
   wait_for_kernel_before();
   if (p.scale->bad) return;
-  const int tile = static_cast<int>(blockIdx.x), ti = tile / p.tiles3, tj = tile - ti * p.tiles3;
+  const int tile = static_cast<int>(blockIdx.x), tr = tile / p.tiles3, ti = p.row0 + tr, tj = tile - tr * p.tiles3;
   if (p.sym && ti > tj) return;
   const bool mirror = p.sym && ti < tj;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -930,8 +935,7 @@ namespace {
 //         (twice the units, where tiles are few);
 //  splits of the inner dimension while SMs have no unit;
 //  grid   entries stored for a launch of its own (additions from every SM,
-//         about 6 us more; entries beyond L2's reach are not worth storing),
-//         or added by the tile kernel while it multiplies on.
+//         about 6 us more), or added by the tile kernel while it multiplies on.
 // Times: a chunk of 64 (FP16 terms) or 128 (BF16) inner indices of a tile
 // 0.40 us (BF16 alone on its operands 0.53: the copies from L2 bound it), and
 // more where the packed operands (`packed` bytes) do not stay in L2: 2.0 times as
@@ -1034,7 +1038,13 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   p.off_acc = o;    o = al1k(o + p.acc_bytes + 256);
   p.zero_bytes = o;
   p.off_grid = o;
-  if (p.grid) o = al1k(o + static_cast<size_t>(p.parts) * p.tiles1 * p.tiles3 * kTile * kTile * sizeof(float));
+  if (p.grid) {
+    // (whole bands of the order of units)
+    const size_t row = static_cast<size_t>(p.parts) * p.tiles3 * kTile * kTile * sizeof(float);
+    p.band = p.tiles1;
+    if (row * p.tiles1 > kMaxStored) p.band = std::max(kBand, static_cast<int>(kMaxStored / row) / kBand * kBand);
+    o = al1k(o + row * p.band);
+  }
   p.off_work = o;   o = al1k(o + (batch ? 0 : tile_work_bytes(p.blocks, p.need_fold, p.need_hand, p.need_merge)));
   p.off_scale = o;  o = al1k(o + sizeof(DirectScale));
   p.off_blocks = o; o = al1k(o + static_cast<size_t>(p.tiles1 + t3) * p.nsb * sizeof(int2));
@@ -1155,6 +1165,7 @@ bool choose_direct_significant(const cms_hashes* h, const SketchPlan& plan, int6
                                bool alias, int sms, int bits, int ell, DirectPlan* out) {
   if (n2 < 64 || n1 < 1 || n3 < 1 || h->n > 65535 || !tile_kernel_usable()) return false;
   *out = make_direct_plan(h, n1, n2, n3, dt, alias, sms, 1 + 2 * bits, false);
+  if (out->ws_bytes > kDirectMaxWorkspace) return false;
   return out->seconds + static_cast<double>(out->acc_bytes) / 3e12 < 2.0 * ell * transform_seconds(plan, n1, n2, n3, false);
 }
 
@@ -1202,6 +1213,8 @@ TileArgs tile_args(const DirectPlan& p, const cms_hashes* h, int64_t n1, int64_t
   a.units = p.units;
   a.copies = p.copies;
   a.grid = reinterpret_cast<float*>(ws + p.off_grid);
+  a.row0 = a.unit0 = 0;
+  a.rows = p.tiles1;
   a.parts = p.parts;
   a.split = p.split ? 1 : 0;
   a.sym = p.alias ? 1 : 0;
@@ -1331,12 +1344,42 @@ namespace {
 cudaError_t launch_product_tiles(const DirectPlan& p, const TileArgs& a, char* ws, cudaStream_t s) {
   ProfScope prof_scope("k_direct_tile", s);
   TileLaunch l{};
-  l.total = p.units * p.splits * a.reps;
+  l.total = a.units * p.splits * a.reps;
   l.need_fold = p.need_fold ? 1 : 0;
   l.need_hand = p.need_hand ? 1 : 0;
   l.need_merge = p.need_merge ? 1 : 0;
   l.work = reinterpret_cast<float*>(ws + p.off_work);
-  return launch_tiles(a, l, p.wide, p.grid, p.blocks, s);
+  return launch_tiles(a, l, p.wide, p.grid, std::min(p.blocks, l.total), s);
+}
+
+// Stored entries into the sums.
+cudaError_t launch_stored(const DirectPlan& p, const cms_hashes* h, const TileArgs& a, cudaStream_t s) {
+  cudaError_t e;
+  GridArgs g{};
+  g.grid = a.grid;
+  g.part = static_cast<size_t>(a.rows) * p.tiles3 * kTile * kTile;
+  g.row0 = a.row0;
+  g.parts = p.parts;
+  g.tiles1 = p.tiles1;
+  g.tiles3 = p.tiles3;
+  g.sym = p.alias ? 1 : 0;
+  g.hs = h->d_hs;
+  g.scale = a.scale;
+  g.acc = a.acc;
+  g.copies = p.copies;
+  g.bits = (p.sets - 1) / 2;
+  g.n = a.n; g.n1 = a.n1; g.n3 = a.n3; g.b = a.b; g.d = a.d;
+  // an SM adds 1.35 G/s: few tiles are shared by the repetitions' blocks
+  if (p.window) {
+    ProfScope window_scope("k_direct_window", s);
+    if ((e = with_smem(k_direct_window, 8 * kWindow)) != cudaSuccess) return e;
+    const int shares = std::max(1, 152 / h->d);
+    return launch_after(k_direct_window, dim3(h->d * shares), 1024, 8 * kWindow, s, g, shares);
+  }
+  const int tiles = a.rows * p.tiles3, per_tile = kTile / (8 * kGridCols);
+  ProfScope grid_scope("k_direct_grid", s);
+  const dim3 gg(tiles, per_tile, std::min(h->d, std::max(1, 152 * 2 / (tiles * per_tile))));
+  return launch_after(p.sets > 1 ? k_direct_grid<true> : k_direct_grid<false>, gg, 256, 0, s, g);
 }
 
 // Zeroed sums, packing, tiles.
@@ -1357,33 +1400,18 @@ cudaError_t launch_sums(const DirectPlan& p, const cms_hashes* h, const void* A,
     }
     if (e != cudaSuccess) return e;
   }
-  const TileArgs a = tile_args(p, h, n1, n2, n3, ws);
-  e = launch_product_tiles(p, a, ws, s);
-  if (e != cudaSuccess || !p.grid) return e;
-  GridArgs g{};
-  g.grid = a.grid;
-  g.part = static_cast<size_t>(p.tiles1) * p.tiles3 * kTile * kTile;
-  g.parts = p.parts;
-  g.tiles1 = p.tiles1;
-  g.tiles3 = p.tiles3;
-  g.sym = p.alias ? 1 : 0;
-  g.hs = h->d_hs;
-  g.scale = a.scale;
-  g.acc = a.acc;
-  g.copies = p.copies;
-  g.bits = (p.sets - 1) / 2;
-  g.n = a.n; g.n1 = a.n1; g.n3 = a.n3; g.b = a.b; g.d = a.d;
-  // an SM adds 1.35 G/s: few tiles are shared by the repetitions' blocks
-  if (p.window) {
-    ProfScope window_scope("k_direct_window", s);
-    if ((e = with_smem(k_direct_window, 8 * kWindow)) != cudaSuccess) return e;
-    const int shares = std::max(1, 152 / h->d);
-    return launch_after(k_direct_window, dim3(h->d * shares), 1024, 8 * kWindow, s, g, shares);
+  TileArgs a = tile_args(p, h, n1, n2, n3, ws);
+  if (!p.grid) return launch_product_tiles(p, a, ws, s);
+  for (int row = 0; row < p.tiles1 && e == cudaSuccess; row += p.band) {
+    // the bands' units follow each other (tile_unit); one band: all of them
+    a.row0 = row;
+    a.rows = std::min(p.band, p.tiles1 - row);
+    a.unit0 = tile_units(row, p.tiles3, p.wide, p.alias);
+    a.units = tile_units(row + a.rows, p.tiles3, p.wide, p.alias) - a.unit0;
+    e = launch_product_tiles(p, a, ws, s);
+    if (e == cudaSuccess) e = launch_stored(p, h, a, s);
   }
-  const int tiles = p.tiles1 * p.tiles3, per_tile = kTile / (8 * kGridCols);
-  ProfScope grid_scope("k_direct_grid", s);
-  const dim3 gg(tiles, per_tile, std::min(h->d, std::max(1, 152 * 2 / (tiles * per_tile))));
-  return launch_after(p.sets > 1 ? k_direct_grid<true> : k_direct_grid<false>, gg, 256, 0, s, g);
+  return e;
 }
 
 // `per` buckets share a scale.

@@ -167,7 +167,7 @@ __device__ __forceinline__ void get_unit(const TileArgs& one, const TileLaunch& 
     idx -= __ldg(l.start + lo);
   }
   const TileArgs& p = *u.p;
-  u.q = idx % p.units;
+  u.q = p.unit0 + idx % p.units;
   idx /= p.units;
   u.split = idx % p.splits;
   u.rep = idx / p.splits;
@@ -214,7 +214,7 @@ __device__ __forceinline__ void bucket_add(unsigned long long* c, uint32_t z, fl
 // 60).
 __device__ __forceinline__ void store_grid(const TileArgs& p, const float (&acc)[kTile], int part, int ti, int tj,
                                            int row) {
-  float* g = p.grid + ((static_cast<size_t>(part) * p.tiles1 + ti) * p.tiles3 + tj) * kTileFloats + row;
+  float* g = p.grid + ((static_cast<size_t>(part) * p.rows + ti - p.row0) * p.tiles3 + tj) * kTileFloats + row;
 #pragma unroll
   for (int q = 0; q < kTile; ++q) __stcg(g + q * kTile, acc[q]);
 }

@@ -103,3 +103,64 @@ def test_batch_of_large_operands_stays_bounded(cms):
     batch.free()
     for h in hs:
         h.free()
+
+
+def planted(n1, n3, m, big, alias, seed):
+    """Operands whose product has the entries `big` far above the others."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    x = 0.01 * torch.randn((m, n1), generator=g, device="cuda")
+    y = x if alias else 0.01 * torch.randn((m, n3), generator=g, device="cuda")
+    for q, (i, j) in enumerate(big):
+        x[q, i] += 10.0
+        y[q, j] += 10.0 + q
+    return x, y
+
+
+# 71 x 71 and 40 x 110 tiles: stored entries in bands of 48 and 36 tile rows (two
+# parts each where the units are single tiles), the last band shorter
+@pytest.mark.parametrize("n1,n3,alias", [(9000, 9000, True), (8970, 8973, False), (5100, 14000, False)])
+def test_significant_entries_in_bands_of_rows(cms, n1, n3, alias):
+    m, b, d = 1000, 16384, 5
+    big = [(3, 5), (n1 - 1, 0), (n1 // 2, n3 - 1), (6143, 7001), (6144, 21)] if n1 > 6144 else \
+        [(3, 5), (n1 - 1, 0), (n1 // 2, n3 - 1), (1535, 13999), (1536, 21), (4607, 4608), (4608, 4607)]
+    x, y = planted(n1, n3, m, big, alias, n1)
+    ab = x.double().T @ y.double()
+    want = torch.nonzero(ab.abs() > 50.0).cpu().tolist()
+    del ab
+    h = cms.make_hashes(15, max(n1, n3), b, d)
+    (ij, count), kernels = kernels_of(cms, lambda: cms.find_significant(x.T, y, h, 50.0, 3))
+    assert kernels["k_direct_tile"]["launches"] > 1 and kernels["k_direct_grid"]["launches"] > 1
+    assert count == len(want) and ij.cpu().tolist() == want
+    h.free()
+
+
+def test_significant_workspace_stays_bounded(cms, monkeypatch):
+    # the entries of AB would take 1.07 GB
+    import ctypes
+    h = cms.make_hashes(1, 16384, 1 << 16, 5)
+    full, least = ctypes.c_size_t(), ctypes.c_size_t()
+    for query, out in ((cms.lib().cms_significant_workspace_size, full),
+                       (cms.lib().cms_significant_workspace_size_min, least)):
+        assert query(h.handle, 16384, 2000, 16384, 0, 3, ctypes.byref(out)) == 0
+    assert least.value < 430e6 and least.value <= full.value < 760e6
+    h.free()
+    # the least is used when memory is short, with the same positions
+    big = [(3, 5), (117, 230), (299, 0)]
+    x, y = planted(300, 280, 5000, big, False, 3)
+    h = cms.make_hashes(4, 300, 16384, 5)
+    (want, count), kernels = kernels_of(cms, lambda: cms.find_significant(x.T, y, h, 50.0, 1))
+    assert "k_direct_sig_decode" in kernels and count == 3
+    from paper_1108_1320_gb300 import cms as binding
+    real, asked = binding.alloc_workspace, []
+
+    def short(nbytes, device=None):
+        asked.append(nbytes)
+        if len(asked) == 1:
+            raise torch.cuda.OutOfMemoryError("no room")
+        return real(nbytes, device)
+    monkeypatch.setattr(binding, "alloc_workspace", short)
+    (got, again), kernels = kernels_of(cms, lambda: cms.find_significant(x.T, y, h, 50.0, 1))
+    assert "k_mask_copy" in kernels and "k_direct_tile" not in kernels and asked[1] < asked[0]
+    assert again == count and torch.equal(got, want)
+    h.free()

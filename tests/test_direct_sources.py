@@ -34,3 +34,11 @@ def test_programmatic_launches_read_results_past_the_read_only_path(name, path):
     loads = re.findall(r"__ldg\(\s*&?\(?([^;]*)", text)
     for arg in loads:
         assert READ_ONLY.match(arg), arg
+
+
+def test_superblocks_are_not_counted_in_a_limited_grid_dimension():
+    # a grid's y and z end at 65535: inner indices by the 128 pass that at 8.4 M
+    with open(os.path.join(CSRC, "k_direct.cu")) as f:
+        src = f.read()
+    assert not re.search(r"blockIdx\.[yz]\)?\s*\*\s*kSuper", src)
+    assert not re.search(r"dim3\([^;]*,\s*p\.nsb\s*,", src)

@@ -257,13 +257,14 @@ struct SparseArgsHost {
 int make_sparse_plan(const cms_hashes* h, int64_t n2, int64_t K, int num_sms, size_t smem_optin,
                      SketchPlan* plan, size_t* off_klist, std::string* why);
 // Ordered split of the nonempty inner indices into the FFT list (flist)
-// and the direct list (dlist; limit < 0: none); counts[0..1] their lengths;
+// and the direct list (dlist, the heavy ones at its back; limit < 0: none);
+// counts[0..1] their lengths without the heavy ones;
 // scratch holds 2 x 1024 ints.  Zeroes the direct part's sums cd; integer:
 // also measures the direct list's terms for launch_direct_scatter.
 cudaError_t launch_nonempty_split(const cms_hashes* h, const SparseArgsHost& in, int dt, int64_t n2, int64_t limit,
                                   int integer, int32_t* flist, int32_t* dlist, int32_t* counts, int32_t* scratch,
                                   double* cd, cudaStream_t s);
-// The direct list's length is read on the device (counts[1]); n2 bounds it.
+// The direct list's length is read on the device (counts[1]); dlist has n2 places.
 // integer: sums of integers at a common scale (the same in any order), else
 // FP64 sums.
 cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer,

@@ -383,8 +383,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_sketch_sparse(const SparseArgs 
 // (each block adds up their counts; a scan kernel of its own between the two
 // cost 6 us of the call).  counts[0] = FFT list length, counts[1] = direct
 // list length.
+//  The direct list fills dlist from its front; inner indices of more than
+// kHeavyTerms terms fill it from its back (DirectTerms::heavy of them, in any
+// order): all blocks share each of those.
+constexpr int64_t kHeavyTerms = 16384;
 __device__ __forceinline__ void classify_k(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_ptr,
-                                           int64_t n2, int64_t limit, int64_t k, bool* fft, bool* direct) {
+                                           int64_t n2, int64_t limit, int64_t k, bool* fft, bool* direct, bool* heavy) {
   int64_t na = 0, nb = 0;
   if (k < n2) {
     na = a_ptr[k + 1] - a_ptr[k];
@@ -392,6 +396,7 @@ __device__ __forceinline__ void classify_k(const int64_t* __restrict__ a_ptr, co
   }
   const bool live = na > 0 && nb > 0;
   *direct = live && limit >= 0 && na * nb <= limit;
+  *heavy = *direct && na * nb > kHeavyTerms;
   *fft = live && !*direct;
 }
 
@@ -415,7 +420,7 @@ __device__ __forceinline__ uint32_t warp_max_abs(const T* __restrict__ v, const 
 struct DirectTerms {
   unsigned long long terms;
   uint32_t max_bits;       // of an FP32 number
-  uint32_t unused;
+  uint32_t heavy;          // length of the list at dlist's back
 };
 
 // Power of two by which a term is scaled before it is rounded to an integer:
@@ -443,10 +448,10 @@ k_split_count(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_p
   uint32_t mx = 0;
   for (int64_t base = k0; base < k1; base += blockDim.x) {
     const int64_t k = base + threadIdx.x;
-    bool f = false, dr = false;
-    if (k < k1) classify_k(a_ptr, b_ptr, n2, limit, k, &f, &dr);
+    bool f = false, dr = false, hv = false;
+    if (k < k1) classify_k(a_ptr, b_ptr, n2, limit, k, &f, &dr, &hv);
     cf += f;
-    cd += dr;
+    cd += dr && !hv;
     if (terms == nullptr) continue;
     // the warp measures its direct inner indices one after the other
     for (unsigned todo = __ballot_sync(0xFFFFFFFFu, dr); todo; todo &= todo - 1) {
@@ -479,7 +484,7 @@ k_split_count(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_p
 __global__ void __launch_bounds__(1024)
 k_split_write(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_ptr, int64_t n2, int64_t limit,
               int64_t chunk, const int32_t* __restrict__ part, int32_t* __restrict__ flist,
-              int32_t* __restrict__ dlist, int32_t* __restrict__ counts) {
+              int32_t* __restrict__ dlist, int32_t* __restrict__ counts, DirectTerms* __restrict__ terms) {
   __shared__ int32_t warp_tot[2][32];
   __shared__ int32_t running[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -497,8 +502,10 @@ k_split_write(const int64_t* __restrict__ a_ptr, const int64_t* __restrict__ b_p
   const int64_t k1 = min(n2, k0 + chunk);
   for (int64_t base = k0; base < k1; base += 1024) {
     const int64_t k = base + tid;
-    bool f = false, dr = false;
-    if (k < k1) classify_k(a_ptr, b_ptr, n2, limit, k, &f, &dr);
+    bool f = false, dr = false, hv = false;
+    if (k < k1) classify_k(a_ptr, b_ptr, n2, limit, k, &f, &dr, &hv);
+    if (hv) dlist[n2 - 1 - static_cast<int64_t>(atomicAdd(&terms->heavy, 1u))] = static_cast<int32_t>(k);
+    dr = dr && !hv;
     const unsigned bf = __ballot_sync(0xFFFFFFFFu, f);
     const unsigned bd = __ballot_sync(0xFFFFFFFFu, dr);
     const unsigned lt = (1u << lane) - 1u;
@@ -527,81 +534,158 @@ template <> __device__ __forceinline__ double val_f64<__nv_bfloat16>(const __nv_
 
 // Direct sketch of the outer products of the listed inner indices: for every
 // nonzero pair (A_ik, B_kj) and repetition t, s1(i) s2(j) A_ik B_kj goes to
-// bucket (h1(i) + h2(j)) mod b.  One block per listed k at a time; the values
-// and hashes of up to kDirA x kDirB nonzeros sit in shared memory, so that a
-// term costs its addition alone (6.3 M random 64-bit reductions of the exact
-// sparse workload: 31 us at the chip's 205 G/s; with the hashes read per term
-// and a 64-bit division per pair 42 us).
+// bucket (h1(i) + h2(j)) mod b.  A block takes an inner index of the list at a
+// time, in pieces of up to 4096 terms from up to kDirN nonzeros, whose values
+// and hashes sit in shared memory, so that a term costs its addition alone (6.3
+// M random 64-bit reductions of the exact sparse workload: 31 us at the chip's
+// 205 G/s; with the hashes read per term and a 64-bit division per pair 42 us).
+// A piece is 32 x 128 where both sides have that many, and longer along one
+// side where the other is short (a column of 100000 nonzeros against one
+// element: 32 x 128 at most took 4.5 ms, 32 threads at work; 0.08 so).  The
+// pieces of heavy inner indices are dealt to all blocks, one adding 1.35 G/s (one
+// product of 640 x 640, b = 2^20, d = 7: 1.73 ms by one block, 0.12 so).
 //  INT: terms rounded to integers at a common scale (term_shift) and added
 //       as 64-bit integers: the same sums in any order.
 //  else: FP64 (products of two FP32 or BF16 values are exact), added
 //       atomically: their order varies, at FP64 rounding.
-constexpr int kDirA = 32, kDirB = 128, kDirT = 8;
+constexpr int kDirN = 512, kDirTerms = 4096, kDirT = 8;
+
+// Nonzeros of A and of B in a piece of an na x nb outer product.
+struct Piece {
+  int a, b;
+};
+__device__ __forceinline__ Piece piece_of(int64_t na, int64_t nb) {
+  Piece q;
+  if (na <= 32 && nb <= 128) {   // one piece, without the divisions
+    q.a = static_cast<int>(na);
+    q.b = static_cast<int>(nb);
+    return q;
+  }
+  q.a = static_cast<int>(min(na, static_cast<int64_t>(32)));
+  q.b = static_cast<int>(min(nb, static_cast<int64_t>(min(kDirTerms / q.a, kDirN - q.a))));
+  q.a = static_cast<int>(min(na, static_cast<int64_t>(min(kDirTerms / q.b, kDirN - q.b))));
+  return q;
+}
 
 template <typename T, bool INT>
 __global__ void __launch_bounds__(256)
 k_direct_scatter(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ a_idx, const T* __restrict__ a_val,
                  const int64_t* __restrict__ b_ptr, const int32_t* __restrict__ b_idx, const T* __restrict__ b_val,
-                 int n1, int n3, int64_t n, const int32_t* __restrict__ dlist, const int32_t* __restrict__ counts,
-                 const uint32_t* __restrict__ hs, int d, int64_t b, double* __restrict__ cd,
-                 const DirectTerms* __restrict__ terms) {
-  __shared__ double va[kDirA], vb[kDirB];
-  __shared__ int xa[kDirA], xb[kDirB];
-  __shared__ uint32_t wa[kDirT][kDirA], wb_[kDirT][kDirB];
-  const int Kd = counts[1];
+                 int n1, int n3, int64_t n, int64_t n2, const int32_t* __restrict__ dlist,
+                 const int32_t* __restrict__ counts, const uint32_t* __restrict__ hs, int d, int64_t b,
+                 double* __restrict__ cd, const DirectTerms* __restrict__ terms) {
+  __shared__ double val[kDirN];            // A's nonzeros, then B's
+  __shared__ int pos[kDirN];
+  __shared__ uint32_t hash[kDirT][kDirN];
+  const int Kd = counts[1], Kh = static_cast<int>(terms->heavy);
   const int tid = threadIdx.x;
   double up = 1.0;
   if (INT) {
-    if (Kd == 0 || terms->max_bits >= 0x7F800000u) return;   // the conversion writes NaN
+    if (Kd + Kh == 0 || terms->max_bits >= 0x7F800000u) return;   // the conversion writes NaN
     up = ldexp(1.0, term_shift(*terms));
   }
-  for (int q = blockIdx.x; q < Kd; q += gridDim.x) {
-    const int64_t k = dlist[q];
+  int q = blockIdx.x;                      // place in the list
+  int64_t ca = 0, cb = 0;                  // nonzeros of the piece's corner
+  __shared__ long long last[256], part[8];   // of 256 heavy ones: pieces up to each
+  int h0 = -256;
+  long long c = 0, total = 0, turn = 0;    // this block's next piece, pieces of these 256, and before them
+  for (;;) {
+    const bool light = q < Kd;
+    int64_t k;
+    if (light) {
+      k = dlist[q];
+    } else {
+      while (c >= total) {
+        turn += total;
+        h0 += 256;
+        if (h0 >= Kh) return;
+        long long pieces = 0;
+        if (h0 + tid < Kh) {
+          const int64_t kk = dlist[n2 - 1 - (h0 + tid)];
+          const int64_t na = a_ptr[kk + 1] - a_ptr[kk], nb = b_ptr[kk + 1] - b_ptr[kk];
+          const Piece pc = piece_of(na, nb);
+          pieces = (na + pc.a - 1) / pc.a * ((nb + pc.b - 1) / pc.b);
+        }
+        const int lane = tid & 31, warp = tid >> 5;
+        for (int o = 1; o < 32; o <<= 1) {
+          const long long y = __shfl_up_sync(0xFFFFFFFFu, pieces, o);
+          if (lane >= o) pieces += y;
+        }
+        __syncthreads();
+        if (lane == 31) part[warp] = pieces;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) pieces += part[w];
+        last[tid] = pieces;
+        __syncthreads();
+        total = last[255];
+        c = (static_cast<long long>(blockIdx.x) + gridDim.x - turn % gridDim.x) % gridDim.x;
+      }
+      int lo = 0, hi = 255;                // the first with last > c
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (last[mid] > c) hi = mid;
+        else lo = mid + 1;
+      }
+      k = dlist[n2 - 1 - (h0 + lo)];
+      ca = c - (lo > 0 ? last[lo - 1] : 0);   // the piece's number, for now
+    }
     const int64_t a0 = a_ptr[k], na = a_ptr[k + 1] - a0;
     const int64_t b0 = b_ptr[k], nb = b_ptr[k + 1] - b0;
-    for (int64_t ca = 0; ca < na; ca += kDirA) {
-      const int la = static_cast<int>(min(na - ca, static_cast<int64_t>(kDirA)));
-      for (int64_t cb = 0; cb < nb; cb += kDirB) {
-        const int lb = static_cast<int>(min(nb - cb, static_cast<int64_t>(kDirB)));
-        __syncthreads();
-        // an index outside the matrix marks its entry as none (-1)
-        if (tid < la) {
-          const int i = a_idx[a0 + ca + tid];
-          xa[tid] = i >= 0 && i < n1 ? i : -1;
-          va[tid] = val_f64<T>(a_val, a0 + ca + tid) * up;
-        } else if (tid >= kDirB && tid - kDirB < lb) {
-          const int j = b_idx[b0 + cb + tid - kDirB];
-          xb[tid - kDirB] = j >= 0 && j < n3 ? j : -1;
-          vb[tid - kDirB] = val_f64<T>(b_val, b0 + cb + tid - kDirB);
+    const Piece pc = piece_of(na, nb);
+    if (!light) {
+      const int64_t per = (nb + pc.b - 1) / pc.b, x = ca;
+      ca = x / per * pc.a;
+      cb = x % per * pc.b;
+    }
+    const int la = static_cast<int>(min(na - ca, static_cast<int64_t>(pc.a)));
+    const int lb = static_cast<int>(min(nb - cb, static_cast<int64_t>(pc.b)));
+    __syncthreads();
+    for (int e = tid; e < la + lb; e += 256) {
+      // an index outside the matrix marks its entry as none (-1)
+      if (e < la) {
+        const int i = a_idx[a0 + ca + e];
+        pos[e] = i >= 0 && i < n1 ? i : -1;
+        val[e] = val_f64<T>(a_val, a0 + ca + e) * up;
+      } else {
+        const int j = b_idx[b0 + cb + e - la];
+        pos[e] = j >= 0 && j < n3 ? j : -1;
+        val[e] = val_f64<T>(b_val, b0 + cb + e - la);
+      }
+    }
+    __syncthreads();
+    for (int t0 = 0; t0 < d; t0 += kDirT) {
+      const int lt = min(kDirT, d - t0);
+      if (t0 > 0) __syncthreads();
+      for (int e = tid; e < lt * (la + lb); e += 256) {
+        const int t = e / (la + lb), x = e - t * (la + lb);
+        const uint32_t* row = hs + (static_cast<size_t>(t0 + t) * 2 + (x < la ? 0 : 1)) * n;
+        hash[t][x] = pos[x] >= 0 ? row[pos[x]] : 0;
+      }
+      __syncthreads();
+      for (int e = tid; e < la * lb; e += 256) {
+        const int i = e / lb, j = la + e - i * lb;
+        if (pos[i] < 0 || pos[j] < 0) continue;
+        // once per pair: FP64 arithmetic is slow beside the additions
+        const double v = val[i] * val[j];
+        const long long iv = INT ? __double2ll_rn(v) : 0;
+        for (int t = 0; t < lt; ++t) {
+          const uint32_t w1 = hash[t][i], w2 = hash[t][j];
+          uint32_t z = (w1 & kBucketMask) + (w2 & kBucketMask);
+          if (z >= static_cast<uint32_t>(b)) z -= static_cast<uint32_t>(b);
+          const bool neg = ((w1 ^ w2) >> 31) != 0;
+          double* dst = cd + static_cast<size_t>(t0 + t) * b + z;
+          if (INT) atomicAdd(reinterpret_cast<unsigned long long*>(dst), static_cast<unsigned long long>(neg ? -iv : iv));
+          else atomicAdd(dst, neg ? -v : v);
         }
-        __syncthreads();
-        for (int t0 = 0; t0 < d; t0 += kDirT) {
-          const int lt = min(kDirT, d - t0);
-          if (t0 > 0) __syncthreads();
-          for (int e = tid; e < lt * (la + lb); e += 256) {
-            const int t = e / (la + lb), x = e - t * (la + lb);
-            const uint32_t* row = hs + static_cast<size_t>(t0 + t) * 2 * n;
-            if (x < la) wa[t][x] = xa[x] >= 0 ? row[xa[x]] : 0;
-            else wb_[t][x - la] = xb[x - la] >= 0 ? row[n + xb[x - la]] : 0;
-          }
-          __syncthreads();
-          for (int e = tid; e < la * lb; e += 256) {
-            const int i = e / lb, j = e - i * lb;
-            if (xa[i] < 0 || xb[j] < 0) continue;
-            // once per pair: FP64 arithmetic is slow beside the additions
-            const double v = va[i] * vb[j];
-            const long long iv = INT ? __double2ll_rn(v) : 0;
-            for (int t = 0; t < lt; ++t) {
-              const uint32_t w1 = wa[t][i], w2 = wb_[t][j];
-              uint32_t z = (w1 & kBucketMask) + (w2 & kBucketMask);
-              if (z >= static_cast<uint32_t>(b)) z -= static_cast<uint32_t>(b);
-              const bool neg = ((w1 ^ w2) >> 31) != 0;
-              double* dst = cd + static_cast<size_t>(t0 + t) * b + z;
-              if (INT) atomicAdd(reinterpret_cast<unsigned long long*>(dst), static_cast<unsigned long long>(neg ? -iv : iv));
-              else atomicAdd(dst, neg ? -v : v);
-            }
-          }
-        }
+      }
+    }
+    if (!light) {
+      c += gridDim.x;
+    } else if ((cb += pc.b) >= nb) {
+      cb = 0;
+      if ((ca += pc.a) >= na) {
+        ca = 0;
+        q += gridDim.x;
       }
     }
   }
@@ -616,7 +700,7 @@ __global__ void k_add_direct(float* __restrict__ c, const double* __restrict__ c
   int shift = 0;
   bool bad = false;
   if (INT) {
-    if (counts[1] == 0 && fft) return;
+    if (terms->terms == 0 && fft) return;
     bad = terms->max_bits >= 0x7F800000u;
     shift = term_shift(*terms);
   }
@@ -728,22 +812,23 @@ cudaError_t launch_nonempty_split(const cms_hashes* h, const SparseArgsHost& in,
   if (dt == CMS_F32) count(static_cast<float*>(nullptr));
   else if (dt == CMS_BF16) count(static_cast<__nv_bfloat16*>(nullptr));
   else count(static_cast<double*>(nullptr));
-  k_split_write<<<g, 1024, 0, s>>>(in.a_ptr, in.b_ptr, n2, limit, chunk, scratch, flist, dlist, counts);
+  k_split_write<<<g, 1024, 0, s>>>(in.a_ptr, in.b_ptr, n2, limit, chunk, scratch, flist, dlist, counts,
+                                   direct_terms(h, cd));
   return cudaGetLastError();
 }
 
 cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer,
                                   const int32_t* dlist, const int32_t* counts, int64_t n2, double* cd, cudaStream_t s) {
   if (n2 <= 0) return cudaSuccess;
-  // the list length is on the device: blocks stride over it and those past
-  // its end return at once
-  const unsigned grid = static_cast<unsigned>(std::min<int64_t>(n2, 152 * 8));
+  // the lists' lengths are on the device: blocks stride over them, and return
+  // at once when they are empty
+  const unsigned grid = 152 * 8;
   ProfScope prof_scope("k_direct_scatter", s);
   auto go = [&](auto* tag, auto integer_tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
     k_direct_scatter<T, decltype(integer_tag)::value><<<grid, 256, 0, s>>>(
         in.a_ptr, in.a_idx, static_cast<const T*>(in.a_val), in.b_ptr, in.b_idx, static_cast<const T*>(in.b_val),
-        in.n1, in.n3, h->n, dlist, counts, h->d_hs, h->d, h->b, cd, direct_terms(h, cd));
+        in.n1, in.n3, h->n, n2, dlist, counts, h->d_hs, h->d, h->b, cd, direct_terms(h, cd));
   };
   auto both = [&](auto* tag) {
     if (integer) go(tag, std::true_type{});

@@ -62,11 +62,13 @@ namespace {
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
-std::string tune_key(const cms_instance& it, const SketchPlan& p, int sms, bool direct = false) {
+// direct: the key of the choice between the direct route and the others (its
+// own plan knows whether A = X^T, B = X for every storage type).
+std::string tune_key(const cms_instance& it, const SketchPlan& p, int sms, const DirectPlan* direct = nullptr) {
   std::ostringstream k;
   k << "b=" << p.b << ",n1=" << it.n1 << ",n2=" << it.n2 << ",n3=" << it.n3 << ",dt=" << it.dt
     << ",d=" << p.d << ",sms=" << sms << ",kernel=" << (direct ? "direct" : p.fast ? "fast" : "generic")
-    << (p.alias ? "-alias" : "");
+    << ((direct ? direct->alias : p.alias) ? "-alias" : "");
   return k.str();
 }
 
@@ -136,20 +138,15 @@ cms_status cuda_fail(cudaError_t e, const char* where) {
   return CMS_ERR_CUDA;
 }
 
-// Time one configuration of one instance with the single-instance launch
-// (on the direct route when `direct` is given).
-cudaError_t time_plan(const SketchPlan& p, const cms_instance& it, char* ws, cudaStream_t s, double* ms,
-                      const DirectPlan* direct = nullptr) {
+// Time of one pass of f, after a first one.
+template <typename F>
+cudaError_t time_passes(F f, cudaStream_t s, double* ms) {
   cudaEvent_t a = nullptr, b = nullptr;
   cudaError_t e = cudaEventCreate(&a);
   if (e == cudaSuccess) e = cudaEventCreate(&b);
-  auto once = [&]() {
-    return direct ? launch_direct(*direct, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, it.c, ws, s)
-                  : launch_sketch(p, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, it.c, ws, s);
-  };
-  if (e == cudaSuccess) e = once();  // warm-up
+  if (e == cudaSuccess) e = f();  // warm-up
   if (e == cudaSuccess) e = cudaEventRecord(a, s);
-  for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = once();
+  for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = f();
   if (e == cudaSuccess) e = cudaEventRecord(b, s);
   if (e == cudaSuccess) e = cudaEventSynchronize(b);
   float t = 0.f;
@@ -157,6 +154,41 @@ cudaError_t time_plan(const SketchPlan& p, const cms_instance& it, char* ws, cud
   *ms = t / 2.0;
   if (a) cudaEventDestroy(a);
   if (b) cudaEventDestroy(b);
+  return e;
+}
+
+// One configuration of one instance with the single-instance launch.
+cudaError_t time_plan(const SketchPlan& p, const cms_instance& it, char* ws, cudaStream_t s, double* ms) {
+  return time_passes(
+      [&]() { return launch_sketch(p, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, it.c, ws, s); }, s, ms);
+}
+
+// One instance on the direct route in the form that the batch runs it (units of
+// two tiles whose entries are added as they leave the tensor cores).
+cudaError_t time_direct(const DirectPlan& d, const SketchPlan& p, const cms_instance& it, char* ws, int sms,
+                        cudaStream_t s, double* ms) {
+  void* args = nullptr;
+  void* inv = nullptr;
+  DirectBatch batch;
+  InverseBatch inverse;
+  const std::vector<DirectSpec> specs{DirectSpec{d, it.h, it.A, it.lda, it.B, it.ldb, it.n1, it.n2, it.n3, it.dt, ws}};
+  const std::vector<InverseSpec> convert{InverseSpec{reinterpret_cast<unsigned long long*>(ws + d.off_acc), d.copies,
+                                                     reinterpret_cast<const DirectScale*>(ws + d.off_scale),
+                                                     direct_scale_log2(d.split), &p, nullptr, nullptr, nullptr, nullptr,
+                                                     it.c}};
+  cudaError_t e = cudaMalloc(&args, direct_batch_bytes(1, sms));
+  if (e == cudaSuccess) e = cudaMalloc(&inv, inverse_batch_bytes(1));
+  if (e == cudaSuccess) e = build_direct_batch(specs, sms, args, &batch, s);
+  if (e == cudaSuccess) e = build_inverse_batch(convert, inv, &inverse, s);
+  if (e == cudaSuccess)
+    e = time_passes(
+        [&]() {
+          const cudaError_t x = launch_direct_batched(batch, s);
+          return x != cudaSuccess ? x : launch_inverse_batched(inverse, s);
+        },
+        s, ms);
+  if (args) cudaFree(args);
+  if (inv) cudaFree(inv);
   return e;
 }
 
@@ -251,26 +283,24 @@ cms_status cms_batch_create(const cms_instance* items, int32_t count, int32_t fl
     if (!b->is_direct[i]) continue;
     // the direct route has no tiles to tune: the cache holds whether it was
     // the faster route (nkc = 0), else the transform route's chunks
-    auto hit = cache.find(tune_key(it, p, sms, true));
+    auto hit = cache.find(tune_key(it, p, sms, &b->direct[i]));
     if (hit != cache.end()) {
       b->is_direct[i] = hit->second.nkc == 0;
     } else if (flags & CMS_BATCH_AUTOTUNE) {
       char* tws = nullptr;
-      // (the batch's own plan leaves the tile kernel's words to the batch)
-      const DirectPlan one = make_direct_plan(it.h, it.n1, it.n2, it.n3, it.dt, b->direct[i].alias, sms, 1, false);
-      cudaError_t e = cudaMalloc(&tws, std::max<size_t>(std::max(p.ws_bytes, one.ws_bytes), 256));
+      cudaError_t e = cudaMalloc(&tws, std::max<size_t>(std::max(p.ws_bytes, b->direct[i].ws_bytes), 256));
       if (e == cudaErrorMemoryAllocation) {   // no room for the packed operands
         cudaGetLastError();
         b->is_direct[i] = 0;
         continue;
       }
       double td = 0.0, tt = 0.0;
-      if (e == cudaSuccess) e = time_plan(p, it, tws, s, &td, &one);
+      if (e == cudaSuccess) e = time_direct(b->direct[i], p, it, tws, sms, s, &td);
       if (e == cudaSuccess) e = time_plan(p, it, tws, s, &tt);
       if (tws) cudaFree(tws);
       if (e != cudaSuccess) { delete b; return cuda_fail(e, "cms_batch_create (autotune)"); }
       b->is_direct[i] = td <= tt;
-      cache[tune_key(it, p, sms, true)] = Tuned{td <= tt ? 0 : p.nkc, 0, std::min(td, tt)};
+      cache[tune_key(it, p, sms, &b->direct[i])] = Tuned{td <= tt ? 0 : p.nkc, 0, std::min(td, tt)};
       cache_dirty = true;
     }
   }

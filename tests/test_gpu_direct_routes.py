@@ -164,3 +164,32 @@ def test_significant_workspace_stays_bounded(cms, monkeypatch):
     assert "k_mask_copy" in kernels and "k_direct_tile" not in kernels and asked[1] < asked[0]
     assert again == count and torch.equal(got, want)
     h.free()
+
+
+def test_tuned_route_of_a_batch_knows_aliased_operands(cms, tmp_path):
+    # FP64 storage: X^T X packs one operand and skips half of the tiles, so that its
+    # tuned route is not that of two operands of the same shape
+    n, m, b, d = 640, 1280, 10240, 2
+    x = torch.randn((m, n), device="cuda", dtype=torch.float64)
+    y = torch.randn((m, n), device="cuda", dtype=torch.float64)
+    hs = [cms.make_hashes(q, n, b, d) for q in range(2)]
+    items = [(x.T, x, hs[0]), (x.T, y, hs[1])]
+    cache = tmp_path / "tune.txt"
+    batch = cms.Batch(items, autotune=True, tune_cache=str(cache))
+    want, _ = kernels_of(cms, batch.run)
+    want = [c.clone() for c in want]
+    lines = [ln for ln in cache.read_text().splitlines() if "kernel=direct" in ln]
+    assert sorted(ln.split()[0].endswith("-alias") for ln in lines) == [False, True]
+    # each key decides for its own instance (a count of chunks: the transform route)
+    tuned = [ln.split()[0] + (" 3 0 1.0" if "-alias" in ln else " 0 0 1.0") for ln in lines]
+    cache.write_text("\n".join(tuned) + "\n")
+    again = cms.Batch(items, tune_cache=str(cache))
+    out, kernels = kernels_of(cms, again.run)
+    assert "k_direct_tile_batched" in kernels and "k_sketch_batched" in kernels
+    assert kernels["k_direct_balance_batched"]["launches"] == 1      # the two operands, by the tiles
+    for c, w in zip(out, want):
+        assert ((c - w).norm() / w.norm()).item() < 1e-5
+    batch.free()
+    again.free()
+    for h in hs:
+        h.free()

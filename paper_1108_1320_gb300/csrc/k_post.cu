@@ -29,7 +29,9 @@ template <> __device__ __forceinline__ double to_f64<__nv_bfloat16>(__nv_bfloat1
 // The sum of A_ik B_ki over k = k0, k0 + step, ...: FP64 storage in FP64, FP32
 // and BF16 storage as the sum and its error in FP32 (products split by a fused
 // multiply-add, additions by Knuth's two-sum; 48 bits, of which the sketch
-// keeps 24), in FP64 where a value leaves FP32's range on the way.
+// keeps 24), in FP64 where a value leaves FP32's range on the way: an infinity,
+// or a sum so small that products may have underflowed (each loses at most 2^-149
+// then, 2^31 of them 2^-118).
 template <typename T>
 __device__ __forceinline__ double diag_part(const T* A, int64_t lda, const T* B, int64_t ldb, int64_t k0, int64_t n2,
                                             int64_t step) {
@@ -43,7 +45,13 @@ __device__ __forceinline__ double diag_part(const T* A, int64_t lda, const T* B,
       e += ((s - (t - v)) + (p - v)) + pe;
       s = t;
     }
-    if (isfinite(s) && isfinite(e)) return static_cast<double>(s) + static_cast<double>(e);
+    if (fabsf(s) >= 0x1p-70f && isfinite(s) && isfinite(e)) return static_cast<double>(s) + static_cast<double>(e);
+    if (s == 0.f && e == 0.f) {   // nothing to add, or all of it underflowed
+      bool any = false;
+#pragma unroll 8
+      for (int64_t k = k0; k < n2; k += step) any |= to_f32(A[k * lda]) != 0.f && to_f32(B[k * ldb]) != 0.f;
+      if (!any) return 0.0;
+    }
   }
   double s = 0.0;
 #pragma unroll 4

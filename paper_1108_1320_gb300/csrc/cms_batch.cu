@@ -135,6 +135,7 @@ cms_status fail(cms_status s, const std::string& msg) {
 
 cms_status cuda_fail(cudaError_t e, const char* where) {
   set_error(std::string(where) + ": " + cudaGetErrorString(e));
+  cudaGetLastError();   // a refused launch is not the next call's error
   return CMS_ERR_CUDA;
 }
 

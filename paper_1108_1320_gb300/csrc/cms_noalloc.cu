@@ -99,6 +99,7 @@ cms_status cms_sketch_product_noalloc(const void* A, int64_t lda, const void* B,
                           static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) {
     set_error(std::string("cms_sketch_product_noalloc: ") + cudaGetErrorString(e));
+    cudaGetLastError();
     return CMS_ERR_CUDA;
   }
   return CMS_OK;

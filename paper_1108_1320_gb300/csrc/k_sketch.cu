@@ -427,11 +427,13 @@ int make_sketch_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, in
     const size_t sm_ws = ws_smem_bytes(p.npad, h->fe_ecap, p.alias ? 1 : 0, p.tw_shift, p.nhi, ovcap);
     const bool ws_ok = allow_ws && dt == CMS_F32 && !p.unal && p.C == kFeC && ovcap >= 64 &&
                        sm_ws <= smem_optin && ws_kernel_usable();
+    // (the lock-step kernels' static shared variables come on top: 128 bytes)
+    const size_t room = smem_optin - std::min<size_t>(smem_optin, 128);
     // the front-end records hold staging indices (< 3 npad) in 16 bits
-    if ((sm <= smem_optin || ws_ok || sm_tm <= smem_optin) && 3 * static_cast<int64_t>(p.npad) <= 65535) {
+    if ((sm <= room || ws_ok || sm_tm <= room) && 3 * static_cast<int64_t>(p.npad) <= 65535) {
       p.fast = true;
       p.ws = ws_ok;
-      p.tmem_rec = !ws_ok && sm > smem_optin;
+      p.tmem_rec = !ws_ok && sm > room;
       p.ovcap = ws_ok ? ovcap : 0;
       p.G = 2;
       p.threads = ws_ok ? 512 : 256;

@@ -127,3 +127,34 @@ def test_smallest_normal_values_times_large_ones(cms, e, n1, n2, n3, b):
         assert "k_direct_tile" in kernels
         assert worst(c, O.sketch_definition(Ad, Xd, O.make_tables(5, max(n1, n3), b, 2))) < TOL
         h.free()
+
+
+@pytest.mark.parametrize("n1,n2,n3,b,kernel", [(300, 500, 260, 16384, "k_direct_grid"), (1400, 200, 1200, 20000, "k_direct_window"),
+                                               (6000, 400, 5000, 1536, "k_pre_pack")])
+def test_two_operands_replayed_from_a_graph(cms, n1, n2, n3, b, kernel):
+    # the balance, the packing and what follows them overlap at their ends; a graph
+    # keeps that, on new values in the same buffers
+    A, B, Ad, Bd = scaled(n1, n2, n3, "f32", 20, 5)
+    h = cms.make_hashes(5, max(n1, n3), b, 2)
+    ws = cms.alloc_workspace(cms.workspace_size(h, n1, n2, n3))
+    c = torch.empty((2, b), device="cuda")
+    cms.profile_enable(True)
+    cms.sketch_product(A, B, h, c=c, ws=ws)
+    torch.cuda.synchronize()
+    assert kernel in cms.profile_summary()
+    cms.profile_enable(False)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        cms.sketch_product(A, B, h, c=c, ws=ws, stream=torch.cuda.current_stream())
+    C, D, Cd, Dd = scaled(n1, n2, n3, "f32", 20, 6)
+    ref = O.sketch_definition(Cd, Dd, O.make_tables(5, max(n1, n3), b, 2))
+    A.copy_(C)
+    B.copy_(D)
+    for _ in range(3):
+        c.zero_()
+        ws.fill_(0x7F)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert worst(c, ref) < TOL
+    cms.check_async()
+    h.free()

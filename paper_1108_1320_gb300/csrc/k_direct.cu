@@ -416,7 +416,6 @@ struct PreArgs {
   int alias;
   int64_t K;
   int nsb, d;
-  int strips;             // of 32 columns
   int hn;                 // hash domain
   int R, C, classes, tiles;   // classes of R buckets per tile of 128 rows
   float* slab[2];         // [superblock][n][128]
@@ -434,15 +433,12 @@ struct PreArgs {
 template <typename T>
 __global__ void __launch_bounds__(256) k_pre_transpose(const PreArgs p) {
   __shared__ float sh[kSuper][33];
-  // strips of 32 columns fastest; superblocks in x as well, which alone has no
-  // limit of 65535 (8388480 inner indices)
   const int side = blockIdx.z;
-  const int strip = static_cast<int>(blockIdx.x) % p.strips, sb = static_cast<int>(blockIdx.x) / p.strips;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t i = static_cast<int64_t>(strip) * 32 + lane;
-  const int64_t k0 = static_cast<int64_t>(sb) * kSuper;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * 32 + lane;
+  const int64_t k0 = static_cast<int64_t>(blockIdx.y) * kSuper;
   wait_for_kernel_before();
-  if (static_cast<int64_t>(strip) * 32 >= p.n[side]) return;
+  if (static_cast<int64_t>(blockIdx.x) * 32 >= p.n[side]) return;
   const T* X = static_cast<const T*>(p.X[side]);
 #pragma unroll
   for (int q = 0; q < kSuper / 8; ++q) {
@@ -455,9 +451,9 @@ __global__ void __launch_bounds__(256) k_pre_transpose(const PreArgs p) {
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int x = q * 8 + warp;
-    const int64_t xi = static_cast<int64_t>(strip) * 32 + x;
+    const int64_t xi = static_cast<int64_t>(blockIdx.x) * 32 + x;
     if (xi >= p.n[side]) continue;
-    float* dst = p.slab[side] + (static_cast<size_t>(sb) * p.n[side] + xi) * kSuper;
+    float* dst = p.slab[side] + (static_cast<size_t>(blockIdx.y) * p.n[side] + xi) * kSuper;
 #pragma unroll
     for (int g = 0; g < 4; ++g) dst[g * 32 + lane] = sh[g * 32 + lane][x];
   }
@@ -1449,7 +1445,6 @@ cudaError_t launch_pre(const DirectPlan& chosen, const cms_hashes* h, const void
   a.alias = alias ? 1 : 0;
   a.K = n2;
   a.nsb = p.nsb;
-  a.strips = static_cast<int>((std::max(n1, n3) + 31) / 32);
   a.d = h->d;
   a.hn = static_cast<int>(h->n);
   a.R = q.R; a.C = q.C; a.classes = q.classes; a.tiles = q.tiles;
@@ -1468,17 +1463,29 @@ cudaError_t launch_pre(const DirectPlan& chosen, const cms_hashes* h, const void
   if (e != cudaSuccess) return e;
   {
     ProfScope prof_scope("k_pre_transpose", s);
-    const dim3 grid(static_cast<unsigned>(a.strips * p.nsb), 1, alias ? 1 : 2);
     void (*const kern)(const PreArgs) = dt == CMS_BF16  ? k_pre_transpose<__nv_bfloat16>
                                         : dt == CMS_F64 ? k_pre_transpose<double>
                                                         : k_pre_transpose<float>;
-    if (alias) {
-      kern<<<grid, 256, 0, s>>>(a);
-      e = cudaGetLastError();
-    } else {
-      e = launch_after(kern, grid, 256, 0, s, a);
+    // 65535 superblocks a launch, the limit of y (8388480 inner indices)
+    const int64_t esz = dt == CMS_BF16 ? 2 : dt == CMS_F64 ? 8 : 4;
+    for (int first = 0; first < p.nsb; first += 65535) {
+      PreArgs part = a;
+      const int64_t k0 = static_cast<int64_t>(first) * kSuper;
+      for (int side = 0; side < 2; ++side) {
+        part.X[side] = static_cast<const char*>(a.X[side]) + k0 * a.ld[side] * esz;
+        part.slab[side] = a.slab[side] + k0 * a.n[side];
+      }
+      if (a.bal != nullptr) part.bal = a.bal + k0;
+      part.K = n2 - k0;
+      const dim3 grid(static_cast<unsigned>((std::max(n1, n3) + 31) / 32), std::min(p.nsb - first, 65535), alias ? 1 : 2);
+      if (alias) {
+        kern<<<grid, 256, 0, s>>>(part);
+        e = cudaGetLastError();
+      } else {
+        e = launch_after(kern, grid, 256, 0, s, part);
+      }
+      if (e != cudaSuccess) return e;
     }
-    if (e != cudaSuccess) return e;
   }
   {
     ProfScope prof_scope("k_pre_lists", s);

@@ -36,9 +36,11 @@ def test_programmatic_launches_read_results_past_the_read_only_path(name, path):
         assert READ_ONLY.match(arg), arg
 
 
-def test_superblocks_are_not_counted_in_a_limited_grid_dimension():
+def test_superblocks_are_counted_within_a_grid_dimension():
     # a grid's y and z end at 65535: inner indices by the 128 pass that at 8.4 M
     with open(os.path.join(CSRC, "k_direct.cu")) as f:
         src = f.read()
-    assert not re.search(r"blockIdx\.[yz]\)?\s*\*\s*kSuper", src)
-    assert not re.search(r"dim3\([^;]*,\s*p\.nsb\s*,", src)
+    for dims in re.findall(r"dim3 \w+\(([^;]*)\);|dim3\(([^;]*)\)", src):
+        y = (dims[0] or dims[1]).split(",", 1)
+        if len(y) == 2 and "nsb" in y[1]:
+            assert "65535)" in y[1]

@@ -125,6 +125,42 @@ def _stream(stream) -> int:
     return int(stream)
 
 
+def _other(stream):
+    """The stream of a call when it is not the current one, else None."""
+    if stream is None or _stream(stream) == torch.cuda.current_stream().cuda_stream:
+        return None
+    return stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(int(stream))
+
+
+def _scratch(nbytes: int, device, stream) -> torch.Tensor:
+    """A workspace in the order of ``stream`` (the caching allocator gives a
+    block to the next user in the order of the stream it came from)."""
+    s = _other(stream)
+    if s is None:
+        return alloc_workspace(nbytes, device)
+    with torch.cuda.stream(s):
+        return alloc_workspace(nbytes, device)
+
+
+def _empty(shape, dtype, device, stream) -> torch.Tensor:
+    """An output that a call on ``stream`` writes and the caller keeps."""
+    s = _other(stream)
+    if s is None:
+        return torch.empty(shape, dtype=dtype, device=device)
+    with torch.cuda.stream(s):
+        out = torch.empty(shape, dtype=dtype, device=device)
+    out.record_stream(torch.cuda.current_stream())
+    return out
+
+
+def _read(t: torch.Tensor, stream):
+    """The number that a call on ``stream`` leaves in t."""
+    s = _other(stream)
+    if s is not None:
+        s.synchronize()
+    return t.item()
+
+
 def _ptr(t: torch.Tensor | None) -> int | None:
     return None if t is None else t.data_ptr()
 
@@ -225,10 +261,10 @@ def _check_buf(t, name: str, device, dtype=None, numel: int = 0) -> None:
         raise ValueError(f"{name} holds {t.numel()} elements, {numel} are needed")
 
 
-def _sketch_out(c, h: "Hashes", device, dtype=torch.float32):
+def _sketch_out(c, h: "Hashes", device, stream, dtype=torch.float32):
     inf = h.info()
     if c is None:
-        return torch.empty((inf["d"], inf["b"]), dtype=dtype, device=device)
+        return _empty((inf["d"], inf["b"]), dtype, device, stream)
     _check_buf(c, "c", device, dtype, inf["d"] * inf["b"])
     return c
 
@@ -274,13 +310,13 @@ def sketch_product(A: torch.Tensor, B: torch.Tensor, h: Hashes, c: torch.Tensor 
     ``ws`` is scratch of workspace_size() bytes, allocated here when None (of
     the smallest size when the device has no room for more)."""
     n1, n2, n3, lda, ldb = _ab_args(A, B)
-    c = _sketch_out(c, h, A.device)
+    c = _sketch_out(c, h, A.device, stream)
     need = workspace_size(h, n1, n2, n3, A.dtype)
     if ws is None:
         try:
-            ws = alloc_workspace(need, A.device)
+            ws = _scratch(need, A.device, stream)
         except torch.cuda.OutOfMemoryError:
-            ws = alloc_workspace(workspace_size(h, n1, n2, n3, A.dtype, smallest=True), A.device)
+            ws = _scratch(workspace_size(h, n1, n2, n3, A.dtype, smallest=True), A.device, stream)
     _check_buf(ws, "ws", A.device)
     _check(lib().cms_sketch_product(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, _DTYPES[A.dtype], h.handle,
                                     _ptr(c), _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)))
@@ -306,7 +342,7 @@ def sketch_product_noalloc(A: torch.Tensor, B: torch.Tensor, h: Hashes,
     (shared by all calls on the device; calls overlapping on the GPU race).
     Returns c, float32 (d, b)."""
     n1, n2, n3, lda, ldb = _ab_args(A, B)
-    c = _sketch_out(c, h, A.device)
+    c = _sketch_out(c, h, A.device, stream)
     _check(lib().cms_sketch_product_noalloc(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, _DTYPES[A.dtype],
                                             h.handle, _ptr(c), _stream(stream)))
     return c
@@ -344,9 +380,9 @@ def sketch_product_csr(a_colptr: torch.Tensor, a_rowidx: torch.Tensor, a_val: to
     for t_, nm in ((a_rowidx, "a_rowidx"), (b_rowptr, "b_rowptr"), (b_colidx, "b_colidx"), (a_val, "a_val"),
                    (b_val, "b_val")):
         _check_buf(t_, nm, dev)
-    c = _sketch_out(c, h, dev)
+    c = _sketch_out(c, h, dev, stream)
     if ws is None:
-        ws = alloc_workspace(sparse_workspace_size(h, n1, n2, n3), dev)
+        ws = _scratch(sparse_workspace_size(h, n1, n2, n3), dev, stream)
     _check_buf(ws, "ws", dev)
     if direct_max_pairs is None:
         _check(lib().cms_sketch_product_csr(_ptr(a_colptr), _ptr(a_rowidx), _ptr(a_val), _ptr(b_rowptr),
@@ -432,9 +468,9 @@ def sketch_product_plain_f64(A: torch.Tensor, B: torch.Tensor, h: Hashes,
     n1, n2, n3, lda, ldb = _ab_args(A, B)
     if A.dtype != torch.float64:
         raise ValueError("the plain path takes float64 A and B")
-    c = _sketch_out(c, h, A.device, torch.float64)
+    c = _sketch_out(c, h, A.device, stream, torch.float64)
     if ws is None:
-        ws = alloc_workspace(plain_workspace_size(h, n1, n2, n3), A.device)
+        ws = _scratch(plain_workspace_size(h, n1, n2, n3), A.device, stream)
     _check_buf(ws, "ws", A.device)
     _check(lib().cms_sketch_product_plain_f64(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, h.handle,
                                               _ptr(c), _ptr(ws), ws.numel() * ws.element_size(),
@@ -456,7 +492,7 @@ def decode(c: torch.Tensor, h: Hashes, ij: torch.Tensor, out: torch.Tensor | Non
     _check_buf(c, "c", c.device, c.dtype, inf["d"] * inf["b"])
     _check_buf(ij, "ij", c.device)
     if out is None:
-        out = torch.empty(q, dtype=c.dtype, device=c.device)
+        out = _empty(q, c.dtype, c.device, stream)
     _check_buf(out, "out", c.device, c.dtype, q)
     if c.dtype == torch.float64:
         _check(lib().cms_decode_f64(_ptr(c), h.handle, _ptr(ij), q, _ptr(out), _stream(stream)))
@@ -474,7 +510,7 @@ def decode_dense(c: torch.Tensor, h: Hashes, n1: int, n3: int, out: torch.Tensor
     inf = h.info()
     _check_buf(c, "c", c.device, torch.float32, inf["d"] * inf["b"])
     if out is None:
-        out = torch.empty((n1, n3), dtype=torch.float32, device=c.device)
+        out = _empty((n1, n3), torch.float32, c.device, stream)
     if (not isinstance(out, torch.Tensor) or not out.is_cuda or out.device != c.device
             or out.dtype != torch.float32 or out.dim() != 2 or tuple(out.shape) != (n1, n3)
             or (n3 > 1 and out.stride(1) != 1)):
@@ -504,20 +540,20 @@ def decode_threshold(c: torch.Tensor, h: Hashes, n1: int, n3: int, tau: float, s
     c = c.contiguous()
     inf = h.info()
     _check_buf(c, "c", dev, torch.float32, inf["d"] * inf["b"])
-    ij = torch.empty((max(capacity, 1), 2), dtype=torch.int64, device=dev)
-    val = torch.empty(max(capacity, 1), dtype=torch.float32, device=dev)
-    cnt = torch.zeros(1, dtype=torch.int64, device=dev)
-    ws = torch.empty(n1 + 1, dtype=torch.int64, device=dev)
+    ij = _empty((max(capacity, 1), 2), torch.int64, dev, stream)
+    val = _empty(max(capacity, 1), torch.float32, dev, stream)
+    cnt = _empty(1, torch.int64, dev, stream)
+    ws = _scratch(8 * (n1 + 1), dev, stream)
     _check(lib().cms_decode_threshold(_ptr(c), h.handle, n1, n3, float(tau), 1 if skip_diagonal else 0,
-                                      _ptr(ij), _ptr(val), capacity, _ptr(cnt), _ptr(ws), ws.numel() * 8,
+                                      _ptr(ij), _ptr(val), capacity, _ptr(cnt), _ptr(ws), ws.numel(),
                                       _stream(stream)))
-    q = int(cnt.item())
+    q = int(_read(cnt, stream))
     k = min(q, capacity)
     return ij[:k], val[:k], q
 
 
-def _sorted_positions(ij: torch.Tensor, count: torch.Tensor, capacity: int):
-    q = int(count.item())
+def _sorted_positions(ij: torch.Tensor, count: torch.Tensor, capacity: int, stream):
+    q = int(_read(count, stream))
     out = ij[:min(q, capacity)]
     if out.shape[0] > 1:
         order = torch.argsort(out[:, 0] * (int(out[:, 1].max()) + 1) + out[:, 1])
@@ -533,17 +569,17 @@ def find_significant(A: torch.Tensor, B: torch.Tensor, h: Hashes, delta: float, 
     need = _SZ()
     _check(lib().cms_significant_workspace_size(h.handle, n1, n2, n3, _DTYPES[A.dtype], rho, ctypes.byref(need)))
     try:
-        ws = alloc_workspace(need.value, A.device)
+        ws = _scratch(need.value, A.device, stream)
     except torch.cuda.OutOfMemoryError:
         _check(lib().cms_significant_workspace_size_min(h.handle, n1, n2, n3, _DTYPES[A.dtype], rho,
                                                         ctypes.byref(need)))
-        ws = alloc_workspace(need.value, A.device)
-    ij = torch.empty((max(capacity, 1), 2), dtype=torch.int64, device=A.device)
-    cnt = torch.zeros(1, dtype=torch.int64, device=A.device)
+        ws = _scratch(need.value, A.device, stream)
+    ij = _empty((max(capacity, 1), 2), torch.int64, A.device, stream)
+    cnt = _empty(1, torch.int64, A.device, stream)
     _check(lib().cms_find_significant(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, _DTYPES[A.dtype], h.handle,
                                       float(delta), rho, _ptr(ij), capacity, _ptr(cnt), _ptr(ws),
                                       ws.numel() * ws.element_size(), _stream(stream)))
-    return _sorted_positions(ij, cnt, capacity)
+    return _sorted_positions(ij, cnt, capacity, stream)
 
 
 def decode_significant(sketches: torch.Tensor, h: Hashes, n1: int, n3: int, delta: float, rho: int = 1,
@@ -556,13 +592,13 @@ def decode_significant(sketches: torch.Tensor, h: Hashes, n1: int, n3: int, delt
     _check_buf(sketches, "sketches", sketches.device, torch.float32)
     need = _SZ()
     _check(lib().cms_significant_decode_workspace_size(h.handle, ctypes.byref(need)))
-    ws = alloc_workspace(need.value, sketches.device)
-    ij = torch.empty((max(capacity, 1), 2), dtype=torch.int64, device=sketches.device)
-    cnt = torch.zeros(1, dtype=torch.int64, device=sketches.device)
+    ws = _scratch(need.value, sketches.device, stream)
+    ij = _empty((max(capacity, 1), 2), torch.int64, sketches.device, stream)
+    cnt = _empty(1, torch.int64, sketches.device, stream)
     _check(lib().cms_decode_significant(_ptr(sketches), h.handle, n1, n3, float(delta), rho, _ptr(ij),
                                         capacity, _ptr(cnt), _ptr(ws), ws.numel() * ws.element_size(),
                                         _stream(stream)))
-    return _sorted_positions(ij, cnt, capacity)
+    return _sorted_positions(ij, cnt, capacity, stream)
 
 
 def nnz_estimate(a_colptr: torch.Tensor, a_rowidx: torch.Tensor, a_val: torch.Tensor,
@@ -574,7 +610,7 @@ def nnz_estimate(a_colptr: torch.Tensor, a_rowidx: torch.Tensor, a_val: torch.Te
     n2 = a_colptr.numel() - 1
     need = _SZ()
     _check(lib().cms_nnz_workspace_size(d, b_max, ctypes.byref(need)))
-    ws = alloc_workspace(need.value, a_colptr.device)
+    ws = _scratch(need.value, a_colptr.device, stream)
     b_out = _I64()
     k_out = _I64()
     _check(lib().cms_nnz_estimate(_ptr(a_colptr), _ptr(a_rowidx), _ptr(a_val), _ptr(b_rowptr), _ptr(b_colidx),
@@ -590,13 +626,13 @@ def frobenius_estimate(A: torch.Tensor, B: torch.Tensor, seed: int, d: int, stre
     n1, n2, n3, lda, ldb = _ab_args(A, B)
     need = _SZ()
     _check(lib().cms_frobenius_workspace_size(n1, n2, n3, d, ctypes.byref(need)))
-    ws = alloc_workspace(need.value, A.device)
-    est = torch.empty(d, dtype=torch.float64, device=A.device)
-    bound = torch.empty(1, dtype=torch.float64, device=A.device)
+    ws = _scratch(need.value, A.device, stream)
+    est = _empty(d, torch.float64, A.device, stream)
+    bound = _empty(1, torch.float64, A.device, stream)
     _check(lib().cms_frobenius_estimate(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, _DTYPES[A.dtype],
                                         seed & ((1 << 64) - 1), d, _ptr(est), _ptr(bound), _ptr(ws),
                                         ws.numel() * ws.element_size(), _stream(stream)))
-    return est, float(bound.item())
+    return est, float(_read(bound, stream))
 
 
 def merge(parts: list[torch.Tensor], out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
@@ -610,7 +646,7 @@ def merge(parts: list[torch.Tensor], out: torch.Tensor | None = None, stream=Non
             raise ValueError("parts must share one (d, b) shape")
         _check_buf(p_, f"parts[{i}]", dev, torch.float32, d * b)
     if out is None:
-        out = torch.empty((d, b), dtype=torch.float32, device=dev)
+        out = _empty((d, b), torch.float32, dev, stream)
     _check_buf(out, "out", dev, torch.float32, d * b)
     arr = (ctypes.c_void_p * len(parts))(*[p.data_ptr() for p in parts])
     _check(lib().cms_merge(arr, len(parts), d, b, _ptr(out), _stream(stream)))

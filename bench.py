@@ -37,8 +37,9 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_sketch_ws_covariance.json")
 # the fused sketch kernels' profiling names: warp-specialised, lock-step,
 # shared-memory (generic)
 SKETCH_KERNEL_NAMES = ("k_sketch_ws", "k_sketch_fast", "k_sketch_fused")
+REDUCTIONS_GS = 205.0    # random 64-bit reductions a second, in G, that L2 takes
 # the direct route's kernels (tensor-core tiles of AB added to the buckets)
-DIRECT_KERNEL_NAMES = ("k_direct_pack", "k_direct_tile", "k_direct_grid", "k_direct_window", "k_direct_finish",
+DIRECT_KERNEL_NAMES = ("k_direct_balance", "k_direct_pack", "k_direct_tile", "k_direct_grid", "k_direct_window", "k_direct_finish",
                        "k_pre_transpose", "k_pre_lists", "k_pre_pack")
 # the sources of the transform route's kernel and its launch: the kernel itself,
 # its helpers, the planner that shapes its launch and the table builder whose
@@ -66,9 +67,11 @@ def total_flops(d: int, K: int, b: int) -> float:
 
 def sketch_roofline(prof: dict, m: int, n: int, b: int, d: int, alu_peak: float) -> dict:
     """Roofline of one product X^T X's kernels as profiled.  The direct route's
-    kernels together against the tensor cores: the products of the symmetric
-    matrix's distinct entries, m n (n + 1) flops, at the measured BF16 rate.
-    The transform route's fused kernel against the FP32 pipe."""
+    kernels together against the additions into the buckets, d n^2 random 64-bit
+    reductions at the rate that they reach alone, which bound them; beside it the
+    products of the symmetric matrix's distinct entries, m n (n + 1) flops, against
+    the measured BF16 rate of the tensor cores.  The transform route's fused kernel
+    against the FP32 pipe."""
     direct = [k for k in DIRECT_KERNEL_NAMES if prof.get(k, {}).get("launches", 0) > 0]
     if direct:
         ms = sum(prof[k]["ms"] / prof[k]["launches"] for k in direct)
@@ -81,9 +84,13 @@ def sketch_roofline(prof: dict, m: int, n: int, b: int, d: int, alu_peak: float)
         peak = peaks.get("bf16_tflops", 1900.0)
         flops = float(m) * n * (n + 1)
         achieved = flops / (ms * 1e-3) / 1e12
-        return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": None, "kernel": " + ".join(direct), "kernel_ms": ms, "alg_flops_per_launch": flops,
-                "peak_source": "measured cuBLAS BF16 burst" if "bf16_tflops" in peaks else "fallback"}
+        adds = float(d) * n * n / (ms * 1e-3) / 1e9
+        return {"bound": "l2_reductions", "achieved": adds, "peak": REDUCTIONS_GS, "unit": "Gadd/s",
+                "frac": adds / REDUCTIONS_GS, "traffic": None, "kernel": " + ".join(direct), "kernel_ms": ms,
+                "alg_flops_per_launch": flops,
+                "peak_source": "measured: random 64-bit integer reductions into L2, whole chip",
+                "tensor": {"achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                           "peak_source": "measured cuBLAS BF16 burst" if "bf16_tflops" in peaks else "fallback"}}
     name = next((k for k in SKETCH_KERNEL_NAMES if prof.get(k, {}).get("launches", 0) > 0), "k_sketch_ws")
     fused = prof.get(name, {"launches": 0, "ms": float("nan")})
     ms = fused["ms"] / max(fused["launches"], 1)

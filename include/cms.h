@@ -199,8 +199,9 @@ CMS_API cms_status cms_plan_kernel(const void* A, int64_t lda, const void* B, in
  *              over k (compensated FP32), then one inverse FFT per repetition;
  *   direct     where b is not much smaller than n1 n3: the entries of AB
  *              from tensor-core tiles, each added to its bucket of every
- *              repetition as the tile leaves the accumulators (integer sums,
- *              so their order does not matter); AB is not stored.
+ *              repetition as the tile leaves the accumulators, or from the
+ *              workspace (integer sums, so their order does not matter); at most
+ *              16.8 M entries of AB are stored at a time.
  * Either gives the same bits in every run.  An infinity or a NaN in A or B
  * makes c NaN.
  *   A   : n1 x n2, column-major, column k at A + k*lda (lda >= n1), so a
@@ -370,7 +371,8 @@ CMS_API cms_status cms_batch_run(cms_batch* b, void* stream);
 CMS_API cms_status cms_batch_run_graph(cms_batch* b, void* stream);
 
 /* Counts of instances, persistent-kernel tasks, kernel launches per run,
- * workspace bytes and instances served by the C = 1024 kernel (any NULL). */
+ * workspace bytes and instances that the register-FFT body serves or would
+ * serve on the transform route (any NULL). */
 CMS_API cms_status cms_batch_info(const cms_batch* b, int32_t* instances, int32_t* tasks,
                                   int32_t* launches, size_t* ws_bytes, int32_t* fast_instances);
 

@@ -327,7 +327,9 @@ KERNEL_NAMES = {0: "shared_memory", 1: "lockstep", 2: "lockstep_tmem", 3: "warp_
 
 
 def plan_kernel(A: torch.Tensor, B: torch.Tensor, h: Hashes) -> str:
-    """The fused kernel sketch_product(A, B, h) would run (see KERNEL_NAMES)."""
+    """The fused kernel of sketch_product(A, B, h) on the transform route (see
+    KERNEL_NAMES).  Which route a call took shows in profile_summary()
+    ("k_direct_tile": the direct route)."""
     n1, n2, n3, lda, ldb = _ab_args(A, B)
     out = _I32()
     _check(lib().cms_plan_kernel(_ptr(A), lda, _ptr(B), ldb, n1, n2, n3, _DTYPES[A.dtype], h.handle,

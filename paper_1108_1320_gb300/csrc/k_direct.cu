@@ -1,7 +1,8 @@
 // k_direct.cu - the sketch from the product's entries, for sketches that are
 // long beside n1 n3: tensor-core tiles of AB whose entries are added to the
 // buckets (h1(i) + h2(j)) mod b of every repetition as they leave the
-// accumulators.  AB itself is never stored.
+// accumulators, or from a buffer of entries: all of them up to 16.8 M, bands of
+// rows for FINDSIGNIFICANTENTRIES.
 //
 // Sec. 2.2 forms c from the spectra of the columns of A and rows of B, d n2
 // transforms of length b.  By the same identity c_t[z] is the signed sum of
@@ -22,7 +23,8 @@
 //    cores.  Entries are scaled to 64-bit integers and added to the buckets
 //    with integer reductions: the order of the additions does not matter, so
 //    the sketch is the same in every run.  Its scatter warps add them while the
-//    next tile is multiplied, or the entries are stored (at most 16.8 M) and
+//    next tile is multiplied, or the entries are stored (at most 16.8 M of a
+//    product) and
 //    k_direct_grid or k_direct_window adds them with the whole chip: a tile's
 //    additions take an SM 12 us a repetition, so that a last wave of few tiles
 //    would wait for them (2265 x 2265 x 503, d = 7: 318 us fused, 24 + 197 us
@@ -35,8 +37,9 @@
 // 32768 BF16, b = 2^20, d = 7 834 -> 50.6 ms; 64 uneven products of n = 512 ..
 // 8192, b = 16 n, d = 3 416 -> 25.2 ms.  What bounds it: the additions into
 // the buckets (random 64-bit reductions run at 205 G/s on the whole chip, one
-// 32-byte sector each), then shared memory, which the operands' copies and the
-// tensor cores' reads of them share (about 110 bytes per clock and SM).
+// 32-byte sector each: 36.7 of the large product's 51 ms), then shared memory,
+// which the operands' copies and the tensor cores' reads of them share (about 110
+// bytes per clock and SM).
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -749,7 +752,8 @@ __device__ __forceinline__ uint32_t window_byte(uint32_t z4) { return z4 ^ ((z4 
 // reductions a second and SM: 4096 x 4096 entries, d = 3, b = 2^16 (44% of the
 // buckets in the window) 228 -> 175 us; 1500 x 1500, d = 5, b = 30000 (all but
 // 4%) 78 -> 45 us, 30 clocks for a warp's 32 additions, most of them latency.
-// Three windows a repetition, every entry read for each: 279 us of the 228.
+// Three windows a repetition, every entry read for each, took 279 us where one
+// takes 175.
 __global__ void __launch_bounds__(1024, 1) k_direct_window(const GridArgs p, int shares) {
   extern __shared__ uint32_t words[];        // low halves, then high halves
   next_kernel_may_start();
@@ -935,7 +939,10 @@ namespace {
 //         (twice the units, where tiles are few);
 //  splits of the inner dimension while SMs have no unit;
 //  grid   entries stored for a launch of its own (additions from every SM,
-//         about 6 us more), or added by the tile kernel while it multiplies on.
+//         about 6 us more; at most 16.8 M, 64 MB of scratch: above that it would
+//         still pay where most buckets are in the window, 4500 x 4500, K = 4000,
+//         b = 30000, d = 5 FP32 560 us against 785, and not elsewhere, 8192 x 8192,
+//         b = 2^17 2186 against 2008), or added by the tile kernel while it multiplies on.
 // Times: a chunk of 64 (FP16 terms) or 128 (BF16) inner indices of a tile
 // 0.40 us (BF16 alone on its operands 0.53: the copies from L2 bound it), and
 // more where the packed operands (`packed` bytes) do not stay in L2: 2.0 times as

@@ -94,7 +94,7 @@ def milliseconds(cms, data, n, h, pairs):
         e[1].record()
         e[1].synchronize()
         out.append(e[0].elapsed_time(e[1]))
-    return sorted(out[2:])[2]
+    return min(out[2:])
 
 
 def test_time_follows_the_terms_not_their_shape(cms):

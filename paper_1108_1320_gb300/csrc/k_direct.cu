@@ -1161,8 +1161,13 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
   }
   // a margin for the estimates' error: where both are mostly launches, and a
   // fourth beyond L2, where 5 of 200 calls of other sizes than the fitted ones
-  // were up to 1.33 slower by the chosen route without it
-  return best * (out->beyond_l2 ? 1.25 : 1.0) + (batch ? 0.0 : kMargin) < transform;
+  // were up to 1.33 slower by the chosen route without it.  In a batch the other
+  // way round with several repetitions: its transform body takes up to 2.6 times
+  // as long as the single call's there (6827 x 58270 FP32, b = 2592, d = 3: 10.9 ms
+  // an instance, 8.1 by the tiles), with one as long (5022 x 19702, b = 3125, d = 1:
+  // 1.03 and 1.69)
+  const double beyond = !out->beyond_l2 ? 1.0 : !batch ? 1.25 : h->d > 1 ? 1.0 / 1.2 : 1.0;
+  return best * beyond + (batch ? 0.0 : kMargin) < transform;
 }
 
 // The masked sums of FINDSIGNIFICANTENTRIES in one pass: an entry is added to

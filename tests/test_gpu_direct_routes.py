@@ -193,3 +193,22 @@ def test_tuned_route_of_a_batch_knows_aliased_operands(cms, tmp_path):
     again.free()
     for h in hs:
         h.free()
+
+
+# long inner dimensions in a batch, packed operands beyond L2 (ms an instance by the
+# tiles, by the spectra)
+@pytest.mark.parametrize("n,m,b,d,dts,direct", [
+    (8975, 30000, 2592, 2, "bf16", True),       # 3.74, 5.79
+    (2001, 28282, 1350, 2, "bf16", True),       # 0.30, 0.91
+    (5022, 19702, 3125, 1, "f32", False),       # 1.69, 1.03
+    (4096, 8192, 4096, 1, "f32", False),        # 0.46, 0.34
+])
+def test_long_inner_dimensions_of_a_batch(cms, n, m, b, d, dts, direct):
+    x = torch.randn((m, n), device="cuda").to(DT[dts])
+    hs = [cms.make_hashes(q, n, b, d) for q in range(2)]
+    batch = cms.Batch([(x.T, x, h) for h in hs])
+    _, kernels = kernels_of(cms, batch.run)
+    assert ("k_direct_tile_batched" in kernels) == direct
+    batch.free()
+    for h in hs:
+        h.free()

@@ -1024,16 +1024,30 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
   const int64_t images = (n2 + per - 1) / per;
   const double entries = static_cast<double>(n1) * static_cast<double>(n3);
   const double packed = static_cast<double>(p.tiles1 + (alias ? 0 : p.tiles3)) * static_cast<double>(images) * kStageBytes;
-  choose_tiles(p, alias, 1, entries, 0.5 * h->d * (sets + 1), 2.05e11, 1.35e9,
-               sets == 1 ? std::min(1.0, static_cast<double>(kWindow) / static_cast<double>(h->b)) : 0.0, packed,
-               !batch && (sets > 1 || entries <= 16.8e6), sets == 1, batch, sms);
+  const int64_t words = static_cast<int64_t>(h->d) * h->b;
+  auto choose = [&](DirectPlan& q, double rate) {
+    choose_tiles(q, alias, 1, entries, 0.5 * h->d * (sets + 1), rate, 1.35e9,
+                 sets == 1 ? std::min(1.0, static_cast<double>(kWindow) / static_cast<double>(h->b)) : 0.0, packed,
+                 !batch && (sets > 1 || entries <= 16.8e6), sets == 1, batch, sms);
+  };
+  choose(p, 2.05e11);
+  // reductions to few words queue up (see sum_copies), and a batch has at most
+  // four copies: few splits of the inner dimension there, each of which adds its
+  // own share (242 x 6456 BF16, b = 64, d = 1: 89 us an instance with the splits for
+  // the full rate, 42 by the spectra, 12 so).  The estimate stays the full rate's,
+  // which the choice of route was fitted with.
+  const double rate = 2.3e10 * std::pow(4.0 * static_cast<double>(words) / 1024.0, 0.53);
+  if (batch && rate < 2.05e11) {
+    const double seconds = p.seconds;
+    choose(p, rate);
+    p.seconds = seconds;
+  }
   // large operands: read (twice where their inner indices are balanced) and
   // packed at 5 TB/s; small ones are in the fixed part
   if (p.beyond_l2) {
     const double values = static_cast<double>(alias ? n1 : n1 + n3) * static_cast<double>(n2);
     p.seconds += (values * (dt == CMS_F64 ? 8.0 : dt == CMS_BF16 ? 2.0 : 4.0) * (alias ? 1.0 : 2.0) + packed) / 5e12;
   }
-  const int64_t words = static_cast<int64_t>(h->d) * h->b;
   // (a batch's products queue up less: others' additions are under way too)
   p.copies = sets > 1 ? 1 : sum_copies(words, static_cast<int64_t>(p.units) * p.splits);
   if (batch) p.copies = std::min(p.copies, 4);

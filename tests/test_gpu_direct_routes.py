@@ -212,3 +212,37 @@ def test_long_inner_dimensions_of_a_batch(cms, n, m, b, d, dts, direct):
     batch.free()
     for h in hs:
         h.free()
+
+
+def test_short_sketches_of_a_batch_split_little(cms, tmp_path):
+    # additions to few buckets queue up: with the inner dimension split for the full
+    # rate the tiles took 89 us an instance where the spectra take 42, now 12
+    n, m, b = 242, 6456, 64
+    xs = [torch.randn((m, n), device="cuda").bfloat16() for _ in range(8)]
+    hs = [cms.make_hashes(q, n, b, 1) for q in range(8)]
+    items = [(x.T, x, h) for x, h in zip(xs, hs)]
+    cache = tmp_path / "tune.txt"
+    cms.Batch(items, autotune=True, tune_cache=str(cache)).free()
+    key = [ln.split()[0] for ln in cache.read_text().splitlines() if "kernel=direct" in ln][0]
+    best, outs = [], []
+    for chunks in (0, 64):                  # the tiles, the spectra
+        cache.write_text(f"{key} {chunks} 0 1.0\n")
+        batch = cms.Batch(items, tune_cache=str(cache))
+        out, kernels = kernels_of(cms, batch.run)
+        assert ("k_direct_tile_batched" in kernels) == (chunks == 0)
+        outs.append([c.clone() for c in out])
+        times = []
+        for _ in range(8):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            batch.run()
+            e[1].record()
+            e[1].synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        best.append(min(times))
+        batch.free()
+    assert best[0] < best[1]
+    for c, w in zip(*outs):
+        assert ((c - w).norm() / w.norm()).item() < 1e-5
+    for h in hs:
+        h.free()

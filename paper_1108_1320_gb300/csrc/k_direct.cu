@@ -1082,7 +1082,10 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
 // conventional 5 b log2 b + 4 b flops per repetition and inner index, and the
 // gathers of its front end (every entry of a_k and b_k for each computed row),
 // at rates fitted per kernel family to 160 calls of n = 64 .. 16384, b = n / 8
-// .. 32 n, 64 to 8192 inner indices (n = 454, K = 142, b = 810, d = 4 BF16:
+// .. 32 n, 64 to 8192 inner indices.  Of 1330 calls of n = 8 .. 17000, b = 2 .. 400 n,
+// 64 to 2 M inner indices, every storage type, 7 are slower by the chosen route than
+// by the spectra by more than 8%, at most by 1.37 (4667 x 14591 x 4018 FP32, b = 600, d
+// = 1: 0.76 and 0.56 ms) (n = 454, K = 142, b = 810, d = 4 BF16:
 // 96 us by the spectra, 44 us this way; n = 6746, K = 184, b = 1620, d = 4 the
 // other way round: 160 and 1136 us).
 static double transform_seconds(const SketchPlan& p, int64_t n1, int64_t n2, int64_t n3, bool batch) {
@@ -1113,6 +1116,7 @@ PrePlan make_pre_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, b
   q.classes = kTile / q.R;
   q.tiles = (q.C + q.classes - 1) / q.classes;
   if (q.tiles > 128) return q;    // b above about 16384 is never cheap
+  if (h->b < 64) return q;        // nor is a tile with few rows (5120 x 415, b = 27, d = 3: 325 us, 175 by the spectra)
   const int64_t rows = static_cast<int64_t>(q.tiles) * kTile;
   DirectPlan& p = q.direct;
   p.split = true;
@@ -1121,10 +1125,15 @@ PrePlan make_pre_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t n3, b
   const double packed = 2.0 * static_cast<double>(rows) * static_cast<double>(n2) * 4.0 * h->d;
   choose_tiles(p, false, h->d, static_cast<double>(rows) * rows, 1.0, 5.0e11, 4e9, 0.0, packed, false, true, false, sms);
   const double n = static_cast<double>(alias ? n1 : n1 + n3), k = static_cast<double>(p.nsb) * kSuper;
-  p.seconds += 14e-6 + n * k * 8.0 / 4e12 + static_cast<double>(n1 + n3) * k * h->d * 4.0 / 5e12 +
+  // sums of rows: 5 TB/s together, 24 GB/s a block of which 304 run at a time
+  // (10847 x 947 x 5263 BF16, b = 128, d = 1: 16 blocks, 0.33 ms, 0.18 by the spectra)
+  const double blocks = 2.0 * p.nsb * q.tiles * h->d;
+  const double sums = std::max(static_cast<double>(n1 + n3) * k * h->d * 4.0 / 5e12,
+                               static_cast<double>(std::max(n1, n3)) * 512.0 / q.tiles * std::max(1.0, blocks / 304.0) / 2.4e10);
+  p.seconds += 14e-6 + n * k * 8.0 / 4e12 + sums +
               2.0 * static_cast<double>(rows) * k * h->d * 4.0 / 3e12;
   // (beyond L2 the measured times were 1.0 to 1.5 of the rest)
-  if (p.beyond_l2) p.seconds = 1.2 * (p.seconds + (alias ? 0.0 : n * k * 4.0 / 5e12));
+  if (p.beyond_l2) p.seconds = 1.1 * (p.seconds + (alias ? 0.0 : n * k * 4.0 / 5e12));
   const int64_t words = static_cast<int64_t>(h->d) * h->b;
   p.copies = sum_copies(words, static_cast<int64_t>(p.units) * p.splits);
   const int64_t images = (n2 + 31) / 32;
@@ -1174,13 +1183,11 @@ bool choose_direct(const cms_hashes* h, const SketchPlan& plan, int64_t n1, int6
     }
   }
   // a margin for the estimates' error: where both are mostly launches, and a
-  // fourth beyond L2, where 5 of 200 calls of other sizes than the fitted ones
-  // were up to 1.33 slower by the chosen route without it.  In a batch the other
-  // way round with several repetitions: its transform body takes up to 2.6 times
-  // as long as the single call's there (6827 x 58270 FP32, b = 2592, d = 3: 10.9 ms
-  // an instance, 8.1 by the tiles), with one as long (5022 x 19702, b = 3125, d = 1:
-  // 1.03 and 1.69)
-  const double beyond = !out->beyond_l2 ? 1.0 : !batch ? 1.25 : h->d > 1 ? 1.0 / 1.2 : 1.0;
+  // tenth beyond L2.  In a batch the other way round there with several
+  // repetitions: its transform body takes up to 2.6 times as long as the single
+  // call's (6827 x 58270 FP32, b = 2592, d = 3: 10.9 ms an instance, 8.1 by the tiles),
+  // with one as long (5022 x 19702, b = 3125, d = 1: 1.03 and 1.69).
+  const double beyond = !out->beyond_l2 ? 1.0 : !batch ? 1.1 : h->d > 1 ? 1.0 / 1.2 : 1.0;
   return best * beyond + (batch ? 0.0 : kMargin) < transform;
 }
 

@@ -246,3 +246,19 @@ def test_short_sketches_of_a_batch_split_little(cms, tmp_path):
         assert ((c - w).norm() / w.norm()).item() < 1e-5
     for h in hs:
         h.free()
+
+
+# few buckets or few inner indices: pre-sketched operands have few blocks to sum them
+# in, or tiles with few rows (ms by them, by the spectra)
+@pytest.mark.parametrize("n1,n2,n3,b,d,dts,alias", [
+    (10847, 947, 5263, 128, 1, "bf16", False),      # 0.33, 0.18
+    (11552, 535, 11552, 144, 1, "bf16", True),      # 0.21, 0.16
+    (5120, 415, 5120, 27, 3, "f64", True),          # 0.32, 0.18
+])
+def test_pre_sketched_operands_need_blocks_to_sum_in(cms, n1, n2, n3, b, d, dts, alias):
+    x = torch.randn((n2, n1), device="cuda").to(DT[dts])
+    y = x if alias else torch.randn((n2, n3), device="cuda").to(DT[dts])
+    h = cms.make_hashes(1, max(n1, n3), b, d)
+    _, kernels = kernels_of(cms, lambda: cms.sketch_product(x.T, y, h))
+    assert "k_pre_pack" not in kernels and "k_direct_tile" not in kernels
+    h.free()

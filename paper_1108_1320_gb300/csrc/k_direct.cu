@@ -1031,13 +1031,14 @@ DirectPlan make_direct_plan(const cms_hashes* h, int64_t n1, int64_t n2, int64_t
                  !batch && (sets > 1 || entries <= 16.8e6), sets == 1, batch, sms);
   };
   choose(p, 2.05e11);
-  // reductions to few words queue up (see sum_copies), and a batch has at most
-  // four copies: few splits of the inner dimension there, each of which adds its
-  // own share (242 x 6456 BF16, b = 64, d = 1: 89 us an instance with the splits for
-  // the full rate, 42 by the spectra, 12 so).  The estimate stays the full rate's,
+  // reductions to few words queue up (see sum_copies), where each split of the
+  // inner dimension adds its own share: few splits there.  A batch has at most four
+  // copies: 242 x 6456 BF16, b = 64, d = 1 took 89 us an instance with the splits for
+  // the full rate, 42 by the spectra, 12 so.  The estimate stays the full rate's,
   // which the choice of route was fitted with.
-  const double rate = 2.3e10 * std::pow(4.0 * static_cast<double>(words) / 1024.0, 0.53);
-  if (batch && rate < 2.05e11) {
+  const double spread = (batch ? 4.0 : sets > 1 ? 1e9 : 256.0) * static_cast<double>(words) / 1024.0;
+  const double rate = 2.3e10 * std::pow(spread, 0.53);
+  if (rate < 2.05e11) {
     const double seconds = p.seconds;
     choose(p, rate);
     p.seconds = seconds;

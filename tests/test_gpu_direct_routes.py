@@ -262,3 +262,30 @@ def test_pre_sketched_operands_need_blocks_to_sum_in(cms, n1, n2, n3, b, d, dts,
     _, kernels = kernels_of(cms, lambda: cms.sketch_product(x.T, y, h))
     assert "k_pre_pack" not in kernels and "k_direct_tile" not in kernels
     h.free()
+
+
+def test_shortest_sketches_split_little(cms):
+    # three buckets: 64 parts of the inner dimension would each add their own share
+    # to them (0.52 ms, 0.33 by the spectra)
+    n1, n2, n3, b = 362, 35456, 209, 3
+    x, y = torch.randn((n2, n1), device="cuda"), torch.randn((n2, n3), device="cuda")
+    h = cms.make_hashes(1, n1, b, 1)
+    least = cms.alloc_workspace(cms.workspace_size(h, n1, n2, n3, smallest=True))
+    room = cms.alloc_workspace(cms.workspace_size(h, n1, n2, n3))
+    want, kernels = kernels_of(cms, lambda: cms.sketch_product(x.T, y, h, ws=least))
+    assert "k_direct_tile" not in kernels
+    got, kernels = kernels_of(cms, lambda: cms.sketch_product(x.T, y, h, ws=room))
+    assert ((got - want).norm() / want.norm()).item() < 1e-5
+    best = []
+    for ws in (room, least):
+        times = []
+        for _ in range(10):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            cms.sketch_product(x.T, y, h, ws=ws)
+            e[1].record()
+            e[1].synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        best.append(min(times))
+    assert best[0] < 1.15 * best[1]
+    h.free()

@@ -494,7 +494,7 @@ cms_status sparse_product(const char* name, const int64_t* a_colptr, const int32
   e = launch_twiddle_tables(twC, static_cast<int>(plan.C), twR, static_cast<int>(plan.R), s, counts);
   if (e == cudaSuccess) e = launch_sketch_sparse(plan, h, in, dt, flist, counts, 1, partial, s);
   if (e == cudaSuccess) e = launch_inverse(plan, partial, V, twC, twR, c, s, counts);
-  if (e == cudaSuccess) e = launch_direct_scatter(h, in, dt, integer, dlist, counts, n2, cd, s);
+  if (e == cudaSuccess) e = launch_direct_scatter(h, in, dt, integer, limit, dlist, counts, n2, cd, s);
   if (e == cudaSuccess) e = launch_add_direct(h, c, cd, integer, counts, s);
   if (e != cudaSuccess) return cuda_fail(e, name);
   return CMS_OK;

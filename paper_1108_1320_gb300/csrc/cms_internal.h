@@ -267,7 +267,7 @@ cudaError_t launch_nonempty_split(const cms_hashes* h, const SparseArgsHost& in,
 // The direct list's length is read on the device (counts[1]); dlist has n2 places.
 // integer: sums of integers at a common scale (the same in any order), else
 // FP64 sums.
-cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer,
+cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer, int64_t limit,
                                   const int32_t* dlist, const int32_t* counts, int64_t n2, double* cd, cudaStream_t s);
 cudaError_t launch_add_direct(const cms_hashes* h, float* c, double* cd, int integer, const int32_t* counts,
                               cudaStream_t s);

@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "cms_internal.h"
+#include "direct_tile.cuh"
 #include "warp_fft.cuh"
 
 namespace cms {
@@ -571,40 +572,65 @@ __device__ __forceinline__ Piece piece_of(int64_t na, int64_t nb) {
   return q;
 }
 
-template <typename T, bool INT>
-__global__ void __launch_bounds__(256)
-k_direct_scatter(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ a_idx, const T* __restrict__ a_val,
-                 const int64_t* __restrict__ b_ptr, const int32_t* __restrict__ b_idx, const T* __restrict__ b_val,
-                 int n1, int n3, int64_t n, int64_t n2, const int32_t* __restrict__ dlist,
-                 const int32_t* __restrict__ counts, const uint32_t* __restrict__ hs, int d, int64_t b,
-                 double* __restrict__ cd, const DirectTerms* __restrict__ terms) {
+struct ScatterArgs {
+  const int64_t* a_ptr;
+  const int32_t* a_idx;
+  const void* a_val;
+  const int64_t* b_ptr;
+  const int32_t* b_idx;
+  const void* b_val;
+  int n1, n3;
+  int64_t n, n2;
+  const int32_t* dlist;
+  const int32_t* counts;
+  const uint32_t* hs;
+  int d;
+  int64_t b;
+  double* cd;
+  const DirectTerms* terms;
+};
+
+template <typename T, bool INT, bool HEAVY>
+__device__ __forceinline__ void scatter(const ScatterArgs& p) {
+  const int64_t* __restrict__ a_ptr = p.a_ptr;
+  const int64_t* __restrict__ b_ptr = p.b_ptr;
+  const int32_t* __restrict__ a_idx = p.a_idx;
+  const int32_t* __restrict__ b_idx = p.b_idx;
+  const T* __restrict__ a_val = static_cast<const T*>(p.a_val);
+  const T* __restrict__ b_val = static_cast<const T*>(p.b_val);
+  const int32_t* __restrict__ dlist = p.dlist;
+  const uint32_t* __restrict__ hs = p.hs;
+  const DirectTerms* __restrict__ terms = p.terms;
+  double* __restrict__ cd = p.cd;
+  const int n1 = p.n1, n3 = p.n3, d = p.d;
+  const int64_t n = p.n, n2 = p.n2, b = p.b;
   __shared__ double val[kDirN];            // A's nonzeros, then B's
   __shared__ int pos[kDirN];
   __shared__ uint32_t hash[kDirT][kDirN];
-  const int Kd = counts[1], Kh = static_cast<int>(terms->heavy);
+  const int count = HEAVY ? static_cast<int>(terms->heavy) : p.counts[1];
   const int tid = threadIdx.x;
   double up = 1.0;
   if (INT) {
-    if (Kd + Kh == 0 || terms->max_bits >= 0x7F800000u) return;   // the conversion writes NaN
+    if (count == 0 || terms->max_bits >= 0x7F800000u) return;   // the conversion writes NaN
     up = ldexp(1.0, term_shift(*terms));
   }
   int q = blockIdx.x;                      // place in the list
   int64_t ca = 0, cb = 0;                  // nonzeros of the piece's corner
-  __shared__ long long last[256], part[8];   // of 256 heavy ones: pieces up to each
+  __shared__ long long last[HEAVY ? 256 : 1], part[8];   // of 256 heavy ones: pieces up to each
   int h0 = -256;
   long long c = 0, total = 0, turn = 0;    // this block's next piece, pieces of these 256, and before them
   for (;;) {
-    const bool light = q < Kd;
     int64_t k;
-    if (light) {
+    if constexpr (!HEAVY) {
+      if (q >= count) return;
       k = dlist[q];
     } else {
       while (c >= total) {
         turn += total;
         h0 += 256;
-        if (h0 >= Kh) return;
+        if (h0 >= count) return;
         long long pieces = 0;
-        if (h0 + tid < Kh) {
+        if (h0 + tid < count) {
           const int64_t kk = dlist[n2 - 1 - (h0 + tid)];
           const int64_t na = a_ptr[kk + 1] - a_ptr[kk], nb = b_ptr[kk + 1] - b_ptr[kk];
           const Piece pc = piece_of(na, nb);
@@ -636,7 +662,7 @@ k_direct_scatter(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ 
     const int64_t a0 = a_ptr[k], na = a_ptr[k + 1] - a0;
     const int64_t b0 = b_ptr[k], nb = b_ptr[k + 1] - b0;
     const Piece pc = piece_of(na, nb);
-    if (!light) {
+    if constexpr (HEAVY) {
       const int64_t per = (nb + pc.b - 1) / pc.b, x = ca;
       ca = x / per * pc.a;
       cb = x % per * pc.b;
@@ -683,7 +709,7 @@ k_direct_scatter(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ 
         }
       }
     }
-    if (!light) {
+    if constexpr (HEAVY) {
       c += gridDim.x;
     } else if ((cb += pc.b) >= nb) {
       cb = 0;
@@ -693,6 +719,19 @@ k_direct_scatter(const int64_t* __restrict__ a_ptr, const int32_t* __restrict__ 
       }
     }
   }
+}
+
+// The list, and beside it (a programmatic launch, where inner indices may be that
+// long) the heavy ones: in one kernel their code cost the list's 2 to 3 us of 37.
+template <typename T, bool INT>
+__global__ void __launch_bounds__(256) k_direct_scatter(const ScatterArgs p) {
+  dtile::next_kernel_may_start();
+  scatter<T, INT, false>(p);
+}
+template <typename T, bool INT>
+__global__ void __launch_bounds__(256) k_direct_scatter_heavy(const ScatterArgs p) {
+  scatter<T, INT, true>(p);
+  dtile::wait_for_kernel_before();   // this kernel's end implies the list's
 }
 
 // c = FFT-route c + direct part (rounded once to FP32), or the direct part
@@ -821,18 +860,26 @@ cudaError_t launch_nonempty_split(const cms_hashes* h, const SparseArgsHost& in,
   return cudaGetLastError();
 }
 
-cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer,
+cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in, int dt, int integer, int64_t limit,
                                   const int32_t* dlist, const int32_t* counts, int64_t n2, double* cd, cudaStream_t s) {
   if (n2 <= 0) return cudaSuccess;
   // the lists' lengths are on the device: blocks stride over them, and return
-  // at once when they are empty
-  const unsigned grid = 152 * 8;
-  ProfScope prof_scope("k_direct_scatter", s);
+  // at once when they are empty (two waves of blocks: with one, those with two
+  // inner indices end last, 40.8 us for 2048 of them and 36.7 with two)
+  const ScatterArgs a{in.a_ptr, in.a_idx, in.a_val, in.b_ptr, in.b_idx, in.b_val, in.n1, in.n3, h->n, n2, dlist,
+                      counts, h->d_hs, h->d, h->b, cd, direct_terms(h, cd)};
+  cudaError_t e = cudaSuccess;
   auto go = [&](auto* tag, auto integer_tag) {
     using T = std::remove_pointer_t<decltype(tag)>;
-    k_direct_scatter<T, decltype(integer_tag)::value><<<grid, 256, 0, s>>>(
-        in.a_ptr, in.a_idx, static_cast<const T*>(in.a_val), in.b_ptr, in.b_idx, static_cast<const T*>(in.b_val),
-        in.n1, in.n3, h->n, n2, dlist, counts, h->d_hs, h->d, h->b, cd, direct_terms(h, cd));
+    constexpr bool kInt = decltype(integer_tag)::value;
+    {
+      ProfScope prof_scope("k_direct_scatter", s);
+      k_direct_scatter<T, kInt><<<static_cast<unsigned>(std::min<int64_t>(n2, 152 * 16)), 256, 0, s>>>(a);
+      e = cudaGetLastError();
+    }
+    if (e != cudaSuccess || limit <= kHeavyTerms) return;
+    ProfScope prof_scope("k_direct_scatter_heavy", s);
+    e = dtile::launch_after(k_direct_scatter_heavy<T, kInt>, dim3(152 * 4), 256, 0, s, a);
   };
   auto both = [&](auto* tag) {
     if (integer) go(tag, std::true_type{});
@@ -841,7 +888,7 @@ cudaError_t launch_direct_scatter(const cms_hashes* h, const SparseArgsHost& in,
   if (dt == CMS_F32) both(static_cast<float*>(nullptr));
   else if (dt == CMS_BF16) both(static_cast<__nv_bfloat16*>(nullptr));
   else both(static_cast<double*>(nullptr));
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_add_direct(const cms_hashes* h, float* c, double* cd, int integer, const int32_t* counts,
